@@ -21,19 +21,38 @@ static constexpr double kPiA = 3.14159265358979323846;
 
 // ---------------------------------------------------------------- kernels used here
 
-// Forces into sorted SoA; the FP32 form also keeps a single-precision copy.
-__global__ void k_gather_f(const double *f, const int *perm, int64_t n, double *fs, float *f32) {
-    int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t j = perm[i];
-    double fx = f[3 * j], fy = f[3 * j + 1], fz = f[3 * j + 2];
-    fs[i] = fx;
-    fs[n + i] = fy;
-    fs[2 * n + i] = fz;
-    if (f32) {
-        f32[i] = float(fx);
-        f32[n + i] = float(fy);
-        f32[2 * n + i] = float(fz);
+// Forces into sorted SoA; the FP32 form also keeps a single-precision copy, the FP64 form the largest component
+// of each system (the high word of its magnitude: NaN and infinity compare highest).
+__global__ void k_gather_f(const double *f, const int *perm, const int *bead_sys, int64_t n, double *fs, float *f32,
+                           int *fmax) {
+    __shared__ int smax;
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (threadIdx.x == 0) smax = 0;
+    int w = 0;
+    if (i < n) {
+        const int64_t j = perm[i];
+        const double fx = f[3 * j], fy = f[3 * j + 1], fz = f[3 * j + 2];
+        fs[i] = fx;
+        fs[n + i] = fy;
+        fs[2 * n + i] = fz;
+        if (f32) {
+            f32[i] = float(fx);
+            f32[n + i] = float(fy);
+            f32[2 * n + i] = float(fz);
+        }
+        w = max(max(__double2hiint(fx) & 0x7fffffff, __double2hiint(fy) & 0x7fffffff), __double2hiint(fz) & 0x7fffffff);
+    }
+    if (!fmax) return;
+    const int64_t b0 = int64_t(blockIdx.x) * blockDim.x, b1 = min(b0 + blockDim.x, n) - 1;
+    const int s0 = bead_sys[b0];
+    if (s0 == bead_sys[b1]) {   // one system in the block (beads are sorted by system)
+        __syncthreads();
+        w = __reduce_max_sync(0xffffffffu, w);
+        if ((threadIdx.x & 31) == 0) atomicMax(&smax, w);
+        __syncthreads();
+        if (threadIdx.x == 0 && smax > *(volatile int *)&fmax[s0]) atomicMax(&fmax[s0], smax);
+    } else if (i < n) {
+        atomicMax(&fmax[bead_sys[i]], w);
     }
 }
 
@@ -60,6 +79,18 @@ __global__ void k_pair_const(int nsys, const double *a_, const double *s_, const
     c.f_nco_c9 = float(-co_cf * 9.0 / (32.0 * a));
     c.f_co_c3 = float(co_cf * 3.0 / (32.0 * a));
     c.f_pad = 0.f;
+    const double xs = near_unit(cube[4 * k + 3]), ap = a * xs;
+    c.d_xs = xs;
+    c.d_ok = ap >= 0x1p-60 && ap <= 0x1p30;
+    auto split = [](double v, float &h, float &l) {
+        h = float(v);
+        l = float(v - double(h));
+    };
+    split(2.0 * ap * ap / 3.0, c.d_k23h, c.d_k23l);
+    split(4.0 / (3.0 * ap), c.d_c43h, c.d_c43l);
+    split(9.0 / (32.0 * ap), c.d_c9h, c.d_c9l);
+    split(1.0 / (8.0 * ap * ap), c.d_c8h, c.d_c8l);
+    c.d_lim = fmaxf(float(4.0 * ap * ap), kDfTiny2);
     pc[k] = c;
 }
 
@@ -339,6 +370,12 @@ static int alloc_tree_arrays(Tree &t, cudaStream_t st) {
     return RPY_OK;
 }
 
+static int alloc_near_f64(Tree &t) {
+    RPY_TRY(dev_alloc(t, (void **)&t.p3, sizeof(float) * 9 * t.n));
+    RPY_TRY(dev_alloc(t, (void **)&t.f2, sizeof(float) * 6 * t.n));
+    return dev_alloc(t, (void **)&t.sys_fmax, sizeof(int) * t.nsys);
+}
+
 int tree_alloc_workspace(Tree &t, cudaStream_t st) {
     const OpTables &h = *t.tabs;
     size_t es = t.params.precision == RPY_FP32 ? sizeof(cpx<float>) : sizeof(cpx<double>);
@@ -354,6 +391,8 @@ int tree_alloc_workspace(Tree &t, cudaStream_t st) {
         if (t.params.precision == RPY_FP32) {
             RPY_TRY(dev_alloc(t, (void **)&t.p32, sizeof(float) * 6 * t.n));
             RPY_TRY(dev_alloc(t, (void **)&t.f32, sizeof(float) * 3 * t.n));
+        } else {
+            RPY_TRY(alloc_near_f64(t));
         }
         RPY_TRY(dev_alloc(t, (void **)&t.u_near, sizeof(double) * 3 * t.n));
         RPY_TRY(dev_alloc(t, (void **)&t.u_far, sizeof(double) * 3 * t.n));
@@ -376,6 +415,8 @@ int tree_alloc_workspace(Tree &t, cudaStream_t st) {
     if (t.params.precision == RPY_FP32) {
         RPY_TRY(dev_alloc(t, (void **)&t.p32, sizeof(float) * 6 * t.n));
         RPY_TRY(dev_alloc(t, (void **)&t.f32, sizeof(float) * 3 * t.n));
+    } else {
+        RPY_TRY(alloc_near_f64(t));
     }
     RPY_TRY(dev_alloc(t, (void **)&t.u_near, sizeof(double) * 3 * t.n));
     RPY_TRY(dev_alloc(t, (void **)&t.u_far, sizeof(double) * 3 * t.n));
@@ -397,6 +438,7 @@ static int do_build(Tree &t, const double *pos_dev, cudaStream_t st) {
     t.dt32 = ds->d32;
     RPY_TRY(tree_alloc_workspace(t, st));
     if (t.params.precision == RPY_FP32) RPY_TRY(split_positions_f32(t, st));
+    else RPY_TRY(split_positions_f64(t, st));
     RPY_CHECK(cudaStreamSynchronize(st));
     mark_done(t, st);
     t.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -492,9 +534,11 @@ int run_matvec(Tree &t, const double *f_dev, const double *s_host, double *u_dev
     SysConst sc{t.sys_cube, t.sys_a, t.sys_s, t.sys_pc};
     t.n_marks = 0;
     prof_mark(t, RPY_STAGE_GATHER, st);
-    k_gather_f<<<nb256(t.n), 256, 0, st>>>(f_dev, t.perm, t.n, t.fs, t.f32);
+    if (t.sys_fmax) RPY_CHECK(cudaMemsetAsync(t.sys_fmax, 0, sizeof(int) * t.nsys, st));
+    k_gather_f<<<nb256(t.n), 256, 0, st>>>(f_dev, t.perm, t.bead_sys, t.n, t.fs, t.f32, t.sys_fmax);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
+    if (t.f2) RPY_TRY(split_forces_f64(t, st));
     bool graph = parts == RPY_PART_ALL && !t.prof && !(t.params.flags & RPY_FLAG_NO_GRAPH) && t.matvecs >= 1;
     if (graph && !t.gexec) RPY_TRY(capture_graph(t, sc));
     if (graph) {
@@ -947,7 +991,7 @@ int rpy_tree_footprint(int64_t n, int digits, int precision, int leaf_cap, int64
     double per_box = es * (2.0 * kSets * ncoef(p) + 2.0 * 2 * xf * kSets * q.half() + 18.0 * ncoef(p) + m2m) +
                      4.0 * (8 + 27 + 3 + 12) + 32.0;
     double per_bead = 3 * 8 /*pos*/ + 8 /*key*/ + 4 + 4 + 9 * 8 /*fs, unear, ufar*/ + 27 * 4 /*U list share*/ +
-                      (precision == RPY_FP32 ? 9 * 4 /*p32, f32*/ : 0);
+                      (precision == RPY_FP32 ? 9 * 4 /*p32, f32*/ : 15 * 4 /*p3, f2*/);
     *bytes = int64_t(nbox * per_box + double(n) * per_bead + 32.0 * 1024 * 1024);
     return RPY_OK;
 }

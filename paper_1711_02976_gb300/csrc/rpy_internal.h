@@ -187,7 +187,32 @@ struct PairConst {
     double C1, C2, icube;         // C1 = s/(8 pi), C2 = s a^2/(12 pi), 1/(side of the root cube)
     float f_a2x4, f_tiny2, f_k23, f_nk2;   // FP32 copies; tiny2 = 1e-6 a^2
     float f_co_cf, f_nco_c9, f_co_c3, f_pad;   // co/cf, -(co/cf) 9/(32a), (co/cf) 3/(32a)
+    // FP64 near field in double-floats, lengths in units of 1/d_xs (a power of two at least the root side),
+    // a' = a d_xs: 2a'^2/3, 4/(3a'), 9/(32a') and 1/(8a'^2) as hi and lo floats; d_lim = max(4a'^2, kDfTiny2);
+    // d_ok: the lengths lie in the range of the form
+    double d_xs;
+    float d_k23h, d_k23l, d_c43h, d_c43l, d_c9h, d_c9l, d_c8h, d_c8l, d_lim;
+    int d_ok;
 };
+
+constexpr float kDfTiny2 = 3.5527136788005009e-15f;   // 2^-48: closer pairs are taken in FP64
+
+// 2^(e - 1023), 0 < e < 2047
+__host__ __device__ __forceinline__ double exp2_of_biased(int e) {
+#ifdef __CUDA_ARCH__
+    return __hiloint2double(e << 20, 0);
+#else
+    return std::ldexp(1.0, e - 1023);
+#endif
+}
+// The double-float near field takes systems whose root side and largest force component (its high word, fmax)
+// lie within 2^-500 .. 2^500.
+__device__ __forceinline__ bool force_range_ok(int w) { return w >= (523 << 20) && w < (1523 << 20); }
+// 2^-e with 2^e > side >= 2^(e-1); 0 when side is out of range (or zero)
+__device__ __forceinline__ double near_unit(double side) {
+    const int w = __double2hiint(side);
+    return force_range_ok(w) ? exp2_of_biased(2045 - (w >> 20)) : 0.0;
+}
 
 struct Tree {
     int device = 0;
@@ -249,6 +274,9 @@ struct Tree {
     double *fs = nullptr;             // sorted forces SoA [3][n]
     float *p32 = nullptr;             // FP32 form: sorted positions as hi + lo floats, [6][n] (x,y,z hi; x,y,z lo)
     float *f32 = nullptr;             // FP32 form: sorted forces [3][n]
+    float *p3 = nullptr;              // FP64 form: sorted positions as three floats per coordinate [9][n]
+    float *f2 = nullptr;              // FP64 form: sorted forces as double-floats [6][n]
+    int *sys_fmax = nullptr;          // FP64 form: [nsys] high word of the largest force component's magnitude
     double *u_near = nullptr, *u_far = nullptr, *u_dir = nullptr;   // sorted [n][3]
     double *host_io = nullptr;        // rpy_tree_matvec_host: positions, forces, velocities [9][n] (caller order),
                                       // allocated on its first call, kept across rebuilds
@@ -333,6 +361,8 @@ constexpr int kCartMaxP = 10, kCartDefaultP = 8;
 constexpr int kListU = 0, kListD = 1, kListM = 2;   // near list: U, direct substitutes, both
 int run_p2p(Tree &t, const double *fs, double *out, const SysConst &sc, cudaStream_t st, int list);
 int split_positions_f32(Tree &t, cudaStream_t st);
+int split_positions_f64(Tree &t, cudaStream_t st);
+int split_forces_f64(Tree &t, cudaStream_t st);
 // the tree of a valid handle, else nullptr
 Tree *tree_of(rpy_tree h);
 

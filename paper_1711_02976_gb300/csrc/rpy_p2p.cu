@@ -12,9 +12,13 @@
 //   r = 0   : s/(6 pi a) F                                           (r -> 0 limit)
 // The self term s/(6 pi a) F_i is added once.
 //
-// FP64 form: every operation in FP64; 1/r from a single-precision seed and
-// one Newton-Raphson step for the reciprocal square root (y <- y (3 - r2 y^2)/2),
-// which brings the relative error from ~1e-7 to ~1e-14.
+// FP64 form (k_p2p_df): every pair value and sum is a double-float, the unevaluated sum of two FP32
+// numbers (about 48 significant bits; two-sum of Knuth, products by FMA as in Dekker 1971 /
+// Ogita, Rump and Oishi 2005).  This part executes 2 FP64 operations per SM and clock but
+// 128 FP32 ones: 24 FP64 operations per pair cost 12 cycles, the 200 FP32 operations of
+// the double-float form under 2.  The running sums go to FP64 every kDfBlock pairs of sources.  Pairs closer
+// than 2^-24 of the root cube's side, leaves below level 17 and systems whose
+// lengths or forces lie outside the FP32 exponent range take every operation in FP64 (near64).
 // FP32 form (precision setting, k_p2p32): positions relative to the target
 // leaf centre in FP32; every thread carries two targets as the two lanes of
 // packed FP32x2 operations and takes two staged sources per iteration; an
@@ -32,7 +36,6 @@
 
 namespace rpy {
 
-constexpr double kPiD = 3.14159265358979323846;
 constexpr int kP2PThreads = 256;
 
 // Reciprocal square root for r2 > 0: an FP32 seed taken from the bit pattern
@@ -69,6 +72,14 @@ __device__ __forceinline__ void overlap_pair(double dx, double dy, double dz, do
         acc[1] += co * fy;
         acc[2] += co * fz;
     }
+}
+
+// Hardware reciprocal square root, flushing subnormals (the argument here is at
+// least 1e-6 a^2, kept normal by k_pair_const).
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 // Source staging: the beads of all source boxes of a leaf's list are streamed
@@ -109,28 +120,23 @@ __device__ __forceinline__ SrcCursor cursor_advance(SrcCursor c, int u1, int t, 
     return c;
 }
 
-// Thread layout: a leaf of T beads uses R = min(T, blockDim) targets per pass and
-// G = blockDim / R groups; group g takes every G-th bead of each staged chunk.
-// Far pairs accumulate in units of s/(8 pi) (applied once per target) with
-// explicit FMAs: 24 FP64 operations per pair and no conversions.
-__global__ void __launch_bounds__(kP2PThreads) k_p2p(const int2 *items, const int *leaves, const int *beg,
-                                                     const int *end, const int *bsys, const int *uoff,
-                                                     const int *uidx, const double *pos, const double *fs, int64_t n,
-                                                     SysConst sc, int add_self, double *out) {
-    __shared__ double sx[kP2PThreads], sy[kP2PThreads], sz[kP2PThreads];
-    __shared__ double sfx[kP2PThreads], sfy[kP2PThreads], sfz[kP2PThreads];
-    __shared__ int sj[kP2PThreads];
-    __shared__ double red[3][kP2PThreads];
-    const int2 item = items[blockIdx.x];
-    const int li = item.x, b = leaves[li], sys = bsys[b];
-    const int tb = item.y, te = min(end[b], item.y + kItemTargets);
-    const PairConst &pc = sc.pc[sys];
+// All pairs of one item in FP64: the general form, for what k_p2p_df cannot represent.  smem
+// holds 9 x kP2PThreads doubles and kP2PThreads ints.
+// Thread layout: R = min(T, blockDim) targets per pass and G = blockDim / R groups; group g takes
+// every G-th bead of each staged chunk.  Far pairs accumulate in units of s/(8 pi) (applied
+// once per target) with explicit FMAs: 24 FP64 operations per pair and no conversions; 1/r from a
+// single-precision seed and one Newton step.
+__device__ __noinline__ void near64(unsigned char *smem, int tb, int te, int u0, int u1, const int *beg,
+                                    const int *end, const int *uidx, const double *pos, const double *fs, int64_t n,
+                                    const PairConst &pc, int add_self, double *out) {
+    double *sx = reinterpret_cast<double *>(smem), *sy = sx + kP2PThreads, *sz = sy + kP2PThreads;
+    double *sfx = sz + kP2PThreads, *sfy = sfx + kP2PThreads, *sfz = sfy + kP2PThreads, *red = sfz + kP2PThreads;
+    int *sj = reinterpret_cast<int *>(red + 3 * kP2PThreads);
     const double a = pc.a, co = pc.co, cf = pc.cf, k23 = pc.k23, nk2 = pc.nk2;
     const long long a2x4 = __double_as_longlong(pc.a2x4);   // r2 >= 4a^2 compared on the bit patterns
-    const int u0 = uoff[li], u1 = uoff[li + 1];
     const int nt = te - tb;
-    const int Rn = nt < int(blockDim.x) ? nt : int(blockDim.x);
-    const int G = int(blockDim.x) / Rn;
+    const int Rn = nt < kP2PThreads ? nt : kP2PThreads;
+    const int G = kP2PThreads / Rn;
     const int tl = threadIdx.x % Rn, g = threadIdx.x / Rn;
     for (int i0 = tb; i0 < te; i0 += Rn) {
         const int i = i0 + tl;
@@ -151,10 +157,10 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p(const int2 *items, const in
                 sfy[threadIdx.x] = fs[n + j];
                 sfz[threadIdx.x] = fs[2 * n + j];
             }
-            cur = cursor_advance(cur, u1, int(blockDim.x), uidx, beg, end);
+            cur = cursor_advance(cur, u1, kP2PThreads, uidx, beg, end);
             __syncthreads();
             if (!act) continue;
-            for (int jj = g; jj < int(blockDim.x); jj += G) {
+            for (int jj = g; jj < kP2PThreads; jj += G) {
                 const int jg = sj[jj];
                 if (jg < 0) break;
                 const double dx = xi - sx[jj], dy = yi - sy[jj], dz = zi - sz[jj];
@@ -180,21 +186,389 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p(const int2 *items, const in
             }
         }
         __syncthreads();
-        red[0][threadIdx.x] = fma(cf, ax, accd[0]);
-        red[1][threadIdx.x] = fma(cf, ay, accd[1]);
-        red[2][threadIdx.x] = fma(cf, az, accd[2]);
+        red[threadIdx.x] = fma(cf, ax, accd[0]);
+        red[kP2PThreads + threadIdx.x] = fma(cf, ay, accd[1]);
+        red[2 * kP2PThreads + threadIdx.x] = fma(cf, az, accd[2]);
         __syncthreads();
         if (act && g == 0) {
             double v[3];
             for (int c = 0; c < 3; ++c) {
-                v[c] = red[c][threadIdx.x];
-                for (int gg = 1; gg < G; ++gg) v[c] += red[c][threadIdx.x + gg * Rn];
+                v[c] = red[c * kP2PThreads + threadIdx.x];
+                for (int gg = 1; gg < G; ++gg) v[c] += red[c * kP2PThreads + threadIdx.x + gg * Rn];
             }
             const double cs = add_self ? co : 0.0;
             out[3 * size_t(i)] = v[0] + cs * fs[i];
             out[3 * size_t(i) + 1] = v[1] + cs * fs[n + i];
             out[3 * size_t(i) + 2] = v[2] + cs * fs[2 * n + i];
         }
+    }
+}
+
+// ---------------------------------------------------------------- FP64 form in double-floats
+
+// Positions of the FP64 form as three floats per coordinate, x' = h + m + l in units of 2^e with e the
+// exponent of the root cube's side, relative to the cube's centre: h a multiple of 2^-23 and m of 2^-46, so
+// that the differences of two h's and of two m's are exact in FP32, and l the rest, rounded
+// at 2^-71: the difference of two FP64 coordinates is kept to its last bit.
+__global__ void k_split3(const double *pos, const int *bead_sys, const double *cube, int64_t n, float *p3) {
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double *c = cube + 4 * bead_sys[i];
+    const double xs = near_unit(c[3]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double x = pos[a * n + i], d = x - c[a];
+        const double bb = d - x, err = (x - (d - bb)) + (-c[a] - bb);   // d + err = x - c exactly
+        const double v = d * xs;
+        const double h = (v + 805306368.0) - 805306368.0;   // 1.5 * 2^29: ulp 2^-23
+        const double r = v - h;
+        const double m = (r + 96.0) - 96.0;                 // 1.5 * 2^6: ulp 2^-46
+        p3[(3 * a) * n + i] = float(h);
+        p3[(3 * a + 1) * n + i] = float(m);
+        p3[(3 * a + 2) * n + i] = float((r - m) + err * xs);
+    }
+}
+
+int split_positions_f64(Tree &t, cudaStream_t st) {
+    k_split3<<<unsigned((t.n + 255) / 256), 256, 0, st>>>(t.pos, t.bead_sys, t.sys_cube, t.n, t.p3);
+    RPY_LAUNCHED(1);
+    RPY_CHECK(cudaGetLastError());
+    return RPY_OK;
+}
+
+// Sorted forces as double-floats in units of 2^e, e the exponent of the system's largest component.
+__global__ void k_split_force(const double *fs, const int *bead_sys, const int *fmax, int64_t n, float *f2) {
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int w = fmax[bead_sys[i]];
+    if (!force_range_ok(w)) return;   // near64 takes this system
+    const double sc = exp2_of_biased(2046 - (w >> 20));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double v = fs[a * n + i] * sc;
+        const float h = float(v);
+        f2[(2 * a) * n + i] = h;
+        f2[(2 * a + 1) * n + i] = float(v - double(h));
+    }
+}
+
+int split_forces_f64(Tree &t, cudaStream_t st) {
+    k_split_force<<<unsigned((t.n + 255) / 256), 256, 0, st>>>(t.fs, t.bead_sys, t.sys_fmax, t.n, t.f2);
+    RPY_LAUNCHED(1);
+    RPY_CHECK(cudaGetLastError());
+    return RPY_OK;
+}
+
+// Packed (two lanes) FP32 operations and double-floats of them.
+struct df2 {
+    float2 h, l;
+};
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// s + e = a + b exactly
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2 &e) {
+    const float2 s = add2(a, b), bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
+}
+// (a.h + a.l) (b.h + b.l)
+__device__ __forceinline__ df2 mul_df(df2 a, df2 b) {
+    df2 r;
+    r.h = mul2(a.h, b.h);
+    r.l = fma2(a.l, b.h, fma2(a.h, b.l, fma2(a.h, b.h, neg2(r.h))));
+    return r;
+}
+
+// The difference of two coordinates held as three floats, normalised.
+__device__ __forceinline__ df2 diff3(float2 xh, float2 xm, float2 xl, float2 sh, float2 sm, float2 sl) {
+    const float2 dh = sub2(xh, sh), dm = sub2(xm, sm), dl = sub2(xl, sl);   // the first two exact
+    df2 r;
+    r.h = add2(dh, dm);                          // dh = 0 or |dh| >= |dm|
+    r.l = add2(sub2(dm, sub2(r.h, dh)), dl);
+    return r;
+}
+
+// What both branches of a pair share: r^2 (hi part r2), 1/r = ri and 1/r^2 = ri2 as
+// double-floats, and R.F.
+struct PairDf {
+    df2 r2, ri, ri2, rf;
+};
+
+__device__ __forceinline__ void pair_r2(const df2 *D, df2 &r2) {
+    const float2 px = mul2(D[0].h, D[0].h), py = mul2(D[1].h, D[1].h), pz = mul2(D[2].h, D[2].h);
+    const float2 ex = fma2(D[0].h, D[0].h, neg2(px)), ey = fma2(D[1].h, D[1].h, neg2(py)),
+                 ez = fma2(D[2].h, D[2].h, neg2(pz));
+    const float2 ll = fma2(D[2].h, D[2].l, fma2(D[1].h, D[1].l, mul2(D[0].h, D[0].l)));
+    float2 t1, t2;
+    r2.h = two_sum2(two_sum2(px, py, t1), pz, t2);
+    r2.l = fma2(dup(2.f), ll, add2(add2(ex, ey), add2(ez, add2(t1, t2))));
+}
+
+// 1/r from the hardware approximation y of 1/sqrt(r2): one Newton step with the residual r^2 y^2 - 1 from
+// u = r^2 y brings y within half an ulp and a bit; then, with exact products, z = r^2 y^2 - 1 again and
+// 1/r = y (1 - z/2 + 3 z^2/8).  (An FP32 residual in the first step leaves y, and with it the roundings of
+// every low part below, 1.5 times as far off.)
+__device__ __forceinline__ void pair_common(const df2 *D, const df2 *F, float2 r2clamped, PairDf &P) {
+    float2 y = make_float2(rsqrt_ftz(r2clamped.x), rsqrt_ftz(r2clamped.y));
+    const float2 u = mul2(P.r2.h, y), eu = fma2(P.r2.l, y, fma2(P.r2.h, y, neg2(u)));
+    y = fma2(mul2(y, dup(-0.5f)), fma2(eu, y, fma2(u, y, dup(-1.f))), y);
+    const float2 p2 = mul2(y, y), e2 = fma2(y, y, neg2(p2));
+    const float2 z = add2(fma2(P.r2.h, p2, dup(-1.f)), fma2(P.r2.h, e2, mul2(P.r2.l, p2)));
+    const float2 d = mul2(z, fma2(dup(0.375f), z, dup(-0.5f)));
+    P.ri.h = y;
+    P.ri.l = mul2(y, d);
+    P.ri2.h = p2;
+    P.ri2.l = fma2(p2, add2(d, d), e2);
+    const float2 qx = mul2(D[0].h, F[0].h), qy = mul2(D[1].h, F[1].h), qz = mul2(D[2].h, F[2].h);
+    const float2 ex = fma2(D[0].h, F[0].h, neg2(qx)), ey = fma2(D[1].h, F[1].h, neg2(qy)),
+                 ez = fma2(D[2].h, F[2].h, neg2(qz));
+    float2 cl = mul2(D[0].h, F[0].l);
+    cl = fma2(D[0].l, F[0].h, cl);
+    cl = fma2(D[1].h, F[1].l, cl);
+    cl = fma2(D[1].l, F[1].h, cl);
+    cl = fma2(D[2].h, F[2].l, cl);
+    cl = fma2(D[2].l, F[2].h, cl);
+    float2 t1, t2;
+    P.rf.h = two_sum2(two_sum2(qx, qy, t1), qz, t2);
+    P.rf.l = add2(add2(add2(ex, ey), add2(ez, add2(t1, t2))), cl);
+}
+
+// r >= 2a:  T1 = ri (1 + V),  T2 = ri^3 (1 - 3V) R.F,  V = (2a^2/3) ri^2 <= 1/6
+__device__ __forceinline__ void pair_far(const PairDf &P, df2 k23, df2 &T1, df2 &T2) {
+    const df2 V = mul_df(P.ri2, k23);
+    df2 a1, a2;
+    a1.h = add2(dup(1.f), V.h);
+    a1.l = add2(sub2(V.h, sub2(a1.h, dup(1.f))), V.l);
+    a2.h = fma2(dup(-3.f), V.h, dup(1.f));
+    a2.l = fma2(dup(-3.f), V.l, fma2(dup(-3.f), V.h, sub2(dup(1.f), a2.h)));
+    T1 = mul_df(P.ri, a1);
+    T2 = mul_df(mul_df(mul_df(P.ri2, a2), P.rf), P.ri);
+}
+
+// 0 < r < 2a, in the same units:  T1 = 4/(3a) (1 - 9r/(32a)),  T2 = 1/(8 a^2) ri R.F
+__device__ __forceinline__ void pair_overlap(const PairDf &P, const PairConst &pc, df2 &T1, df2 &T2) {
+    const df2 c9{dup(pc.d_c9h), dup(pc.d_c9l)}, c43{dup(pc.d_c43h), dup(pc.d_c43l)}, c8{dup(pc.d_c8h), dup(pc.d_c8l)};
+    const df2 v = mul_df(mul_df(P.r2, P.ri), c9);   // <= 9/16
+    df2 b;
+    b.h = sub2(dup(1.f), v.h);
+    b.l = sub2(sub2(sub2(dup(1.f), b.h), v.h), v.l);
+    T1 = mul_df(b, c43);
+    T2 = mul_df(mul_df(P.ri, c8), P.rf);
+}
+
+// S + C += T1 F + T2 D, renormalised
+__device__ __forceinline__ void accumulate_df(df2 T1, df2 F, df2 T2, df2 D, float2 &S, float2 &C) {
+    const df2 q1 = mul_df(T1, F), q2 = mul_df(T2, D);
+    float2 t1, t2;
+    const float2 h = two_sum2(q1.h, q2.h, t1);
+    const float2 lo = add2(add2(q1.l, q2.l), t1);
+    const float2 s = two_sum2(S, h, t2);
+    const float2 c = add2(t2, add2(C, lo));
+    S = add2(s, c);
+    C = sub2(c, sub2(S, s));
+}
+
+// A pair closer than 2^-24 of the root cube's side, from the FP64 positions.
+__device__ __noinline__ void pair_tiny_f64(int j, int i, const PairConst &pc, const double *pos, const double *fs,
+                                           int64_t n, double *acc) {
+    const double dx = pos[i] - pos[j], dy = pos[n + i] - pos[n + j], dz = pos[2 * n + i] - pos[2 * n + j];
+    const double fx = fs[j], fy = fs[n + j], fz = fs[2 * n + j], r2 = dx * dx + dy * dy + dz * dz;
+    if (r2 >= pc.a2x4) {
+        const double ri = 1.0 / sqrt(r2), ri2 = ri * ri;
+        const double t1 = pc.cf * fma(pc.k23, ri2 * ri, ri);
+        const double t2 = pc.cf * ri * ri2 * fma(pc.nk2, ri2, 1.0) * (dx * fx + dy * fy + dz * fz);
+        acc[0] += t1 * fx + t2 * dx;
+        acc[1] += t1 * fy + t2 * dy;
+        acc[2] += t1 * fz + t2 * dz;
+    } else {
+        overlap_pair(dx, dy, dz, r2, fx, fy, fz, pc.a, pc.co, acc);
+    }
+}
+
+constexpr int kDfThreads = kP2PThreads;
+constexpr int kDfChunk = 512;    // sources staged per pass
+constexpr int kDfList = 256;     // list boxes per prefix segment
+constexpr int kDfStride = 9;     // float4 per staged pair of sources: 15 packed values, 2 indices, 1 of padding
+constexpr int kDfBlock = 8;      // pairs of sources per double-float block between FP64 sums
+constexpr int kDfMaxLevel = 17;  // deeper leaves hold pairs closer than the three-float split resolves
+constexpr size_t kDfSmem = sizeof(float4) * kDfStride * (kDfChunk / 2) + sizeof(double) * 6 * kDfThreads +
+                           sizeof(int) * (2 * kDfList + 4);
+static_assert(sizeof(float4) * kDfStride * (kDfChunk / 2) >= kP2PThreads * (9 * sizeof(double) + sizeof(int)),
+              "near64 works in the staging buffer");
+
+// Thread layout: an item of T targets uses G = blockDim / T groups of T threads; the list's beads are staged
+// in chunks as pairs (two sources in the two lanes of the packed operations), and group g takes every G-th
+// pair.  The list's boxes are prefix-summed in shared memory and each staged bead finds its box by binary
+// search.  A pair of sources stands in 9 float4 (8 used): the groups of a warp then read different banks.
+__global__ void __launch_bounds__(kDfThreads, 2)
+    k_p2p_df(const int2 *items, const int *leaves, const int *beg, const int *end, const int *bsys, const int *lvl,
+             const int *uoff, const int *uidx, const float *p3, const float *f2, const int *fmax, const double *pos,
+             const double *fs, int64_t n, SysConst sc, int add_self, double *out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4 *sS = reinterpret_cast<float4 *>(smem_raw);
+    double *sU = reinterpret_cast<double *>(sS + kDfStride * (kDfChunk / 2));   // [3][threads] running sums
+    double *sD = sU + 3 * kDfThreads;                                            // [threads][3] FP64 pairs
+    int *lb = reinterpret_cast<int *>(sD + 3 * kDfThreads), *lpre = lb + kDfList;
+    int *any64 = lpre + kDfList + 1;
+    const int2 item = items[blockIdx.x];
+    const int li = item.x, b = leaves[li], sys = bsys[b];
+    const int tb = item.y, te = min(end[b], item.y + kItemTargets), nt = te - tb;
+    const int u0 = uoff[li], u1 = uoff[li + 1];
+    const PairConst &pc = sc.pc[sys];
+    const int fw = fmax[sys];
+    if (!pc.d_ok || !force_range_ok(fw) || lvl[b] > kDfMaxLevel) {
+        near64(smem_raw, tb, te, u0, u1, beg, end, uidx, pos, fs, n, pc, add_self, out);
+        return;
+    }
+    const float lim = pc.d_lim, tiny = kDfTiny2;
+    const df2 k23{dup(pc.d_k23h), dup(pc.d_k23l)};
+    const int G = kDfThreads / nt;
+    const int tl = threadIdx.x % nt, g = threadIdx.x / nt;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = tb + tl;
+    const bool act = g < G;
+    float2 X[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X[k] = dup(p3[k * n + i]);
+    for (int c = 0; c < 3; ++c) {
+        sU[c * kDfThreads + threadIdx.x] = 0.0;
+        sD[3 * threadIdx.x + c] = 0.0;
+    }
+    if (threadIdx.x == 0) *any64 = 0;
+    for (int us = u0; us < u1; us += kDfList) {
+        const int L = min(kDfList, u1 - us);
+        __syncthreads();
+        if (warp == 0) {   // prefix of the box sizes of this list segment
+            int carry = 0;
+            for (int q0 = 0; q0 < L; q0 += 32) {
+                const int q = q0 + lane;
+                int cnt = 0;
+                if (q < L) {
+                    const int C = uidx[us + q];
+                    lb[q] = beg[C];
+                    cnt = end[C] - beg[C];
+                }
+                int v = cnt;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int w = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += w;
+                }
+                if (q < L) lpre[q + 1] = carry + v;
+                carry += __shfl_sync(0xffffffffu, v, 31);
+            }
+            if (lane == 0) lpre[0] = 0;
+        }
+        __syncthreads();
+        const int Ns = lpre[L];
+        for (int c0 = 0; c0 < Ns; c0 += kDfChunk) {
+            const int nS = min(kDfChunk, Ns - c0), nP = (nS + 1) >> 1;
+            // the barrier after the prefix or after the previous chunk's pairs orders these writes
+            for (int e = threadIdx.x; e < 2 * nP; e += kDfThreads) {
+                float *w = reinterpret_cast<float *>(sS + kDfStride * (e >> 1)) + (e & 1);
+                if (e < nS) {
+                    const int q = c0 + e;
+                    int lo = 0, hi = L;   // box: lpre[lo] <= q < lpre[lo + 1]
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (lpre[mid] <= q) lo = mid;
+                        else hi = mid;
+                    }
+                    const int j = lb[lo] + (q - lpre[lo]);
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) w[2 * k] = p3[k * n + j];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) w[18 + 2 * k] = f2[k * n + j];
+                    reinterpret_cast<int *>(w)[30] = j;
+                } else {   // an odd last source gets a partner outside the cube, without force
+#pragma unroll
+                    for (int k = 0; k < 15; ++k) w[2 * k] = k == 0 ? 4.f : 0.f;
+                    reinterpret_cast<int *>(w)[30] = -1;
+                }
+            }
+            __syncthreads();
+            if (act) {
+                for (int e0 = g; e0 < nP; e0 += kDfBlock * G) {
+                    float2 S[3], C[3];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) S[c] = C[c] = dup(0.f);
+                    const int e1 = min(nP, e0 + kDfBlock * G);
+                    for (int e = e0; e < e1; e += G) {
+                        const float4 *s = sS + kDfStride * e;
+                        const float4 v0 = s[0], v1 = s[1], v2 = s[2], v3 = s[3], v4 = s[4], v5 = s[5], v6 = s[6], v7 = s[7];
+                        df2 D[3], F[3];
+                        D[0] = diff3(X[0], X[1], X[2], make_float2(v0.x, v0.y), make_float2(v0.z, v0.w),
+                                     make_float2(v1.x, v1.y));
+                        D[1] = diff3(X[3], X[4], X[5], make_float2(v1.z, v1.w), make_float2(v2.x, v2.y),
+                                     make_float2(v2.z, v2.w));
+                        D[2] = diff3(X[6], X[7], X[8], make_float2(v3.x, v3.y), make_float2(v3.z, v3.w),
+                                     make_float2(v4.x, v4.y));
+                        F[0] = df2{make_float2(v4.z, v4.w), make_float2(v5.x, v5.y)};
+                        F[1] = df2{make_float2(v5.z, v5.w), make_float2(v6.x, v6.y)};
+                        F[2] = df2{make_float2(v6.z, v6.w), make_float2(v7.x, v7.y)};
+                        PairDf P;
+                        pair_r2(D, P.r2);
+                        df2 T1, T2;
+                        if (__all_sync(__activemask(), fminf(P.r2.h.x, P.r2.h.y) >= lim)) {
+                            pair_common(D, F, P.r2.h, P);
+                            pair_far(P, k23, T1, T2);
+                        } else {
+                            // some lane has an overlapping, very close or self pair: both branches with selects
+                            pair_common(D, F, make_float2(fmaxf(P.r2.h.x, tiny), fmaxf(P.r2.h.y, tiny)), P);
+                            df2 O1, O2;
+                            pair_far(P, k23, T1, T2);
+                            pair_overlap(P, pc, O1, O2);
+                            const bool fx = P.r2.h.x >= lim, fy = P.r2.h.y >= lim;
+                            const bool ox = P.r2.h.x > tiny, oy = P.r2.h.y > tiny;
+                            auto pick = [&](float2 far, float2 near) {
+                                return make_float2(fx ? far.x : (ox ? near.x : 0.f), fy ? far.y : (oy ? near.y : 0.f));
+                            };
+                            T1.h = pick(T1.h, O1.h);
+                            T1.l = pick(T1.l, O1.l);
+                            T2.h = pick(T2.h, O2.h);
+                            T2.l = pick(T2.l, O2.l);
+                            if (!ox || !oy) {
+                                const int jx = __float_as_int(v7.z), jy = __float_as_int(v7.w);
+                                if (!ox && jx != i) {
+                                    pair_tiny_f64(jx, i, pc, pos, fs, n, sD + 3 * threadIdx.x);
+                                    *any64 = 1;
+                                }
+                                if (!oy && jy != i) {
+                                    pair_tiny_f64(jy, i, pc, pos, fs, n, sD + 3 * threadIdx.x);
+                                    *any64 = 1;
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) accumulate_df(T1, F[c], T2, D[c], S[c], C[c]);
+                    }
+                    // the two lanes of the block into the FP64 sums
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        const float s = S[c].x + S[c].y, bb = s - S[c].x;
+                        const float e = (S[c].x - (s - bb)) + (S[c].y - bb);
+                        sU[c * kDfThreads + threadIdx.x] += double(s) + double((C[c].x + C[c].y) + e);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    // one thread per (component, target) adds the groups in order
+    const double unit = pc.cf * pc.d_xs * exp2_of_biased(fw >> 20), co = pc.co;
+    const bool any = *any64 != 0;
+    for (int q = threadIdx.x; q < 3 * nt; q += kDfThreads) {
+        const int c = q / nt, tt = q - c * nt, it = tb + tt;
+        double v = 0.0;
+        for (int gg = 0; gg < G; ++gg) v += sU[c * kDfThreads + tt + gg * nt];
+        double u = unit * v;
+        if (any)
+            for (int gg = 0; gg < G; ++gg) u += sD[3 * (tt + gg * nt) + c];
+        out[3 * size_t(it) + c] = u + (add_self ? co * fs[c * n + it] : 0.0);
     }
 }
 
@@ -236,14 +610,6 @@ __device__ __forceinline__ void pair_tiny64(int jg, int i, double a, double co, 
                                             int64_t n, double *acc) {
     double ddx = pos[i] - pos[jg], ddy = pos[n + i] - pos[n + jg], ddz = pos[2 * n + i] - pos[2 * n + jg];
     overlap_pair(ddx, ddy, ddz, ddx * ddx + ddy * ddy + ddz * ddz, fs[jg], fs[n + jg], fs[2 * n + jg], a, co, acc);
-}
-
-// Hardware reciprocal square root, flushing subnormals (the argument here is at
-// least 1e-6 a^2, kept normal by k_pair_const).
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 
 // One pair, both branches without divergence, in units of s/(8 pi), with
@@ -553,9 +919,9 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, con
     }
 }
 
-// The dynamic shared memory of k_p2p32 exceeds the default 48 KB: raise the
+// The dynamic shared memory of both near-field kernels exceeds the default 48 KB: raise the
 // limit once per device.
-static cudaError_t set_p2p32_smem() {
+static cudaError_t set_near_smem() {
     static std::mutex mu;
     static std::set<int> done;
     int dev = 0;
@@ -564,6 +930,7 @@ static cudaError_t set_p2p32_smem() {
     std::lock_guard<std::mutex> lk(mu);
     if (done.count(dev)) return cudaSuccess;
     e = cudaFuncSetAttribute(k_p2p32, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kP32Smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_p2p_df, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kDfSmem));
     if (e == cudaSuccess) done.insert(dev);
     return e;
 }
@@ -577,14 +944,15 @@ int run_p2p(Tree &t, const double *fs, double *out, const SysConst &sc, cudaStre
     int add_self = direct_list ? 0 : 1;
     const int2 *items = merged ? t.m_items : (direct_list ? t.d_items : t.u_items);
     if (t.n_items == 0) return RPY_OK;
+    RPY_CHECK(set_near_smem());
     if (t.params.precision == RPY_FP32) {
-        RPY_CHECK(set_p2p32_smem());
         k_p2p32<<<t.n_items, kP32Threads, kP32Smem, st>>>(items, t.leaves, t.b_begin, t.b_end, t.b_sys, t.b_center,
                                                           off, idx, t.p32, t.f32, t.pos, fs, t.n, sc, add_self, out);
         RPY_LAUNCHED(1);
     } else {
-        k_p2p<<<t.n_items, kP2PThreads, 0, st>>>(items, t.leaves, t.b_begin, t.b_end, t.b_sys, off, idx, t.pos, fs,
-                                                 t.n, sc, add_self, out);
+        k_p2p_df<<<t.n_items, kDfThreads, kDfSmem, st>>>(items, t.leaves, t.b_begin, t.b_end, t.b_sys, t.b_level, off,
+                                                         idx, t.p3, t.f2, t.sys_fmax, t.pos, fs, t.n, sc, add_self,
+                                                         out);
         RPY_LAUNCHED(1);
     }
     RPY_CHECK(cudaGetLastError());

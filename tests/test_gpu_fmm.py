@@ -208,6 +208,85 @@ def test_fp32_close_pairs_beyond_the_queue():
     np.testing.assert_allclose(u[:48], ref[:48], rtol=0, atol=2e-6 * np.abs(ref[:48]).max())
 
 
+def _near_case(name, n, seed):
+    """(positions, forces, a) of one system for the FP64 near field: the layouts its double-float kernel
+    has to get right."""
+    rng = np.random.default_rng(seed)
+    pos, f, a = rng.random((n, 3)), rng.standard_normal((n, 3)), 1e-3
+    if name == "overlap":          # most near pairs closer than 2a
+        a = 0.1
+    elif name == "close":          # partners in (0, 2a), within 1e-4 a and coincident
+        a = 0.002
+        pos, f = _close_pairs(n, a, seed)
+    elif name == "below_split":    # pairs on both sides of the distance below which FP64 takes over
+        a = 1e-9
+        k = n // 8
+        d = rng.standard_normal((k, 3))
+        d *= (2.0 ** rng.uniform(-30, -18, k) / np.linalg.norm(d, axis=1))[:, None]
+        pos[:k] = np.clip(pos[k:2 * k] + d, 0, 1)
+    elif name == "offset":         # far from the origin: the differences keep the last bits of the positions
+        pos += 1000.0
+    elif name == "si":             # micrometres and piconewtons, near the ends of the FP32 range when squared
+        pos, f, a = 1e-12 * pos, 1e-30 * f, 2e-15
+    elif name == "huge":
+        pos, f, a = 1e15 * pos, 1e25 * f, 1e13
+    elif name == "uneven_forces":  # 30 decades between the forces of one system
+        f *= 10.0 ** rng.uniform(-30, 0, n)[:, None]
+    return pos, f, a
+
+
+@pytest.mark.parametrize("n,leaf_cap", [(2, 4), (33, 64), (255, 300), (256, 300), (257, 300), (513, 600),
+                                        (4097, 40)])
+@pytest.mark.parametrize("name", ["plain", "overlap", "close", "below_split", "offset", "si", "huge",
+                                  "uneven_forces"])
+def test_fp64_near_part_in_double_floats(name, n, leaf_cap):
+    """The FP64 near field sums in double-floats (2^-48 per operation, some 30 roundings per pair
+    value).  A target's error stays below 2^-40 of the sum of the magnitudes of its terms, which is what
+    rounding of any order of summation is bounded by."""
+    if name == "close" and n < 700:
+        pytest.skip("330 partners need more beads")
+    pos, f, a = _near_case(name, n, 7 + n)
+    s = 6 * math.pi * a
+    u, t = matvec(pos, f, a, s, 3, leaf_cap=leaf_cap, parts=rp.RPY_PART_NEAR)
+    ref = _near_oracle(t, pos, f, a, s)
+    lm, leaves, ul = leaf_members(t), rp.rpy_tree_export(t, "leaves"), csr(t, "u_off", "u_idx")
+    for li, b in enumerate(leaves):
+        mem, src = lm[int(b)], np.concatenate([lm[int(c)] for c in ul[li]])
+        # both branches, and the self term: |term| <= (s / 8 pi) (8/3) |F| / max(r, a)
+        r = np.linalg.norm(pos[mem][:, None, :] - pos[src][None, :, :], axis=2)
+        mag = (s / (8 * math.pi)) * (8.0 / 3.0) * (np.linalg.norm(f[src], axis=1) / np.maximum(r, a)).sum(axis=1)
+        assert (np.abs(u[mem] - ref[mem]).max(axis=1) <= 2.0 ** -40 * mag).all(), name
+
+
+def test_fp64_near_part_outside_the_double_float_range():
+    """A system whose forces hold an infinity, or lie below the range the double-floats cover, takes the
+    all-FP64 form; in a forest the other system is untouched."""
+    import torch
+    rng = np.random.default_rng(3)
+    pos, f = rng.random((600, 3)), rng.standard_normal((600, 3))
+    a, off = [1e-3, 1e-3], [0, 300, 600]
+    t = rp.rpy_forest_build(cuda_tensor(pos), off, a, 3, leaf_cap=400)
+    s = [6 * math.pi * 1e-3] * 2
+
+    def run(g):
+        F = cuda_tensor(g)
+        U = torch.empty_like(F)
+        rp.rpy_forest_matvec(t, F, s, U)
+        rp.rpy_tree_sync(t)
+        return U.cpu().numpy()
+    u0 = run(f)
+    tiny = f.copy()
+    tiny[300:] *= 1e-200
+    u1 = run(tiny)
+    assert np.array_equal(u1[:300], u0[:300])
+    np.testing.assert_allclose(u1[300:], 1e-200 * u0[300:], rtol=1e-10, atol=1e-213)
+    bad = f.copy()
+    bad[450, 0] = np.inf
+    u2 = run(bad)
+    assert np.array_equal(u2[:300], u0[:300])
+    assert not np.isfinite(u2[300:, 0]).any()
+
+
 # ---------------------------------------------------------------- far field operators
 
 @pytest.mark.parametrize("digits,tol", [(3, 1e-3), (6, 1e-6), (9, 1e-9)])
