@@ -21,6 +21,21 @@ static constexpr double kPiA = 3.14159265358979323846;
 
 // ---------------------------------------------------------------- kernels used here
 
+// fmax[system] = max over the block's beads of w (beads are sorted by system; i the thread's bead).
+__device__ __forceinline__ void block_sys_max(int w, int64_t i, int64_t n, const int *bead_sys, int *smax, int *fmax) {
+    const int64_t b0 = int64_t(blockIdx.x) * blockDim.x, b1 = min(b0 + blockDim.x, n) - 1;
+    const int s0 = bead_sys[b0];
+    if (s0 == bead_sys[b1]) {   // one system in the block
+        __syncthreads();
+        w = __reduce_max_sync(0xffffffffu, w);
+        if ((threadIdx.x & 31) == 0) atomicMax(smax, w);
+        __syncthreads();
+        if (threadIdx.x == 0 && *smax > *(volatile int *)&fmax[s0]) atomicMax(&fmax[s0], *smax);
+    } else if (i < n) {
+        atomicMax(&fmax[bead_sys[i]], w);
+    }
+}
+
 // Forces into sorted SoA; the FP32 form also keeps a single-precision copy, the FP64 form the largest component
 // of each system (the high word of its magnitude: NaN and infinity compare highest).
 __global__ void k_gather_f(const double *f, const int *perm, const int *bead_sys, int64_t n, double *fs, float *f32,
@@ -42,18 +57,7 @@ __global__ void k_gather_f(const double *f, const int *perm, const int *bead_sys
         }
         w = max(max(__double2hiint(fx) & 0x7fffffff, __double2hiint(fy) & 0x7fffffff), __double2hiint(fz) & 0x7fffffff);
     }
-    if (!fmax) return;
-    const int64_t b0 = int64_t(blockIdx.x) * blockDim.x, b1 = min(b0 + blockDim.x, n) - 1;
-    const int s0 = bead_sys[b0];
-    if (s0 == bead_sys[b1]) {   // one system in the block (beads are sorted by system)
-        __syncthreads();
-        w = __reduce_max_sync(0xffffffffu, w);
-        if ((threadIdx.x & 31) == 0) atomicMax(&smax, w);
-        __syncthreads();
-        if (threadIdx.x == 0 && smax > *(volatile int *)&fmax[s0]) atomicMax(&fmax[s0], smax);
-    } else if (i < n) {
-        atomicMax(&fmax[bead_sys[i]], w);
-    }
+    if (fmax) block_sys_max(w, i, n, bead_sys, &smax, fmax);
 }
 
 __global__ void k_pair_const(int nsys, const double *a_, const double *s_, const double *cube, PairConst *pc) {
@@ -81,7 +85,7 @@ __global__ void k_pair_const(int nsys, const double *a_, const double *s_, const
     c.f_pad = 0.f;
     const double xs = near_unit(cube[4 * k + 3]), ap = a * xs;
     c.d_xs = xs;
-    c.d_ok = ap >= 0x1p-60 && ap <= 0x1p30;
+    c.d_ok = near_range_ok(__double2hiint(cube[4 * k + 3])) && ap >= 0x1p-60 && ap <= 0x1p30;
     auto split = [](double v, float &h, float &l) {
         h = float(v);
         l = float(v - double(h));
@@ -94,11 +98,20 @@ __global__ void k_pair_const(int nsys, const double *a_, const double *s_, const
     pc[k] = c;
 }
 
-__global__ void k_gather_q4(const double *q, const int *perm, int64_t n, double *qs) {
-    int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t j = perm[i];
-    for (int k = 0; k < 4; ++k) qs[4 * i + k] = q[4 * j + k];
+__global__ void k_gather_q4(const double *q, const int *perm, const int *bead_sys, int64_t n, double *qs, int *fmax) {
+    __shared__ int smax;
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (threadIdx.x == 0) smax = 0;
+    int w = 0;
+    if (i < n) {
+        const int64_t j = perm[i];
+        for (int k = 0; k < 4; ++k) {
+            const double v = q[4 * j + k];
+            qs[4 * i + k] = v;
+            w = max(w, __double2hiint(v) & 0x7fffffff);
+        }
+    }
+    if (fmax) block_sys_max(w, i, n, bead_sys, &smax, fmax);
 }
 
 __global__ void k_combine(const int *perm, int64_t n, const double *un, const double *uf, const double *ud, int parts,
@@ -114,11 +127,13 @@ __global__ void k_combine(const int *perm, int64_t n, const double *un, const do
     }
 }
 
-__global__ void k_unperm_lap(const int *perm, int64_t n, const double *src, double *dst) {
+__global__ void k_unperm_lap(const int *perm, int64_t n, const double *src, const int *bead_sys, const int *fmax,
+                             double *dst) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int64_t j = perm[i];
-    for (int c = 0; c < 52; ++c) dst[52 * j + c] = src[52 * i + c];
+    const double unit = fmax ? force_unit(fmax[bead_sys[i]]) : 1.0;   // FP64 form: charges were scaled
+    for (int c = 0; c < 52; ++c) dst[52 * j + c] = unit * src[52 * i + c];
 }
 
 static inline int nb256(int64_t n) { return int((n + 255) / 256); }
@@ -152,7 +167,7 @@ void prof_mark(Tree &t, int k, cudaStream_t st) {
 
 struct DevTableSet {
     void *mem = nullptr;
-    DevTables<double> d64{};
+    DevTables<dfl> d64{};
     DevTables<float> d32{};
 };
 
@@ -306,7 +321,7 @@ static int device_tables(int dev, int p, int digits, DevTableSet **out) {
     }
     std::vector<char> b64, b32;
     std::vector<size_t> o64, o32;
-    pack_tables<double>(*h, b64, o64);
+    pack_tables<dfl>(*h, b64, o64);
     pack_tables<float>(*h, b32, o32);
     size_t off32 = (b64.size() + 255) / 256 * 256;
     void *mem = nullptr;
@@ -319,7 +334,7 @@ static int device_tables(int dev, int p, int digits, DevTableSet **out) {
     }
     DevTableSet *s = new DevTableSet();
     s->mem = mem;
-    s->d64 = bind_tables<double>(*h, static_cast<char *>(mem), o64);
+    s->d64 = bind_tables<dfl>(*h, static_cast<char *>(mem), o64);
     s->d32 = bind_tables<float>(*h, static_cast<char *>(mem) + off32, o32);
     g_dev_tabs[key] = s;
     *out = s;
@@ -373,6 +388,8 @@ static int alloc_tree_arrays(Tree &t, cudaStream_t st) {
 static int alloc_near_f64(Tree &t) {
     RPY_TRY(dev_alloc(t, (void **)&t.p3, sizeof(float) * 9 * t.n));
     RPY_TRY(dev_alloc(t, (void **)&t.f2, sizeof(float) * 6 * t.n));
+    RPY_TRY(dev_alloc(t, (void **)&t.c3, sizeof(float) * 9 * size_t(t.nbox)));
+    RPY_TRY(dev_alloc(t, (void **)&t.side_u, sizeof(double) * size_t(t.nbox)));
     return dev_alloc(t, (void **)&t.sys_fmax, sizeof(int) * t.nsys);
 }
 
@@ -488,7 +505,7 @@ static int matvec_body(Tree &t, const SysConst &sc, int parts, cudaStream_t st, 
         } else if (t.params.precision == RPY_FP32) {
             RPY_TRY(run_far_t<float>(t, t.dt32, t.fs, nullptr, t.u_far, nullptr, sc, st));
         } else {
-            RPY_TRY(run_far_t<double>(t, t.dt64, t.fs, nullptr, t.u_far, nullptr, sc, st));
+            RPY_TRY(run_far_t<dfl>(t, t.dt64, t.fs, nullptr, t.u_far, nullptr, sc, st));
         }
     }
     if (side) {
@@ -531,7 +548,7 @@ static int capture_graph(Tree &t, const SysConst &sc) {
 int run_matvec(Tree &t, const double *f_dev, const double *s_host, double *u_dev, int parts, cudaStream_t st) {
     if (!t.built) return RPY_ERR_STATE;
     RPY_TRY(upload_s(t, s_host, st));
-    SysConst sc{t.sys_cube, t.sys_a, t.sys_s, t.sys_pc};
+    SysConst sc{t.sys_cube, t.sys_a, t.sys_s, t.sys_pc, t.p3, t.c3, t.f2, t.sys_fmax};
     t.n_marks = 0;
     prof_mark(t, RPY_STAGE_GATHER, st);
     if (t.sys_fmax) RPY_CHECK(cudaMemsetAsync(t.sys_fmax, 0, sizeof(int) * t.nsys, st));
@@ -571,16 +588,17 @@ int run_laplace_far(Tree &t, const double *q_dev, double *out_dev, cudaStream_t 
     double *lap_out = nullptr;
     Tree scratch;
     RPY_TRY(dev_alloc(scratch, (void **)&lap_out, sizeof(double) * 52 * t.n));
-    SysConst sc{t.sys_cube, t.sys_a, t.sys_s, t.sys_pc};
-    k_gather_q4<<<nb256(t.n), 256, 0, st>>>(q_dev, t.perm, t.n, t.lap_q);
+    SysConst sc{t.sys_cube, t.sys_a, t.sys_s, t.sys_pc, t.p3, t.c3, t.f2, t.sys_fmax};
+    if (t.sys_fmax) RPY_CHECK(cudaMemsetAsync(t.sys_fmax, 0, sizeof(int) * t.nsys, st));
+    k_gather_q4<<<nb256(t.n), 256, 0, st>>>(q_dev, t.perm, t.bead_sys, t.n, t.lap_q, t.sys_fmax);
     RPY_LAUNCHED(1);
     int s;
     if (t.params.precision == RPY_FP32)
         s = run_far_t<float>(t, t.dt32, nullptr, t.lap_q, nullptr, lap_out, sc, st);
     else
-        s = run_far_t<double>(t, t.dt64, nullptr, t.lap_q, nullptr, lap_out, sc, st);
+        s = run_far_t<dfl>(t, t.dt64, nullptr, t.lap_q, nullptr, lap_out, sc, st);
     if (s == RPY_OK) {
-        k_unperm_lap<<<nb256(t.n), 256, 0, st>>>(t.perm, t.n, lap_out, out_dev);
+        k_unperm_lap<<<nb256(t.n), 256, 0, st>>>(t.perm, t.n, lap_out, t.bead_sys, t.sys_fmax, out_dev);
         RPY_LAUNCHED(1);
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) s = check_cuda("laplace far", e);
@@ -989,7 +1007,7 @@ int rpy_tree_footprint(int64_t n, int digits, int precision, int leaf_cap, int64
     // slot for the boxes of one level, counted here for every box
     const double m2m = (precision != RPY_FP32 || p >= 12) ? 8.0 * kSets * ncoef(p) : 0.0;
     double per_box = es * (2.0 * kSets * ncoef(p) + 2.0 * 2 * xf * kSets * q.half() + 18.0 * ncoef(p) + m2m) +
-                     4.0 * (8 + 27 + 3 + 12) + 32.0;
+                     4.0 * (8 + 27 + 3 + 12) + 32.0 + (precision == RPY_FP32 ? 0.0 : 9 * 4.0 + 8.0 /*c3, side_u*/);
     double per_bead = 3 * 8 /*pos*/ + 8 /*key*/ + 4 + 4 + 9 * 8 /*fs, unear, ufar*/ + 27 * 4 /*U list share*/ +
                       (precision == RPY_FP32 ? 9 * 4 /*p32, f32*/ : 15 * 4 /*p3, f2*/);
     *bytes = int64_t(nbox * per_box + double(n) * per_bead + 32.0 * 1024 * 1024);

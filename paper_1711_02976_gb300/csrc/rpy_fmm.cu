@@ -5,6 +5,15 @@
 // Charge sets (Sec. 2): q_1..q_3 = F^1..F^3, q_4 = F . (r - c0) with c0 the
 // centre of the system's bounding cube (Eq. 2.8 holds for any common origin).
 //
+// Number types: T = float in the FP32 form, T = dfl (two FP32 numbers, about 48 bits: rpy_dfl.h) in the
+// FP64 form, whose kernels were bound by the FP64 pipe (91 to 95% busy) at 64 times the cost of an FP32
+// operation; a multiply-add is 12 FP32 operations in dfl.  Lengths are in units of a power of two at the root
+// cube's side and forces in units of each system's largest (SysConst), so that every value lies well
+// inside the FP32 exponent range.  Measured, matvec of the 1M-bead sphere and cube at 6 digits: 104 -> 45.5 ms
+// (M2X 23.4 -> 8.8, X2L 20.1 -> 8.9, X2X 11.9 -> 5.4, L2P and M2P 16.6 -> 4.8, P2M and P2L 14.5 -> 4.0 ms); the
+// velocities of whole matvecs move by 1e-14 ... 1.2e-13, the error of the expansions being 1e-10
+// at 9 digits.
+//
 // Kernels, in launch order:
 //   k_p2m      S->M   leaves: M_n^m = sum_j q_j conj(y_n^m(eta_j))
 //   k_m2m_child, k_m2m_sum  M->M   per child: rotate to the shift axis, z-shift, rotate back;
@@ -43,7 +52,7 @@ __device__ __forceinline__ int deg_of(int idx) {
 // Lanes per point: columns m and P - m share a lane, so every lane runs P + 2
 // recurrence steps (a column per lane would leave the lanes of high m idle
 // while column 0 runs P + 1 steps, and lanes above P idle altogether; the
-// FP64 pipe is charged per warp instruction).
+// arithmetic pipes are charged per warp instruction).
 __host__ __device__ constexpr int harm_lanes(int P) { return P / 2 + 1; }
 
 // Solid harmonics (regular, or irregular when IRREG) of one point into out[],
@@ -70,7 +79,7 @@ __device__ void lane_harmonics(T x, T y, T z, int P, const T *ra, const T *rb, c
         for (int n = m + 1; n <= P; ++n) {
             const int i = tri(n, m);
             const T A = ra[i] * zz, B = rb[i] * rr;
-            const cpx<T> cn = mk(fma(A, p1.x, -B * p2.x), fma(A, p1.y, -B * p2.y));
+            const cpx<T> cn = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
             out[i] = cn;
             p2 = p1;
             p1 = cn;
@@ -99,23 +108,27 @@ __device__ void eval_fields(T x, T y, T z, int P, const cpx<T> *E, int stride, c
 #pragma unroll
             for (int q = 0; q < NE; ++q) {
                 const cpx<T> e = E[q * stride + i];
-                acc[q] = fma(-e.y, hw.y, fma(e.x, hw.x, acc[q]));
+                macc(acc[q], e.x, hw.x);
+                macc(acc[q], -e.y, hw.y);
             }
         }
         for (int n = m + 1; n <= P; ++n) {
             const int i = tri(n, m);
             const T A = ra[i] * zz, B = rb[i] * rr;
-            const cpx<T> c = mk(fma(A, p1.x, -B * p2.x), fma(A, p1.y, -B * p2.y));
+            const cpx<T> c = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
             const cpx<T> hw = W2 ? c : mk(wm * c.x, wm * c.y);
 #pragma unroll
             for (int q = 0; q < NE; ++q) {
                 const cpx<T> e = E[q * stride + i];
-                acc[q] = fma(-e.y, hw.y, fma(e.x, hw.x, acc[q]));
+                macc(acc[q], e.x, hw.x);
+                macc(acc[q], -e.y, hw.y);
             }
             p2 = p1;
             p1 = c;
         }
     }
+#pragma unroll
+    for (int q = 0; q < NE; ++q) acc[q] = closed(acc[q]);
 }
 
 // ---------------------------------------------------------------- derivative expansions
@@ -271,6 +284,15 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
     const double c0x = rb ? cx : sc.cube[4 * sy], c0y = rb ? cy : sc.cube[4 * sy + 1],
                  c0z = rb ? cz : sc.cube[4 * sy + 2];   // origin of q4
     const double ih = sc.pc[sy].icube * pow2i(lvl[b]);   // 1 / side[b], exactly
+    // double-floats: the box centre in the split units of the positions, and 1 / side in them
+    float c3[9];
+    T ihs = T(0);
+    double qs = 1.0;   // scale of given charges
+    if constexpr (kIsDf<T>) {
+        for (int k = 0; k < 9; ++k) c3[k] = sc.c3[9 * size_t(b) + k];
+        ihs = T(inv_side_u(sc.pc[sy], lvl[b]));
+        qs = force_scale(sc.fmax[sy]);
+    }
     int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     // harmonics: hG points per warp, lane -> (point hg, column pair hc)
     const int hL = harm_lanes(p), hG = 32 / hL, hg = (threadIdx.x & 31) / hL, hc = (threadIdx.x & 31) - hg * hL;
@@ -284,14 +306,32 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
                 const int t = t0 + hg;
                 if (hg < hG && t < cnt) {
                     int j = jc + t;
-                    T ex = T((pos[j] - cx) * ih), ey = T((pos[n + j] - cy) * ih), ez = T((pos[2 * n + j] - cz) * ih);
+                    T ex, ey, ez;
+                    if constexpr (kIsDf<T>) {
+                        ex = coord_diff(sc.p3, n, j, 0, c3) * ihs;
+                        ey = coord_diff(sc.p3, n, j, 1, c3) * ihs;
+                        ez = coord_diff(sc.p3, n, j, 2, c3) * ihs;
+                    } else {
+                        ex = T((pos[j] - cx) * ih), ey = T((pos[n + j] - cy) * ih), ez = T((pos[2 * n + j] - cz) * ih);
+                    }
                     lane_harmonics<T, MODE == 1>(ex, ey, ez, p, R.a, R.b, R.cm, ybuf + t * nc, hc);
                 }
             }
             for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
                 int j = jc + t;
                 if (lapq) {
-                    for (int k = 0; k < kSets; ++k) q[4 * t + k] = T(lapq[4 * j + k]);
+                    for (int k = 0; k < kSets; ++k) q[4 * t + k] = T(kIsDf<T> ? qs * lapq[4 * j + k] : lapq[4 * j + k]);
+                } else if constexpr (kIsDf<T>) {
+                    // scaled forces; q4 in the split units of length, its origin at the cube's or the box's centre
+                    float o3[9];
+                    for (int k = 0; k < 9; ++k) o3[k] = rb ? c3[k] : 0.f;
+                    T q4 = T(0);
+                    for (int a = 0; a < 3; ++a) {
+                        const T fa(sc.f2[(2 * a) * n + j], sc.f2[(2 * a + 1) * n + j]);
+                        q[4 * t + a] = fa;
+                        macc(q4, fa, coord_diff(sc.p3, n, j, a, o3));
+                    }
+                    q[4 * t + 3] = closed(q4);
                 } else {
                     double fx = fs[j], fy = fs[n + j], fz = fs[2 * n + j];
                     q[4 * t] = T(fx);
@@ -307,8 +347,8 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
                 for (int t = 0; t < cnt; ++t) {
                     cpx<T> yv = ybuf[t * nc + i];
                     T qq = q[4 * t + k];
-                    a.x += qq * yv.x;
-                    a.y -= qq * yv.y;   // conj
+                    macc(a.x, qq, yv.x);
+                    macc(a.y, -qq, yv.y);   // conj
                 }
                 if constexpr (sizeof(T) == 4) {
                     // a leaf (or an X-list source) may hold hundreds to thousands of beads: the
@@ -323,7 +363,7 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
                     acc[e] = sum;
                     cmp[e] = c;
                 } else {
-                    acc[e] = a;
+                    acc[e] = mk(closed(a.x), closed(a.y));
                 }
             }
             __syncthreads();
@@ -431,7 +471,7 @@ __device__ void rotate_sets_f(const T *rf, const int *foff, int p, const cpx<T> 
         const T *za = rf + foff[n];
         const T c = za[2 * m], sn = za[2 * m + 1];
         const cpx<T> v = src[st * nc + i];
-        tmp[e] = mk(fma(c, v.x, -sn * v.y), fma(sn, v.x, c * v.y));
+        tmp[e] = mk(mul_diff(c, v.x, sn, v.y), mul_diff(sn, v.x, -c, v.y));
     }
     __syncthreads();
     for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
@@ -443,17 +483,19 @@ __device__ void rotate_sets_f(const T *rf, const int *foff, int p, const cpx<T> 
         if (QUARTER) {
             // middle angle pi/2 (the frame rotations): the y blocks are checkerboards
             // (checked when the tables are built); Im of m = 0 is zero for real fields
-            for (int k = (m + n) & 1; k < q; k += 2) re = fma(yre[k], in[k].x, re);
+            for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k], in[k].x);
             if (m > 0)
-                for (int k = 1 + ((m + n) & 1); k < q; k += 2) im = fma(yim[k], in[k].y, im);
+                for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k], in[k].y);
         } else {
             for (int k = 0; k < q; ++k) {
-                re = fma(yre[k], in[k].x, re);
-                im = fma(yim[k], in[k].y, im);
+                macc(re, yre[k], in[k].x);
+                macc(im, yim[k], in[k].y);
             }
         }
+        re = closed(re);
+        im = closed(im);
         const T c = o[2 * q + 2 * m], sn = o[2 * q + 2 * m + 1];
-        dst[st * nc + i] = mk(fma(c, re, -sn * im), fma(sn, re, c * im));
+        dst[st * nc + i] = mk(mul_diff(c, re, sn, im), mul_diff(sn, re, -c, im));
     }
 }
 
@@ -488,8 +530,12 @@ __global__ void k_m2m_child(int c0, int pb0, DevTables<T> D, const int *par, con
         int n = deg_of(i), m = i - tri(n, 0);
         const T *z = D.zm2m + size_t(i) * P1;
         cpx<T> a = mk<T>(0, 0);
-        for (int k = m; k <= n; ++k) a += z[k] * Y[st * nc + tri(k, m)];
-        X[e] = a;
+        for (int k = m; k <= n; ++k) {
+            const cpx<T> y = Y[st * nc + tri(k, m)];
+            macc(a.x, z[k], y.x);
+            macc(a.y, z[k], y.y);
+        }
+        X[e] = mk(closed(a.x), closed(a.y));
     }
     __syncthreads();
     rotate_sets_f(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
@@ -548,8 +594,12 @@ __global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const 
         int n = deg_of(i), m = i - tri(n, 0);
         const T *z = D.zl2l + size_t(i) * P1;
         cpx<T> a = mk<T>(0, 0);
-        for (int k = n; k <= p; ++k) a += z[k] * Y[st * nc + tri(k, m)];
-        X[e] = a;
+        for (int k = n; k <= p; ++k) {
+            const cpx<T> y = Y[st * nc + tri(k, m)];
+            macc(a.x, z[k], y.x);
+            macc(a.y, z[k], y.y);
+        }
+        X[e] = mk(closed(a.x), closed(a.y));
     }
     __syncthreads();
     rotate_sets_f(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
@@ -608,17 +658,17 @@ __global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *X
                 T evx = 0, evy = 0, odx = 0, ody = 0;
                 for (int n = m; n <= p; n += 2) {
                     const int i = tri(n, m);
-                    evx = fma(cc[i], Ms[i].x, evx);
-                    evy = fma(cc[i], Ms[i].y, evy);
+                    macc(evx, cc[i], Ms[i].x);
+                    macc(evy, cc[i], Ms[i].y);
                 }
                 for (int n = m + 1; n <= p; n += 2) {
                     const int i = tri(n, m);
-                    odx = fma(cc[i], Ms[i].x, odx);
-                    ody = fma(cc[i], Ms[i].y, ody);
+                    macc(odx, cc[i], Ms[i].x);
+                    macc(ody, cc[i], Ms[i].y);
                 }
-                const T sg = m == 0 ? T(1) : (((m >> 1) & 1) ? T(-2) : T(2));   // 2 i^m up to i for odd m
-                AE[k * NS + m * kSets + st] = mk(sg * evx, sg * evy);
-                AO[k * NS + m * kSets + st] = mk(sg * odx, sg * ody);
+                const float sg = m == 0 ? 1.f : (((m >> 1) & 1) ? -2.f : 2.f);   // 2 i^m up to i for odd m
+                AE[k * NS + m * kSets + st] = mk(scale2(sg, closed(evx)), scale2(sg, closed(evy)));
+                AO[k * NS + m * kSets + st] = mk(scale2(sg, closed(odx)), scale2(sg, closed(ody)));
             }
         }
         __syncthreads();
@@ -658,10 +708,10 @@ __global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *X
     #pragma unroll
                     for (int st = 0; st < kSets; ++st) {
                         const cpx<T> a = ae[m * kSets + st], o = ao[m * kSets + st];
-                        pe[st] = fma(a.x, z.x, pe[st]);
-                        qe[st] = fma(a.y, z.y, qe[st]);
-                        po[st] = fma(o.x, z.x, po[st]);
-                        qo[st] = fma(o.y, z.y, qo[st]);
+                        macc(pe[st], a.x, z.x);
+                        macc(qe[st], a.y, z.y);
+                        macc(po[st], o.x, z.x);
+                        macc(qo[st], o.y, z.y);
                     }
                 }
                 // real parts: even m; + direction A = AE + AO, - direction AE - AO
@@ -686,10 +736,10 @@ __global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *X
     #pragma unroll
                     for (int st = 0; st < kSets; ++st) {
                         const cpx<T> a = ae[m * kSets + st], o = ao[m * kSets + st];
-                        pe[st] = fma(a.x, z.x, pe[st]);
-                        qe[st] = fma(a.y, z.y, qe[st]);
-                        po[st] = fma(o.x, z.x, po[st]);
-                        qo[st] = fma(o.y, z.y, qo[st]);
+                        macc(pe[st], a.x, z.x);
+                        macc(qe[st], a.y, z.y);
+                        macc(po[st], o.x, z.x);
+                        macc(qo[st], o.y, z.y);
                     }
                     idx += step2;
                     if (idx >= Mk) idx -= Mk;
@@ -861,12 +911,14 @@ __global__ void k_x2x(const int *parents, DevTables<T> D, const int *coll, const
             if constexpr (FAC) {
                 const cpx<T> a = sX[vox[z] + j], b = sY[voy[z] + j];
                 const T c = sZ[voz[z] + j];
-                sh = mk(c * fmaf(a.x, b.x, -a.y * b.y), c * fmaf(a.x, b.y, a.y * b.x));
+                sh = mk(c * mul_diff(a.x, b.x, a.y, b.y), c * mul_diff(a.x, b.y, -a.y, b.x));
             } else {
                 sh = D.shift[size_t(vsh[z]) * S + j];
             }
-            ga.x = fma(-x.y, sh.y, fma(x.x, sh.x, ga.x));
-            ga.y = fma(x.y, sh.x, fma(x.x, sh.y, ga.y));
+            macc(ga.x, x.x, sh.x);
+            macc(ga.x, -x.y, sh.y);
+            macc(ga.y, x.x, sh.y);
+            macc(ga.y, x.y, sh.x);
             const int mask = vend[z];   // block-uniform
             if (mask) {
 #pragma unroll
@@ -995,14 +1047,16 @@ __global__ void k_x2x4(const int *parents, DevTables<T> D, const int *coll, cons
             if constexpr (FAC) {
                 const cpx<T> a = sX[vox[z] + j], b = sY[voy[z] + j];
                 const T c = sZ[voz[z] + j];
-                sh = mk(c * fma(a.x, b.x, -a.y * b.y), c * fma(a.x, b.y, a.y * b.x));
+                sh = mk(c * mul_diff(a.x, b.x, a.y, b.y), c * mul_diff(a.x, b.y, -a.y, b.x));
             } else {
                 sh = D.shift[size_t(vsh[z]) * S + j];
             }
 #pragma unroll
             for (int k = 0; k < kSets; ++k) {
-                ga[k].x = fma(-x[k].y, sh.y, fma(x[k].x, sh.x, ga[k].x));
-                ga[k].y = fma(x[k].y, sh.x, fma(x[k].x, sh.y, ga[k].y));
+                macc(ga[k].x, x[k].x, sh.x);
+                macc(ga[k].x, -x[k].y, sh.y);
+                macc(ga[k].y, x[k].x, sh.y);
+                macc(ga[k].y, x[k].y, sh.x);
             }
             const int mask = vend[z];   // block-uniform
             if (mask) {
@@ -1347,10 +1401,10 @@ __global__ void k_x2l(int b0, int nb, DevTables<T> D, const cpx<T> *Xi, cpx<T> *
                 int idx = 0;
                 for (int u = u0; u < u1; ++u) {
                     const cpx<T> r = rt[idx];
-                    bpx = fma(xp[u], r.x, bpx);
-                    bpy = fma(-yp[u], r.y, bpy);
-                    bmx = fma(xm[u], r.x, bmx);
-                    bmy = fma(-ym[u], r.y, bmy);
+                    macc(bpx, xp[u], r.x);
+                    macc(bpy, -yp[u], r.y);
+                    macc(bmx, xm[u], r.x);
+                    macc(bmy, -ym[u], r.y);
                     idx += mm;
                     if (idx >= Mk) idx -= Mk;
                 }
@@ -1368,10 +1422,10 @@ __global__ void k_x2l(int b0, int nb, DevTables<T> D, const cpx<T> *Xi, cpx<T> *
                 for (int k = 0; k < s; ++k) {
                     T c = D.x2l_c[size_t(k) * nc + i];
                     cpx<T> bb = Bs[k * P1 + m];
-                    a.x = fma(c, bb.x, a.x);
-                    a.y = fma(c, bb.y, a.y);
+                    macc(a.x, c, bb.x);
+                    macc(a.y, c, bb.y);
                 }
-                Lf[st * nc + i] = mul_ipow(mk(2 * a.x, 2 * a.y), m + (m & 1));
+                Lf[st * nc + i] = mul_ipow(mk(scale2(2.f, closed(a.x)), scale2(2.f, closed(a.y))), m + (m & 1));
             }
         }
         __syncthreads();
@@ -1516,8 +1570,8 @@ constexpr int kNF2 = 6;   // evaluated per bead in the one-expansion-per-compone
 // Build the 18 evaluation expansions of Eq. (2.8) from 4 source expansions.
 // IRREG = multipole source (degrees grow by one per derivative), else local.
 template <typename T, bool IRREG>
-__device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<T> *tmp, double cbx, double cby,
-                               double cbz, const Lad<T> &G) {
+__device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<T> *tmp, T cbx, T cby, T cbz,
+                               const Lad<T> &G) {
     const int st = ncoef(P);
     // 0..2 values
     for (int i = threadIdx.x; i < 3 * st; i += blockDim.x) {
@@ -1532,16 +1586,16 @@ __device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<
     }
     __syncthreads();
     // 12..14: G4'_a = dL4_a - sum_k cb_k dL_k,a ; tmp[3] = L_C = dxL1 + dyL2 + dzL3
-    T cb[3] = {T(cbx), T(cby), T(cbz)};
+    const T cb[3] = {cbx, cby, cbz};
     for (int i = threadIdx.x; i < st; i += blockDim.x) {
         for (int a = 0; a < 3; ++a) {
             cpx<T> g = tmp[a * st + i];
             for (int k = 0; k < 3; ++k) {
                 cpx<T> v = EV[(3 + 3 * k + a) * st + i];
-                g.x -= cb[k] * v.x;
-                g.y -= cb[k] * v.y;
+                macc(g.x, -cb[k], v.x);
+                macc(g.y, -cb[k], v.y);
             }
-            EV[(12 + a) * st + i] = g;
+            EV[(12 + a) * st + i] = mk(closed(g.x), closed(g.y));
         }
         cpx<T> lc = EV[(3 + 0) * st + i] + EV[(3 + 3 + 1) * st + i] + EV[(3 + 6 + 2) * st + i];
         tmp[3 * st + i] = lc;
@@ -1574,6 +1628,9 @@ __global__ void k_far_eval(const int *leaves, DevTables<T> D, const int *beg, co
     const double C1 = sc.pc[sy].C1, C2 = sc.pc[sy].C2, icube = sc.pc[sy].icube;
     double c0x = sc.cube[4 * sy], c0y = sc.cube[4 * sy + 1], c0z = sc.cube[4 * sy + 2];
     double cbx = ctr[3 * b], cby = ctr[3 * b + 1], cbz = ctr[3 * b + 2];
+    float c3b[9];
+    if constexpr (kIsDf<T>)
+        for (int k = 0; k < 9; ++k) c3b[k] = sc.c3[9 * size_t(b) + k];
     int j0 = beg[b], j1 = end[b];
     int nw = woff[li + 1] - woff[li];
     if (nw == 0) return;
@@ -1583,27 +1640,46 @@ __global__ void k_far_eval(const int *leaves, DevTables<T> D, const int *beg, co
         double x = act ? pos[j] : cbx, y = act ? pos[n + j] : cby, z = act ? pos[2 * n + j] : cbz;
         double u[3] = {0, 0, 0};
         for (int w = 0; w < nw; ++w) {
-            int C = w < 0 ? b : widx[woff[li] + w];
-            const cpx<T> *E = w < 0 ? L + size_t(C) * kSets * nc : M + size_t(C) * kSets * nc;
+            const int C = widx[woff[li] + w];
+            const cpx<T> *E = M + size_t(C) * kSets * nc;
             __syncthreads();
             for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) srcs[i] = E[i];
             __syncthreads();
             // origin of the source expansion's q4: its own centre (box origin) or the cube centre
-            const double ox = rb ? ctr[3 * C] : c0x, oy = rb ? ctr[3 * C + 1] : c0y, oz = rb ? ctr[3 * C + 2] : c0z;
-            if (w < 0) build_eval_set<T, false>(srcs, p, P, EV, tmp, cbx - ox, cby - oy, cbz - oz, G);
-            else build_eval_set<T, true>(srcs, p, P, EV, tmp, cbx - ox, cby - oy, cbz - oz, G);
-            double ih = icube * pow2i(lvl[C]);   // 1 / side[C], exactly
             T acc[kNE];
 #pragma unroll
-            for (int q = 0; q < kNE; ++q) acc[q] = 0;
-            T vx = T((x - ctr[3 * C]) * ih), vy = T((y - ctr[3 * C + 1]) * ih), vz = T((z - ctr[3 * C + 2]) * ih);
-            if (w < 0) eval_fields<T, kNE, false>(vx, vy, vz, p, EV, st, R.a, R.b, R.c, acc);
-            else eval_fields<T, kNE, true>(vx, vy, vz, P, EV, st, R.a, R.b, R.c, acc);
-            double xi[3] = {(x - cbx) * ih, (y - cby) * ih, (z - cbz) * ih};
-            for (int d = 0; d < 3; ++d) {
-                double v = double(acc[d]);
-                for (int k = 0; k < 3; ++k) v -= xi[k] * double(acc[3 + 3 * k + d]);
-                u[d] += C1 * ih * v + C1 * ih * ih * double(acc[12 + d]) - C2 * ih * ih * ih * double(acc[15 + d]);
+            for (int q = 0; q < kNE; ++q) acc[q] = T(0);
+            if constexpr (kIsDf<T>) {
+                // lengths in the split units; L4 and the C2 term carry their factors here
+                T cb[3], v[3], xi[3];
+                const double ihd = inv_side_u(sc.pc[sy], lvl[C]);
+                const T ihs = T(ihd);
+                for (int a = 0; a < 3; ++a) {
+                    cb[a] = rb ? coord_diff(c3b, sc.c3 + 9 * size_t(C), a) : dfl3(c3b[3 * a], c3b[3 * a + 1], c3b[3 * a + 2]);
+                    v[a] = act ? coord_diff(sc.p3, n, j, a, sc.c3 + 9 * size_t(C)) * ihs : T(1);
+                    xi[a] = act ? coord_diff(sc.p3, n, j, a, c3b) * ihs : T(0);
+                }
+                build_eval_set<T, true>(srcs, p, P, EV, tmp, cb[0], cb[1], cb[2], G);
+                eval_fields<T, kNE, true>(v[0], v[1], v[2], P, EV, st, R.a, R.b, R.c, acc);
+                const T cc = T(double(sc.pc[sy].d_k23h) + double(sc.pc[sy].d_k23l)) * ihs;
+                const double w1 = sc.pc[sy].C1 * sc.pc[sy].d_xs * force_unit(sc.fmax[sy]) * ihd;
+                for (int d = 0; d < 3; ++d) {
+                    T t = acc[d] + ihs * (acc[12 + d] - cc * acc[15 + d]);
+                    for (int k = 0; k < 3; ++k) t -= xi[k] * acc[3 + 3 * k + d];
+                    u[d] += w1 * double(t);
+                }
+            } else {
+                const double ox = rb ? ctr[3 * C] : c0x, oy = rb ? ctr[3 * C + 1] : c0y, oz = rb ? ctr[3 * C + 2] : c0z;
+                build_eval_set<T, true>(srcs, p, P, EV, tmp, T(cbx - ox), T(cby - oy), T(cbz - oz), G);
+                double ih = icube * pow2i(lvl[C]);   // 1 / side[C], exactly
+                T vx = T((x - ctr[3 * C]) * ih), vy = T((y - ctr[3 * C + 1]) * ih), vz = T((z - ctr[3 * C + 2]) * ih);
+                eval_fields<T, kNE, true>(vx, vy, vz, P, EV, st, R.a, R.b, R.c, acc);
+                double xi[3] = {(x - cbx) * ih, (y - cby) * ih, (z - cbz) * ih};
+                for (int d = 0; d < 3; ++d) {
+                    double v = double(acc[d]);
+                    for (int k = 0; k < 3; ++k) v -= xi[k] * double(acc[3 + 3 * k + d]);
+                    u[d] += C1 * ih * v + C1 * ih * ih * double(acc[12 + d]) - C2 * ih * ih * ih * double(acc[15 + d]);
+                }
             }
         }
         if (act)
@@ -1632,20 +1708,34 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
     __syncthreads();
     int sy = bsys[b];
     cpx<T> *EV = EVg + size_t(li) * kNE * nc;
-    if (rb) build_eval_set<T, false>(srcs, p, p, EV, tmp, 0.0, 0.0, 0.0, G);
-    else
-        build_eval_set<T, false>(srcs, p, p, EV, tmp, ctr[3 * b] - sc.cube[4 * sy],
-                                 ctr[3 * b + 1] - sc.cube[4 * sy + 1], ctr[3 * b + 2] - sc.cube[4 * sy + 2], G);
+    if (rb) {
+        build_eval_set<T, false>(srcs, p, p, EV, tmp, T(0), T(0), T(0), G);
+    } else if constexpr (kIsDf<T>) {
+        const float *c = sc.c3 + 9 * size_t(b);
+        build_eval_set<T, false>(srcs, p, p, EV, tmp, dfl3(c[0], c[1], c[2]), dfl3(c[3], c[4], c[5]),
+                                 dfl3(c[6], c[7], c[8]), G);
+    } else {
+        build_eval_set<T, false>(srcs, p, p, EV, tmp, T(ctr[3 * b] - sc.cube[4 * sy]),
+                                 T(ctr[3 * b + 1] - sc.cube[4 * sy + 1]), T(ctr[3 * b + 2] - sc.cube[4 * sy + 2]), G);
+    }
     // Fold the terms of Eq. (2.8) that are not multiplied by a coordinate into
     // fields 0..2 (in units of C1/h):  L_d + h^-1 dL4'_d - (C2/C1) h^-2 dL_C,d.
     // The bead evaluation then needs fields 0..11 only.
     const double ih = sc.pc[sy].icube * pow2i(lvl[b]);
-    const T c4 = T(ih), cc = T(sc.pc[sy].C2 / sc.pc[sy].C1 * ih * ih);
+    T c4 = T(ih), cc = T(sc.pc[sy].C2 / sc.pc[sy].C1 * ih * ih);
+    if constexpr (kIsDf<T>) {   // lengths in the split units: C2 / C1 = 2a^2/3 there
+        const double ihs = inv_side_u(sc.pc[sy], lvl[b]);
+        c4 = T(ihs);
+        cc = T((double(sc.pc[sy].d_k23h) + double(sc.pc[sy].d_k23l)) * ihs * ihs);
+    }
     for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x) {
         int d = i / nc, c = i - d * nc;
         cpx<T> v = EV[d * nc + c], g4 = EV[(12 + d) * nc + c], gc = EV[(15 + d) * nc + c];
-        v.x = fma(c4, g4.x, fma(-cc, gc.x, v.x));
-        v.y = fma(c4, g4.y, fma(-cc, gc.y, v.y));
+        macc(v.x, -cc, gc.x);
+        macc(v.x, c4, g4.x);
+        macc(v.y, -cc, gc.y);
+        macc(v.y, c4, g4.y);
+        v = mk(closed(v.x), closed(v.y));
         EV[d * nc + c] = v;
     }
     int nf = kNF;
@@ -1689,7 +1779,7 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
         int c = i % nc, n = deg_of(c);
         if (c != tri(n, 0)) {
             cpx<T> v = EV[i];
-            EV[i] = mk(2 * v.x, 2 * v.y);
+            EV[i] = mk(scale2(2.f, v.x), scale2(2.f, v.y));
         }
     }
 }
@@ -1710,12 +1800,30 @@ __global__ void k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
         const int p = D.p, nc = ncoef(p);
         int sy = bsys[b];
         const double C1 = sc.pc[sy].C1;
+        T acc[NF];
+#pragma unroll
+        for (int q = 0; q < NF; ++q) acc[q] = T(0);
+        if constexpr (kIsDf<T>) {
+            const float *c = sc.c3 + 9 * size_t(b);
+            const double ihd = inv_side_u(sc.pc[sy], lvl[b]);
+            const T ihs = T(ihd);
+            const T xi[3] = {coord_diff(sc.p3, n, i, 0, c) * ihs, coord_diff(sc.p3, n, i, 1, c) * ihs,
+                             coord_diff(sc.p3, n, i, 2, c) * ihs};
+            eval_fields<T, NF, false, true>(xi[0], xi[1], xi[2], p, EVg + size_t(li) * kNE * nc, nc, D.rec_a, D.rec_b,
+                                            D.rec_c, acc);
+            const double w1 = C1 * sc.pc[sy].d_xs * force_unit(sc.fmax[sy]) * ihd;
+            const T r2 = fma(xi[2], xi[2], fma(xi[1], xi[1], xi[0] * xi[0]));
+            for (int d = 0; d < 3; ++d) {
+                T v = acc[d];
+                if constexpr (NF == kNF2) v -= r2 * acc[3 + d];
+                else
+                    for (int k = 0; k < 3; ++k) v -= xi[k] * acc[3 + 3 * k + d];
+                u[d] = w1 * double(v);
+            }
+        } else {
         const double ih = sc.pc[sy].icube * pow2i(lvl[b]);   // 1 / side[b], exactly
         double xi[3] = {(pos[i] - ctr[3 * b]) * ih, (pos[n + i] - ctr[3 * b + 1]) * ih,
                         (pos[2 * n + i] - ctr[3 * b + 2]) * ih};
-        T acc[NF];
-#pragma unroll
-        for (int q = 0; q < NF; ++q) acc[q] = 0;
         eval_fields<T, NF, false, true>(T(xi[0]), T(xi[1]), T(xi[2]), p, EVg + size_t(li) * kNE * nc, nc, D.rec_a,
                                         D.rec_b, D.rec_c, acc);
         if constexpr (NF == kNF2) {
@@ -1729,6 +1837,7 @@ __global__ void k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
                 for (int k = 0; k < 3; ++k) v -= xi[k] * double(acc[3 + 3 * k + d]);
                 u[d] = C1 * ih * v;
             }
+        }
         }
     }
     for (int d = 0; d < 3; ++d) ufar[3 * i + d] = u[d];
@@ -1883,22 +1992,24 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     int n2 = nbx - b2;
     // origin of q4 (RPY charges only; the Laplace diagnostic takes its charges as given):
     // each expansion's own box centre by default in the FP32 form at 6 digits, the cube
-    // centre otherwise (in FP64, and at 3 digits, its rounding stays far below the setting)
+    // centre otherwise (in the FP64 form, and at 3 digits, its rounding stays far below the setting)
     const int fl = t.params.flags;
     const int rb = lapq ? 0
                         : (fl & RPY_FLAG_BOX_ORIGIN) ? 1
                         : (fl & RPY_FLAG_CUBE_ORIGIN) ? 0
                         : (sizeof(T) == 4 && t.params.digits >= 6);
+    // box sides in the units of the expansions' lengths
+    const double *side = kIsDf<T> ? t.side_u : t.b_side;
     // upward pass
     size_t sp = smem_p2x<T>(p, 128);
     RPY_TRY(set_smem(k_p2x<T, 0>, sp));
     RPY_TRY(set_smem(k_p2x<T, 1>, sp));
-    k_p2x<T, 0><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, t.b_side, t.b_level, t.b_leaf,
+    k_p2x<T, 0><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
                                      t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, M, rb);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
     prof_mark(t, RPY_STAGE_M2M, st);
-    // FP64: rotation-based M2M and L2L (fewer FP64 operations).  FP32: the dense
+    // FP64 form: rotation-based M2M and L2L (fewer operations).  FP32: the dense
     // operators below p = 12, the rotation forms (one child per block) from there
     const bool rot_l = sizeof(T) == 8 || p >= 12;
     size_t smr2 = sizeof(cpx<T>) * 3 * kSets * nc;
@@ -1906,8 +2017,10 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     size_t smd = sizeof(T) * kSets * Dd;
     RPY_TRY(set_smem(k_l2l_rot<T>, smr2));
     RPY_TRY(set_smem(k_m2m_child<T>, smr2));
-    RPY_TRY(set_smem(k_m2m<T>, smd));
-    RPY_TRY(set_smem(k_l2l<T>, smd));
+    if constexpr (sizeof(T) == 4) {
+        RPY_TRY(set_smem(k_m2m<T>, smd));
+        RPY_TRY(set_smem(k_l2l<T>, smd));
+    }
     for (int l = t.nlevels - 2; l >= 2; --l) {
         int lb = t.level_off[l], ln = t.level_off[l + 1] - lb;
         if (ln > 0) {
@@ -1917,12 +2030,12 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
                 if (cn > 0) {
                     if (!t.m2m_scratch) return RPY_ERR_INTERNAL;
                     cpx<T> *Sc = static_cast<cpx<T> *>(t.m2m_scratch);
-                    k_m2m_child<T><<<cn, 256, smr2, st>>>(cb, lb, D, t.b_parent, t.b_cell, t.b_side, rb, M, Sc);
+                    k_m2m_child<T><<<cn, 256, smr2, st>>>(cb, lb, D, t.b_parent, t.b_cell, side, rb, M, Sc);
                     k_m2m_sum<T><<<ln, 256, 0, st>>>(lb, kSets * nc, t.b_leaf, t.b_child, Sc, M);
                     RPY_LAUNCHED(2);
                 }
-            } else {
-                k_m2m<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_leaf, t.b_child, t.b_side, rb, M);
+            } else if constexpr (sizeof(T) == 4) {
+                k_m2m<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_leaf, t.b_child, side, rb, M);
                 RPY_LAUNCHED(1);
             }
         }
@@ -1946,39 +2059,32 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
         prof_mark(t, RPY_STAGE_X2X, st);
         if (t.n_x2x_par > 0) {
             dim3 g(t.n_x2x_par, 2 * nf);
-            // FP32 (and the box-origin form): the four sets of a wave in one thread.  FP32 with
-            // up to 256 stored waves: shifts from per-axis factors in shared memory (measured
-            // faster there; at more waves the shared memory costs occupancy and the table is
-            // faster)
-            if (sizeof(T) == 4 && !rb && D.S <= 256) {
-                // cube origin, few plane waves: one set per thread, shifts from per-axis factors
-                const size_t sxx = sizeof(T) * ((6 * D.S + 3) & ~3) + 2 * sizeof(cpx<T>) * 6 * D.S;
-                k_x2x<T, true><<<g, x2x_threads(D.S), sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf, Xo,
-                                                                 Xi, f0, nf);
-            } else if (sizeof(T) == 4 || rb) {
-                bool fac = false;
-                if constexpr (sizeof(T) == 4) {
-                    if (D.S > 256 && D.S <= 480) {
-                        // a producer warp stages the sources through shared memory by bulk copies
-                        // (measured faster than per-thread loads from 323 stored waves up; at 3 digits,
-                        // 134 waves, the per-thread loads below keep two to three blocks per SM and win)
-                        const size_t sxx = x2x_tma_smem(D.S);
-                        RPY_TRY(set_smem(k_x2x_tma, sxx));
-                        k_x2x_tma<<<g, (D.S + 31) / 32 * 32 + 32, sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child,
-                                                                             t.b_leaf, t.b_side, Xo, Xi, f0, nf, rb,
-                                                                             t.dev_status);
-                        fac = true;
-                    } else if (D.S <= 256) {
-                        const size_t sxx = sizeof(T) * ((6 * D.S + 3) & ~3) + 2 * sizeof(cpx<T>) * 6 * D.S;
+            if constexpr (sizeof(T) == 4) {
+                if (D.S > 256 && D.S <= 480) {
+                    // a producer warp stages the sources through shared memory by bulk copies
+                    // (measured faster than per-thread loads from 323 stored waves up; at 3 digits,
+                    // 134 waves, the per-thread loads below keep two to three blocks per SM and win)
+                    const size_t sxx = x2x_tma_smem(D.S);
+                    RPY_TRY(set_smem(k_x2x_tma, sxx));
+                    k_x2x_tma<<<g, (D.S + 31) / 32 * 32 + 32, sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
+                                                                         side, Xo, Xi, f0, nf, rb, t.dev_status);
+                } else if (D.S <= 256) {
+                    // shifts from per-axis factors in shared memory (measured faster there; at more
+                    // waves the shared memory costs occupancy and the table is faster)
+                    const size_t sxx = sizeof(T) * ((6 * D.S + 3) & ~3) + 2 * sizeof(cpx<T>) * 6 * D.S;
+                    if (rb)
                         k_x2x4<T, true><<<g, even_threads(D.S), sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child,
-                                                                           t.b_leaf, t.b_side, Xo, Xi, f0, nf, rb);
-                        fac = true;
-                    }
-                }
-                if (!fac) {
+                                                                           t.b_leaf, side, Xo, Xi, f0, nf, rb);
+                    else   // cube origin, few plane waves: one set per thread
+                        k_x2x<T, true><<<g, x2x_threads(D.S), sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
+                                                                         Xo, Xi, f0, nf);
+                } else {
                     k_x2x4<T, false><<<g, even_threads(D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                      t.b_side, Xo, Xi, f0, nf, rb);
+                                                                      side, Xo, Xi, f0, nf, rb);
                 }
+            } else if (rb) {
+                k_x2x4<T, false><<<g, even_threads(D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf, side,
+                                                                  Xo, Xi, f0, nf, rb);
             } else {
                 k_x2x<T, false><<<g, x2x_threads(D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf, Xo, Xi,
                                                                 f0, nf);
@@ -1998,7 +2104,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     }
     // X list
     prof_mark(t, RPY_STAGE_P2L, st);
-    k_p2x<T, 1><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, t.b_side, t.b_level, t.b_leaf,
+    k_p2x<T, 1><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
                                      t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, L, rb);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
@@ -2007,8 +2113,8 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     for (int l = 3; l < t.nlevels; ++l) {
         int lb = t.level_off[l], ln = t.level_off[l + 1] - lb;
         if (ln > 0) {
-            if (rot_l) k_l2l_rot<T><<<ln, 256, smr2, st>>>(lb, ln, D, t.b_parent, t.b_cell, t.b_side, rb, L);
-            else k_l2l<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_parent, t.b_cell, t.b_side, rb, L);
+            if (rot_l) k_l2l_rot<T><<<ln, 256, smr2, st>>>(lb, ln, D, t.b_parent, t.b_cell, side, rb, L);
+            else if constexpr (sizeof(T) == 4) k_l2l<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_parent, t.b_cell, side, rb, L);
             RPY_LAUNCHED(1);
         }
     }
@@ -2025,15 +2131,15 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
         RPY_LAUNCHED(1);
         const int ga = int((t.n + 127) / 128);
         if (per_comp)
-            k_eval_apply<T, kNF2><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, t.b_side, t.b_level,
+            k_eval_apply<T, kNF2><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, side, t.b_level,
                                                       t.b_sys, t.pos, sc, EVg, ufar);
         else
-            k_eval_apply<T, kNF><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, t.b_side, t.b_level,
+            k_eval_apply<T, kNF><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, side, t.b_level,
                                                      t.b_sys, t.pos, sc, EVg, ufar);
         RPY_LAUNCHED(1);
         size_t sf = smem_far<T>(p);
         RPY_TRY(set_smem(k_far_eval<T>, sf));
-        k_far_eval<T><<<t.nleaf, 64, sf, st>>>(t.leaves, D, t.b_begin, t.b_end, t.b_center, t.b_side, t.b_level,
+        k_far_eval<T><<<t.nleaf, 64, sf, st>>>(t.leaves, D, t.b_begin, t.b_end, t.b_center, side, t.b_level,
                                                 t.b_sys, t.w_off, t.w_idx, t.pos, t.n, sc, L, M, ufar, rb);
         RPY_LAUNCHED(1);
         RPY_CHECK(cudaGetLastError());
@@ -2049,7 +2155,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     return RPY_OK;
 }
 
-template int run_far_t<double>(Tree &, const DevTables<double> &, const double *, const double *, double *, double *,
+template int run_far_t<dfl>(Tree &, const DevTables<dfl> &, const double *, const double *, double *, double *,
                                const SysConst &, cudaStream_t);
 template int run_far_t<float>(Tree &, const DevTables<float> &, const double *, const double *, double *, double *,
                               const SysConst &, cudaStream_t);

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/rpyfmm.h"
+#include "rpy_dfl.h"
 
 #define RPY_HD __host__ __device__ __forceinline__
 
@@ -205,14 +206,37 @@ __host__ __device__ __forceinline__ double exp2_of_biased(int e) {
     return std::ldexp(1.0, e - 1023);
 #endif
 }
-// The double-float near field takes systems whose root side and largest force component (its high word, fmax)
-// lie within 2^-500 .. 2^500.
-__device__ __forceinline__ bool force_range_ok(int w) { return w >= (523 << 20) && w < (1523 << 20); }
-// 2^-e with 2^e > side >= 2^(e-1); 0 when side is out of range (or zero)
+// Lengths of the FP64 form's double-floats: multiples of 2^e with 2^e > side >= 2^(e-1) (near_unit = 2^-e).
 __device__ __forceinline__ double near_unit(double side) {
-    const int w = __double2hiint(side);
-    return force_range_ok(w) ? exp2_of_biased(2045 - (w >> 20)) : 0.0;
+    return exp2_of_biased(min(max(2045 - (__double2hiint(side) >> 20), 1), 2045));
 }
+// Forces: multiples of 2^e, e the exponent of the system's largest component (w its high word);
+// infinities and NaN keep their values.
+__device__ __forceinline__ int force_exp(int w) { return (w >> 20) >= 2047 ? 1023 : max(w >> 20, 1); }
+__device__ __forceinline__ double force_unit(int w) { return exp2_of_biased(force_exp(w)); }
+__device__ __forceinline__ double force_scale(int w) { return exp2_of_biased(2046 - force_exp(w)); }
+// The double-float near field takes systems whose root side and largest force lie within 2^-500 .. 2^500.
+__device__ __forceinline__ bool near_range_ok(int w) { return w >= (523 << 20) && w < (1523 << 20); }
+// 1 / side of a box of level l in the units of lengths
+__device__ __forceinline__ double inv_side_u(const PairConst &pc, int l) {
+    return pc.icube * exp2_of_biased(2046 - (__double2hiint(pc.d_xs) >> 20)) * __hiloint2double((1023 + l) << 20, 0);
+}
+
+// A coordinate of the FP64 form, or the difference of two, from its three floats (k_split3), normalised.
+__device__ __forceinline__ dfl dfl3(float h, float m, float l) {
+    const float s = __fadd_rn(h, m);   // h = 0 or |h| >= |m|, and no rounding below 2^-46
+    return dfl(s, __fadd_rn(__fsub_rn(m, __fsub_rn(s, h)), l));
+}
+__device__ __forceinline__ dfl coord_diff(const float *p3, int64_t n, int64_t j, int a, const float *c) {
+    return dfl3(__fsub_rn(p3[3 * a * n + j], c[3 * a]), __fsub_rn(p3[(3 * a + 1) * n + j], c[3 * a + 1]),
+                __fsub_rn(p3[(3 * a + 2) * n + j], c[3 * a + 2]));
+}
+__device__ __forceinline__ dfl coord_diff(const float *b, const float *c, int a) {
+    return dfl3(__fsub_rn(b[3 * a], c[3 * a]), __fsub_rn(b[3 * a + 1], c[3 * a + 1]),
+                __fsub_rn(b[3 * a + 2], c[3 * a + 2]));
+}
+template <typename T> constexpr bool kIsDf = false;
+template <> inline constexpr bool kIsDf<dfl> = true;
 
 struct Tree {
     int device = 0;
@@ -275,6 +299,8 @@ struct Tree {
     float *p32 = nullptr;             // FP32 form: sorted positions as hi + lo floats, [6][n] (x,y,z hi; x,y,z lo)
     float *f32 = nullptr;             // FP32 form: sorted forces [3][n]
     float *p3 = nullptr;              // FP64 form: sorted positions as three floats per coordinate [9][n]
+    float *c3 = nullptr;              // FP64 form: box centres split like p3 [nbox][9]
+    double *side_u = nullptr;         // FP64 form: box sides in units of p3 [nbox]
     float *f2 = nullptr;              // FP64 form: sorted forces as double-floats [6][n]
     int *sys_fmax = nullptr;          // FP64 form: [nsys] high word of the largest force component's magnitude
     double *u_near = nullptr, *u_far = nullptr, *u_dir = nullptr;   // sorted [n][3]
@@ -293,7 +319,7 @@ struct Tree {
     // tables
     const OpTables *tabs = nullptr;   // the cached host tables of (p, quadrature rule); never freed
     void *dtabs_mem = nullptr;        // one device block holding all tables
-    DevTables<double> dt64{};
+    DevTables<dfl> dt64{};
     DevTables<float> dt32{};
     // device memory: blocks in use, and free blocks kept for the next rebuild
     struct Block {
@@ -344,6 +370,8 @@ struct SysConst {
     const double *a;      // [nsys]
     const double *s;      // [nsys] kT/eta
     const PairConst *pc;  // [nsys]
+    const float *p3, *c3, *f2;   // FP64 form: split positions, box centres and forces
+    const int *fmax;             // FP64 form: [nsys] high word of the largest force component
 };
 
 // 2^l as a double, by its bit pattern (0 <= l < 1000)

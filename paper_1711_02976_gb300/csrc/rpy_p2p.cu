@@ -210,27 +210,41 @@ __device__ __noinline__ void near64(unsigned char *smem, int tb, int te, int u0,
 // exponent of the root cube's side, relative to the cube's centre: h a multiple of 2^-23 and m of 2^-46, so
 // that the differences of two h's and of two m's are exact in FP32, and l the rest, rounded
 // at 2^-71: the difference of two FP64 coordinates is kept to its last bit.
-__global__ void k_split3(const double *pos, const int *bead_sys, const double *cube, int64_t n, float *p3) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double *c = cube + 4 * bead_sys[i];
-    const double xs = near_unit(c[3]);
+__device__ __forceinline__ void split3(double x, double c, double xs, float &fh, float &fm, float &fl) {
+    const double d = x - c, bb = d - x, err = (x - (d - bb)) + (-c - bb);   // d + err = x - c exactly
+    const double v = d * xs;
+    const double h = (v + 805306368.0) - 805306368.0;   // 1.5 * 2^29: ulp 2^-23
+    const double r = v - h;
+    const double m = (r + 96.0) - 96.0;                 // 1.5 * 2^6: ulp 2^-46
+    fh = float(h);
+    fm = float(m);
+    fl = float((r - m) + err * xs);
+}
+
+// The beads [9][n] and the box centres [nbox][9], and the box sides in the same units.
+__global__ void k_split3(const double *pos, const int *bead_sys, const double *cube, int64_t n, const double *ctr,
+                         const double *side, const int *bsys, int nbox, float *p3, float *c3, double *side_u) {
+    int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i < n) {
+        const double *c = cube + 4 * bead_sys[i];
+        const double xs = near_unit(c[3]);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double x = pos[a * n + i], d = x - c[a];
-        const double bb = d - x, err = (x - (d - bb)) + (-c[a] - bb);   // d + err = x - c exactly
-        const double v = d * xs;
-        const double h = (v + 805306368.0) - 805306368.0;   // 1.5 * 2^29: ulp 2^-23
-        const double r = v - h;
-        const double m = (r + 96.0) - 96.0;                 // 1.5 * 2^6: ulp 2^-46
-        p3[(3 * a) * n + i] = float(h);
-        p3[(3 * a + 1) * n + i] = float(m);
-        p3[(3 * a + 2) * n + i] = float((r - m) + err * xs);
+        for (int a = 0; a < 3; ++a)
+            split3(pos[a * n + i], c[a], xs, p3[3 * a * n + i], p3[(3 * a + 1) * n + i], p3[(3 * a + 2) * n + i]);
+        return;
     }
+    i -= n;
+    if (i >= nbox) return;
+    const double *c = cube + 4 * bsys[i];
+    const double xs = near_unit(c[3]);
+    side_u[i] = side[i] * xs;
+    for (int a = 0; a < 3; ++a)
+        split3(ctr[3 * i + a], c[a], xs, c3[9 * i + 3 * a], c3[9 * i + 3 * a + 1], c3[9 * i + 3 * a + 2]);
 }
 
 int split_positions_f64(Tree &t, cudaStream_t st) {
-    k_split3<<<unsigned((t.n + 255) / 256), 256, 0, st>>>(t.pos, t.bead_sys, t.sys_cube, t.n, t.p3);
+    k_split3<<<unsigned((t.n + t.nbox + 255) / 256), 256, 0, st>>>(t.pos, t.bead_sys, t.sys_cube, t.n, t.b_center,
+                                                                   t.b_side, t.b_sys, t.nbox, t.p3, t.c3, t.side_u);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
     return RPY_OK;
@@ -240,9 +254,7 @@ int split_positions_f64(Tree &t, cudaStream_t st) {
 __global__ void k_split_force(const double *fs, const int *bead_sys, const int *fmax, int64_t n, float *f2) {
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int w = fmax[bead_sys[i]];
-    if (!force_range_ok(w)) return;   // near64 takes this system
-    const double sc = exp2_of_biased(2046 - (w >> 20));
+    const double sc = force_scale(fmax[bead_sys[i]]);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double v = fs[a * n + i] * sc;
@@ -420,7 +432,7 @@ __global__ void __launch_bounds__(kDfThreads, 2)
     const int u0 = uoff[li], u1 = uoff[li + 1];
     const PairConst &pc = sc.pc[sys];
     const int fw = fmax[sys];
-    if (!pc.d_ok || !force_range_ok(fw) || lvl[b] > kDfMaxLevel) {
+    if (!pc.d_ok || !near_range_ok(fw) || lvl[b] > kDfMaxLevel) {
         near64(smem_raw, tb, te, u0, u1, beg, end, uidx, pos, fs, n, pc, add_self, out);
         return;
     }
@@ -559,7 +571,7 @@ __global__ void __launch_bounds__(kDfThreads, 2)
     }
     __syncthreads();
     // one thread per (component, target) adds the groups in order
-    const double unit = pc.cf * pc.d_xs * exp2_of_biased(fw >> 20), co = pc.co;
+    const double unit = pc.cf * pc.d_xs * force_unit(fw), co = pc.co;
     const bool any = *any64 != 0;
     for (int q = threadIdx.x; q < 3 * nt; q += kDfThreads) {
         const int c = q / nt, tt = q - c * nt, it = tb + tt;

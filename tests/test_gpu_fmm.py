@@ -396,6 +396,28 @@ def test_fp32_precision_form_3digit():
     _check(sysm.pos, sysm.f, sysm.a, sysm.s, 3, 1e-3, leaf_cap=40, precision=rp.RPY_FP32)
 
 
+@pytest.mark.parametrize("digits,n,flags", [(3, 3000, 0), (6, 9001, 0), (6, 9001, rp.RPY_FLAG_BOX_ORIGIN),
+                                            (6, 9001, rp.RPY_FLAG_EVAL_PER_POTENTIAL), (9, 9001, 0)])
+def test_fp64_far_field_in_any_units(digits, n, flags):
+    """The FP64 form's expansions are double-floats in units of the root cube and of the largest force:
+    lengths scaled by a power of two and forces by another (far outside the FP32 range) scale
+    every result exactly; a factor that is not a power of two changes it by rounding only (2^-48 per operation,
+    thousands of them per velocity: 1e-11)."""
+    sysm = synth.sphere_plus_cube(n, 33, 1e-3)
+    kw = dict(leaf_cap=20, direct_w=-1, direct_x=-1, flags=flags)
+    u0, t0 = matvec(sysm.pos, sysm.f, sysm.a, sysm.s, digits, **kw)
+    st = rp.rpy_tree_stats(t0)
+    assert st["n_wlist"] > 0 and st["n_xlist"] > 0 and st["n_dlist"] == 0
+    for ln, fo in ((2.0 ** -40, 2.0 ** -300), (2.0 ** 70, 2.0 ** 400), (1.0, 2.0 ** -900)):
+        u, _ = matvec(ln * sysm.pos, fo * sysm.f, ln * sysm.a, ln * sysm.s, digits, **kw)
+        if fo > 2.0 ** -500:
+            assert np.array_equal(u, fo * u0), (ln, fo)   # s / a unchanged: velocities scale with the forces
+        else:   # forces below the range of the double-float near field: FP64 there
+            assert oracle.rel_l2(u / fo, u0) < 1e-11
+    u, _ = matvec(3.7e-9 * sysm.pos, 4.1e-12 * sysm.f, 3.7e-9 * sysm.a, 3.7e-9 * sysm.s, digits, **kw)
+    assert oracle.rel_l2(u / 4.1e-12, u0) < 1e-11
+
+
 # ---------------------------------------------------------------- edge cases
 
 @pytest.mark.parametrize("precision", [rp.RPY_FP64, rp.RPY_FP32])
