@@ -235,12 +235,34 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
     putT(h.lad);      // 23
     putT(h.orot_fwd); // 24
     putT(h.orot_bwd); // 25
-    putT(h.zm2m);     // 26
-    putT(h.zl2l);     // 27
-    putT(h.frot_fwd); // 28
-    putT(h.frot_bwd); // 29
-    putT(h.forot_fwd);// 30
-    putT(h.forot_bwd);// 31
+    auto put_transposed = [&](const std::vector<double> &v) {   // [coefficient][k] -> [k][coefficient]
+        const size_t P1 = size_t(h.p) + 1, nc = v.size() / P1;
+        std::vector<double> w(v.size());
+        for (size_t i = 0; i < nc; ++i)
+            for (size_t k = 0; k < P1; ++k) w[k * nc + i] = v[i * P1 + k];
+        putT(w);
+    };
+    put_transposed(h.zm2m);     // 26
+    put_transposed(h.zl2l);     // 27
+    // factored rotations: the y blocks as [k][m] where the kernels read them so (y_by_column)
+    auto put_factored = [&](const std::vector<double> &v) {
+        std::vector<double> w(v);
+        const int FL = h.frot_off.back();
+        for (size_t r = 0; y_by_column(sizeof(T), h.p) && r < v.size(); r += FL)
+            for (int n = 0; n <= h.p; ++n) {
+                const int q = n + 1;
+                for (int half = 0; half < 2; ++half) {   // real and imaginary block
+                    const size_t o = r + h.frot_off[n] + 4 * q + half * q * q;
+                    for (int m = 0; m < q; ++m)
+                        for (int k = 0; k < q; ++k) w[o + k * q + m] = v[o + m * q + k];
+                }
+            }
+        putT(w);
+    };
+    put_factored(h.frot_fwd); // 28
+    put_factored(h.frot_bwd); // 29
+    put_factored(h.forot_fwd);// 30
+    put_factored(h.forot_bwd);// 31
     putI(h.frot_off); // 32
     putI(h.u_k);      // 33
     putI(h.u_start);  // 34

@@ -463,7 +463,8 @@ __global__ void k_l2l(int b0, int nb, DevTables<T> D, const int *par, const int 
 // The factorized rotation of the four sets: tmp <- za (src) (one 2x2 rotation per
 // coefficient), then dst <- zc (Y tmp), Y acting on real and imaginary parts
 // separately.  src and dst may not alias tmp; the caller synchronises after.
-template <typename T, bool QUARTER = false>
+// COL: the y blocks stand as [k][m] (y_by_column).
+template <typename T, bool QUARTER, bool COL>
 __device__ void rotate_sets_f(const T *rf, const int *foff, int p, const cpx<T> *src, cpx<T> *tmp, cpx<T> *dst) {
     const int nc = ncoef(p);
     for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
@@ -477,19 +478,20 @@ __device__ void rotate_sets_f(const T *rf, const int *foff, int p, const cpx<T> 
     for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
         const int st = e / nc, i = e - st * nc, n = deg_of(i), m = i - tri(n, 0), q = n + 1;
         const T *o = rf + foff[n];
-        const T *yre = o + 4 * q + m * q, *yim = o + 4 * q + q * q + m * q;
+        const T *yre = o + 4 * q + (COL ? m : m * q), *yim = yre + q * q;
+        const int sk = COL ? q : 1;   // stride of k
         const cpx<T> *in = tmp + st * nc + tri(n, 0);
         T re = 0, im = 0;
         if (QUARTER) {
             // middle angle pi/2 (the frame rotations): the y blocks are checkerboards
             // (checked when the tables are built); Im of m = 0 is zero for real fields
-            for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k], in[k].x);
+            for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k * sk], in[k].x);
             if (m > 0)
-                for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k], in[k].y);
+                for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k * sk], in[k].y);
         } else {
             for (int k = 0; k < q; ++k) {
-                macc(re, yre[k], in[k].x);
-                macc(im, yim[k], in[k].y);
+                macc(re, yre[k * sk], in[k].x);
+                macc(im, yim[k * sk], in[k].y);
             }
         }
         re = closed(re);
@@ -515,7 +517,7 @@ __global__ void k_m2m_child(int c0, int pb0, DevTables<T> D, const int *par, con
                             int rb, const cpx<T> *M, cpx<T> *Sc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int c = c0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p), P1 = p + 1;
+    const int p = D.p, nc = ncoef(p);
     cpx<T> *X = reinterpret_cast<cpx<T> *>(smem_raw);
     cpx<T> *Y = X + kSets * nc;
     cpx<T> *Tm = Y + kSets * nc;   // rotation scratch
@@ -523,22 +525,22 @@ __global__ void k_m2m_child(int c0, int pb0, DevTables<T> D, const int *par, con
     const cpx<T> *src = M + size_t(c) * kSets * nc;
     for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) X[i] = src[i];
     __syncthreads();
-    rotate_sets_f(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
+    rotate_sets_f<T, false, true>(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
     __syncthreads();
     for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
         int st = e / nc, i = e - st * nc;
         int n = deg_of(i), m = i - tri(n, 0);
-        const T *z = D.zm2m + size_t(i) * P1;
+        const T *z = D.zm2m + i;   // stored [k][coefficient]
         cpx<T> a = mk<T>(0, 0);
         for (int k = m; k <= n; ++k) {
             const cpx<T> y = Y[st * nc + tri(k, m)];
-            macc(a.x, z[k], y.x);
-            macc(a.y, z[k], y.y);
+            macc(a.x, z[k * nc], y.x);
+            macc(a.y, z[k * nc], y.y);
         }
         X[e] = mk(closed(a.x), closed(a.y));
     }
     __syncthreads();
-    rotate_sets_f(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
+    rotate_sets_f<T, false, true>(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
     __syncthreads();
     cpx<T> *dst = Sc + (size_t(par[c] - pb0) * 8 + o) * kSets * nc;
     const double h = 0.5 * side[c];
@@ -579,7 +581,7 @@ __global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int b = b0 + blockIdx.x;
     int P = par[b];
-    const int p = D.p, nc = ncoef(p), P1 = p + 1;
+    const int p = D.p, nc = ncoef(p);
     cpx<T> *X = reinterpret_cast<cpx<T> *>(smem_raw);
     cpx<T> *Y = X + kSets * nc;
     cpx<T> *Tm = Y + kSets * nc;   // rotation scratch
@@ -587,22 +589,22 @@ __global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const 
     const cpx<T> *src = L + size_t(P) * kSets * nc;
     for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) X[i] = src[i];
     __syncthreads();
-    rotate_sets_f(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
+    rotate_sets_f<T, false, true>(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
     __syncthreads();
     for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
         int st = e / nc, i = e - st * nc;
         int n = deg_of(i), m = i - tri(n, 0);
-        const T *z = D.zl2l + size_t(i) * P1;
+        const T *z = D.zl2l + i;   // stored [k][coefficient]
         cpx<T> a = mk<T>(0, 0);
         for (int k = n; k <= p; ++k) {
             const cpx<T> y = Y[st * nc + tri(k, m)];
-            macc(a.x, z[k], y.x);
-            macc(a.y, z[k], y.y);
+            macc(a.x, z[k * nc], y.x);
+            macc(a.y, z[k * nc], y.y);
         }
         X[e] = mk(closed(a.x), closed(a.y));
     }
     __syncthreads();
-    rotate_sets_f(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
+    rotate_sets_f<T, false, true>(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
     __syncthreads();
     cpx<T> *dst = L + size_t(b) * kSets * nc;
     const double h = 0.5 * side[b];
@@ -619,7 +621,7 @@ __global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const 
 }
 
 // ---------------------------------------------------------------- M2X
-template <typename T>
+template <typename T, bool COL>
 __global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *Xo, int f0, int nf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int b = b0 + blockIdx.x;
@@ -640,7 +642,7 @@ __global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *X
     for (int f = f0; f < f0 + nf; ++f) {
         const cpx<T> *Mu = Mw;
         if (f > 0) {
-            rotate_sets_f<T, true>(D.frot_fwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Mw, Tm, Mf);
+            rotate_sets_f<T, true, COL>(D.frot_fwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Mw, Tm, Mf);
             __syncthreads();
             Mu = Mf;
         }
@@ -1432,7 +1434,7 @@ __global__ void k_x2l(int b0, int nb, DevTables<T> D, const cpx<T> *Xi, cpx<T> *
         if (f == 0) {
             for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lf[i];
         } else {
-            rotate_sets_f<T, true>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Lf, Tm, Lr);
+            rotate_sets_f<T, true, true>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Lf, Tm, Lr);
             __syncthreads();
             for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lr[i];
         }
@@ -1447,6 +1449,7 @@ __global__ void k_x2l(int b0, int nb, DevTables<T> D, const cpx<T> *Xi, cpx<T> *
 // parts in another), so that the real DFT, which takes the real parts for even m
 // and the imaginary parts for odd m, reads four sets with one 16-byte load per
 // wave and direction; one root lookup then serves sixteen FMAs.
+template <bool COL>
 __global__ void k_x2l4(int b0, int nb, DevTables<float> D, const cpx<float> *Xi, cpx<float> *L, int f0, int nf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int b = b0 + blockIdx.x;
@@ -1547,7 +1550,7 @@ __global__ void k_x2l4(int b0, int nb, DevTables<float> D, const cpx<float> *Xi,
         if (f == 0) {
             for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lf[i];
         } else {
-            rotate_sets_f<float, false>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Lf, Tm, Lr);
+            rotate_sets_f<float, false, COL>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Lf, Tm, Lr);
             __syncthreads();
             for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lr[i];
         }
@@ -2047,13 +2050,16 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     // M2X, X2X and X2L launches are timed under their own stages).
     const int nf = t.x_frames;
     size_t smx = smem_m2x<T>(p, D.s);
-    RPY_TRY(set_smem(k_m2x<T>, smx));
+    const bool col = y_by_column(sizeof(T), p);
+    auto m2x = col ? k_m2x<T, true> : k_m2x<T, sizeof(T) == 8>;
+    RPY_TRY(set_smem(m2x, smx));
     size_t sxl = sizeof(T) == 4 ? smem_x2l4(p, D.s, D.S) : smem_x2l<T>(p, D.s, D.NU);
-    if constexpr (sizeof(T) == 4) RPY_TRY(set_smem(k_x2l4, sxl));
+    auto x2l4 = col ? k_x2l4<true> : k_x2l4<false>;
+    if constexpr (sizeof(T) == 4) RPY_TRY(set_smem(x2l4, sxl));
     else RPY_TRY(set_smem(k_x2l<T>, sxl));
     for (int f0 = 0; f0 < 3; f0 += nf) {
         prof_mark(t, RPY_STAGE_M2X, st);
-        k_m2x<T><<<n2, even_threads(sizeof(T) == 8 ? D.NU : D.S), smx, st>>>(b2, n2, D, M, Xo, f0, nf);
+        m2x<<<n2, even_threads(sizeof(T) == 8 ? D.NU : D.S), smx, st>>>(b2, n2, D, M, Xo, f0, nf);
         RPY_LAUNCHED(1);
         RPY_CHECK(cudaGetLastError());
         prof_mark(t, RPY_STAGE_X2X, st);
@@ -2097,7 +2103,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
         // order; at high order the shared memory already limits the blocks per SM
         // and 256 threads hide latency better
         const int tx = D.s * (p + 1) <= 256 ? even_threads(D.s * (p + 1)) : 256;
-        if constexpr (sizeof(T) == 4) k_x2l4<<<n2, tx, sxl, st>>>(b2, n2, D, Xi, L, f0, nf);
+        if constexpr (sizeof(T) == 4) x2l4<<<n2, tx, sxl, st>>>(b2, n2, D, Xi, L, f0, nf);
         else k_x2l<T><<<n2, 256, sxl, st>>>(b2, n2, D, Xi, L, f0, nf);
         RPY_LAUNCHED(1);
         RPY_CHECK(cudaGetLastError());

@@ -151,6 +151,12 @@ struct OpTables {
 constexpr int kGroupMax = 32;
 
 int build_tables(int p, int digits, OpTables &t);   // host computation, no CUDA
+// The y blocks of the factored rotations, indexed by output m and input k, stand as [k][m] on the device
+// from p = 12 and in double-floats: a warp's lanes take consecutive m, and at a row of 13 and
+// more values the [m][k] order costs a 128-byte line per lane (200k-bead tree at 9 digits: M2M 4.4 -> 1.9, L2L
+// 3.9 -> 1.6 ms; FP32, 1M beads, p = 15: M2M 0.92 -> 0.82, L2L 0.89 -> 0.78, X2L 2.28 -> 2.07 ms).  FP32 below p = 12 keeps [m][k],
+// whose immediate offsets are 2% faster there (15M-bead cube, p = 6: M2X 4.61 against 4.70 ms).
+constexpr bool y_by_column(size_t elem_bytes, int p) { return elem_bytes == 8 || p >= 12; }
 
 // device copies
 template <typename T>
