@@ -271,30 +271,6 @@ int split_forces_f64(Tree &t, cudaStream_t st) {
     return RPY_OK;
 }
 
-// Packed (two lanes) FP32 operations and double-floats of them.
-struct df2 {
-    float2 h, l;
-};
-__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// s + e = a + b exactly
-__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2 &e) {
-    const float2 s = add2(a, b), bb = sub2(s, a);
-    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-    return s;
-}
-// (a.h + a.l) (b.h + b.l)
-__device__ __forceinline__ df2 mul_df(df2 a, df2 b) {
-    df2 r;
-    r.h = mul2(a.h, b.h);
-    r.l = fma2(a.l, b.h, fma2(a.h, b.l, fma2(a.h, b.h, neg2(r.h))));
-    return r;
-}
-
 // The difference of two coordinates held as three floats, normalised.
 __device__ __forceinline__ df2 diff3(float2 xh, float2 xm, float2 xl, float2 sh, float2 sm, float2 sl) {
     const float2 dh = sub2(xh, sh), dm = sub2(xm, sm), dl = sub2(xl, sl);   // the first two exact
