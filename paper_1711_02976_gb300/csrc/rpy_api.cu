@@ -264,7 +264,14 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
     put_factored(h.forot_fwd);// 30
     put_factored(h.forot_bwd);// 31
     putI(h.frot_off); // 32
-    putI(h.u_k);      // 33
+    {                 // 33: per wave-pair unit (node, first stored wave, stored waves, t)
+        std::vector<int> v;
+        for (size_t u = 0; u < h.u_k.size(); ++u) {
+            const int k = h.u_k[u];
+            v.insert(v.end(), {k, h.k_start[k], h.k_start[k + 1] - h.k_start[k], int(u) - h.u_start[k]});
+        }
+        putI(v);
+    }
     putI(h.u_start);  // 34
     putT(h.shz);      // 35
     putT(h.shx);      // 36
@@ -320,7 +327,7 @@ static DevTables<T> bind_tables(const OpTables &h, char *base, const std::vector
     d.forot_bwd = reinterpret_cast<const T *>(base + o[31]);
     d.frot_off = reinterpret_cast<const int *>(base + o[32]);
     d.frot_len = h.frot_off.back();
-    d.u_k = reinterpret_cast<const int *>(base + o[33]);
+    d.u_info = reinterpret_cast<const int4 *>(base + o[33]);
     d.u_start = reinterpret_cast<const int *>(base + o[34]);
     d.NU = int(h.u_k.size());
     d.shz = reinterpret_cast<const T *>(base + o[35]);

@@ -37,24 +37,12 @@
 #include <map>
 #include <mutex>
 
+#include "rpy_far.h"
 #include "rpy_harmonics.h"
 
 namespace rpy {
 
-__device__ __forceinline__ int deg_of(int idx) {
-    int n = int((sqrtf(8.0f * idx + 1.0f) - 1.0f) * 0.5f);
-    while (tri(n + 1, 0) <= idx) ++n;
-    while (tri(n, 0) > idx) --n;
-    return n;
-}
-
 // ---------------------------------------------------------------- harmonics, several points per warp
-// Lanes per point: columns m and P - m share a lane, so every lane runs P + 2
-// recurrence steps (a column per lane would leave the lanes of high m idle
-// while column 0 runs P + 1 steps, and lanes above P idle altogether; the
-// arithmetic pipes are charged per warp instruction).
-__host__ __device__ constexpr int harm_lanes(int P) { return P / 2 + 1; }
-
 // Solid harmonics (regular, or irregular when IRREG) of one point into out[],
 // columns c and P - c of it.
 template <typename T, bool IRREG>
@@ -620,1276 +608,6 @@ __global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const 
     }
 }
 
-// ---------------------------------------------------------------- M2X
-template <typename T, bool COL>
-__global__ void k_m2x(int b0, int nb, DevTables<T> D, const cpx<T> *M, cpx<T> *Xo, int f0, int nf) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int b = b0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p), s = D.s, S = D.S, P1 = p + 1;
-    // A per node k: [P1][4 sets] at stride NS = 4 P1 + 1, so that the units of
-    // neighbouring nodes in one warp read different shared-memory banks
-    const int NS = kSets * P1 + 1;
-    cpx<T> *Mw = reinterpret_cast<cpx<T> *>(smem_raw);
-    cpx<T> *Mf = Mw + kSets * nc;
-    cpx<T> *AE = Mf + kSets * nc;       // [s][NS]
-    cpx<T> *AO = AE + s * NS;
-    cpx<T> *Tm = AO + s * NS;           // rotation scratch
-    const cpx<T> *src = M + size_t(b) * kSets * nc;
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Mw[i] = src[i];
-    __syncthreads();
-    size_t base = size_t(b) * (2 * nf) * kSets * S;   // frames f0 .. f0 + nf - 1 of this pass
-    const int hP = harm_lanes(p);
-    for (int f = f0; f < f0 + nf; ++f) {
-        const cpx<T> *Mu = Mw;
-        if (f > 0) {
-            rotate_sets_f<T, true, COL>(D.frot_fwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Mw, Tm, Mf);
-            __syncthreads();
-            Mu = Mf;
-        }
-        // A_k^m split by parity of n + m (the - direction is the reflection (-1)^{n+m}),
-        // stored as 2 i^m A_k^m so that the wave sum below needs no sign logic:
-        // even m feed the real part, odd m the imaginary part.  One thread per
-        // (set, node k, column pair (m, p - m)): p + 2 terms each.
-        for (int e = threadIdx.x; e < kSets * s * hP; e += blockDim.x) {
-            const int st = e / (s * hP), r = e - st * s * hP, k = r / hP, c = r - k * hP;
-            const T *cc = D.m2x_c + size_t(k) * nc;
-            const cpx<T> *Ms = Mu + st * nc;
-            for (int h = 0; h < 2; ++h) {
-                const int m = h ? p - c : c;
-                if (h && m == c) break;
-                T evx = 0, evy = 0, odx = 0, ody = 0;
-                for (int n = m; n <= p; n += 2) {
-                    const int i = tri(n, m);
-                    macc(evx, cc[i], Ms[i].x);
-                    macc(evy, cc[i], Ms[i].y);
-                }
-                for (int n = m + 1; n <= p; n += 2) {
-                    const int i = tri(n, m);
-                    macc(odx, cc[i], Ms[i].x);
-                    macc(ody, cc[i], Ms[i].y);
-                }
-                const float sg = m == 0 ? 1.f : (((m >> 1) & 1) ? -2.f : 2.f);   // 2 i^m up to i for odd m
-                AE[k * NS + m * kSets + st] = mk(scale2(sg, closed(evx)), scale2(sg, closed(evy)));
-                AO[k * NS + m * kSets + st] = mk(scale2(sg, closed(odx)), scale2(sg, closed(ody)));
-            }
-        }
-        __syncthreads();
-        {
-            // FP32: one wave per thread (the kernel is not bound by its FMAs, and
-            // twice the threads hide more latency)
-            // W_j = (w_k/M_k) [A^0 + 2 sum_m i^m Re(A^m e^{i m a_j})], A = AE +- AO, all four
-            // sets per wave (one root lookup and index update serve four sets)
-            for (int j = threadIdx.x; j < S; j += blockDim.x) {
-                const int k = D.e_k[j];
-                const int j0 = D.k_start[k], jl = j - j0, Mk = 2 * (D.k_start[k + 1] - j0);
-                const cpx<T> *rt = D.roots + 2 * j0;
-                const cpx<T> *ae = AE + k * NS;
-                const cpx<T> *ao = AO + k * NS;
-                T er[kSets], orr[kSets], ei[kSets], oi[kSets];
-    #pragma unroll
-                for (int st = 0; st < kSets; ++st) {
-                    er[st] = ae[st].x;
-                    orr[st] = ao[st].x;
-                    ei[st] = 0;
-                    oi[st] = 0;
-                }
-                int step2 = 2 * jl;
-                if (step2 >= Mk) step2 -= Mk;
-                int idx = 0;   // (m jl) mod Mk for even m
-                for (int m = 2; m <= p; m += 2) {
-                    idx += step2;
-                    if (idx >= Mk) idx -= Mk;
-                    const cpx<T> z = rt[idx];
-    #pragma unroll
-                    for (int st = 0; st < kSets; ++st) {
-                        const cpx<T> a = ae[m * kSets + st], o = ao[m * kSets + st];
-                        er[st] = fma(-a.y, z.y, fma(a.x, z.x, er[st]));
-                        orr[st] = fma(-o.y, z.y, fma(o.x, z.x, orr[st]));
-                    }
-                }
-                idx = jl;      // odd m, starting at m = 1
-                for (int m = 1; m <= p; m += 2) {
-                    const cpx<T> z = rt[idx];
-    #pragma unroll
-                    for (int st = 0; st < kSets; ++st) {
-                        const cpx<T> a = ae[m * kSets + st], o = ao[m * kSets + st];
-                        ei[st] = fma(-a.y, z.y, fma(a.x, z.x, ei[st]));
-                        oi[st] = fma(-o.y, z.y, fma(o.x, z.x, oi[st]));
-                    }
-                    idx += step2;
-                    if (idx >= Mk) idx -= Mk;
-                }
-                const T wm = D.e_wm[j];
-    #pragma unroll
-                for (int st = 0; st < kSets; ++st) {
-                    Xo[base + size_t(2 * (f - f0)) * kSets * S + st * S + j] =
-                        mk(wm * (er[st] + orr[st]), wm * (ei[st] + oi[st]));
-                    Xo[base + size_t(2 * (f - f0) + 1) * kSets * S + st * S + j] =
-                        mk(wm * (er[st] - orr[st]), wm * (ei[st] - oi[st]));
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------- X2X merge-and-shift
-template <typename T, bool FAC>
-__global__ void k_x2x(const int *parents, DevTables<T> D, const int *coll, const int *child, const int *leaf,
-                      const cpx<T> *Xo, cpx<T> *Xi, int f0, int nf) {
-    __shared__ int src[216];
-    __shared__ int vsrc[216], vsh[216], vpre[217];   // the present sources, compacted in slot order
-    __shared__ int vend[216];   // child mask of its group at the last present source of a group, else 0
-    // FAC (FP32, few plane waves): the shift of a source as the product of its
-    // per-axis factors, from shared memory (z offsets x S, x offsets, y offsets);
-    // otherwise the shift table
-    __shared__ int voz[216], vox[216], voy[216];
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int P = parents[blockIdx.x];
-    const int dl = blockIdx.y, d = 2 * f0 + dl;   // direction, and its slot in this pass's buffers
-    const int S = D.S;
-    for (int sl = threadIdx.x; sl < 216; sl += blockDim.x) {
-        int q = sl >> 3, o = sl & 7;
-        int Q = coll[27 * P + q];
-        src[sl] = (Q >= 0 && !leaf[Q]) ? child[8 * Q + o] : -1;
-    }
-    __syncthreads();
-    int ng = D.grp_n[d];
-    const int *goff = D.grp_off + d * (kGroupMax + 1);
-    const int *gmask = D.grp_mask + d * kGroupMax;
-    const int *slots = D.slot_list + d * 216;
-    // warp 0: keep the slots whose source box exists; vpre[z] = present slots before z,
-    // so group g covers vsrc[vpre[goff[g]] .. vpre[goff[g + 1]])
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x, nsl = goff[ng];
-        int carry = 0;
-        for (int z0 = 0; z0 < nsl; z0 += 32) {
-            const int z = z0 + lane;
-            int ent = 0, sb = -1;
-            if (z < nsl) {
-                ent = slots[z];
-                sb = src[ent & 255];
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, sb >= 0);
-            const int pos = carry + __popc(bal & ((1u << lane) - 1u));
-            if (z < nsl) vpre[z] = pos;
-            if (sb >= 0) {
-                vsrc[pos] = sb;
-                vsh[pos] = ent >> 8;
-            }
-            carry += __popc(bal);
-        }
-        if (lane == 0) vpre[nsl] = carry;
-    }
-    __syncthreads();
-    const int nz = vpre[goff[ng]];
-    for (int z = threadIdx.x; z < nz; z += blockDim.x) {
-        vend[z] = 0;
-        const int o = vsh[z];
-        vox[z] = (o % 6) * S;
-        voy[z] = ((o / 6) % 6) * S;
-        voz[z] = (o / 36) * S;
-    }
-    T *sZ = reinterpret_cast<T *>(smem_raw);
-    cpx<T> *sX = reinterpret_cast<cpx<T> *>(sZ + ((6 * S + 3) & ~3));
-    cpx<T> *sY = sX + 6 * S;
-    if constexpr (FAC) {
-        for (int i = threadIdx.x; i < 6 * S; i += blockDim.x) {
-            sZ[i] = D.shz[i];
-            sX[i] = D.shx[i];
-            sY[i] = D.shy[i];
-        }
-    }
-    __syncthreads();
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-        const int z1 = vpre[goff[g + 1]];
-        if (z1 > vpre[goff[g]]) vend[z1 - 1] = gmask[g];
-    }
-    __syncthreads();
-    int ch[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) ch[t] = child[8 * P + t];
-    const size_t dstride = size_t(2 * nf) * kSets * S;
-    const cpx<T> *Xd = Xo + size_t(dl) * kSets * S;
-    for (int e = threadIdx.x; e < kSets * S; e += blockDim.x) {
-        int j = e % S;
-        cpx<T> acc[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) acc[t] = mk<T>(0, 0);
-        // one pass over all present sources (group boundaries marked by vend), so
-        // that the unrolled loads run ahead across groups (measured: 8 in flight for the
-        // FP32 table form, 4 elsewhere)
-        constexpr int kUnroll = (sizeof(T) == 4 && !FAC) ? 8 : 4;
-        cpx<T> ga = mk<T>(0, 0);
-#pragma unroll kUnroll
-        for (int z = 0; z < nz; ++z) {
-            const cpx<T> x = Xd[size_t(vsrc[z]) * dstride + e];
-            cpx<T> sh;
-            if constexpr (FAC) {
-                const cpx<T> a = sX[vox[z] + j], b = sY[voy[z] + j];
-                const T c = sZ[voz[z] + j];
-                sh = mk(c * mul_diff(a.x, b.x, a.y, b.y), c * mul_diff(a.x, b.y, -a.y, b.x));
-            } else {
-                sh = D.shift[size_t(vsh[z]) * S + j];
-            }
-            macc(ga.x, x.x, sh.x);
-            macc(ga.x, -x.y, sh.y);
-            macc(ga.y, x.x, sh.y);
-            macc(ga.y, x.y, sh.x);
-            const int mask = vend[z];   // block-uniform
-            if (mask) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    if ((mask >> t) & 1) acc[t] += ga;
-                ga = mk<T>(0, 0);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (ch[t] < 0) continue;
-            cpx<T> sh = D.shift[size_t(D.child_shift[d * 8 + t]) * S + j];
-            Xi[(size_t(ch[t]) * (2 * nf) + dl) * kSets * S + e] = acc[t] * sh;
-        }
-    }
-}
-
-// Merge-and-shift with the four charge sets of a plane wave in one thread (the
-// FP32 form, and the box-origin form in either precision).  With rb (box origin
-// of q4 = F . (r - o)), set 4 travels with its origin at the centre of the box
-// whose expansion it is: each source's set 4 moves to the parent centre as it is
-// merged, X4 += (c_source - c_parent) . X_F, and each merged sum moves to the
-// child as it is shifted there, X4 += (c_parent - c_child) . X_F, with X_F the
-// force sets 1..3 of the same wave (rotations of the frames act on the plane-wave
-// variables only, so the world offsets apply as they are).
-template <typename T, bool FAC>
-__global__ void k_x2x4(const int *parents, DevTables<T> D, const int *coll, const int *child, const int *leaf,
-                       const double *side, const cpx<T> *Xo, cpx<T> *Xi, int f0, int nf, int rb) {
-    __shared__ int src[216];
-    __shared__ int vsrc[216], vsh[216], vpre[217], vend[216];
-    __shared__ int voz[216], vox[216], voy[216];
-    __shared__ T vd[3][216];   // source centre - parent centre (world axes), set-4 origin move
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int P = parents[blockIdx.x];
-    const int dl = blockIdx.y, d = 2 * f0 + dl;
-    const int S = D.S;
-    const double hc = 0.5 * side[P];   // side of P's children (and of the sources)
-    for (int sl = threadIdx.x; sl < 216; sl += blockDim.x) {
-        int q = sl >> 3, o = sl & 7;
-        int Q = coll[27 * P + q];
-        src[sl] = (Q >= 0 && !leaf[Q]) ? child[8 * Q + o] : -1;
-    }
-    __syncthreads();
-    const int ng = D.grp_n[d];
-    const int *goff = D.grp_off + d * (kGroupMax + 1);
-    const int *gmask = D.grp_mask + d * kGroupMax;
-    const int *slots = D.slot_list + d * 216;
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x, nsl = goff[ng];
-        int carry = 0;
-        for (int z0 = 0; z0 < nsl; z0 += 32) {
-            const int z = z0 + lane;
-            int ent = 0, sb = -1;
-            if (z < nsl) {
-                ent = slots[z];
-                sb = src[ent & 255];
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, sb >= 0);
-            const int pos = carry + __popc(bal & ((1u << lane) - 1u));
-            if (z < nsl) vpre[z] = pos;
-            if (sb >= 0) {
-                vsrc[pos] = sb;
-                vsh[pos] = ent >> 8;
-                // slot = colleague (dx, dy, dz in -1..1, index 9 dz + 3 dy + dx + 13) x 8 + child octant:
-                // source centre - P's centre = hc (2 d + bit - 1/2) per axis, in world axes
-                const int sl = ent & 255, q = sl >> 3, o = sl & 7;
-                vd[0][pos] = T(hc * (2 * (q % 3 - 1) + (o & 1) - 0.5));
-                vd[1][pos] = T(hc * (2 * ((q / 3) % 3 - 1) + ((o >> 1) & 1) - 0.5));
-                vd[2][pos] = T(hc * (2 * (q / 9 - 1) + ((o >> 2) & 1) - 0.5));
-            }
-            carry += __popc(bal);
-        }
-        if (lane == 0) vpre[nsl] = carry;
-    }
-    __syncthreads();
-    const int nz = vpre[goff[ng]];
-    for (int z = threadIdx.x; z < nz; z += blockDim.x) {
-        vend[z] = 0;
-        const int o = vsh[z];
-        vox[z] = (o % 6) * S;
-        voy[z] = ((o / 6) % 6) * S;
-        voz[z] = (o / 36) * S;
-    }
-    T *sZ = reinterpret_cast<T *>(smem_raw);
-    cpx<T> *sX = reinterpret_cast<cpx<T> *>(sZ + ((6 * S + 3) & ~3));
-    cpx<T> *sY = sX + 6 * S;
-    if constexpr (FAC) {
-        for (int i = threadIdx.x; i < 6 * S; i += blockDim.x) {
-            sZ[i] = D.shz[i];
-            sX[i] = D.shx[i];
-            sY[i] = D.shy[i];
-        }
-    }
-    __syncthreads();
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-        const int z1 = vpre[goff[g + 1]];
-        if (z1 > vpre[goff[g]]) vend[z1 - 1] = gmask[g];
-    }
-    __syncthreads();
-    int ch[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) ch[t] = child[8 * P + t];
-    const size_t dstride = size_t(2 * nf) * kSets * S;
-    const cpx<T> *Xd = Xo + size_t(dl) * kSets * S;
-    for (int j = threadIdx.x; j < S; j += blockDim.x) {
-        cpx<T> acc[8][kSets];
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-#pragma unroll
-            for (int k = 0; k < kSets; ++k) acc[t][k] = mk<T>(0, 0);
-        cpx<T> ga[kSets];
-#pragma unroll
-        for (int k = 0; k < kSets; ++k) ga[k] = mk<T>(0, 0);
-#pragma unroll 2
-        for (int z = 0; z < nz; ++z) {
-            const cpx<T> *xs = Xd + size_t(vsrc[z]) * dstride + j;
-            cpx<T> x[kSets];
-#pragma unroll
-            for (int k = 0; k < kSets; ++k) x[k] = xs[size_t(k) * S];
-            if (rb) {
-                const T ex = vd[0][z], ey = vd[1][z], ez = vd[2][z];
-                x[3].x = fma(ez, x[2].x, fma(ey, x[1].x, fma(ex, x[0].x, x[3].x)));
-                x[3].y = fma(ez, x[2].y, fma(ey, x[1].y, fma(ex, x[0].y, x[3].y)));
-            }
-            cpx<T> sh;
-            if constexpr (FAC) {
-                const cpx<T> a = sX[vox[z] + j], b = sY[voy[z] + j];
-                const T c = sZ[voz[z] + j];
-                sh = mk(c * mul_diff(a.x, b.x, a.y, b.y), c * mul_diff(a.x, b.y, -a.y, b.x));
-            } else {
-                sh = D.shift[size_t(vsh[z]) * S + j];
-            }
-#pragma unroll
-            for (int k = 0; k < kSets; ++k) {
-                macc(ga[k].x, x[k].x, sh.x);
-                macc(ga[k].x, -x[k].y, sh.y);
-                macc(ga[k].y, x[k].x, sh.y);
-                macc(ga[k].y, x[k].y, sh.x);
-            }
-            const int mask = vend[z];   // block-uniform
-            if (mask) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    if ((mask >> t) & 1)
-#pragma unroll
-                        for (int k = 0; k < kSets; ++k) acc[t][k] += ga[k];
-#pragma unroll
-                for (int k = 0; k < kSets; ++k) ga[k] = mk<T>(0, 0);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (ch[t] < 0) continue;
-            if (rb) {   // P's centre - child t's centre = -(hc / 2) (2 bit - 1) per axis
-                const double h = 0.5 * hc;
-                const T ex = T((t & 1) ? -h : h), ey = T((t & 2) ? -h : h), ez = T((t & 4) ? -h : h);
-                acc[t][3].x = fma(ez, acc[t][2].x, fma(ey, acc[t][1].x, fma(ex, acc[t][0].x, acc[t][3].x)));
-                acc[t][3].y = fma(ez, acc[t][2].y, fma(ey, acc[t][1].y, fma(ex, acc[t][0].y, acc[t][3].y)));
-            }
-            const cpx<T> sh = D.shift[size_t(D.child_shift[d * 8 + t]) * S + j];
-            cpx<T> *dst = Xi + (size_t(ch[t]) * (2 * nf) + dl) * kSets * S + j;
-#pragma unroll
-            for (int k = 0; k < kSets; ++k) dst[size_t(k) * S] = acc[t][k] * sh;
-        }
-    }
-}
-
-// ---------------------------------------------------------------- bulk copies and mbarriers
-// One-dimensional bulk copies global -> shared (the TMA engine) completing on an
-// mbarrier: a thread announces the bytes to arrive (expect_tx), issues the copies,
-// and every thread waits for the barrier's phase.  Waits give up after about a
-// second (a copy that never lands), so that no kernel can hang the device.
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return unsigned(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect(uint64_t *bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, uint64_t limit_ns = 1000000000ull) {
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_test(bar, parity))
-        if (global_ns() - t0 > limit_ns) return false;
-    return true;
-}
-
-// Self-test of the bounded wait: one thread waits for an mbarrier phase that no
-// arrival will ever complete (no copy is issued), gives up after limit_ns and
-// reports the timeout through the status word, as the pipelined kernels do.
-__global__ void k_wait_selftest(uint64_t limit_ns, unsigned *status) {
-    __shared__ __align__(8) uint64_t bar;
-    if (threadIdx.x != 0) return;
-    mbar_init(&bar, 1);
-    mbar_init_fence();
-    if (!mbar_wait(&bar, 0, limit_ns)) atomicOr(status, DEVERR_TIMEOUT);
-}
-
-int wait_selftest(double limit_ms, cudaStream_t st) {
-    unsigned *d = nullptr;
-    RPY_CHECK(cudaMalloc(&d, sizeof(unsigned)));
-    unsigned h = 0;
-    cudaError_t e = cudaMemsetAsync(d, 0, sizeof(unsigned), st);
-    if (e == cudaSuccess) {
-        k_wait_selftest<<<1, 32, 0, st>>>(uint64_t(limit_ms * 1e6), d);
-        RPY_LAUNCHED(1);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d);
-    if (e != cudaSuccess) return check_cuda("wait self-test", e);
-    return (h & DEVERR_TIMEOUT) ? RPY_ERR_TIMEOUT : RPY_OK;
-}
-// orders this thread's earlier generic-proxy accesses to shared memory before later bulk copies
-__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
-// Bulk-copy pipeline of the FP32 X2X: kX2XStages buffers, each holding one source's
-// outgoing waves in one direction (4 S values) and its shift row (S values, rows
-// padded to an even length).
-constexpr int kX2XStages = 4;
-__host__ __device__ inline int x2x_tma_stage_elems(int S) { return 4 * S + ((S + 1) & ~1); }
-__host__ inline size_t x2x_tma_smem(int S) { return sizeof(cpx<float>) * size_t(kX2XStages) * x2x_tma_stage_elems(S); }
-
-// FP32 merge-and-shift, one consumer thread per plane wave (the four charge sets
-// and the box-origin move of set 4 as in k_x2x4), fed by a producer warp: the
-// present sources are staged through shared memory by bulk copies (TMA) into
-// kX2XStages buffers.  Buffer q is "full" when its copies have landed (an mbarrier
-// with the transaction count) and "empty" when every consumer warp has read it
-// (an mbarrier with one arrival per consumer warp); the producer refills a buffer
-// as soon as it is empty, so the consumers never wait on a global load and the
-// block needs no barrier per source.
-__global__ void __launch_bounds__(512, 1) k_x2x_tma(const int *parents, DevTables<float> D, const int *coll,
-                                                    const int *child, const int *leaf, const double *side,
-                                                    const cpx<float> *Xo, cpx<float> *Xi, int f0, int nf, int rb,
-                                                    unsigned *status) {
-    __shared__ int src[216];
-    __shared__ int vsrc[216], vsh[216], vpre[217], vend[216];
-    __shared__ float vd[3][216];
-    __shared__ __align__(8) uint64_t full[kX2XStages], empty[kX2XStages];
-    __shared__ int bad, issued;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int P = parents[blockIdx.x];
-    const int dl = blockIdx.y, d = 2 * f0 + dl;
-    const int S = D.S, Sp = D.Sp;
-    const int ncw = (S + 31) / 32;                 // consumer warps; the last warp produces
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double hc = 0.5 * side[P];
-    for (int sl = threadIdx.x; sl < 216; sl += blockDim.x) {
-        int q = sl >> 3, o = sl & 7;
-        int Q = coll[27 * P + q];
-        src[sl] = (Q >= 0 && !leaf[Q]) ? child[8 * Q + o] : -1;
-    }
-    if (threadIdx.x == 0) {
-        bad = 0;
-        issued = 0;
-        for (int q = 0; q < kX2XStages; ++q) {
-            mbar_init(&full[q], 1);
-            mbar_init(&empty[q], unsigned(ncw));
-        }
-        mbar_init_fence();
-    }
-    __syncthreads();
-    const int ng = D.grp_n[d];
-    const int *goff = D.grp_off + d * (kGroupMax + 1);
-    const int *gmask = D.grp_mask + d * kGroupMax;
-    const int *slots = D.slot_list + d * 216;
-    if (warp == 0) {
-        const int nsl = goff[ng];
-        int carry = 0;
-        for (int z0 = 0; z0 < nsl; z0 += 32) {
-            const int z = z0 + lane;
-            int ent = 0, sb = -1;
-            if (z < nsl) {
-                ent = slots[z];
-                sb = src[ent & 255];
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, sb >= 0);
-            const int pos = carry + __popc(bal & ((1u << lane) - 1u));
-            if (z < nsl) vpre[z] = pos;
-            if (sb >= 0) {
-                vsrc[pos] = sb;
-                vsh[pos] = ent >> 8;
-                const int sl = ent & 255, q = sl >> 3, o = sl & 7;
-                vd[0][pos] = float(hc * (2 * (q % 3 - 1) + (o & 1) - 0.5));
-                vd[1][pos] = float(hc * (2 * ((q / 3) % 3 - 1) + ((o >> 1) & 1) - 0.5));
-                vd[2][pos] = float(hc * (2 * (q / 9 - 1) + ((o >> 2) & 1) - 0.5));
-            }
-            carry += __popc(bal);
-        }
-        if (lane == 0) vpre[nsl] = carry;
-    }
-    __syncthreads();
-    const int nz = vpre[goff[ng]];
-    for (int z = threadIdx.x; z < nz; z += blockDim.x) vend[z] = 0;
-    __syncthreads();
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-        const int z1 = vpre[goff[g + 1]];
-        if (z1 > vpre[goff[g]]) vend[z1 - 1] = gmask[g];
-    }
-    __syncthreads();
-    const int stage_elems = x2x_tma_stage_elems(S);
-    cpx<float> *stage0 = reinterpret_cast<cpx<float> *>(smem_raw);
-    if (warp == ncw) {
-        // producer: one lane issues the copies, refilling each buffer once it is empty
-        if (lane == 0) {
-            const size_t dstride = size_t(2 * nf) * kSets * S;
-            const cpx<float> *Xd = Xo + size_t(dl) * kSets * S;
-            const unsigned src_bytes = 32u * unsigned(S), sh_bytes = 8u * unsigned(Sp);
-            for (int z = 0; z < nz; ++z) {
-                const int q = z % kX2XStages;
-                if (z >= kX2XStages && !mbar_wait(&empty[q], unsigned(z / kX2XStages - 1) & 1u)) {
-                    bad = 1;
-                    break;
-                }
-                if (*(volatile int *)&bad) break;
-                cpx<float> *buf = stage0 + size_t(q) * stage_elems;
-                mbar_expect(&full[q], src_bytes + sh_bytes);
-                bulk_load(buf, Xd + size_t(vsrc[z]) * dstride, src_bytes, &full[q]);
-                bulk_load(buf + 4 * S, D.shiftp + size_t(vsh[z]) * Sp, sh_bytes, &full[q]);
-                issued = z + 1;
-            }
-        }
-    } else {
-        int ch[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) ch[t] = child[8 * P + t];
-        const int j = threadIdx.x;
-        const bool act = j < S;
-        cpx<float> acc[8][kSets];
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-#pragma unroll
-            for (int k = 0; k < kSets; ++k) acc[t][k] = mk(0.f, 0.f);
-        cpx<float> ga[kSets];
-#pragma unroll
-        for (int k = 0; k < kSets; ++k) ga[k] = mk(0.f, 0.f);
-        for (int z = 0; z < nz; ++z) {
-            const int q = z % kX2XStages;
-            if (!mbar_wait(&full[q], unsigned(z / kX2XStages) & 1u) || *(volatile int *)&bad) {
-                bad = 1;
-                break;
-            }
-            if (act) {
-                const cpx<float> *buf = stage0 + size_t(q) * stage_elems;
-                cpx<float> x[kSets];
-#pragma unroll
-                for (int k = 0; k < kSets; ++k) x[k] = buf[k * S + j];
-                if (rb) {
-                    const float ex = vd[0][z], ey = vd[1][z], ez = vd[2][z];
-                    x[3].x = fmaf(ez, x[2].x, fmaf(ey, x[1].x, fmaf(ex, x[0].x, x[3].x)));
-                    x[3].y = fmaf(ez, x[2].y, fmaf(ey, x[1].y, fmaf(ex, x[0].y, x[3].y)));
-                }
-                const cpx<float> sh = buf[4 * S + j];
-#pragma unroll
-                for (int k = 0; k < kSets; ++k) {
-                    ga[k].x = fmaf(-x[k].y, sh.y, fmaf(x[k].x, sh.x, ga[k].x));
-                    ga[k].y = fmaf(x[k].y, sh.x, fmaf(x[k].x, sh.y, ga[k].y));
-                }
-                const int mask = vend[z];   // block-uniform
-                if (mask) {
-#pragma unroll
-                    for (int t = 0; t < 8; ++t)
-                        if ((mask >> t) & 1)
-#pragma unroll
-                            for (int k = 0; k < kSets; ++k) acc[t][k] += ga[k];
-#pragma unroll
-                    for (int k = 0; k < kSets; ++k) ga[k] = mk(0.f, 0.f);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[q]);   // this warp is done with buffer q
-        }
-        if (!*(volatile int *)&bad && act) {
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                if (ch[t] < 0) continue;
-                if (rb) {   // P's centre - child t's centre = -(hc / 2) (2 bit - 1) per axis
-                    const float h = float(0.5 * hc);
-                    const float ex = (t & 1) ? -h : h, ey = (t & 2) ? -h : h, ez = (t & 4) ? -h : h;
-                    acc[t][3].x = fmaf(ez, acc[t][2].x, fmaf(ey, acc[t][1].x, fmaf(ex, acc[t][0].x, acc[t][3].x)));
-                    acc[t][3].y = fmaf(ez, acc[t][2].y, fmaf(ey, acc[t][1].y, fmaf(ex, acc[t][0].y, acc[t][3].y)));
-                }
-                const cpx<float> sh = D.shift[size_t(D.child_shift[d * 8 + t]) * S + j];
-                cpx<float> *dst = Xi + (size_t(ch[t]) * (2 * nf) + dl) * kSets * S + j;
-#pragma unroll
-                for (int k = 0; k < kSets; ++k) dst[size_t(k) * S] = acc[t][k] * sh;
-            }
-        }
-    }
-    __syncthreads();
-    if (bad && threadIdx.x == 0) {
-        // a wait gave up: let every copy issued land (bounded) before the block's shared
-        // memory is released, and flag the failure
-        for (int q = 0; q < min(issued, kX2XStages); ++q) {
-            const int zl = q + ((issued - 1 - q) / kX2XStages) * kX2XStages;   // last copy issued into buffer q
-            mbar_wait(&full[q], unsigned(zl / kX2XStages) & 1u);
-        }
-        atomicOr(status, DEVERR_TIMEOUT);
-    }
-}
-
-// ---------------------------------------------------------------- X2L
-// FP32 form of X2L: the four charge sets in one pass.  The incoming waves of a
-// frame are staged planar (real parts of the four sets in one float4, imaginary
-// parts in another), so that the real DFT, which takes the real parts for even m
-// and the imaginary parts for odd m, reads four sets with one 16-byte load per
-// wave and direction; one root lookup then serves sixteen FMAs.
-template <bool COL>
-__global__ void k_x2l4(int b0, int nb, DevTables<float> D, const cpx<float> *Xi, cpx<float> *L, int f0, int nf) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int b = b0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p), s = D.s, S = D.S, P1 = p + 1;
-    float4 *PRe = reinterpret_cast<float4 *>(smem_raw);   // [S] + direction, real parts of sets 0..3
-    float4 *PIm = PRe + S;
-    float4 *MRe = PIm + S;                                  // - direction
-    float4 *MIm = MRe + S;
-    // b+ + b- (Bs) and b+ - b- (Bd) per (node, m), as planes of set pairs: (re, im) of sets
-    // 0 and 1, then of sets 2 and 3, so that each thread's 16-byte stores are contiguous
-    // across lanes (one [s][P1][4] array took four 8-byte stores 32 bytes apart)
-    const int SP = s * P1;
-    float4 *Bs01 = MIm + S, *Bs23 = Bs01 + SP, *Bd01 = Bs23 + SP, *Bd23 = Bd01 + SP;
-    cpx<float> *Lf = reinterpret_cast<cpx<float> *>(Bd23 + SP);                  // [4][nc]
-    cpx<float> *Lw = Lf + kSets * nc;
-    cpx<float> *Lr = Lw + kSets * nc;
-    cpx<float> *Tm = Lr + kSets * nc;                             // rotation scratch
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] = mk<float>(0, 0);
-    for (int f = f0; f < f0 + nf; ++f) {
-        __syncthreads();
-        const cpx<float> *sp = Xi + (size_t(b) * (2 * nf) + 2 * (f - f0)) * kSets * S;
-        const cpx<float> *sm = Xi + (size_t(b) * (2 * nf) + 2 * (f - f0) + 1) * kSets * S;
-        for (int j = threadIdx.x; j < S; j += blockDim.x) {
-            const cpx<float> p0 = sp[j], p1 = sp[S + j], p2 = sp[2 * S + j], p3 = sp[3 * S + j];
-            const cpx<float> m0 = sm[j], m1 = sm[S + j], m2 = sm[2 * S + j], m3 = sm[3 * S + j];
-            PRe[j] = make_float4(p0.x, p1.x, p2.x, p3.x);
-            PIm[j] = make_float4(p0.y, p1.y, p2.y, p3.y);
-            MRe[j] = make_float4(m0.x, m1.x, m2.x, m3.x);
-            MIm[j] = make_float4(m0.y, m1.y, m2.y, m3.y);
-        }
-        __syncthreads();
-        // b_k^m = 2 sum_j Re(I_j) e^{-i m a_j} (m even), 2i sum_j Im(I_j) e^{-i m a_j} (m odd)
-        // (node, m) items at a stride of PA = 8 per node when p + 1 <= 8, so that a
-        // quarter-warp never straddles two nodes (its wave loads are then broadcasts)
-        const int PA = P1 <= 8 ? 8 : P1;
-        for (int ea = threadIdx.x; ea < s * PA; ea += blockDim.x) {
-            const int k = ea / PA, m = ea - k * PA;
-            if (m >= P1) continue;
-            const int e = k * P1 + m;
-            const int j0 = D.k_start[k], j1 = D.k_start[k + 1];
-            const int Mk = 2 * (j1 - j0), mm = m % Mk;
-            const cpx<float> *rt = D.roots + 2 * j0;
-            const float4 *vp = (m & 1) ? PIm : PRe;
-            const float4 *vm = (m & 1) ? MIm : MRe;
-            float bpx[kSets] = {0, 0, 0, 0}, bpy[kSets] = {0, 0, 0, 0};
-            float bmx[kSets] = {0, 0, 0, 0}, bmy[kSets] = {0, 0, 0, 0};
-            int idx = 0;
-            for (int j = j0; j < j1; ++j) {
-                const cpx<float> r = rt[idx];
-                const float4 a = vp[j], c = vm[j];
-                const float av[kSets] = {a.x, a.y, a.z, a.w}, cv[kSets] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-                for (int st = 0; st < kSets; ++st) {
-                    bpx[st] = fmaf(av[st], r.x, bpx[st]);
-                    bpy[st] = fmaf(-av[st], r.y, bpy[st]);
-                    bmx[st] = fmaf(cv[st], r.x, bmx[st]);
-                    bmy[st] = fmaf(-cv[st], r.y, bmy[st]);
-                }
-                idx += mm;
-                if (idx >= Mk) idx -= Mk;
-            }
-            Bs01[e] = make_float4(bpx[0] + bmx[0], bpy[0] + bmy[0], bpx[1] + bmx[1], bpy[1] + bmy[1]);
-            Bs23[e] = make_float4(bpx[2] + bmx[2], bpy[2] + bmy[2], bpx[3] + bmx[3], bpy[3] + bmy[3]);
-            Bd01[e] = make_float4(bpx[0] - bmx[0], bpy[0] - bmy[0], bpx[1] - bmx[1], bpy[1] - bmy[1]);
-            Bd23[e] = make_float4(bpx[2] - bmx[2], bpy[2] - bmy[2], bpx[3] - bmx[3], bpy[3] - bmy[3]);
-        }
-        __syncthreads();
-        // L_n^m = i^m sum_k (-lambda_k)^n / sqrt((n-m)!(n+m)!) b_k^m, the - direction reflected
-        for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-            const int n = deg_of(i), m = i - tri(n, 0);
-            const bool odd = (n + m) & 1;
-            const float4 *B01 = odd ? Bd01 : Bs01, *B23 = odd ? Bd23 : Bs23;
-            // sum over the quadrature nodes with compensated (Kahan) addition: the terms
-            // (-lambda_k)^n b_k^m alternate in sign and cancel strongly at high degree
-            float ax[kSets] = {0, 0, 0, 0}, ay[kSets] = {0, 0, 0, 0};
-            float cx[kSets] = {0, 0, 0, 0}, cy[kSets] = {0, 0, 0, 0};
-            auto kahan = [](float &sum, float &c, float v) {
-                const float y = v - c, t = sum + y;
-                c = (t - sum) - y;
-                sum = t;
-            };
-            for (int k = 0; k < s; ++k) {
-                const float c = D.x2l_c[size_t(k) * nc + i];
-                const float4 b01 = B01[k * P1 + m], b23 = B23[k * P1 + m];
-                kahan(ax[0], cx[0], c * b01.x);
-                kahan(ay[0], cy[0], c * b01.y);
-                kahan(ax[1], cx[1], c * b01.z);
-                kahan(ay[1], cy[1], c * b01.w);
-                kahan(ax[2], cx[2], c * b23.x);
-                kahan(ay[2], cy[2], c * b23.y);
-                kahan(ax[3], cx[3], c * b23.z);
-                kahan(ay[3], cy[3], c * b23.w);
-            }
-#pragma unroll
-            for (int st = 0; st < kSets; ++st) Lf[st * nc + i] = mul_ipow(mk(2 * ax[st], 2 * ay[st]), m + (m & 1));
-        }
-        __syncthreads();
-        if (f == 0) {
-            for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lf[i];
-        } else {
-            rotate_sets_f<float, false, COL>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, p, Lf, Tm, Lr);
-            __syncthreads();
-            for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) Lw[i] += Lr[i];
-        }
-    }
-    __syncthreads();
-    cpx<float> *dst = L + size_t(b) * kSets * nc;
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) dst[i] += Lw[i];
-}
-
-static size_t smem_x2l4(int p, int s, int S) {
-    const int nc = ncoef(p);
-    return sizeof(float4) * 4 * size_t(S) + sizeof(cpx<float>) * (2 * kSets * s * (p + 1) + 4 * kSets * nc);
-}
-
-// ---------------------------------------------------------------- double-float plane waves, sets packed
-// M2X, X2X and X2L of the FP64 form.  Every table value serves the four charge sets alike, so a thread
-// carries two sets in the lanes of packed operations: half the FMA instructions of scalar double-floats,
-// and one table load, index update and loop step for two sets (all four in one thread: 106 to 118
-// registers and 12 to 14 warps per SM, M2X 6.2 and X2L 8.3 ms where this form takes 5.4 and 7.2, 1M-bead sphere
-// at 6 digits).
-// A quantity of a pair of sets stands as one float4 (h, h', l, l').
-// Plane waves: Xo and Xi [box][direction][wave][4] float4: re {0,1}, re {2,3}, im {0,1}, im {2,3}.
-// Neighbouring lanes carry the two pairs of one item: they share its table loads.
-__device__ __forceinline__ df2 zero_df2() { return df2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-__device__ __forceinline__ df2 operator+(df2 a, df2 b) { return renorm(sum_raw(a, b)); }
-__device__ __forceinline__ df2 operator-(df2 a, df2 b) { return renorm(sum_raw(a, -b)); }
-__device__ __forceinline__ df2 closed(df2 a) { return renorm(a); }
-__device__ __forceinline__ void macc(df2 &acc, dfl s, df2 b) { macc(acc, dup(s), b); }
-// a x + b y with scalar a, b
-__device__ __forceinline__ df2 lin2(dfl a, df2 x, dfl b, df2 y) {
-    return renorm(sum_raw(mul_df(dup(a), x), mul_df(dup(b), y)));
-}
-
-// n complex coefficients of four sets in shared memory: real parts [n][pair], then imaginary parts,
-// 16 bytes each, so that consecutive threads touch consecutive banks.  pr: the pair of sets.
-struct Planes {
-    float4 *p;
-    int n;
-    __device__ __forceinline__ df2 x(int pr, int i) const { return as_df2(p[2 * i + pr]); }
-    __device__ __forceinline__ df2 y(int pr, int i) const { return as_df2(p[2 * (n + i) + pr]); }
-    __device__ __forceinline__ void set(int pr, int i, df2 a, df2 b) const {
-        p[2 * i + pr] = as_float4(a);
-        p[2 * (n + i) + pr] = as_float4(b);
-    }
-};
-// coefficient i of the pair's sets in global memory ([set][nc] cpx<dfl>)
-__device__ __forceinline__ void load_pair(const cpx<dfl> *g, int nc, int pr, int i, df2 &x, df2 &y) {
-    const cpx<dfl> u = g[2 * pr * nc + i], v = g[(2 * pr + 1) * nc + i];
-    x = df2{make_float2(u.x.h, v.x.h), make_float2(u.x.l, v.x.l)};
-    y = df2{make_float2(u.y.h, v.y.h), make_float2(u.y.l, v.y.l)};
-}
-
-// The factored rotation of the four sets (rotate_sets_f): rotate_z forms tmp from a source of (x, y) per item,
-// rotate_y the result in dst.  An item is (coefficient, pair of sets).
-template <typename F>
-__device__ __forceinline__ void rotate_z(const dfl *rf, const int *foff, int nc, Planes tmp, F source) {
-    for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) {
-        const int pr = e & 1, i = e >> 1, n = deg_of(i), m = i - tri(n, 0);
-        const dfl *za = rf + foff[n];
-        const dfl c = za[2 * m], sn = za[2 * m + 1];
-        df2 x, y;
-        source(pr, i, x, y);
-        tmp.set(pr, i, lin2(c, x, -sn, y), lin2(sn, x, c, y));
-    }
-}
-__device__ __forceinline__ void rotate_y(const dfl *rf, const int *foff, int nc, Planes tmp, Planes dst) {
-    for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) {
-        const int pr = e & 1, i = e >> 1, n = deg_of(i), m = i - tri(n, 0), q = n + 1, t0 = tri(n, 0);
-        const dfl *o = rf + foff[n], *yre = o + 4 * q + m, *yim = yre + q * q;
-        df2 re = zero_df2(), im = re;
-        // the frame rotations' middle angle is pi/2: checkerboard y blocks, Im of m = 0 zero
-        for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k * q], tmp.x(pr, t0 + k));
-        if (m > 0)
-            for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k * q], tmp.y(pr, t0 + k));
-        re = closed(re);
-        im = closed(im);
-        const dfl c = o[2 * q + 2 * m], sn = o[2 * q + 2 * m + 1];
-        dst.set(pr, i, lin2(c, re, -sn, im), lin2(sn, re, c, im));
-    }
-}
-
-// A_k^m rows of one node at an odd stride, so that neighbouring nodes fall on different banks
-__host__ __device__ inline int a_stride(int p) { return (p + 1) | 1; }
-
-// M2X: one box per block, kc quadrature nodes at a time.
-__global__ void __launch_bounds__(256, 3)
-    k_m2x_df(int b0, DevTables<dfl> D, const cpx<dfl> *M, float4 *Xo, int f0, int nf, int kc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int b = b0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p), s = D.s, S = D.S, NS = a_stride(p);
-    const Planes Mu{reinterpret_cast<float4 *>(smem_raw), nc};
-    const Planes AE{Mu.p + 4 * nc, kc * NS}, AO{AE.p + 4 * kc * NS, kc * NS};
-    const Planes Tm{AE.p, nc};   // rotation scratch, before the A rows are formed (node_chunk leaves room)
-    const cpx<dfl> *src = M + size_t(b) * kSets * nc;
-    const int hP = harm_lanes(p);
-    for (int f = f0; f < f0 + nf; ++f) {
-        if (f > 0) {
-            const dfl *rf = D.frot_fwd + size_t(f - 1) * D.frot_len;
-            rotate_z(rf, D.frot_off, nc, Tm, [&](int pr, int i, df2 &x, df2 &y) { load_pair(src, nc, pr, i, x, y); });
-            __syncthreads();
-            rotate_y(rf, D.frot_off, nc, Tm, Mu);
-        } else {
-            for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) {
-                df2 x, y;
-                load_pair(src, nc, e & 1, e >> 1, x, y);
-                Mu.set(e & 1, e >> 1, x, y);
-            }
-        }
-        __syncthreads();
-        float4 *out = Xo + (size_t(b) * (2 * nf) + 2 * (f - f0)) * 4 * S;   // + direction; - direction 4 S further
-        for (int k0 = 0; k0 < s; k0 += kc) {
-            const int kn = min(kc, s - k0);
-            // A_k^m split by parity of n + m (the - direction is the reflection (-1)^{n+m}), stored as
-            // 2 i^m A_k^m so that the wave sum needs no sign logic: even m feed the real part, odd m the
-            // imaginary part.  One thread per (pair of sets, node, column pair (m, p - m)): p + 2 terms.
-            for (int e = threadIdx.x; e < 2 * kn * hP; e += blockDim.x) {
-                const int pr = e & 1, r = e >> 1, kk = r / hP, c = r - kk * hP;
-                const dfl *cc = D.m2x_c + size_t(k0 + kk) * nc;
-                for (int h = 0; h < 2; ++h) {
-                    const int m = h ? p - c : c;
-                    if (h && m == c) break;
-                    df2 evx = zero_df2(), evy = evx, odx = evx, ody = evx;
-                    int n = m, i = tri(m, m);
-                    for (; n < p; n += 2) {   // degrees n and n + 1
-                        const int i1 = i + n + 1;
-                        const dfl c0 = cc[i], c1 = cc[i1];
-                        macc(evx, c0, Mu.x(pr, i));
-                        macc(evy, c0, Mu.y(pr, i));
-                        macc(odx, c1, Mu.x(pr, i1));
-                        macc(ody, c1, Mu.y(pr, i1));
-                        i = i1 + n + 2;
-                    }
-                    if (n == p) {
-                        const dfl c0 = cc[i];
-                        macc(evx, c0, Mu.x(pr, i));
-                        macc(evy, c0, Mu.y(pr, i));
-                    }
-                    const float sg = m == 0 ? 1.f : (((m >> 1) & 1) ? -2.f : 2.f);   // 2 i^m up to i for odd m
-                    AE.set(pr, kk * NS + m, scale2(sg, closed(evx)), scale2(sg, closed(evy)));
-                    AO.set(pr, kk * NS + m, scale2(sg, closed(odx)), scale2(sg, closed(ody)));
-                }
-            }
-            __syncthreads();
-            // W_j = (w_k/M_k) [A^0 + 2 sum_m i^m Re(A^m e^{i m a_j})], A = AE +- AO.  Waves t and
-            // M_k/2 - t of a node have angles a and pi - a: e^{i m (pi - a)} = (-1)^m conj(e^{i m a}), so with
-            // P = sum a.x z.x and Q = sum a.y z.y over even (or odd) m, Re(A z) = P - Q serves wave t and
-            // (-1)^m Re(A conj z) = +-(P + Q) its partner: two multiply-adds per (m, set) for both waves.
-            const int ub = D.u_start[k0], un = D.u_start[k0 + kn] - ub;
-            for (int e = threadIdx.x; e < 2 * un; e += blockDim.x) {
-                const int pr = e & 1, u = ub + (e >> 1);
-                const int k = D.u_k[u], row = (k - k0) * NS;
-                const int j0 = D.k_start[k], H = D.k_start[k + 1] - j0, t = u - D.u_start[k], Mk = 2 * H;
-                const bool pair = t > 0 && 2 * t != H;
-                const cpx<dfl> *rt = D.roots + 2 * j0;
-                const dfl wm = D.e_wm[j0 + t];
-                int step2 = 2 * t;
-                if (step2 >= Mk) step2 -= Mk;
-#pragma unroll 1
-                for (int odd = 0; odd < 2; ++odd) {
-                    df2 pe = zero_df2(), qe = pe, po = pe, qo = pe;
-                    int idx = t, m = 1;
-                    if (!odd) {
-                        pe = AE.x(pr, row);
-                        po = AO.x(pr, row);
-                        idx = step2;
-                        m = 2;
-                    }
-                    for (; m <= p; m += 2) {
-                        const cpx<dfl> z = rt[idx];
-                        const int i = row + m;
-                        macc(pe, z.x, AE.x(pr, i));
-                        macc(qe, z.y, AE.y(pr, i));
-                        macc(po, z.x, AO.x(pr, i));
-                        macc(qo, z.y, AO.y(pr, i));
-                        idx += step2;
-                        if (idx >= Mk) idx -= Mk;
-                    }
-                    // real (even m) or imaginary (odd m) parts: + direction A = AE + AO, - direction AE - AO
-                    auto put = [&](int j, df2 a, df2 o) {
-                        float4 *d = out + 4 * j + 2 * odd + pr;
-                        const df2 W = dup(wm);
-                        d[0] = as_float4(renorm(mul_df(W, a + o)));
-                        d[4 * S] = as_float4(renorm(mul_df(W, a - o)));
-                    };
-                    put(j0 + t, pe - qe, po - qo);
-                    if (pair) {   // the partner, with sign (-1)^m
-                        const df2 eb = pe + qe, ob = po + qo;
-                        put(j0 + H - t, odd ? -eb : eb, odd ? -ob : ob);
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// X2X merge-and-shift (k_x2x), one thread per (wave, pair of sets).  Plain loads, two sources in flight: staging
-// each thread's sources through shared memory by asynchronous copies four steps ahead was slower
-// (1M-bead sphere 4.17 -> 4.46 ms, 15M-bead cube 25.7 -> 29.4 ms: it adds shared-memory instructions and
-// takes a third of the L1).
-// Blocks of 128 threads at 96 registers (five per SM) on large grids; of 256 threads (two per SM) where the
-// grid leaves the SMs room and a block's own length counts (1M-bead sphere 4.24 -> 3.71 ms and 15M-bead cube
-// 26.1 -> 23.0 ms from 256 to 128; 20k-bead sphere 0.133 -> 0.191 ms, 4,096 beads 0.058 -> 0.094 ms).
-constexpr int kX2XSmallGrid = 3000;   // blocks
-template <int THREADS, int BLOCKS>
-__global__ void __launch_bounds__(THREADS, BLOCKS)
-    k_x2x_df(const int *parents, DevTables<dfl> D, const int *coll, const int *child, const int *leaf,
-             const float4 *Xo, float4 *Xi, int f0, int nf) {
-    __shared__ int src[216];
-    __shared__ int vsrc[216], vsh[216], vpre[217];   // the present sources, compacted in slot order
-    __shared__ int vend[216];   // child mask of its group at the last present source of a group, else 0
-    const int P = parents[blockIdx.x];
-    const int dl = blockIdx.y, d = 2 * f0 + dl;   // direction, and its slot in this pass's buffers
-    const int S = D.S;
-    for (int sl = threadIdx.x; sl < 216; sl += blockDim.x) {
-        const int q = sl >> 3, o = sl & 7;
-        const int Q = coll[27 * P + q];
-        src[sl] = (Q >= 0 && !leaf[Q]) ? child[8 * Q + o] : -1;
-    }
-    __syncthreads();
-    const int ng = D.grp_n[d];
-    const int *goff = D.grp_off + d * (kGroupMax + 1);
-    const int *gmask = D.grp_mask + d * kGroupMax;
-    const int *slots = D.slot_list + d * 216;
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x, nsl = goff[ng];
-        int carry = 0;
-        for (int z0 = 0; z0 < nsl; z0 += 32) {
-            const int z = z0 + lane;
-            int ent = 0, sb = -1;
-            if (z < nsl) {
-                ent = slots[z];
-                sb = src[ent & 255];
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, sb >= 0);
-            const int pos = carry + __popc(bal & ((1u << lane) - 1u));
-            if (z < nsl) vpre[z] = pos;
-            if (sb >= 0) {
-                vsrc[pos] = sb;
-                vsh[pos] = (ent >> 8) * S;
-            }
-            carry += __popc(bal);
-        }
-        if (lane == 0) vpre[nsl] = carry;
-    }
-    __syncthreads();
-    const int nz = vpre[goff[ng]];
-    for (int z = threadIdx.x; z < nz; z += blockDim.x) vend[z] = 0;
-    __syncthreads();
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-        const int z1 = vpre[goff[g + 1]];
-        if (z1 > vpre[goff[g]]) vend[z1 - 1] = gmask[g];
-    }
-    __syncthreads();
-    const size_t dstride = size_t(2 * nf) * 4 * S;
-    const float4 *Xd = Xo + size_t(dl) * 4 * S;
-    for (int e = threadIdx.x; e < 2 * S; e += blockDim.x) {
-        const int j = e >> 1, pr = e & 1;
-        df2 ax[8], ay[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) ax[t] = ay[t] = zero_df2();
-        df2 gx = zero_df2(), gy = gx;
-#pragma unroll 2
-        for (int z = 0; z < nz; ++z) {
-            const float4 *xs = Xd + size_t(vsrc[z]) * dstride + 4 * j + pr;
-            const df2 x = as_df2(xs[0]), y = as_df2(xs[2]);
-            const cpx<dfl> sh = D.shift[vsh[z] + j];
-            const df2 sx = dup(sh.x), sy = dup(sh.y);
-            macc(gx, sx, x);
-            macc(gx, -sy, y);
-            macc(gy, sy, x);
-            macc(gy, sx, y);
-            const int mask = vend[z];   // block-uniform
-            if (mask) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    if ((mask >> t) & 1) {
-                        ax[t] = sum_raw(ax[t], gx);
-                        ay[t] = sum_raw(ay[t], gy);
-                    }
-                gx = gy = zero_df2();
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const int ch = child[8 * P + t];
-            if (ch < 0) continue;
-            const cpx<dfl> sh = D.shift[size_t(D.child_shift[d * 8 + t]) * S + j];
-            const df2 x = renorm(ax[t]), y = renorm(ay[t]);
-            float4 *dst = Xi + (size_t(ch) * (2 * nf) + dl) * 4 * S + 4 * j + pr;
-            dst[0] = as_float4(lin2(sh.x, x, -sh.y, y));
-            dst[2] = as_float4(lin2(sh.y, x, sh.x, y));
-        }
-    }
-}
-
-// X2L: one box per block, kc quadrature nodes at a time (umax wave-pair units at most).
-__global__ void __launch_bounds__(256, 3)
-    k_x2l_df(int b0, DevTables<dfl> D, const float4 *Xi, cpx<dfl> *L, int f0, int nf, int kc, int umax) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int b = b0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p), s = D.s, S = D.S, P1 = p + 1, NS = a_stride(p);
-    const Planes Lf{reinterpret_cast<float4 *>(smem_raw), nc};   // the frame's sums
-    // b+ + b- and b+ - b- per (node, m)
-    const Planes Bs{Lf.p + 4 * nc, kc * NS}, Bd{Bs.p + 4 * kc * NS, kc * NS};
-    // per unit (waves t and M_k/2 - t of a node): sums and differences of the pair's real and imaginary
-    // parts, UQ[direction][re +, re -, im +, im -][unit][pair of sets]
-    float4 *UQ = Bd.p + 4 * kc * NS;
-    const Planes Tm{Bs.p, nc};   // rotation scratch over the B rows and the units (node_chunk leaves room)
-    cpx<dfl> *dst = L + size_t(b) * kSets * nc;
-    for (int f = f0; f < f0 + nf; ++f) {
-        const float4 *in = Xi + (size_t(b) * (2 * nf) + 2 * (f - f0)) * 4 * S;
-        for (int k0 = 0; k0 < s; k0 += kc) {
-            const int kn = min(kc, s - k0);
-            const int ub = D.u_start[k0], un = D.u_start[k0 + kn] - ub;
-            __syncthreads();
-            for (int e = threadIdx.x; e < 4 * un; e += blockDim.x) {   // (unit, direction, pair of sets)
-                const int u = e >> 2, dir = (e >> 1) & 1, pr = e & 1;
-                const int k = D.u_k[ub + u], j0 = D.k_start[k], H = D.k_start[k + 1] - j0, t = ub + u - D.u_start[k];
-                const bool pair = t > 0 && 2 * t != H;
-                const float4 *w = in + dir * 4 * S + pr;
-                const df2 ax = as_df2(w[4 * (j0 + t)]), ay = as_df2(w[4 * (j0 + t) + 2]);
-                df2 bx = zero_df2(), by = bx;
-                if (pair) {
-                    bx = as_df2(w[4 * (j0 + H - t)]);
-                    by = as_df2(w[4 * (j0 + H - t) + 2]);
-                }
-                float4 *q = UQ + 8 * dir * umax + 2 * u + pr;
-                q[0] = as_float4(ax + bx);
-                q[2 * umax] = as_float4(ax - bx);
-                q[4 * umax] = as_float4(ay + by);
-                q[6 * umax] = as_float4(ay - by);
-            }
-            __syncthreads();
-            // b_k^m = sum_{j < M_k/2} (I_j + (-1)^m conj I_j) e^{-i m a_j}
-            //       = 2 sum_j Re(I_j) e^{-i m a_j}      (m even)
-            //       = 2i sum_j Im(I_j) e^{-i m a_j}     (m odd; the factor i is applied below)
-            // With e^{-i m (pi - a)} = (-1)^m conj(e^{-i m a}), a wave pair adds
-            // (v + (-1)^m v') cos(m a) - i (v - (-1)^m v') sin(m a): even m take the
-            // sum and difference of the real parts, odd m those of the imaginary parts.
-            // A thread takes node kk and its mirror kn - 1 - kk: the nodes' wave counts grow with k, so
-            // the sums over two mirrored nodes are about equally long.
-            const int items = ((kn + 1) >> 1) * P1;
-            for (int e = threadIdx.x; e < 2 * items; e += blockDim.x) {
-                const int pr = e & 1, r = e >> 1, ka = r / P1, m = r - ka * P1;
-                for (int h = 0; h < 2; ++h) {
-                    const int kk = h ? kn - 1 - ka : ka, k = k0 + kk;
-                    if (h && kk == ka) break;
-                    const int j0 = D.k_start[k], Mk = 2 * (D.k_start[k + 1] - j0);
-                    const int u0 = D.u_start[k] - ub, u1 = D.u_start[k + 1] - ub;
-                    const int mm = m % Mk;
-                    const cpx<dfl> *rt = D.roots + 2 * j0;
-                    const float4 *xp = UQ + ((m & 1) ? 6 : 0) * umax + pr, *yp = UQ + ((m & 1) ? 4 : 2) * umax + pr;
-                    df2 bpx = zero_df2(), bpy = bpx, bmx = bpx, bmy = bpx;
-                    int idx = 0;
-                    for (int u = u0; u < u1; ++u) {
-                        const cpx<dfl> z = rt[idx];
-                        macc(bpx, z.x, as_df2(xp[2 * u]));
-                        macc(bpy, -z.y, as_df2(yp[2 * u]));
-                        macc(bmx, z.x, as_df2(xp[8 * umax + 2 * u]));
-                        macc(bmy, -z.y, as_df2(yp[8 * umax + 2 * u]));
-                        idx += mm;
-                        if (idx >= Mk) idx -= Mk;
-                    }
-                    // the + direction and the reflected - direction enter L through
-                    // b+ + b- (n + m even) and b+ - b- (n + m odd)
-                    Bs.set(pr, kk * NS + m, bpx + bmx, bpy + bmy);
-                    Bd.set(pr, kk * NS + m, bpx - bmx, bpy - bmy);
-                }
-            }
-            __syncthreads();
-            // L_n^m = i^m sum_k (-lambda_k)^n / sqrt((n-m)!(n+m)!) b_k^m, the - direction reflected
-            for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) {
-                const int pr = e & 1, i = e >> 1, n = deg_of(i), m = i - tri(n, 0);
-                const Planes B = ((n + m) & 1) ? Bd : Bs;
-                df2 x = zero_df2(), y = x;
-                if (k0) {
-                    x = Lf.x(pr, i);
-                    y = Lf.y(pr, i);
-                }
-                const dfl *c = D.x2l_c + size_t(k0) * nc + i;
-                for (int kk = 0; kk < kn; ++kk, c += nc) {
-                    macc(x, *c, B.x(pr, kk * NS + m));
-                    macc(y, *c, B.y(pr, kk * NS + m));
-                }
-                x = closed(x);
-                y = closed(y);
-                if (k0 + kc >= s) {   // the last nodes: times 2 i^(m + (m & 1))
-                    const float sg = ((m + (m & 1)) & 2) ? -2.f : 2.f;
-                    x = scale2(sg, x);
-                    y = scale2(sg, y);
-                }
-                Lf.set(pr, i, x, y);
-            }
-        }
-        __syncthreads();
-        if (f > 0) {   // back to world axes; Lf is free once rotated about z
-            const dfl *rf = D.frot_bwd + size_t(f - 1) * D.frot_len;
-            rotate_z(rf, D.frot_off, nc, Tm, [&](int pr, int i, df2 &x, df2 &y) {
-                x = Lf.x(pr, i);
-                y = Lf.y(pr, i);
-            });
-            __syncthreads();
-            rotate_y(rf, D.frot_off, nc, Tm, Lf);
-            __syncthreads();
-        }
-        for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) {
-            const int pr = e & 1, i = e >> 1;
-            const df2 x = Lf.x(pr, i), y = Lf.y(pr, i);
-            cpx<dfl> *d0 = dst + 2 * pr * nc + i, *d1 = d0 + nc;
-            cpx<dfl> u = *d0, v = *d1;
-            u += mk(dfl(x.h.x, x.l.x), dfl(y.h.x, y.l.x));
-            v += mk(dfl(x.h.y, x.l.y), dfl(y.h.y, y.l.y));
-            *d0 = u;
-            *d1 = v;
-        }
-    }
-}
-
-// Four sets in one thread, for the box-origin form below.
-struct df4 {
-    df2 v[2];
-};
-__device__ __forceinline__ df4 zero_df4() { return df4{{zero_df2(), zero_df2()}}; }
-__device__ __forceinline__ void macc(df4 &acc, dfl s, const df4 &b) {
-    macc(acc.v[0], s, b.v[0]);
-    macc(acc.v[1], s, b.v[1]);
-}
-__device__ __forceinline__ df4 operator+(const df4 &a, const df4 &b) { return df4{{a.v[0] + b.v[0], a.v[1] + b.v[1]}}; }
-__device__ __forceinline__ df4 lin2(dfl a, const df4 &x, dfl b, const df4 &y) {
-    return df4{{lin2(a, x.v[0], b, y.v[0]), lin2(a, x.v[1], b, y.v[1])}};
-}
-
-// X2X with the box origin of q4 (k_x2x4), one thread per wave, all four sets.
-__global__ void __launch_bounds__(256, 1) k_x2x4_df(const int *parents, DevTables<dfl> D, const int *coll, const int *child, const int *leaf,
-                          const double *side, const float4 *Xo, float4 *Xi, int f0, int nf) {
-    __shared__ int src[216];
-    const int P = parents[blockIdx.x];
-    const int dl = blockIdx.y, d = 2 * f0 + dl;
-    const int S = D.S;
-    const double hc = 0.5 * side[P];   // side of P's children (and of the sources)
-    for (int sl = threadIdx.x; sl < 216; sl += blockDim.x) {
-        const int q = sl >> 3, o = sl & 7;
-        const int Q = coll[27 * P + q];
-        src[sl] = (Q >= 0 && !leaf[Q]) ? child[8 * Q + o] : -1;
-    }
-    __syncthreads();
-    const int ng = D.grp_n[d];
-    const int *goff = D.grp_off + d * (kGroupMax + 1);
-    const int *gmask = D.grp_mask + d * kGroupMax;
-    const int *slots = D.slot_list + d * 216;
-    const size_t dstride = size_t(2 * nf) * 4 * S;
-    const float4 *Xd = Xo + size_t(dl) * 4 * S;
-    // set 3 += (dx, dy, dz) . sets 0..2 of one part (re or im)
-    auto move = [](df4 &v, dfl dx, dfl dy, dfl dz) {
-        dfl a(v.v[1].h.y, v.v[1].l.y);
-        macc(a, dx, dfl(v.v[0].h.x, v.v[0].l.x));
-        macc(a, dy, dfl(v.v[0].h.y, v.v[0].l.y));
-        macc(a, dz, dfl(v.v[1].h.x, v.v[1].l.x));
-        a = closed(a);
-        v.v[1].h.y = a.h;
-        v.v[1].l.y = a.l;
-    };
-    for (int j = threadIdx.x; j < S; j += blockDim.x) {
-        df4 ax[8], ay[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) ax[t] = ay[t] = zero_df4();
-        for (int g = 0; g < ng; ++g) {
-            df4 gx = zero_df4(), gy = gx;
-            bool any = false;
-            for (int z = goff[g]; z < goff[g + 1]; ++z) {
-                const int ent = slots[z], sl = ent & 255, sb = src[sl];
-                if (sb < 0) continue;
-                any = true;
-                const float4 *xs = Xd + size_t(sb) * dstride + 4 * j;
-                df4 x{{as_df2(xs[0]), as_df2(xs[1])}}, y{{as_df2(xs[2]), as_df2(xs[3])}};
-                // slot = colleague (dx, dy, dz in -1..1, index 9 dz + 3 dy + dx + 13) x 8 + child octant:
-                // source centre - P's centre = hc (2 d + bit - 1/2) per axis, in world axes
-                const int q = sl >> 3, o = sl & 7;
-                const dfl ex(hc * (2 * (q % 3 - 1) + (o & 1) - 0.5)), ey(hc * (2 * ((q / 3) % 3 - 1) + ((o >> 1) & 1) - 0.5)),
-                    ez(hc * (2 * (q / 9 - 1) + ((o >> 2) & 1) - 0.5));
-                move(x, ex, ey, ez);
-                move(y, ex, ey, ez);
-                const cpx<dfl> sh = D.shift[size_t(ent >> 8) * S + j];
-                macc(gx, sh.x, x);
-                macc(gx, -sh.y, y);
-                macc(gy, sh.y, x);
-                macc(gy, sh.x, y);
-            }
-            if (!any) continue;
-            const int mask = gmask[g];
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-                if ((mask >> t) & 1) {
-                    ax[t] = ax[t] + gx;
-                    ay[t] = ay[t] + gy;
-                }
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const int ch = child[8 * P + t];
-            if (ch < 0) continue;
-            // P's centre - child t's centre = -(hc / 2) (2 bit - 1) per axis
-            const double h = 0.5 * hc;
-            const dfl ex((t & 1) ? -h : h), ey((t & 2) ? -h : h), ez((t & 4) ? -h : h);
-            move(ax[t], ex, ey, ez);
-            move(ay[t], ex, ey, ez);
-            const cpx<dfl> sh = D.shift[size_t(D.child_shift[d * 8 + t]) * S + j];
-            const df4 x = lin2(sh.x, ax[t], -sh.y, ay[t]), y = lin2(sh.y, ax[t], sh.x, ay[t]);
-            float4 *dst = Xi + (size_t(ch) * (2 * nf) + dl) * 4 * S + 4 * j;
-            dst[0] = as_float4(x.v[0]);
-            dst[1] = as_float4(x.v[1]);
-            dst[2] = as_float4(y.v[0]);
-            dst[3] = as_float4(y.v[1]);
-        }
-    }
-}
-
-
 // ---------------------------------------------------------------- far-field evaluation
 constexpr int kNE = 18;   // evaluation expansions of Eq. (2.8) per box
 constexpr int kNF = 12;   // evaluated per bead after the fold of k_eval_prep (per-potential form)
@@ -2246,16 +964,28 @@ __global__ void k_lap_eval(const int *leaves, DevTables<T> D, const int *beg, co
 
 // ---------------------------------------------------------------- driver
 
+// (never while a stream is being captured: the first, uncaptured matvec sets every limit it needs)
+static std::mutex g_smem_mu;
+static std::map<std::pair<int, const void *>, size_t> g_smem_done;
+
+int raise_smem(const void *kernel, size_t bytes) {
+    if (bytes <= 40 * 1024) return RPY_OK;   // below the default limit, static shared memory included
+    int dev = 0;
+    RPY_CHECK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(g_smem_mu);
+    size_t &d = g_smem_done[{dev, kernel}];
+    if (bytes > d) {
+        RPY_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+        d = bytes;
+    }
+    return RPY_OK;
+}
+
 template <typename T>
 static size_t smem_p2x(int p, int threads) {
     const int nc = ncoef(p), chunk = p2x_chunk(p, threads);
     return sizeof(T) * ((rec_floats<T>(p) + 1) & ~1) + sizeof(cpx<T>) * (chunk * nc + 2 * kSets * nc) +
            sizeof(T) * 4 * chunk + 64;
-}
-template <typename T>
-static size_t smem_m2x(int p, int s) {
-    int nc = ncoef(p);
-    return sizeof(cpx<T>) * (3 * kSets * nc + 2 * s * (kSets * (p + 1) + 1));
 }
 template <typename T>
 static size_t smem_far(int p) {
@@ -2266,147 +996,6 @@ template <typename T>
 static size_t smem_lap(int p) {
     int st = ncoef(p + 2);
     return sizeof(T) * tab_floats<T>(p) + sizeof(cpx<T>) * (13 * st + 3 * st + ncoef(p)) + 64;
-}
-
-// Raise a kernel's dynamic shared-memory limit once per device and kernel
-// (never while a stream is being captured: the first, uncaptured matvec sets
-// every limit it needs).
-static std::mutex g_smem_mu;
-static std::map<std::pair<int, const void *>, size_t> g_smem_done;
-
-template <typename K>
-static int set_smem(K kernel, size_t bytes) {
-    if (bytes <= 40 * 1024) return RPY_OK;   // below the default limit, static shared memory included
-    int dev = 0;
-    RPY_CHECK(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lk(g_smem_mu);
-    size_t &d = g_smem_done[{dev, reinterpret_cast<const void *>(kernel)}];
-    if (bytes > d) {
-        RPY_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
-        d = bytes;
-    }
-    return RPY_OK;
-}
-
-// Threads of an X2X block: each handles elements e, e + blockDim, ... of the
-// 4 S merged plane waves; the fewest warps that keep the number of rounds of
-// 256 threads, so that the last round is not left nearly empty.
-static int even_threads(int items, int most = 256) {
-    const int rounds = (items + most - 1) / most;
-    return std::max(64, ((items + rounds - 1) / rounds + 31) / 32 * 32);
-}
-static int x2x_threads(int S) { return even_threads(kSets * S); }
-
-// Node chunks of the double-float M2X and X2L (equal ones): one for all nodes, split until the block's
-// shared memory (fixed bytes + per-node bytes + 256 bytes per wave-pair unit when units are staged) is at most
-// 48 KB (56 KB with units), or until a chunk of X2L holds at most 200 (node, m) sums, below which its phases
-// run out of threads.  Measured: X2L of the 1M-bead sphere (p = 16) 7.2 / 9.9 ms at 49 / 98 KB; of the 200k sphere at 9
-// digits (p = 25) 13.9 / 8.5 / 7.5 ms at 56 / 72 / 100 KB; M2X there 11.4 / 5.3 / 5.5 ms at 30 / 48 / 60 KB.
-struct NodeChunk {
-    int kc, umax;
-    size_t smem;
-};
-static NodeChunk node_chunk(const OpTables &h, bool stage_units) {
-    const int nc = ncoef(h.p), NS = a_stride(h.p);
-    NodeChunk c{};
-    for (int nch = 1; nch <= h.s; ++nch) {   // equal chunks
-        const int kc = (h.s + nch - 1) / nch;
-        int um = 0;
-        for (int k0 = 0; k0 < h.s; k0 += kc) um = std::max(um, h.u_start[std::min(h.s, k0 + kc)] - h.u_start[k0]);
-        // the rotation scratch (4 nc float4) shares the memory of the rows and the staged units
-        const size_t work = std::max(size_t(8) * kc * NS + (stage_units ? 16 * size_t(um) : 0), size_t(4) * nc);
-        c = NodeChunk{kc, um, sizeof(float4) * (4 * size_t(nc) + work)};
-        if (c.smem <= (stage_units ? 56u : 48u) * 1024 || (stage_units && kc * (h.p + 1) <= 200)) break;
-    }
-    return c;
-}
-
-static int run_waves_df(Tree &t, const DevTables<dfl> &D, const cpx<dfl> *M, cpx<dfl> *L, int rb, cudaStream_t st) {
-    const int nf = t.x_frames, b2 = t.level_off[2], n2 = t.nbox - b2, p = D.p;
-    float4 *Xo = static_cast<float4 *>(t.Xo), *Xi = static_cast<float4 *>(t.Xi);
-    const NodeChunk cm = node_chunk(*t.tabs, false), cl = node_chunk(*t.tabs, true);
-    RPY_TRY(set_smem(k_m2x_df, cm.smem));
-    RPY_TRY(set_smem(k_x2l_df, cl.smem));
-    for (int f0 = 0; f0 < 3; f0 += nf) {
-        prof_mark(t, RPY_STAGE_M2X, st);
-        k_m2x_df<<<n2, even_threads(2 * cm.umax), cm.smem, st>>>(b2, D, M, Xo, f0, nf, cm.kc);
-        RPY_LAUNCHED(1);
-        RPY_CHECK(cudaGetLastError());
-        prof_mark(t, RPY_STAGE_X2X, st);
-        if (t.n_x2x_par > 0) {
-            const dim3 g(t.n_x2x_par, 2 * nf);
-            if (rb)
-                k_x2x4_df<<<g, even_threads(D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf, t.side_u, Xo,
-                                                           Xi, f0, nf);
-            else if (t.n_x2x_par * 2 * nf < kX2XSmallGrid)
-                k_x2x_df<256, 2><<<g, even_threads(2 * D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf, Xo,
-                                                                      Xi, f0, nf);
-            else
-                k_x2x_df<128, 5><<<g, even_threads(2 * D.S, 128), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                           Xo, Xi, f0, nf);
-            RPY_LAUNCHED(1);
-            RPY_CHECK(cudaGetLastError());
-        }
-        prof_mark(t, RPY_STAGE_X2L, st);
-        k_x2l_df<<<n2, even_threads((cl.kc + 1) / 2 * (p + 1) * 2), cl.smem, st>>>(b2, D, Xi, L, f0, nf, cl.kc, cl.umax);
-        RPY_LAUNCHED(1);
-        RPY_CHECK(cudaGetLastError());
-    }
-    return RPY_OK;
-}
-
-static int run_waves_f32(Tree &t, const DevTables<float> &D, const cpx<float> *M, cpx<float> *L, int rb,
-                         cudaStream_t st) {
-    const int nf = t.x_frames, b2 = t.level_off[2], n2 = t.nbox - b2, p = D.p;
-    cpx<float> *Xo = static_cast<cpx<float> *>(t.Xo), *Xi = static_cast<cpx<float> *>(t.Xi);
-    const size_t smx = smem_m2x<float>(p, D.s), sxl = smem_x2l4(p, D.s, D.S);
-    const bool col = y_by_column(sizeof(float), p);
-    auto m2x = col ? k_m2x<float, true> : k_m2x<float, false>;
-    auto x2l = col ? k_x2l4<true> : k_x2l4<false>;
-    RPY_TRY(set_smem(m2x, smx));
-    RPY_TRY(set_smem(x2l, sxl));
-    for (int f0 = 0; f0 < 3; f0 += nf) {
-        prof_mark(t, RPY_STAGE_M2X, st);
-        m2x<<<n2, even_threads(D.S), smx, st>>>(b2, n2, D, M, Xo, f0, nf);
-        RPY_LAUNCHED(1);
-        RPY_CHECK(cudaGetLastError());
-        prof_mark(t, RPY_STAGE_X2X, st);
-        if (t.n_x2x_par > 0) {
-            const dim3 g(t.n_x2x_par, 2 * nf);
-            if (D.S > 256 && D.S <= 480) {
-                // a producer warp stages the sources through shared memory by bulk copies
-                // (measured faster than per-thread loads from 323 stored waves up; at 3 digits,
-                // 134 waves, the per-thread loads below keep two to three blocks per SM and win)
-                const size_t sxx = x2x_tma_smem(D.S);
-                RPY_TRY(set_smem(k_x2x_tma, sxx));
-                k_x2x_tma<<<g, (D.S + 31) / 32 * 32 + 32, sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                     t.b_side, Xo, Xi, f0, nf, rb, t.dev_status);
-            } else if (D.S <= 256) {
-                // shifts from per-axis factors in shared memory (measured faster there; at more
-                // waves the shared memory costs occupancy and the table is faster)
-                const size_t sxx = sizeof(float) * ((6 * D.S + 3) & ~3) + 2 * sizeof(cpx<float>) * 6 * D.S;
-                if (rb)
-                    k_x2x4<float, true><<<g, even_threads(D.S), sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                           t.b_side, Xo, Xi, f0, nf, rb);
-                else   // cube origin, few plane waves: one set per thread
-                    k_x2x<float, true><<<g, x2x_threads(D.S), sxx, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                         Xo, Xi, f0, nf);
-            } else {
-                k_x2x4<float, false><<<g, even_threads(D.S), 0, st>>>(t.x2x_par, D, t.b_coll, t.b_child, t.b_leaf,
-                                                                      t.b_side, Xo, Xi, f0, nf, rb);
-            }
-            RPY_LAUNCHED(1);
-            RPY_CHECK(cudaGetLastError());
-        }
-        prof_mark(t, RPY_STAGE_X2L, st);
-        // blocks sized to the (node, m) items of the widest phase at low order; at high order the
-        // shared memory already limits the blocks per SM and 256 threads hide latency better
-        const int tx = D.s * (p + 1) <= 256 ? even_threads(D.s * (p + 1)) : 256;
-        x2l<<<n2, tx, sxl, st>>>(b2, n2, D, Xi, L, f0, nf);
-        RPY_LAUNCHED(1);
-        RPY_CHECK(cudaGetLastError());
-    }
-    return RPY_OK;
 }
 
 template <typename T>
@@ -2479,8 +1068,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     // plane-wave buffers of six directions would not fit) one frame per pass,
     // each pass adding its frame's share into L (with profiling on, every pass's
     // M2X, X2X and X2L launches are timed under their own stages).
-    if constexpr (kIsDf<T>) RPY_TRY(run_waves_df(t, D, M, L, rb, st));
-    else RPY_TRY(run_waves_f32(t, D, M, L, rb, st));
+    RPY_TRY(run_waves_t(t, D, M, L, rb, st));
     // X list
     prof_mark(t, RPY_STAGE_P2L, st);
     k_p2x<T, 1><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,

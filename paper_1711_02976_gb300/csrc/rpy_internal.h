@@ -173,7 +173,8 @@ struct DevTables {
     const cpx<T> *roots;
     const T *m2x_c, *x2l_c;
     const int *e_k, *k_start;
-    const int *u_k, *u_start;   // wave-pair units
+    const int *u_start;         // wave-pair units: first unit of node k
+    const int4 *u_info;         // per unit: node, first stored wave of the node, waves of the node, t
     int NU;
     const T *e_cos, *e_sin, *e_wm;
     const cpx<T> *shift;
