@@ -562,9 +562,9 @@ __global__ void __launch_bounds__(kDfThreads, 2)
 
 // ---------------------------------------------------------------- FP32 form
 constexpr int kP32Threads = 256;
-constexpr int kP32Chunk = 512;     // sources staged per pass
+constexpr int kP32Chunk = 1024;    // sources staged per pass at most
 constexpr int kP32List = 256;      // list boxes per prefix segment
-constexpr int kP32Block = 32;      // sources per plain FP32 block between Kahan merges
+constexpr int kP32Block = 32;      // source pairs per plain FP32 block (terms per lane) between Kahan merges
 
 struct P32Const {
     float a2x4, tiny2, k23, nk2;
@@ -622,23 +622,16 @@ __device__ __forceinline__ void pair32(float dx, float dy, float dz, float r2, f
     pz = fmaf(t2, dz, fmaf(t1, fz, pz));
 }
 
-// Packed forms over the two targets of a thread (lane .x target a, lane .y
-// target b) and one staged source.  x - x_j is formed as x + (-x_j), which
-// rounds as the difference does.
-__device__ __forceinline__ float2 packed_d(float2 X, float nx0, float nx1) {
-    return __fadd2_rn(X, make_float2(nx0, nx1));
-}
-
+// Packed forms over a pair of staged sources (lanes .x and .y) and the thread's target.
+// x - x_j is formed as x + (-x_j), which rounds as the difference does.
 __device__ __forceinline__ float2 packed_r2(float2 DX, float2 DY, float2 DZ) {
     return __ffma2_rn(DZ, DZ, __ffma2_rn(DY, DY, __fmul2_rn(DX, DX)));
 }
 
-// The r >= 2a branch of pair32 on both lanes, for pairs known to be far (the
-// clamp and the selects of pair32 are then the identity): the same operations
-// in the same order, hence the same rounding lane by lane.
-__device__ __forceinline__ void far_packed(float2 DX, float2 DY, float2 DZ, float2 R2, float2 FX, float2 FY,
+// The r >= 2a branch of pair32 on both lanes, for pairs known to be far (the clamp and the selects of pair32
+// are then the identity): the same operations in the same order, hence the same rounding lane by lane.
+__device__ __forceinline__ void far_packed(float2 DX, float2 DY, float2 DZ, float2 RI, float2 FX, float2 FY,
                                            float2 FZ, float2 K23, float2 NK2, float2 &AX, float2 &AY, float2 &AZ) {
-    const float2 RI = make_float2(rsqrt_ftz(R2.x), rsqrt_ftz(R2.y));
     const float2 RI2 = __fmul2_rn(RI, RI);
     const float2 B = __fmul2_rn(RI, RI2);
     const float2 T1 = __ffma2_rn(K23, B, RI);
@@ -648,6 +641,7 @@ __device__ __forceinline__ void far_packed(float2 DX, float2 DY, float2 DZ, floa
     AY = __ffma2_rn(T2, DY, __ffma2_rn(T1, FY, AY));
     AZ = __ffma2_rn(T2, DZ, __ffma2_rn(T1, FZ, AZ));
 }
+__device__ __forceinline__ float2 rsqrt2(float2 r2) { return make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)); }
 
 __device__ __forceinline__ void kahan_merge(float &s, float &c, float v) {
     float y = v - c;
@@ -656,14 +650,18 @@ __device__ __forceinline__ void kahan_merge(float &s, float &c, float v) {
     s = t;
 }
 
-// A leaf of T beads: R = min(ceil(T/2), blockDim) threads per pass carry
-// targets i0 + t and i0 + R + t (the two lanes of each packed chain);
-// G = blockDim / R groups split every staged chunk.  The U list's boxes are
-// prefix-summed in shared memory and each staged bead finds its box by
-// binary search.
+// An item of T targets uses G = blockDim / T groups of T threads, one target each; the list's beads are staged
+// as pairs and group g takes every G-th pair, two pairs (four sources) per iteration.  The list's boxes are
+// prefix-summed in shared memory and each staged bead finds its box by binary search.  Chunks are of equal size.
+// A vote picks the form of each iteration: all pairs of the warp far (the packed far branch alone), otherwise
+// both branches with selects.
+// Bound by the FP32 FMA pipe (63% busy) and the issue slots.  Sources rather than targets in the two lanes: half the
+// staging memory per source, so chunks of 1,024 instead of 512, and half the running sums; 15M-bead cube
+// 22.25 -> 22.1 ms, 256 systems 29.2 -> 28.5, noise 50k 0.071 -> 0.064.  A third form for iterations that are far but for
+// self pairs (1 in 27 on a uniform system, with 1/r = 0 there) was no faster: 22.2 and 29.2 ms.
 constexpr int kP32Queue = 256;   // FP64 pairs of one staged chunk handled after its FP32 loop
-constexpr size_t kP32Smem = sizeof(float4) * 3 * kP32Chunk + sizeof(int) * kP32Chunk +
-                            sizeof(float2) * 6 * kP32Threads + sizeof(double) * 6 * kP32Threads +
+constexpr size_t kP32Smem = sizeof(float4) * 3 * (kP32Chunk / 2) + sizeof(float2) * 3 * kP32Threads +
+                            sizeof(double) * 3 * kP32Threads + sizeof(int) * kP32Chunk +
                             sizeof(int) * (2 * kP32List + 2) + sizeof(float) * 6 + sizeof(int) * (kP32Queue + 2);
 
 __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, const int *leaves, const int *beg,
@@ -673,16 +671,16 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, con
                                                          const double *pos, const double *fs, int64_t n, SysConst sc,
                                                          int add_self, double *out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // staged source e, relative to the target leaf centre, each value twice (both lanes of a
-    // packed pair): sS[3e] = (-x, -x, -y, -y), sS[3e+1] = (-z, -z, fx, fx), sS[3e+2] = (fy, fy, fz, fz)
+    // staged pair e, relative to the target leaf centre: sS[3e] = (-x, -x', -y, -y'),
+    // sS[3e+1] = (-z, -z', fx, fx'), sS[3e+2] = (fy, fy', fz, fz')
     float4 *sS = reinterpret_cast<float4 *>(smem_raw);
-    float2 *sK = reinterpret_cast<float2 *>(sS + 3 * kP32Chunk);   // [6][kP32Threads] Kahan states (S, C)
-    double *sD = reinterpret_cast<double *>(sK + 6 * kP32Threads);   // [kP32Threads][6] FP64 pairs
-    int *sJ = reinterpret_cast<int *>(sD + 6 * kP32Threads);
+    float2 *sK = reinterpret_cast<float2 *>(sS + 3 * (kP32Chunk / 2));   // [3][kP32Threads] Kahan states (S, C)
+    double *sD = reinterpret_cast<double *>(sK + 3 * kP32Threads);       // [kP32Threads][3] FP64 pairs
+    int *sJ = reinterpret_cast<int *>(sD + 3 * kP32Threads);
     int *lb = sJ + kP32Chunk, *lpre = lb + kP32List;
     float *sCtr = reinterpret_cast<float *>(lpre + kP32List + 2);   // target leaf centre, hi and lo floats
-    int *sQn = reinterpret_cast<int *>(sCtr + 6);   // [0] queue length, [1] any FP64 pair in this pass
-    int *sQ = sQn + 2;                              // queued pairs: thread << 11 | source slot << 1 | target
+    int *sQn = reinterpret_cast<int *>(sCtr + 6);   // [0] queue length, [1] any FP64 pair of this item
+    int *sQ = sQn + 2;                              // queued pairs: thread << 11 | source slot
     const int2 item = items[blockIdx.x];
     const int li = item.x, b = leaves[li], sys = bsys[b];
     const PairConst &pc = sc.pc[sys];
@@ -701,209 +699,194 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, con
         sCtr[threadIdx.x] = h;
         sCtr[3 + threadIdx.x] = float(c - double(h));
     }
-    if (threadIdx.x == 0) sQn[0] = 0;
+    if (threadIdx.x == 0) sQn[0] = sQn[1] = 0;
     __syncthreads();
     const float chx = sCtr[0], chy = sCtr[1], chz = sCtr[2], clx = sCtr[3], cly = sCtr[4], clz = sCtr[5];
     const float *xh = p32, *yh = p32 + n, *zh = p32 + 2 * n, *xl = p32 + 3 * n, *yl = p32 + 4 * n, *zl = p32 + 5 * n;
     const float2 K23 = make_float2(k.k23, k.k23), NK2 = make_float2(k.nk2, k.nk2);
     const int u0 = uoff[li], u1 = uoff[li + 1];
     const int tb = item.y, te = min(end[b], item.y + kItemTargets), nt = te - tb;
-    const int half = (nt + 1) / 2;
-    const int Rn = half < kP32Threads ? half : kP32Threads;
-    const int G = kP32Threads / Rn;
-    const int tl = threadIdx.x % Rn, g = threadIdx.x / Rn;
+    const int G = kP32Threads / nt;
+    const int tl = threadIdx.x % nt, g = threadIdx.x / nt;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i0 = tb; i0 < te; i0 += 2 * Rn) {
-        const int ia = i0 + tl, ib = i0 + Rn + tl;
-        const bool act = g < G && ia < te;
-        const bool actb = act && ib < te;
-        // an absent second target sits far away: its chain stays on the far branch
-        const float xa = act ? (xh[ia] - chx) + (xl[ia] - clx) : 0.f;
-        const float ya = act ? (yh[ia] - chy) + (yl[ia] - cly) : 0.f;
-        const float za = act ? (zh[ia] - chz) + (zl[ia] - clz) : 0.f;
-        const float xb = actb ? (xh[ib] - chx) + (xl[ib] - clx) : 1e15f;
-        const float yb = actb ? (yh[ib] - chy) + (yl[ib] - cly) : 1e15f;
-        const float zb = actb ? (zh[ib] - chz) + (zl[ib] - clz) : 1e15f;
-        const float2 X = make_float2(xa, xb), Y = make_float2(ya, yb), Z = make_float2(za, zb);
-        for (int c = 0; c < 6; ++c) {
-            sK[c * kP32Threads + threadIdx.x] = make_float2(0.f, 0.f);
-            sD[6 * threadIdx.x + c] = 0.0;
-        }
-        if (threadIdx.x == 0) sQn[1] = 0;
-        for (int us = u0; us < u1; us += kP32List) {
-            const int L = min(kP32List, u1 - us);
-            __syncthreads();
-            // prefix of the box sizes of this list segment (warp 0)
-            if (warp == 0) {
-                int carry = 0;
-                for (int q0 = 0; q0 < L; q0 += 32) {
-                    int q = q0 + lane, cnt = 0;
-                    if (q < L) {
-                        int C = uidx[us + q];
-                        lb[q] = beg[C];
-                        cnt = end[C] - beg[C];
-                    }
-                    int v = cnt;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        int w = __shfl_up_sync(0xffffffffu, v, o);
-                        if (lane >= o) v += w;
-                    }
-                    if (q < L) lpre[q + 1] = carry + v;
-                    carry += __shfl_sync(0xffffffffu, v, 31);
+    const int i = tb + tl;
+    const bool act = g < G;
+    const float xa = (xh[i] - chx) + (xl[i] - clx), ya = (yh[i] - chy) + (yl[i] - cly), za = (zh[i] - chz) + (zl[i] - clz);
+    const float2 X = make_float2(xa, xa), Y = make_float2(ya, ya), Z = make_float2(za, za);
+    for (int c = 0; c < 3; ++c) {
+        sK[c * kP32Threads + threadIdx.x] = make_float2(0.f, 0.f);
+        sD[3 * threadIdx.x + c] = 0.0;
+    }
+    for (int us = u0; us < u1; us += kP32List) {
+        const int L = min(kP32List, u1 - us);
+        __syncthreads();
+        // prefix of the box sizes of this list segment (warp 0)
+        if (warp == 0) {
+            int carry = 0;
+            for (int q0 = 0; q0 < L; q0 += 32) {
+                int q = q0 + lane, cnt = 0;
+                if (q < L) {
+                    int C = uidx[us + q];
+                    lb[q] = beg[C];
+                    cnt = end[C] - beg[C];
                 }
-                if (lane == 0) lpre[0] = 0;
+                int v = cnt;
+                for (int o = 1; o < 32; o <<= 1) {
+                    int w = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += w;
+                }
+                if (q < L) lpre[q + 1] = carry + v;
+                carry += __shfl_sync(0xffffffffu, v, 31);
             }
-            __syncthreads();
-            const int Ns = lpre[L];
-            for (int c0 = 0; c0 < Ns; c0 += kP32Chunk) {
-                const int nS = min(kP32Chunk, Ns - c0);
-                // no barrier here: the one after the prefix (first chunk) or after the
-                // previous chunk's compute (and its FP64 queue pass) already orders
-                // every read of sS and sJ before this chunk's writes
-                for (int e = threadIdx.x; e < nS; e += kP32Threads) {
+            if (lane == 0) lpre[0] = 0;
+        }
+        __syncthreads();
+        const int Ns = lpre[L];
+        const int nch = (Ns + kP32Chunk - 1) / kP32Chunk;
+        const int csz = nch ? ((Ns + nch - 1) / nch + 1) & ~1 : 2;   // equal chunks of whole pairs
+        for (int c0 = 0; c0 < Ns; c0 += csz) {
+            const int nS = min(csz, Ns - c0), nP = (nS + 1) >> 1;
+            // no barrier here: the one after the prefix (first chunk) or after the
+            // previous chunk's compute (and its FP64 queue pass) already orders
+            // every read of sS and sJ before this chunk's writes
+            for (int e = threadIdx.x; e < 2 * nP; e += kP32Threads) {
+                float *w = reinterpret_cast<float *>(sS + 3 * (e >> 1)) + (e & 1);
+                float px = 1e15f, py = 1e15f, pz = 1e15f, fx = 0.f, fy = 0.f, fz = 0.f;
+                int j = -1;   // an odd last source gets a far partner without force
+                if (e < nS) {
                     int q = c0 + e, lo = 0, hi = L;   // box: lpre[lo] <= q < lpre[lo + 1]
                     while (hi - lo > 1) {
                         int mid = (lo + hi) >> 1;
                         if (lpre[mid] <= q) lo = mid;
                         else hi = mid;
                     }
-                    int j = lb[lo] + (q - lpre[lo]);
-                    const float px = (xh[j] - chx) + (xl[j] - clx), py = (yh[j] - chy) + (yl[j] - cly),
-                                pz = (zh[j] - chz) + (zl[j] - clz);
-                    const float fx = f32[j], fy = f32[n + j], fz = f32[2 * n + j];
-                    sS[3 * e] = make_float4(-px, -px, -py, -py);
-                    sS[3 * e + 1] = make_float4(-pz, -pz, fx, fx);
-                    sS[3 * e + 2] = make_float4(fy, fy, fz, fz);
-                    sJ[e] = j;
+                    j = lb[lo] + (q - lpre[lo]);
+                    px = (xh[j] - chx) + (xl[j] - clx);
+                    py = (yh[j] - chy) + (yl[j] - cly);
+                    pz = (zh[j] - chz) + (zl[j] - clz);
+                    fx = f32[j];
+                    fy = f32[n + j];
+                    fz = f32[2 * n + j];
                 }
-                __syncthreads();
-                if (act) {
-                    for (int jb = g; jb < nS; jb += kP32Block * G) {
-                        const int je = min(nS, jb + kP32Block * G);
-                        // accumulators: lane .x for target a, lane .y for target b
-                        float2 AX = make_float2(0.f, 0.f), AY = AX, AZ = AX;
-                        // both branches with selects per target, and the close-pair queue
-                        auto slow = [&](int jj, float2 DX, float2 DY, float2 DZ, float2 R2, float2 FX, float2 FY,
-                                        float2 FZ) {
-                            pair32(DX.x, DY.x, DZ.x, R2.x, FX.x, FY.x, FZ.x, k, AX.x, AY.x, AZ.x);
-                            pair32(DX.y, DY.y, DZ.y, R2.y, FX.x, FY.x, FZ.x, k, AX.y, AY.y, AZ.y);
-                            if (!(R2.x > k.tiny2) || !(R2.y > k.tiny2)) {
-                                // the self pair, or beads within 1e-3 a: queue all but the self pair
-                                const int jg = sJ[jj];
-                                if (!(R2.x > k.tiny2) && jg != ia) {
-                                    int q = atomicAdd(&sQn[0], 1);
-                                    if (q < kP32Queue) sQ[q] = (threadIdx.x << 11) | (jj << 1);
-                                }
-                                if (actb && !(R2.y > k.tiny2) && jg != ib) {
-                                    int q = atomicAdd(&sQn[0], 1);
-                                    if (q < kP32Queue) sQ[q] = (threadIdx.x << 11) | (jj << 1) | 1;
-                                }
+                w[0] = -px;
+                w[2] = -py;
+                w[4] = -pz;
+                w[6] = fx;
+                w[8] = fy;
+                w[10] = fz;
+                sJ[e] = j;
+            }
+            __syncthreads();
+            if (act) {
+                for (int eb = g; eb < nP; eb += kP32Block * G) {
+                    const int ee = min(nP, eb + kP32Block * G);
+                    float2 AX = make_float2(0.f, 0.f), AY = AX, AZ = AX;   // lane sums of this block
+                    // pairs at most 1e-3 a apart other than the self pair: to FP64
+                    auto close = [&](int e, float2 R2) {
+                        for (int h = 0; h < 2; ++h)
+                            if (!((h ? R2.y : R2.x) > k.tiny2) && sJ[2 * e + h] != i) {
+                                const int q = atomicAdd(&sQn[0], 1);
+                                if (q < kP32Queue) sQ[q] = (threadIdx.x << 11) | (2 * e + h);
                             }
-                        };
-                        // Two staged sources per iteration: two independent packed chains.  When
-                        // every pair of the lanes running the iteration is far (a warp-uniform
-                        // vote), the far branch alone on packed pairs, the same operations as
-                        // pair32's far branch lane by lane; otherwise the slow form above.
-                        int jj = jb;
-                        for (; jj + G < je; jj += 2 * G) {
-                            const int j1 = jj + G;
-                            const float4 S0 = sS[3 * jj], S1 = sS[3 * jj + 1], S2 = sS[3 * jj + 2];
-                            const float4 U0 = sS[3 * j1], U1 = sS[3 * j1 + 1], U2 = sS[3 * j1 + 2];
-                            const float2 DX = packed_d(X, S0.x, S0.y), DY = packed_d(Y, S0.z, S0.w),
-                                         DZ = packed_d(Z, S1.x, S1.y);
-                            const float2 EX = packed_d(X, U0.x, U0.y), EY = packed_d(Y, U0.z, U0.w),
-                                         EZ = packed_d(Z, U1.x, U1.y);
-                            const float2 R2 = packed_r2(DX, DY, DZ), Q2 = packed_r2(EX, EY, EZ);
-                            const float2 FX = make_float2(S1.z, S1.w), FY = make_float2(S2.x, S2.y),
-                                         FZ = make_float2(S2.z, S2.w);
-                            const float2 GX = make_float2(U1.z, U1.w), GY = make_float2(U2.x, U2.y),
-                                         GZ = make_float2(U2.z, U2.w);
-                            if (__all_sync(__activemask(), fminf(fminf(R2.x, R2.y), fminf(Q2.x, Q2.y)) >= k.a2x4)) {
-                                far_packed(DX, DY, DZ, R2, FX, FY, FZ, K23, NK2, AX, AY, AZ);
-                                far_packed(EX, EY, EZ, Q2, GX, GY, GZ, K23, NK2, AX, AY, AZ);
-                                continue;
-                            }
-                            slow(jj, DX, DY, DZ, R2, FX, FY, FZ);
-                            slow(j1, EX, EY, EZ, Q2, GX, GY, GZ);
+                    };
+                    // both branches with selects
+                    auto slow = [&](int e, float2 DX, float2 DY, float2 DZ, float2 R2, float2 FX, float2 FY, float2 FZ) {
+                        pair32(DX.x, DY.x, DZ.x, R2.x, FX.x, FY.x, FZ.x, k, AX.x, AY.x, AZ.x);
+                        pair32(DX.y, DY.y, DZ.y, R2.y, FX.y, FY.y, FZ.y, k, AX.y, AY.y, AZ.y);
+                        if (!(R2.x > k.tiny2) || !(R2.y > k.tiny2)) close(e, R2);
+                    };
+                    int e = eb;
+                    for (; e + G < ee; e += 2 * G) {
+                        const int e1 = e + G;
+                        const float4 S0 = sS[3 * e], S1 = sS[3 * e + 1], S2 = sS[3 * e + 2];
+                        const float4 U0 = sS[3 * e1], U1 = sS[3 * e1 + 1], U2 = sS[3 * e1 + 2];
+                        const float2 DX = __fadd2_rn(X, make_float2(S0.x, S0.y)), DY = __fadd2_rn(Y, make_float2(S0.z, S0.w)),
+                                     DZ = __fadd2_rn(Z, make_float2(S1.x, S1.y));
+                        const float2 EX = __fadd2_rn(X, make_float2(U0.x, U0.y)), EY = __fadd2_rn(Y, make_float2(U0.z, U0.w)),
+                                     EZ = __fadd2_rn(Z, make_float2(U1.x, U1.y));
+                        const float2 R2 = packed_r2(DX, DY, DZ), Q2 = packed_r2(EX, EY, EZ);
+                        const float2 FX = make_float2(S1.z, S1.w), FY = make_float2(S2.x, S2.y),
+                                     FZ = make_float2(S2.z, S2.w);
+                        const float2 GX = make_float2(U1.z, U1.w), GY = make_float2(U2.x, U2.y),
+                                     GZ = make_float2(U2.z, U2.w);
+                        if (__all_sync(__activemask(), fminf(fminf(R2.x, R2.y), fminf(Q2.x, Q2.y)) >= k.a2x4)) {
+                            far_packed(DX, DY, DZ, rsqrt2(R2), FX, FY, FZ, K23, NK2, AX, AY, AZ);
+                            far_packed(EX, EY, EZ, rsqrt2(Q2), GX, GY, GZ, K23, NK2, AX, AY, AZ);
+                        } else {
+                            slow(e, DX, DY, DZ, R2, FX, FY, FZ);
+                            slow(e1, EX, EY, EZ, Q2, GX, GY, GZ);
                         }
-                        if (jj < je) {
-                            const float4 S0 = sS[3 * jj], S1 = sS[3 * jj + 1], S2 = sS[3 * jj + 2];
-                            const float2 DX = packed_d(X, S0.x, S0.y), DY = packed_d(Y, S0.z, S0.w),
-                                         DZ = packed_d(Z, S1.x, S1.y);
-                            const float2 R2 = packed_r2(DX, DY, DZ);
-                            const float2 FX = make_float2(S1.z, S1.w), FY = make_float2(S2.x, S2.y),
-                                         FZ = make_float2(S2.z, S2.w);
-                            if (__all_sync(__activemask(), fminf(R2.x, R2.y) >= k.a2x4))
-                                far_packed(DX, DY, DZ, R2, FX, FY, FZ, K23, NK2, AX, AY, AZ);
-                            else
-                                slow(jj, DX, DY, DZ, R2, FX, FY, FZ);
-                        }
-                        const float Pv[6] = {AX.x, AY.x, AZ.x, AX.y, AY.y, AZ.y};
+                    }
+                    if (e < ee) {
+                        const float4 S0 = sS[3 * e], S1 = sS[3 * e + 1], S2 = sS[3 * e + 2];
+                        const float2 DX = __fadd2_rn(X, make_float2(S0.x, S0.y)), DY = __fadd2_rn(Y, make_float2(S0.z, S0.w)),
+                                     DZ = __fadd2_rn(Z, make_float2(S1.x, S1.y));
+                        const float2 R2 = packed_r2(DX, DY, DZ);
+                        const float2 FX = make_float2(S1.z, S1.w), FY = make_float2(S2.x, S2.y),
+                                     FZ = make_float2(S2.z, S2.w);
+                        if (__all_sync(__activemask(), fminf(R2.x, R2.y) >= k.a2x4))
+                            far_packed(DX, DY, DZ, rsqrt2(R2), FX, FY, FZ, K23, NK2, AX, AY, AZ);
+                        else
+                            slow(e, DX, DY, DZ, R2, FX, FY, FZ);
+                    }
+                    const float Pv[3][2] = {{AX.x, AX.y}, {AY.x, AY.y}, {AZ.x, AZ.y}};
 #pragma unroll
-                        for (int c = 0; c < 6; ++c) {
-                            float2 kc = sK[c * kP32Threads + threadIdx.x];
-                            kahan_merge(kc.x, kc.y, Pv[c]);
-                            sK[c * kP32Threads + threadIdx.x] = kc;
+                    for (int c = 0; c < 3; ++c) {
+                        float2 kc = sK[c * kP32Threads + threadIdx.x];
+                        kahan_merge(kc.x, kc.y, Pv[c][0]);
+                        kahan_merge(kc.x, kc.y, Pv[c][1]);
+                        sK[c * kP32Threads + threadIdx.x] = kc;
+                    }
+                }
+            }
+            __syncthreads();
+            const int nq = sQn[0];
+            if (nq > 0) {
+                // FP64 pairs of this chunk: from the queue, or (queue overflow)
+                // by every thread re-scanning its own sources
+                if (nq <= kP32Queue) {
+                    for (int e = threadIdx.x; e < nq; e += kP32Threads) {
+                        const int v = sQ[e], t = v >> 11, jj = v & 2047;
+                        double acc[3] = {0, 0, 0};
+                        pair_tiny64(sJ[jj], tb + t % nt, a, co, pos, fs, n, acc);
+                        for (int c = 0; c < 3; ++c) atomicAdd(&sD[3 * t + c], acc[c]);
+                    }
+                } else if (act) {
+                    for (int e = g; e < nP; e += G) {
+                        const float4 S0 = sS[3 * e], S1 = sS[3 * e + 1];
+                        for (int h = 0; h < 2; ++h) {
+                            const float dx = xa + (h ? S0.y : S0.x), dy = ya + (h ? S0.w : S0.z), dz = za + (h ? S1.y : S1.x);
+                            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                            const int jg = sJ[2 * e + h];
+                            if (!(r2 > k.tiny2) && jg != i) pair_tiny64(jg, i, a, co, pos, fs, n, &sD[3 * threadIdx.x]);
                         }
                     }
                 }
                 __syncthreads();
-                const int nq = sQn[0];
-                if (nq > 0) {
-                    // FP64 pairs of this chunk: from the queue, or (queue overflow)
-                    // by every thread re-scanning its own sources
-                    if (nq <= kP32Queue) {
-                        for (int e = threadIdx.x; e < nq; e += kP32Threads) {
-                            const int v = sQ[e], t = v >> 11, jj = (v >> 1) & 1023, h = v & 1;
-                            const int i = i0 + (t % Rn) + h * Rn;
-                            double acc[3] = {0, 0, 0};
-                            pair_tiny64(sJ[jj], i, a, co, pos, fs, n, acc);
-                            for (int c = 0; c < 3; ++c) atomicAdd(&sD[6 * t + 3 * h + c], acc[c]);
-                        }
-                    } else if (act) {
-                        for (int jj = g; jj < nS; jj += G) {
-                            const float4 S0 = sS[3 * jj], S1 = sS[3 * jj + 1];
-                            const int jg = sJ[jj];
-                            for (int h = 0; h < 2; ++h) {
-                                const float dx = (h ? xb : xa) + S0.x, dy = (h ? yb : ya) + S0.z, dz = (h ? zb : za) + S1.x;
-                                const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                                const int i = h ? ib : ia;
-                                if (!(r2 > k.tiny2) && jg != i && (h == 0 || actb))
-                                    pair_tiny64(jg, i, a, co, pos, fs, n, &sD[6 * threadIdx.x + 3 * h]);
-                            }
-                        }
-                    }
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        sQn[0] = 0;
-                        sQn[1] = 1;
-                    }
+                if (threadIdx.x == 0) {
+                    sQn[0] = 0;
+                    sQn[1] = 1;
                 }
             }
         }
-        // group reduction: one thread per (target, component) merges the Kahan
-        // states (S, C) of the G groups in FP32 (Kahan over the S, plain sum of
-        // the small C) and forms the FP64 result once
-        __syncthreads();
-        const bool tiny = sQn[1] != 0;   // read before the barrier: the next pass resets it after
-        __syncthreads();
-        for (int q = threadIdx.x; q < 6 * Rn; q += kP32Threads) {
-            const int hc = q / Rn, tt = q - hc * Rn, h = hc / 3, c = hc - 3 * h;
-            const int i = i0 + h * Rn + tt;
-            if (i < te) {
-                float S = 0.f, C = 0.f, Cs = 0.f;
-                for (int gg = 0; gg < G; ++gg) {
-                    const float2 v = sK[hc * kP32Threads + tt + gg * Rn];
-                    kahan_merge(S, C, v.x);
-                    Cs += v.y;
-                }
-                double u = cf * (double(S) - (double(C) + double(Cs)));
-                if (tiny)
-                    for (int gg = 0; gg < G; ++gg) u += sD[6 * (tt + gg * Rn) + 3 * h + c];
-                out[3 * size_t(i) + c] = u + (add_self ? co * fs[c * n + i] : 0.0);
-            }
+    }
+    // group reduction: one thread per (component, target) merges the Kahan
+    // states (S, C) of the G groups in FP32 (Kahan over the S, plain sum of
+    // the small C) and forms the FP64 result once
+    __syncthreads();
+    const bool tiny = sQn[1] != 0;
+    for (int q = threadIdx.x; q < 3 * nt; q += kP32Threads) {
+        const int c = q / nt, tt = q - c * nt, it = tb + tt;
+        float S = 0.f, C = 0.f, Cs = 0.f;
+        for (int gg = 0; gg < G; ++gg) {
+            const float2 v = sK[c * kP32Threads + tt + gg * nt];
+            kahan_merge(S, C, v.x);
+            Cs += v.y;
         }
-        __syncthreads();   // the next pass clears sK and sD
+        double u = cf * (double(S) - (double(C) + double(Cs)));
+        if (tiny)
+            for (int gg = 0; gg < G; ++gg) u += sD[3 * (tt + gg * nt) + c];
+        out[3 * size_t(it) + c] = u + (add_self ? co * fs[c * n + it] : 0.0);
     }
 }
 
