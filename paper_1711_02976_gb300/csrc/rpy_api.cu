@@ -209,32 +209,22 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
         put(c.data(), sizeof(T) * c.size());
     };
     auto putI = [&](const std::vector<int> &v) { put(v.data(), sizeof(int) * v.size()); };
-    putT(h.m2m_t);    // 0
-    putT(h.l2l_t);    // 1
-    putT(h.rot_fwd);  // 2
-    putT(h.rot_bwd);  // 3
-    putI(h.rot_off);  // 4
-    putT(h.rec_a);    // 5
-    putT(h.rec_b);    // 6
-    putT(h.rec_c);    // 7
-    putT(h.rec_cm);   // 8
-    putT(h.roots);    // 9
-    putT(h.m2x_c);    // 10
-    putT(h.x2l_c);    // 11
-    putI(h.e_k);      // 12
-    putI(h.k_start);  // 13
-    putT(h.e_cos);    // 14
-    putT(h.e_sin);    // 15
-    putT(h.e_wm);     // 16
-    putT(h.shift);    // 17
-    putI(h.grp_off);  // 18
-    putI(h.grp_n);    // 19
-    putI(h.grp_mask); // 20
-    putI(h.slot_list);// 21
-    putI(h.child_shift); // 22
-    putT(h.lad);      // 23
-    putT(h.orot_fwd); // 24
-    putT(h.orot_bwd); // 25
+    putT(h.rec_a);
+    putT(h.rec_b);
+    putT(h.rec_c);
+    putT(h.rec_cm);
+    putT(h.roots);
+    putT(h.m2x_c);
+    putT(h.x2l_c);
+    putI(h.k_start);
+    putT(h.e_wm);
+    putT(h.shift);
+    putI(h.grp_off);
+    putI(h.grp_n);
+    putI(h.grp_mask);
+    putI(h.slot_list);
+    putI(h.child_shift);
+    putT(h.lad);
     auto put_transposed = [&](const std::vector<double> &v) {   // [coefficient][k] -> [k][coefficient]
         const size_t P1 = size_t(h.p) + 1, nc = v.size() / P1;
         std::vector<double> w(v.size());
@@ -242,8 +232,8 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
             for (size_t k = 0; k < P1; ++k) w[k * nc + i] = v[i * P1 + k];
         putT(w);
     };
-    put_transposed(h.zm2m);     // 26
-    put_transposed(h.zl2l);     // 27
+    put_transposed(h.zm2m);
+    put_transposed(h.zl2l);
     // factored rotations: the y blocks as [k][m] where the kernels read them so (y_by_column)
     auto put_factored = [&](const std::vector<double> &v) {
         std::vector<double> w(v);
@@ -259,12 +249,12 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
             }
         putT(w);
     };
-    put_factored(h.frot_fwd); // 28
-    put_factored(h.frot_bwd); // 29
-    put_factored(h.forot_fwd);// 30
-    put_factored(h.forot_bwd);// 31
-    putI(h.frot_off); // 32
-    {                 // 33: per wave-pair unit (node, first stored wave, stored waves, t)
+    put_factored(h.frot_fwd);
+    put_factored(h.frot_bwd);
+    put_factored(h.forot_fwd);
+    put_factored(h.forot_bwd);
+    putI(h.frot_off);
+    {                 // per wave-pair unit (node, first stored wave, stored waves, t)
         std::vector<int> v;
         for (size_t u = 0; u < h.u_k.size(); ++u) {
             const int k = h.u_k[u];
@@ -272,11 +262,8 @@ static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<
         }
         putI(v);
     }
-    putI(h.u_start);  // 34
-    putT(h.shz);      // 35
-    putT(h.shx);      // 36
-    putT(h.shy);      // 37
-    {                 // 38: shift rows padded to an even length
+    putI(h.u_start);
+    {                 // shift rows padded to an even length
         const int S = h.S, Sp = (S + 1) & ~1;
         std::vector<double> v(size_t(216) * Sp * 2, 0.0);
         for (int o = 0; o < 216; ++o)
@@ -292,48 +279,35 @@ static DevTables<T> bind_tables(const OpTables &h, char *base, const std::vector
     d.nc = h.nc;
     d.s = h.s;
     d.S = h.S;
-    d.rot_len = h.rot_off.back();
-    d.m2m_t = reinterpret_cast<const T *>(base + o[0]);
-    d.l2l_t = reinterpret_cast<const T *>(base + o[1]);
-    d.rot_fwd = reinterpret_cast<const T *>(base + o[2]);
-    d.rot_bwd = reinterpret_cast<const T *>(base + o[3]);
-    d.rot_off = reinterpret_cast<const int *>(base + o[4]);
-    d.rec_a = reinterpret_cast<const T *>(base + o[5]);
-    d.rec_b = reinterpret_cast<const T *>(base + o[6]);
-    d.rec_c = reinterpret_cast<const T *>(base + o[7]);
-    d.rec_cm = reinterpret_cast<const T *>(base + o[8]);
-    d.roots = reinterpret_cast<const cpx<T> *>(base + o[9]);
-    d.m2x_c = reinterpret_cast<const T *>(base + o[10]);
-    d.x2l_c = reinterpret_cast<const T *>(base + o[11]);
-    d.e_k = reinterpret_cast<const int *>(base + o[12]);
-    d.k_start = reinterpret_cast<const int *>(base + o[13]);
-    d.e_cos = reinterpret_cast<const T *>(base + o[14]);
-    d.e_sin = reinterpret_cast<const T *>(base + o[15]);
-    d.e_wm = reinterpret_cast<const T *>(base + o[16]);
-    d.shift = reinterpret_cast<const cpx<T> *>(base + o[17]);
-    d.grp_off = reinterpret_cast<const int *>(base + o[18]);
-    d.grp_n = reinterpret_cast<const int *>(base + o[19]);
-    d.grp_mask = reinterpret_cast<const int *>(base + o[20]);
-    d.slot_list = reinterpret_cast<const int *>(base + o[21]);
-    d.child_shift = reinterpret_cast<const int *>(base + o[22]);
-    d.lad = reinterpret_cast<const T *>(base + o[23]);
-    d.orot_fwd = reinterpret_cast<const T *>(base + o[24]);
-    d.orot_bwd = reinterpret_cast<const T *>(base + o[25]);
-    d.zm2m = reinterpret_cast<const T *>(base + o[26]);
-    d.zl2l = reinterpret_cast<const T *>(base + o[27]);
-    d.frot_fwd = reinterpret_cast<const T *>(base + o[28]);
-    d.frot_bwd = reinterpret_cast<const T *>(base + o[29]);
-    d.forot_fwd = reinterpret_cast<const T *>(base + o[30]);
-    d.forot_bwd = reinterpret_cast<const T *>(base + o[31]);
-    d.frot_off = reinterpret_cast<const int *>(base + o[32]);
+    int k = 0;   // in the order of pack_tables
+    auto next = [&](auto &ptr) { ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(base + o[k++]); };
+    next(d.rec_a);
+    next(d.rec_b);
+    next(d.rec_c);
+    next(d.rec_cm);
+    next(d.roots);
+    next(d.m2x_c);
+    next(d.x2l_c);
+    next(d.k_start);
+    next(d.e_wm);
+    next(d.shift);
+    next(d.grp_off);
+    next(d.grp_n);
+    next(d.grp_mask);
+    next(d.slot_list);
+    next(d.child_shift);
+    next(d.lad);
+    next(d.zm2m);
+    next(d.zl2l);
+    next(d.frot_fwd);
+    next(d.frot_bwd);
+    next(d.forot_fwd);
+    next(d.forot_bwd);
+    next(d.frot_off);
+    next(d.u_info);
+    next(d.u_start);
+    next(d.shiftp);
     d.frot_len = h.frot_off.back();
-    d.u_info = reinterpret_cast<const int4 *>(base + o[33]);
-    d.u_start = reinterpret_cast<const int *>(base + o[34]);
-    d.NU = int(h.u_k.size());
-    d.shz = reinterpret_cast<const T *>(base + o[35]);
-    d.shx = reinterpret_cast<const cpx<T> *>(base + o[36]);
-    d.shy = reinterpret_cast<const cpx<T> *>(base + o[37]);
-    d.shiftp = reinterpret_cast<const cpx<T> *>(base + o[38]);
     d.Sp = (h.S + 1) & ~1;
     return d;
 }
@@ -451,12 +425,6 @@ int tree_alloc_workspace(Tree &t, cudaStream_t st) {
     RPY_TRY(dev_alloc(t, &t.Xo, es * nb * 2 * t.x_frames * kSets * h.S));
     RPY_TRY(dev_alloc(t, &t.Xi, es * nb * 2 * t.x_frames * kSets * h.S));
     RPY_TRY(dev_alloc(t, &t.EVg, es * size_t(t.nleaf) * 18 * h.nc));
-    if (t.params.precision != RPY_FP32 || h.p >= 12) {   // rotation-based M2M (see run_far_t)
-        size_t wide = 0;   // the widest parent level of the M2M pass (levels 2 .. nlevels - 2)
-        for (int l = 2; l <= t.nlevels - 2; ++l)
-            wide = std::max(wide, size_t(t.level_off[l + 1] - t.level_off[l]));
-        if (wide > 0) RPY_TRY(dev_alloc(t, &t.m2m_scratch, es * wide * 8 * kSets * h.nc));
-    }
     RPY_TRY(dev_alloc(t, (void **)&t.fs, sizeof(double) * 3 * t.n));
     if (t.params.precision == RPY_FP32) {
         RPY_TRY(dev_alloc(t, (void **)&t.p32, sizeof(float) * 6 * t.n));
@@ -1032,10 +1000,8 @@ int rpy_tree_footprint(int64_t n, int digits, int precision, int leaf_cap, int64
     // boxes: leaves ~ 2n/cap on clustered data, plus internal boxes (< leaves/7 * 8)
     double nbox = 4.0 * double(n) / double(leaf_cap) + 64.0;
     const int xf = plane_wave_frames(nbox, es, q.half());
-    // M, L, plane waves, L2P scratch, and (rotation-based M2M) a per-octant share
-    // slot for the boxes of one level, counted here for every box
-    const double m2m = (precision != RPY_FP32 || p >= 12) ? 8.0 * kSets * ncoef(p) : 0.0;
-    double per_box = es * (2.0 * kSets * ncoef(p) + 2.0 * 2 * xf * kSets * q.half() + 18.0 * ncoef(p) + m2m) +
+    // M, L, plane waves and L2P scratch
+    double per_box = es * (2.0 * kSets * ncoef(p) + 2.0 * 2 * xf * kSets * q.half() + 18.0 * ncoef(p)) +
                      4.0 * (8 + 27 + 3 + 12) + 32.0 + (precision == RPY_FP32 ? 0.0 : 9 * 4.0 + 8.0 /*c3, side_u*/);
     double per_bead = 3 * 8 /*pos*/ + 8 /*key*/ + 4 + 4 + 9 * 8 /*fs, unear, ufar*/ + 27 * 4 /*U list share*/ +
                       (precision == RPY_FP32 ? 9 * 4 /*p32, f32*/ : 15 * 4 /*p3, f2*/);

@@ -38,4 +38,10 @@ inline int even_threads(int items, int most = 256) {
 template <typename T>
 int run_waves_t(Tree &t, const DevTables<T> &D, const cpx<T> *M, cpx<T> *L, int rb, cudaStream_t st);
 
+// Upward and downward shifts, level by level
+template <typename T>
+int run_m2m_t(Tree &t, const DevTables<T> &D, cpx<T> *M, int rb, cudaStream_t st);
+template <typename T>
+int run_l2l_t(Tree &t, const DevTables<T> &D, cpx<T> *L, int rb, cudaStream_t st);
+
 }  // namespace rpy

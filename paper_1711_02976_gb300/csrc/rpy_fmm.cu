@@ -364,250 +364,6 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
     }
 }
 
-// ---------------------------------------------------------------- M2M / L2L
-
-// Dense per-octant operators (used by the FP32 form, where one streaming pass
-// over the operator beats the rotation's extra synchronisation).
-// M2M: parent M = sum over children of T_o [child M]; output degree n uses inputs of degree <= n.
-// rb (box origin of q4): the child's set 4 moves its origin from the child's
-// centre to the parent's first, M4 += (c_child - c_parent) . M_F (sets 1..3).
-template <typename T>
-__global__ void k_m2m(int b0, int nb, DevTables<T> D, const int *leaf, const int *child, const double *side,
-                      int rb, cpx<T> *M) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int b = b0 + blockIdx.x;
-    if (leaf[b]) return;
-    const int nc = ncoef(D.p), Dd = 2 * nc;
-    T *X = reinterpret_cast<T *>(smem_raw);
-    int r = threadIdx.x;
-    int kmax = r < Dd ? 2 * ncoef(deg_of(r >> 1)) : 0;
-    T acc[kSets] = {0, 0, 0, 0};
-    for (int o = 0; o < 8; ++o) {
-        int c = child[8 * b + o];
-        if (c < 0) continue;
-        const T *src = reinterpret_cast<const T *>(M + size_t(c) * kSets * nc);
-        __syncthreads();
-        for (int i = threadIdx.x; i < kSets * Dd; i += blockDim.x) X[i] = src[i];
-        __syncthreads();
-        if (rb) {
-            const double h = 0.5 * side[c];   // child centre - parent centre = h (2 bit - 1) per axis
-            const T dx = T((o & 1) ? h : -h), dy = T((o & 2) ? h : -h), dz = T((o & 4) ? h : -h);
-            for (int i = threadIdx.x; i < Dd; i += blockDim.x)
-                X[3 * Dd + i] = fma(dz, X[2 * Dd + i], fma(dy, X[Dd + i], fma(dx, X[i], X[3 * Dd + i])));
-            __syncthreads();
-        }
-        if (r < Dd) {
-            const T *Tt = D.m2m_t + size_t(o) * Dd * Dd;
-            for (int k = 0; k < kmax; ++k) {
-                T t = Tt[size_t(k) * Dd + r];
-#pragma unroll
-                for (int s = 0; s < kSets; ++s) acc[s] += t * X[s * Dd + k];
-            }
-        }
-    }
-    if (r < Dd) {
-        T *dst = reinterpret_cast<T *>(M + size_t(b) * kSets * nc);
-        for (int s = 0; s < kSets; ++s) dst[s * Dd + r] = acc[s];
-    }
-}
-
-// L2L: child L += S_o [parent L]; output degree k uses inputs of degree >= k.
-// rb (box origin of q4): the shifted set 4 moves its origin from the parent's
-// centre to the child's, L4 += (c_parent - c_child) . L_F.
-template <typename T>
-__global__ void k_l2l(int b0, int nb, DevTables<T> D, const int *par, const int *cell, const double *side, int rb,
-                      cpx<T> *L) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int b = b0 + blockIdx.x;
-    int P = par[b];
-    const int nc = ncoef(D.p), Dd = 2 * nc;
-    T *X = reinterpret_cast<T *>(smem_raw);
-    const T *src = reinterpret_cast<const T *>(L + size_t(P) * kSets * nc);
-    for (int i = threadIdx.x; i < kSets * Dd; i += blockDim.x) X[i] = src[i];
-    __syncthreads();
-    int r = threadIdx.x;
-    if (r >= Dd) return;
-    int o = (cell[3 * b] & 1) | ((cell[3 * b + 1] & 1) << 1) | ((cell[3 * b + 2] & 1) << 2);
-    int kdeg = deg_of(r >> 1);
-    int k0 = 2 * tri(kdeg, 0);
-    const T *St = D.l2l_t + size_t(o) * Dd * Dd;
-    T acc[kSets] = {0, 0, 0, 0};
-    for (int k = k0; k < Dd; ++k) {
-        T t = St[size_t(k) * Dd + r];
-#pragma unroll
-        for (int s = 0; s < kSets; ++s) acc[s] += t * X[s * Dd + k];
-    }
-    if (rb) {
-        const double h = 0.5 * side[b];   // parent centre - child centre = -h (2 bit - 1) per axis
-        const T dx = T((o & 1) ? -h : h), dy = T((o & 2) ? -h : h), dz = T((o & 4) ? -h : h);
-        acc[3] = fma(dz, acc[2], fma(dy, acc[1], fma(dx, acc[0], acc[3])));
-    }
-    T *dst = reinterpret_cast<T *>(L + size_t(b) * kSets * nc);
-    for (int s = 0; s < kSets; ++s) dst[s * Dd + r] += acc[s];
-}
-
-// ---------------------------------------------------------------- rotations
-// dst[s] = R src[s] per degree block (real 2-layout, block size 2(n+1)).
-// The factorized rotation of the four sets: tmp <- za (src) (one 2x2 rotation per
-// coefficient), then dst <- zc (Y tmp), Y acting on real and imaginary parts
-// separately.  src and dst may not alias tmp; the caller synchronises after.
-// COL: the y blocks stand as [k][m] (y_by_column).
-template <typename T, bool QUARTER, bool COL>
-__device__ void rotate_sets_f(const T *rf, const int *foff, int p, const cpx<T> *src, cpx<T> *tmp, cpx<T> *dst) {
-    const int nc = ncoef(p);
-    for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-        const int st = e / nc, i = e - st * nc, n = deg_of(i), m = i - tri(n, 0);
-        const T *za = rf + foff[n];
-        const T c = za[2 * m], sn = za[2 * m + 1];
-        const cpx<T> v = src[st * nc + i];
-        tmp[e] = mk(mul_diff(c, v.x, sn, v.y), mul_diff(sn, v.x, -c, v.y));
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-        const int st = e / nc, i = e - st * nc, n = deg_of(i), m = i - tri(n, 0), q = n + 1;
-        const T *o = rf + foff[n];
-        const T *yre = o + 4 * q + (COL ? m : m * q), *yim = yre + q * q;
-        const int sk = COL ? q : 1;   // stride of k
-        const cpx<T> *in = tmp + st * nc + tri(n, 0);
-        T re = 0, im = 0;
-        if (QUARTER) {
-            // middle angle pi/2 (the frame rotations): the y blocks are checkerboards
-            // (checked when the tables are built); Im of m = 0 is zero for real fields
-            for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k * sk], in[k].x);
-            if (m > 0)
-                for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k * sk], in[k].y);
-        } else {
-            for (int k = 0; k < q; ++k) {
-                macc(re, yre[k * sk], in[k].x);
-                macc(im, yim[k * sk], in[k].y);
-            }
-        }
-        re = closed(re);
-        im = closed(im);
-        const T c = o[2 * q + 2 * m], sn = o[2 * q + 2 * m + 1];
-        dst[st * nc + i] = mk(mul_diff(c, re, sn, im), mul_diff(sn, re, -c, im));
-    }
-}
-
-// ---------------------------------------------------------------- rotation-based M2M / L2L
-// Child octant o: rotate into the frame whose z axis is the shift direction,
-// apply the m-diagonal z-shift, rotate back (O(p^3) per child instead of the
-// O(p^4) dense operator).
-// One child per block (the children of one level): rotate into the frame
-// whose z axis is the shift direction, apply the m-diagonal z-shift, rotate back
-// (O(p^3) per child instead of the O(p^4) dense operator), and write the
-// child's share to its slot Sc[parent][octant]; k_m2m_sum adds the slots of each
-// parent in octant order (a fixed order: the result does not depend on timing).
-// rb (box origin of q4): the share's set 4 moves its origin from the child's
-// centre to the parent's, M4 += (c_child - c_parent) . M_F.
-template <typename T>
-__global__ void k_m2m_child(int c0, int pb0, DevTables<T> D, const int *par, const int *cell, const double *side,
-                            int rb, const cpx<T> *M, cpx<T> *Sc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int c = c0 + blockIdx.x;
-    const int p = D.p, nc = ncoef(p);
-    cpx<T> *X = reinterpret_cast<cpx<T> *>(smem_raw);
-    cpx<T> *Y = X + kSets * nc;
-    cpx<T> *Tm = Y + kSets * nc;   // rotation scratch
-    const int o = (cell[3 * c] & 1) | ((cell[3 * c + 1] & 1) << 1) | ((cell[3 * c + 2] & 1) << 2);
-    const cpx<T> *src = M + size_t(c) * kSets * nc;
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) X[i] = src[i];
-    __syncthreads();
-    rotate_sets_f<T, false, true>(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
-    __syncthreads();
-    for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-        int st = e / nc, i = e - st * nc;
-        int n = deg_of(i), m = i - tri(n, 0);
-        const T *z = D.zm2m + i;   // stored [k][coefficient]
-        cpx<T> a = mk<T>(0, 0);
-        for (int k = m; k <= n; ++k) {
-            const cpx<T> y = Y[st * nc + tri(k, m)];
-            macc(a.x, z[k * nc], y.x);
-            macc(a.y, z[k * nc], y.y);
-        }
-        X[e] = mk(closed(a.x), closed(a.y));
-    }
-    __syncthreads();
-    rotate_sets_f<T, false, true>(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
-    __syncthreads();
-    cpx<T> *dst = Sc + (size_t(par[c] - pb0) * 8 + o) * kSets * nc;
-    const double h = 0.5 * side[c];
-    const T dx = T((o & 1) ? h : -h), dy = T((o & 2) ? h : -h), dz = T((o & 4) ? h : -h);
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) {
-        cpx<T> v = Y[i];
-        if (rb && i >= 3 * nc) {
-            const int k = i - 3 * nc;
-            const cpx<T> fx = Y[k], fy = Y[nc + k], fz = Y[2 * nc + k];
-            v = mk(fma(dz, fz.x, fma(dy, fy.x, fma(dx, fx.x, v.x))), fma(dz, fz.y, fma(dy, fy.y, fma(dx, fx.y, v.y))));
-        }
-        dst[i] = v;
-    }
-}
-
-template <typename T>
-__global__ void k_m2m_sum(int b0, int nc4, const int *leaf, const int *child, const cpx<T> *Sc, cpx<T> *M) {
-    const int b = b0 + blockIdx.x;
-    if (leaf[b]) return;
-    int ch[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) ch[o] = child[8 * b + o];
-    const cpx<T> *src = Sc + size_t(blockIdx.x) * 8 * nc4;
-    for (int i = threadIdx.x; i < nc4; i += blockDim.x) {
-        cpx<T> acc = mk<T>(0, 0);
-#pragma unroll
-        for (int o = 0; o < 8; ++o)
-            if (ch[o] >= 0) acc += src[size_t(o) * nc4 + i];
-        M[size_t(b) * nc4 + i] = acc;
-    }
-}
-
-// rb (box origin of q4): the shifted set 4 moves its origin from the parent's
-// centre to the child's, L4 += (c_parent - c_child) . L_F.
-template <typename T>
-__global__ void k_l2l_rot(int b0, int nb, DevTables<T> D, const int *par, const int *cell, const double *side,
-                          int rb, cpx<T> *L) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int b = b0 + blockIdx.x;
-    int P = par[b];
-    const int p = D.p, nc = ncoef(p);
-    cpx<T> *X = reinterpret_cast<cpx<T> *>(smem_raw);
-    cpx<T> *Y = X + kSets * nc;
-    cpx<T> *Tm = Y + kSets * nc;   // rotation scratch
-    int o = (cell[3 * b] & 1) | ((cell[3 * b + 1] & 1) << 1) | ((cell[3 * b + 2] & 1) << 2);
-    const cpx<T> *src = L + size_t(P) * kSets * nc;
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) X[i] = src[i];
-    __syncthreads();
-    rotate_sets_f<T, false, true>(D.forot_fwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
-    __syncthreads();
-    for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-        int st = e / nc, i = e - st * nc;
-        int n = deg_of(i), m = i - tri(n, 0);
-        const T *z = D.zl2l + i;   // stored [k][coefficient]
-        cpx<T> a = mk<T>(0, 0);
-        for (int k = n; k <= p; ++k) {
-            const cpx<T> y = Y[st * nc + tri(k, m)];
-            macc(a.x, z[k * nc], y.x);
-            macc(a.y, z[k * nc], y.y);
-        }
-        X[e] = mk(closed(a.x), closed(a.y));
-    }
-    __syncthreads();
-    rotate_sets_f<T, false, true>(D.forot_bwd + size_t(o) * D.frot_len, D.frot_off, p, X, Tm, Y);
-    __syncthreads();
-    cpx<T> *dst = L + size_t(b) * kSets * nc;
-    const double h = 0.5 * side[b];
-    const T dx = T((o & 1) ? -h : h), dy = T((o & 2) ? -h : h), dz = T((o & 4) ? -h : h);
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) {
-        cpx<T> v = Y[i];
-        if (rb && i >= 3 * nc) {
-            const int k = i - 3 * nc;
-            const cpx<T> fx = Y[k], fy = Y[nc + k], fz = Y[2 * nc + k];
-            v = mk(fma(dz, fz.x, fma(dy, fy.x, fma(dx, fx.x, v.x))), fma(dz, fz.y, fma(dy, fy.y, fma(dx, fx.y, v.y))));
-        }
-        dst[i] += v;
-    }
-}
-
 // ---------------------------------------------------------------- far-field evaluation
 constexpr int kNE = 18;   // evaluation expansions of Eq. (2.8) per box
 constexpr int kNF = 12;   // evaluated per bead after the fold of k_eval_prep (per-potential form)
@@ -1032,38 +788,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
     prof_mark(t, RPY_STAGE_M2M, st);
-    // FP64 form: rotation-based M2M and L2L (fewer operations).  FP32: the dense
-    // operators below p = 12, the rotation forms (one child per block) from there
-    const bool rot_l = sizeof(T) == 8 || p >= 12;
-    size_t smr2 = sizeof(cpx<T>) * 3 * kSets * nc;
-    int Dd = 2 * nc, thr = ((Dd + 31) / 32) * 32;
-    size_t smd = sizeof(T) * kSets * Dd;
-    RPY_TRY(set_smem(k_l2l_rot<T>, smr2));
-    RPY_TRY(set_smem(k_m2m_child<T>, smr2));
-    if constexpr (sizeof(T) == 4) {
-        RPY_TRY(set_smem(k_m2m<T>, smd));
-        RPY_TRY(set_smem(k_l2l<T>, smd));
-    }
-    for (int l = t.nlevels - 2; l >= 2; --l) {
-        int lb = t.level_off[l], ln = t.level_off[l + 1] - lb;
-        if (ln > 0) {
-            const int cb = t.level_off[l + 1], cn = t.level_off[l + 2] - cb;   // their children
-            if (rot_l) {
-                // the share slots exist whenever a level >= 2 does (tree_alloc_workspace)
-                if (cn > 0) {
-                    if (!t.m2m_scratch) return RPY_ERR_INTERNAL;
-                    cpx<T> *Sc = static_cast<cpx<T> *>(t.m2m_scratch);
-                    k_m2m_child<T><<<cn, 256, smr2, st>>>(cb, lb, D, t.b_parent, t.b_cell, side, rb, M, Sc);
-                    k_m2m_sum<T><<<ln, 256, 0, st>>>(lb, kSets * nc, t.b_leaf, t.b_child, Sc, M);
-                    RPY_LAUNCHED(2);
-                }
-            } else if constexpr (sizeof(T) == 4) {
-                k_m2m<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_leaf, t.b_child, side, rb, M);
-                RPY_LAUNCHED(1);
-            }
-        }
-    }
-    RPY_CHECK(cudaGetLastError());
+    RPY_TRY(run_m2m_t(t, D, M, rb, st));
     // plane-wave M2L: all three frames in one pass, or (large trees, where the
     // plane-wave buffers of six directions would not fit) one frame per pass,
     // each pass adding its frame's share into L (with profiling on, every pass's
@@ -1077,15 +802,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     RPY_CHECK(cudaGetLastError());
     // downward pass
     prof_mark(t, RPY_STAGE_L2L, st);
-    for (int l = 3; l < t.nlevels; ++l) {
-        int lb = t.level_off[l], ln = t.level_off[l + 1] - lb;
-        if (ln > 0) {
-            if (rot_l) k_l2l_rot<T><<<ln, 256, smr2, st>>>(lb, ln, D, t.b_parent, t.b_cell, side, rb, L);
-            else if constexpr (sizeof(T) == 4) k_l2l<T><<<ln, thr, smd, st>>>(lb, ln, D, t.b_parent, t.b_cell, side, rb, L);
-            RPY_LAUNCHED(1);
-        }
-    }
-    RPY_CHECK(cudaGetLastError());
+    RPY_TRY(run_l2l_t(t, D, L, rb, st));
     prof_mark(t, RPY_STAGE_EVAL, st);
     if (ufar) {
         cpx<T> *EVg = static_cast<cpx<T> *>(t.EVg);

@@ -161,27 +161,22 @@ constexpr bool y_by_column(size_t elem_bytes, int p) { return elem_bytes == 8 ||
 // device copies
 template <typename T>
 struct DevTables {
-    int p, nc, s, S, rot_len;
-    const T *m2m_t, *l2l_t, *rot_fwd, *rot_bwd;
-    const int *rot_off;
+    int p, nc, s, S;
     const T *rec_a, *rec_b, *rec_c, *rec_cm;
     const T *lad;
-    const T *orot_fwd, *orot_bwd, *zm2m, *zl2l;
-    const T *frot_fwd, *frot_bwd, *forot_fwd, *forot_bwd;
+    const T *zm2m, *zl2l;       // [k][coefficient]
+    const T *frot_fwd, *frot_bwd, *forot_fwd, *forot_bwd;   // y blocks as y_by_column
     const int *frot_off;
     int frot_len;
     const cpx<T> *roots;
     const T *m2x_c, *x2l_c;
-    const int *e_k, *k_start;
+    const int *k_start;
     const int *u_start;         // wave-pair units: first unit of node k
     const int4 *u_info;         // per unit: node, first stored wave of the node, waves of the node, t
-    int NU;
-    const T *e_cos, *e_sin, *e_wm;
+    const T *e_wm;
     const cpx<T> *shift;
     const cpx<T> *shiftp;   // the same rows with stride Sp (S rounded up to even: 16-byte rows for bulk copies)
     int Sp;
-    const T *shz;
-    const cpx<T> *shx, *shy;
     const int *grp_off, *grp_n, *grp_mask, *slot_list, *child_shift;
 };
 
@@ -300,7 +295,6 @@ struct Tree {
     // expansions and matvec workspace
     void *M = nullptr, *L = nullptr, *Xo = nullptr, *Xi = nullptr;
     int x_frames = 3;                 // plane-wave frames per pass (3 or 1)
-    void *m2m_scratch = nullptr;      // FP64 M2M: [boxes of the widest level][8 octants][4][nc] child shares
     void *EVg = nullptr;              // [nleaf][18][ncoef(p)] derived local expansions of Eq. (2.8)
     double *fs = nullptr;             // sorted forces SoA [3][n]
     float *p32 = nullptr;             // FP32 form: sorted positions as hi + lo floats, [6][n] (x,y,z hi; x,y,z lo)

@@ -15,6 +15,7 @@
 // 2.48, 2.03, 2.07 -> 1.50, 2.05, 1.66; 15M-bead cube 4.61, 10.9, 4.47 -> 2.87, 6.7, 4.6; 256 systems, 11.5M beads,
 // 8.26, 9.8, 6.7 -> 4.4, 6.4, 6.4.
 #include "rpy_far.h"
+#include "rpy_quad.h"
 
 namespace rpy {
 
@@ -94,144 +95,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 }
 
 
-// ---------------------------------------------------------------- sets of one item in packed operations
-// Quad<T>: N threads share the four sets of an item (pr = 0 .. N - 1), each holding V; a V stands as one
-// float4 in memory: four floats, or two double-floats as (h, h', l, l').
-struct f4 {
-    float2 a, b;   // sets 0 1, 2 3
-};
-template <typename T> struct Quad;
-template <> struct Quad<float> {
-    using V = f4;
-    static constexpr int N = 1, SH = 0;   // N = 1 << SH
-};
-template <> struct Quad<dfl> {
-    using V = df2;
-    static constexpr int N = 2, SH = 1;
-};
-__device__ __forceinline__ void get(float4 m, f4 &v) { v = f4{make_float2(m.x, m.y), make_float2(m.z, m.w)}; }
-__device__ __forceinline__ void get(float4 m, df2 &v) { v = as_df2(m); }
-__device__ __forceinline__ float4 put(f4 v) { return make_float4(v.a.x, v.a.y, v.b.x, v.b.y); }
-__device__ __forceinline__ float4 put(df2 v) { return as_float4(v); }
-template <typename V> __device__ __forceinline__ V zero();
-template <> __device__ __forceinline__ f4 zero<f4>() { return f4{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-template <> __device__ __forceinline__ df2 zero<df2>() { return df2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-template <> __device__ __forceinline__ float2 zero<float2>() { return make_float2(0.f, 0.f); }
-
-__device__ __forceinline__ df2 operator+(df2 a, df2 b) { return renorm(sum_raw(a, b)); }
-__device__ __forceinline__ df2 operator-(df2 a, df2 b) { return renorm(sum_raw(a, -b)); }
-__device__ __forceinline__ df2 closed(df2 a) { return renorm(a); }
-__device__ __forceinline__ void macc(df2 &acc, dfl s, df2 b) { macc(acc, dup(s), b); }
-__device__ __forceinline__ df2 times(dfl s, df2 a) { return renorm(mul_df(dup(s), a)); }
-// a x + b y with scalar a, b
-__device__ __forceinline__ df2 lin2(dfl a, df2 x, dfl b, df2 y) {
-    return renorm(sum_raw(mul_df(dup(a), x), mul_df(dup(b), y)));
-}
-
-__device__ __forceinline__ float2 sum_raw(float2 a, float2 b) { return add2(a, b); }
-__device__ __forceinline__ float2 closed(float2 a) { return a; }
-__device__ __forceinline__ void macc(float2 &acc, float s, float2 b) { acc = fma2(dup(s), b, acc); }
-__device__ __forceinline__ float2 lin2(float a, float2 x, float b, float2 y) { return fma2(dup(a), x, mul2(dup(b), y)); }
-
-__device__ __forceinline__ f4 operator-(f4 a) { return f4{neg2(a.a), neg2(a.b)}; }
-__device__ __forceinline__ f4 operator+(f4 a, f4 b) { return f4{add2(a.a, b.a), add2(a.b, b.b)}; }
-__device__ __forceinline__ f4 operator-(f4 a, f4 b) { return f4{sub2(a.a, b.a), sub2(a.b, b.b)}; }
-__device__ __forceinline__ f4 sum_raw(f4 a, f4 b) { return a + b; }
-__device__ __forceinline__ f4 closed(f4 a) { return a; }
-__device__ __forceinline__ void macc(f4 &acc, float s, f4 b) {
-    macc(acc.a, s, b.a);
-    macc(acc.b, s, b.b);
-}
-__device__ __forceinline__ f4 scale2(float s, f4 a) { return f4{mul2(dup(s), a.a), mul2(dup(s), a.b)}; }
-__device__ __forceinline__ f4 times(float s, f4 a) { return scale2(s, a); }
-__device__ __forceinline__ f4 lin2(float a, f4 x, float b, f4 y) { return f4{lin2(a, x.a, b, y.a), lin2(a, x.b, b, y.b)}; }
-
-// n complex coefficients of four sets in shared memory: real parts [n][N], then imaginary parts,
-// 16 bytes each, so that consecutive threads touch consecutive banks.
-template <typename T>
-struct Planes {
-    using V = typename Quad<T>::V;
-    static constexpr int N = Quad<T>::N;
-    float4 *p;
-    int n;
-    __device__ __forceinline__ V x(int pr, int i) const {
-        V v;
-        get(p[N * i + pr], v);
-        return v;
-    }
-    __device__ __forceinline__ V y(int pr, int i) const {
-        V v;
-        get(p[N * (n + i) + pr], v);
-        return v;
-    }
-    __device__ __forceinline__ void set(int pr, int i, V a, V b) const {
-        p[N * i + pr] = put(a);
-        p[N * (n + i) + pr] = put(b);
-    }
-};
-
-// coefficient i of the thread's sets in global memory ([set][nc])
-__device__ __forceinline__ void load_sets(const cpx<dfl> *g, int nc, int pr, int i, df2 &x, df2 &y) {
-    const cpx<dfl> u = g[2 * pr * nc + i], v = g[(2 * pr + 1) * nc + i];
-    x = df2{make_float2(u.x.h, v.x.h), make_float2(u.x.l, v.x.l)};
-    y = df2{make_float2(u.y.h, v.y.h), make_float2(u.y.l, v.y.l)};
-}
-__device__ __forceinline__ void load_sets(const cpx<float> *g, int nc, int, int i, f4 &x, f4 &y) {
-    const cpx<float> a = g[i], b = g[nc + i], c = g[2 * nc + i], d = g[3 * nc + i];
-    x = f4{make_float2(a.x, b.x), make_float2(c.x, d.x)};
-    y = f4{make_float2(a.y, b.y), make_float2(c.y, d.y)};
-}
-__device__ __forceinline__ void add_sets(cpx<dfl> *g, int nc, int pr, int i, df2 x, df2 y) {
-    cpx<dfl> *d0 = g + 2 * pr * nc + i, *d1 = d0 + nc;
-    cpx<dfl> u = *d0, v = *d1;
-    u += mk(dfl(x.h.x, x.l.x), dfl(y.h.x, y.l.x));
-    v += mk(dfl(x.h.y, x.l.y), dfl(y.h.y, y.l.y));
-    *d0 = u;
-    *d1 = v;
-}
-__device__ __forceinline__ void add_sets(cpx<float> *g, int nc, int, int i, f4 x, f4 y) {
-    g[i] += mk(x.a.x, y.a.x);
-    g[nc + i] += mk(x.a.y, y.a.y);
-    g[2 * nc + i] += mk(x.b.x, y.b.x);
-    g[3 * nc + i] += mk(x.b.y, y.b.y);
-}
-
-// The factored rotation of the four sets (a z rotation, the y block on real and imaginary parts, a z
-// rotation): rotate_z forms tmp from a source of (x, y) per item, rotate_y the result in dst.
-// COL: the y blocks stand as [k][m] (y_by_column).
-template <typename T, typename F>
-__device__ __forceinline__ void rotate_z(const T *rf, const int *foff, int nc, Planes<T> tmp, F source) {
-    constexpr int N = Quad<T>::N, SH = Quad<T>::SH;
-    for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
-        const int pr = e & (N - 1), i = e >> SH, n = deg_of(i), m = i - tri(n, 0);
-        const T *za = rf + foff[n];
-        const T c = za[2 * m], sn = za[2 * m + 1];
-        typename Quad<T>::V x, y;
-        source(pr, i, x, y);
-        tmp.set(pr, i, lin2(c, x, -sn, y), lin2(sn, x, c, y));
-    }
-}
-template <typename T, bool COL>
-__device__ __forceinline__ void rotate_y(const T *rf, const int *foff, int nc, Planes<T> tmp, Planes<T> dst) {
-    using V = typename Quad<T>::V;
-    constexpr int N = Quad<T>::N, SH = Quad<T>::SH;
-    for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
-        const int pr = e & (N - 1), i = e >> SH, n = deg_of(i), m = i - tri(n, 0), q = n + 1, t0 = tri(n, 0);
-        const T *o = rf + foff[n], *yre = o + 4 * q + (COL ? m : m * q), *yim = yre + q * q;
-        const int sk = COL ? q : 1;
-        V re = zero<V>(), im = re;
-        // the frame rotations' middle angle is pi/2: checkerboard y blocks (checked when the tables are
-        // built), Im of m = 0 zero
-        for (int k = (m + n) & 1; k < q; k += 2) macc(re, yre[k * sk], tmp.x(pr, t0 + k));
-        if (m > 0)
-            for (int k = 1 + ((m + n) & 1); k < q; k += 2) macc(im, yim[k * sk], tmp.y(pr, t0 + k));
-        re = closed(re);
-        im = closed(im);
-        const T c = o[2 * q + 2 * m], sn = o[2 * q + 2 * m + 1];
-        dst.set(pr, i, lin2(c, re, -sn, im), lin2(sn, re, c, im));
-    }
-}
-
 // A_k^m rows of one node at an odd stride, so that neighbouring nodes fall on different banks
 __host__ __device__ inline int a_stride(int p) { return (p + 1) | 1; }
 
@@ -253,9 +116,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 3)
     for (int f = f0; f < f0 + nf; ++f) {
         if (f > 0) {
             const T *rf = D.frot_fwd + size_t(f - 1) * D.frot_len;
-            rotate_z(rf, D.frot_off, nc, Tm, [&](int pr, int i, V &x, V &y) { load_sets(src, nc, pr, i, x, y); });
+            for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
+                V x, y;
+                load_sets(src, nc, e & (N - 1), e >> SH, x, y);
+                rotate_z(rf, D.frot_off, e >> SH, e & (N - 1), x, y, Tm);
+            }
             __syncthreads();
-            rotate_y<T, COL>(rf, D.frot_off, nc, Tm, Mu);
+            for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
+                V x, y;
+                rotate_y<true, COL>(rf, D.frot_off, e >> SH, e & (N - 1), Tm, x, y);
+                Mu.set(e & (N - 1), e >> SH, x, y);
+            }
         } else {
             for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
                 V x, y;
@@ -426,8 +297,6 @@ __device__ __forceinline__ float2 get_pair(float2 m) { return m; }
 __device__ __forceinline__ df2 get_pair(float4 m) { return as_df2(m); }
 __device__ __forceinline__ float2 put_pair(float2 v) { return v; }
 __device__ __forceinline__ float4 put_pair(df2 v) { return as_float4(v); }
-__device__ __forceinline__ float neg1(float a) { return -a; }
-__device__ __forceinline__ dfl neg1(dfl a) { return -a; }
 
 // One thread per (wave, pair of sets).
 // Plain loads, two sources in flight (double-floats): staging each thread's sources through shared memory by
@@ -867,18 +736,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 5)
             }
         }
         __syncthreads();
-        if (f > 0) {   // back to world axes; Lf is free once rotated about z
+        if (f > 0) {   // back to world axes
             const T *rf = D.frot_bwd + size_t(f - 1) * D.frot_len;
-            rotate_z(rf, D.frot_off, nc, Tm, [&](int pr, int i, V &x, V &y) {
-                x = Lf.x(pr, i);
-                y = Lf.y(pr, i);
-            });
-            __syncthreads();
-            rotate_y<T, COL>(rf, D.frot_off, nc, Tm, Lf);
+            for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
+                const int pr = e & (N - 1), i = e >> SH;
+                rotate_z(rf, D.frot_off, i, pr, Lf.x(pr, i), Lf.y(pr, i), Tm);
+            }
             __syncthreads();
         }
-        for (int e = threadIdx.x; e < N * nc; e += blockDim.x)
-            add_sets(dst, nc, e & (N - 1), e >> SH, Lf.x(e & (N - 1), e >> SH), Lf.y(e & (N - 1), e >> SH));
+        for (int e = threadIdx.x; e < N * nc; e += blockDim.x) {
+            const int pr = e & (N - 1), i = e >> SH;
+            V x = Lf.x(pr, i), y = Lf.y(pr, i);
+            if (f > 0) rotate_y<true, COL>(D.frot_bwd + size_t(f - 1) * D.frot_len, D.frot_off, i, pr, Tm, x, y);
+            add_sets(dst, nc, pr, i, x, y);
+        }
     }
 }
 

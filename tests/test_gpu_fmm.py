@@ -418,6 +418,25 @@ def test_fp64_far_field_in_any_units(digits, n, flags):
     assert oracle.rel_l2(u / 4.1e-12, u0) < 1e-11
 
 
+@pytest.mark.parametrize("order", [2, 3, 6, 7, 11, 12, 15, 20, 27])
+@pytest.mark.parametrize("n,leaf_cap", [(3000, 4), (60000, 3)])
+def test_both_precision_forms_agree_at_every_order(order, n, leaf_cap):
+    """The translation kernels change shape with the order (planes, node chunks, children per block, table
+    orders from p = 12) and with the number of parents on a level (clusters, split children).  At one order
+    both precision forms carry the same truncation, so they differ by FP32 rounding only: some hundred
+    operations of 2^-24 with signs (a bound of 100 x 2^-24 = 6e-6), and the two plane-wave rules
+    agree to the accuracy of the 3-digit one."""
+    sysm = synth.sphere_plus_cube(n, 91, 1e-3)
+    u = {}
+    for prec, digits in ((rp.RPY_FP64, 6), (rp.RPY_FP32, 6), (rp.RPY_FP64, 3), (rp.RPY_FP32, 3)):
+        u[prec, digits], t = matvec(sysm.pos, sysm.f, sysm.a, sysm.s, digits, leaf_cap=leaf_cap, precision=prec,
+                                    order_p=order, direct_w=-1, direct_x=-1, parts=rp.RPY_PART_FAR)
+        t.close()
+    for digits in (3, 6):
+        assert oracle.rel_l2(u[rp.RPY_FP32, digits], u[rp.RPY_FP64, digits]) < 6e-6
+    assert oracle.rel_l2(u[rp.RPY_FP64, 3], u[rp.RPY_FP64, 6]) < 3e-3
+
+
 # ---------------------------------------------------------------- edge cases
 
 @pytest.mark.parametrize("precision", [rp.RPY_FP64, rp.RPY_FP32])
