@@ -89,7 +89,17 @@ inline int plane_wave_frames(double nbox, double elem_bytes, int S) {
 }
 constexpr int kMaxP = 29;         // largest supported expansion order (p + 2 < 32 warp lanes)
 constexpr int kMaxLevel = 21;
-constexpr int kItemTargets = 256;   // targets per near-field work item
+constexpr int kItemTargets = 256;   // targets per near-field work item at most, and threads of its block
+// Near-field items of a leaf of T beads: full ones, then the rest, in halves where the block then holds three
+// groups of threads instead of one (141 targets: 55% of the threads in one item, 83% in two; FP32 near field
+// of 6,859 beads on a sphere in such leaves 114 -> 50 us).  Elsewhere one item wins, for each stages
+// all sources of its leaf again: items of at most 128 cost the 256 systems 28.5 -> 29.9 ms, and equal
+// items for all of a large leaf (224 instead of 256 of 895 targets) a Plummer cluster 653 -> 705 us.
+RPY_HD bool rest_in_halves(int r) { return r > kItemTargets / 2 && 3 * ((r + 1) / 2) <= kItemTargets; }
+RPY_HD int item_count(int T) {
+    const int r = T % kItemTargets;
+    return T / kItemTargets + (r > 0) + rest_in_halves(r);
+}
 
 struct ExpQuad {                  // plane-wave quadrature (box units)
     int s = 0;                    // lambda nodes
@@ -282,14 +292,14 @@ struct Tree {
     int n_x2x_par = 0, *x2x_par = nullptr;
     // direct (P2P) substitutes for small W and X interactions, per leaf
     int *d_off = nullptr, *d_idx = nullptr;
-    // near-field work items (leaf, first target) of at most kItemTargets targets, in
+    // near-field work items (leaf index, box, first target, end) of at most kItemTargets targets, in
     // decreasing cost order for the U-list pass and for the direct-substitute pass
     int n_items = 0;
-    int2 *u_items = nullptr, *d_items = nullptr;
+    int4 *u_items = nullptr, *d_items = nullptr;
     // the near list of the full matvec: per leaf the U list, then the direct substitutes;
     // its work items in decreasing cost order (one pass for both)
     int *m_off = nullptr, *m_idx = nullptr;
-    int2 *m_items = nullptr;
+    int4 *m_items = nullptr;
     int64_t n_d = 0, d_pairs = 0;
     int direct_w = 0, direct_x = 0;    // bead-count thresholds in use (0 = none)
     // expansions and matvec workspace

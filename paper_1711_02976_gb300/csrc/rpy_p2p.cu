@@ -204,6 +204,23 @@ __device__ __noinline__ void near64(unsigned char *smem, int tb, int te, int u0,
     }
 }
 
+// Thread layout of k_p2p_df: an item of T targets is taken in P parts of R = ceil(T / P) targets, G = threads / R
+// groups of R threads each; every group takes its share of the staged sources for the thread's target of
+// each part in turn.  T G / (P threads) of the lanes do work; another part must raise that by 6%, since each
+// has its own block sums (T = 57: one part 89%, three 97%).  15M-bead cube: one part 155.4 ms, at most three 149.1, four
+// 147.9; without the 6% small leaves lose (4,096 beads 0.024 -> 0.034 ms).
+struct TargetParts {
+    int P, R, G;
+};
+__device__ __forceinline__ TargetParts target_parts(int nt, int threads, int most) {
+    TargetParts b{1, nt, threads / nt};
+    for (int P = 2; P <= most; ++P) {
+        const int R = (nt + P - 1) / P, G = threads / R;
+        if (16 * G * b.P > 17 * b.G * P) b = TargetParts{P, R, G};
+    }
+    return b;
+}
+
 // ---------------------------------------------------------------- FP64 form in double-floats
 
 // Positions of the FP64 form as three floats per coordinate, x' = h + m + l in units of 2^e with e the
@@ -383,28 +400,29 @@ constexpr int kDfList = 256;     // list boxes per prefix segment
 constexpr int kDfStride = 9;     // float4 per staged pair of sources: 15 packed values, 2 indices, 1 of padding
 constexpr int kDfBlock = 8;      // pairs of sources per double-float block between FP64 sums
 constexpr int kDfMaxLevel = 17;  // deeper leaves hold pairs closer than the three-float split resolves
-constexpr size_t kDfSmem = sizeof(float4) * kDfStride * (kDfChunk / 2) + sizeof(double) * 6 * kDfThreads +
+constexpr int kDfParts = 4;      // parts of an item's targets at most
+constexpr size_t kDfSmem = sizeof(float4) * kDfStride * (kDfChunk / 2) + sizeof(double) * 6 * kDfParts * kDfThreads +
                            sizeof(int) * (2 * kDfList + 4);
 static_assert(sizeof(float4) * kDfStride * (kDfChunk / 2) >= kP2PThreads * (9 * sizeof(double) + sizeof(int)),
               "near64 works in the staging buffer");
 
-// Thread layout: an item of T targets uses G = blockDim / T groups of T threads; the list's beads are staged
-// in chunks as pairs (two sources in the two lanes of the packed operations), and group g takes every G-th
-// pair.  The list's boxes are prefix-summed in shared memory and each staged bead finds its box by binary
-// search.  A pair of sources stands in 9 float4 (8 used): the groups of a warp then read different banks.
+// The list's beads are staged in chunks as pairs (two sources in the two lanes of the packed operations), and
+// group g takes every G-th pair for the thread's target of each part.  The list's boxes are prefix-summed in shared
+// memory and each staged bead finds its box by binary search.  A pair of sources stands in 9 float4 (8 used): the
+// groups of a warp then read different banks.
 __global__ void __launch_bounds__(kDfThreads, 2)
-    k_p2p_df(const int2 *items, const int *leaves, const int *beg, const int *end, const int *bsys, const int *lvl,
+    k_p2p_df(const int4 *items, const int *beg, const int *end, const int *bsys, const int *lvl,
              const int *uoff, const int *uidx, const float *p3, const float *f2, const int *fmax, const double *pos,
              const double *fs, int64_t n, SysConst sc, int add_self, double *out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *sS = reinterpret_cast<float4 *>(smem_raw);
-    double *sU = reinterpret_cast<double *>(sS + kDfStride * (kDfChunk / 2));   // [3][threads] running sums
-    double *sD = sU + 3 * kDfThreads;                                            // [threads][3] FP64 pairs
-    int *lb = reinterpret_cast<int *>(sD + 3 * kDfThreads), *lpre = lb + kDfList;
+    double *sU = reinterpret_cast<double *>(sS + kDfStride * (kDfChunk / 2));   // [part][3][threads] running sums
+    double *sD = sU + 3 * kDfParts * kDfThreads;                                 // [part][threads][3] FP64 pairs
+    int *lb = reinterpret_cast<int *>(sD + 3 * kDfParts * kDfThreads), *lpre = lb + kDfList;
     int *any64 = lpre + kDfList + 1;
-    const int2 item = items[blockIdx.x];
-    const int li = item.x, b = leaves[li], sys = bsys[b];
-    const int tb = item.y, te = min(end[b], item.y + kItemTargets), nt = te - tb;
+    const int4 item = items[blockIdx.x];
+    const int li = item.x, b = item.y, sys = bsys[b];
+    const int tb = item.z, te = item.w, nt = te - tb;
     const int u0 = uoff[li], u1 = uoff[li + 1];
     const PairConst &pc = sc.pc[sys];
     const int fw = fmax[sys];
@@ -414,17 +432,12 @@ __global__ void __launch_bounds__(kDfThreads, 2)
     }
     const float lim = pc.d_lim, tiny = kDfTiny2;
     const df2 k23{dup(pc.d_k23h), dup(pc.d_k23l)};
-    const int G = kDfThreads / nt;
-    const int tl = threadIdx.x % nt, g = threadIdx.x / nt;
+    const TargetParts tp = target_parts(nt, kDfThreads, kDfParts);
+    const int G = tp.G, tl = threadIdx.x % tp.R, g = threadIdx.x / tp.R;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = tb + tl;
-    const bool act = g < G;
-    float2 X[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) X[k] = dup(p3[k * n + i]);
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 3 * tp.P; ++c) {
         sU[c * kDfThreads + threadIdx.x] = 0.0;
-        sD[3 * threadIdx.x + c] = 0.0;
+        sD[c * kDfThreads + threadIdx.x] = 0.0;
     }
     if (threadIdx.x == 0) *any64 = 0;
     for (int us = u0; us < u1; us += kDfList) {
@@ -478,7 +491,14 @@ __global__ void __launch_bounds__(kDfThreads, 2)
                 }
             }
             __syncthreads();
-            if (act) {
+            for (int part = 0; part < tp.P && g < G; ++part) {
+                const int i = tb + part * tp.R + tl;
+                if (i >= te) break;
+                float2 X[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) X[k] = dup(p3[k * n + i]);
+                double *const U = sU + 3 * part * kDfThreads + threadIdx.x;
+                double *const tiny64 = sD + 3 * (part * kDfThreads + threadIdx.x);
                 for (int e0 = g; e0 < nP; e0 += kDfBlock * G) {
                     float2 S[3], C[3];
 #pragma unroll
@@ -521,11 +541,11 @@ __global__ void __launch_bounds__(kDfThreads, 2)
                             if (!ox || !oy) {
                                 const int jx = __float_as_int(v7.z), jy = __float_as_int(v7.w);
                                 if (!ox && jx != i) {
-                                    pair_tiny_f64(jx, i, pc, pos, fs, n, sD + 3 * threadIdx.x);
+                                    pair_tiny_f64(jx, i, pc, pos, fs, n, tiny64);
                                     *any64 = 1;
                                 }
                                 if (!oy && jy != i) {
-                                    pair_tiny_f64(jy, i, pc, pos, fs, n, sD + 3 * threadIdx.x);
+                                    pair_tiny_f64(jy, i, pc, pos, fs, n, tiny64);
                                     *any64 = 1;
                                 }
                             }
@@ -538,7 +558,7 @@ __global__ void __launch_bounds__(kDfThreads, 2)
                     for (int c = 0; c < 3; ++c) {
                         const float s = S[c].x + S[c].y, bb = s - S[c].x;
                         const float e = (S[c].x - (s - bb)) + (S[c].y - bb);
-                        sU[c * kDfThreads + threadIdx.x] += double(s) + double((C[c].x + C[c].y) + e);
+                        U[c * kDfThreads] += double(s) + double((C[c].x + C[c].y) + e);
                     }
                 }
             }
@@ -550,12 +570,12 @@ __global__ void __launch_bounds__(kDfThreads, 2)
     const double unit = pc.cf * pc.d_xs * force_unit(fw), co = pc.co;
     const bool any = *any64 != 0;
     for (int q = threadIdx.x; q < 3 * nt; q += kDfThreads) {
-        const int c = q / nt, tt = q - c * nt, it = tb + tt;
+        const int c = q / nt, tt = q - c * nt, it = tb + tt, part = tt / tp.R, t0 = tt - part * tp.R;
         double v = 0.0;
-        for (int gg = 0; gg < G; ++gg) v += sU[c * kDfThreads + tt + gg * nt];
+        for (int gg = 0; gg < G; ++gg) v += sU[(3 * part + c) * kDfThreads + t0 + gg * tp.R];
         double u = unit * v;
         if (any)
-            for (int gg = 0; gg < G; ++gg) u += sD[3 * (tt + gg * nt) + c];
+            for (int gg = 0; gg < G; ++gg) u += sD[3 * (part * kDfThreads + t0 + gg * tp.R) + c];
         out[3 * size_t(it) + c] = u + (add_self ? co * fs[c * n + it] : 0.0);
     }
 }
@@ -657,14 +677,14 @@ __device__ __forceinline__ void kahan_merge(float &s, float &c, float v) {
 // both branches with selects.
 // Bound by the FP32 FMA pipe (63% busy) and the issue slots.  Sources rather than targets in the two lanes: half the
 // staging memory per source, so chunks of 1,024 instead of 512, and half the running sums; 15M-bead cube
-// 22.25 -> 22.1 ms, 256 systems 29.2 -> 28.5, noise 50k 0.071 -> 0.064.  A third form for iterations that are far but for
+// 22.25 -> 22.1 ms, 256 systems 29.2 -> 28.5, noise 50k 0.071 -> 0.064.  Items that carry their box and target range: 22.0.  A third form for iterations that are far but for
 // self pairs (1 in 27 on a uniform system, with 1/r = 0 there) was no faster: 22.2 and 29.2 ms.
 constexpr int kP32Queue = 256;   // FP64 pairs of one staged chunk handled after its FP32 loop
 constexpr size_t kP32Smem = sizeof(float4) * 3 * (kP32Chunk / 2) + sizeof(float2) * 3 * kP32Threads +
                             sizeof(double) * 3 * kP32Threads + sizeof(int) * kP32Chunk +
                             sizeof(int) * (2 * kP32List + 2) + sizeof(float) * 6 + sizeof(int) * (kP32Queue + 2);
 
-__global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, const int *leaves, const int *beg,
+__global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int4 *items, const int *beg,
                                                          const int *end,
                                                          const int *bsys, const double *ctr, const int *uoff,
                                                          const int *uidx, const float *p32, const float *f32,
@@ -681,8 +701,8 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, con
     float *sCtr = reinterpret_cast<float *>(lpre + kP32List + 2);   // target leaf centre, hi and lo floats
     int *sQn = reinterpret_cast<int *>(sCtr + 6);   // [0] queue length, [1] any FP64 pair of this item
     int *sQ = sQn + 2;                              // queued pairs: thread << 11 | source slot
-    const int2 item = items[blockIdx.x];
-    const int li = item.x, b = leaves[li], sys = bsys[b];
+    const int4 item = items[blockIdx.x];
+    const int li = item.x, b = item.y, sys = bsys[b];
     const PairConst &pc = sc.pc[sys];
     const double a = pc.a, cf = pc.cf, co = pc.co;
     P32Const k;
@@ -705,7 +725,7 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int2 *items, con
     const float *xh = p32, *yh = p32 + n, *zh = p32 + 2 * n, *xl = p32 + 3 * n, *yl = p32 + 4 * n, *zl = p32 + 5 * n;
     const float2 K23 = make_float2(k.k23, k.k23), NK2 = make_float2(k.nk2, k.nk2);
     const int u0 = uoff[li], u1 = uoff[li + 1];
-    const int tb = item.y, te = min(end[b], item.y + kItemTargets), nt = te - tb;
+    const int tb = item.z, te = item.w, nt = te - tb;
     const int G = kP32Threads / nt;
     const int tl = threadIdx.x % nt, g = threadIdx.x / nt;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -913,15 +933,15 @@ int run_p2p(Tree &t, const double *fs, double *out, const SysConst &sc, cudaStre
     const int *off = merged ? t.m_off : (direct_list ? t.d_off : t.u_off);
     const int *idx = merged ? t.m_idx : (direct_list ? t.d_idx : t.u_idx);
     int add_self = direct_list ? 0 : 1;
-    const int2 *items = merged ? t.m_items : (direct_list ? t.d_items : t.u_items);
+    const int4 *items = merged ? t.m_items : (direct_list ? t.d_items : t.u_items);
     if (t.n_items == 0) return RPY_OK;
     RPY_CHECK(set_near_smem());
     if (t.params.precision == RPY_FP32) {
-        k_p2p32<<<t.n_items, kP32Threads, kP32Smem, st>>>(items, t.leaves, t.b_begin, t.b_end, t.b_sys, t.b_center,
+        k_p2p32<<<t.n_items, kP32Threads, kP32Smem, st>>>(items, t.b_begin, t.b_end, t.b_sys, t.b_center,
                                                           off, idx, t.p32, t.f32, t.pos, fs, t.n, sc, add_self, out);
         RPY_LAUNCHED(1);
     } else {
-        k_p2p_df<<<t.n_items, kDfThreads, kDfSmem, st>>>(items, t.leaves, t.b_begin, t.b_end, t.b_sys, t.b_level, off,
+        k_p2p_df<<<t.n_items, kDfThreads, kDfSmem, st>>>(items, t.b_begin, t.b_end, t.b_sys, t.b_level, off,
                                                          idx, t.p3, t.f2, t.sys_fmax, t.pos, fs, t.n, sc, add_self,
                                                          out);
         RPY_LAUNCHED(1);

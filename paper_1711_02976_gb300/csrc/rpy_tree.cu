@@ -850,7 +850,7 @@ __global__ void k_item_count(int nleaf, const int *leaves, const int *beg, const
         return;
     }
     int b = leaves[li];
-    cnt[li] = (end[b] - beg[b] + kItemTargets - 1) / kItemTargets;
+    cnt[li] = item_count(end[b] - beg[b]);
 }
 
 __device__ __forceinline__ uint64_t cost_key(unsigned long long c) {
@@ -858,7 +858,7 @@ __device__ __forceinline__ uint64_t cost_key(unsigned long long c) {
 }
 
 __global__ void k_item_fill(int nleaf, const int *leaves, const int *beg, const int *end, const int *uoff,
-                            const int *uidx, const int *doff, const int *didx, const int *ioff, int2 *items,
+                            const int *uidx, const int *doff, const int *didx, const int *ioff, int4 *items,
                             uint64_t *ku, uint32_t *vu, uint64_t *kd, uint32_t *vd, uint64_t *km, uint32_t *vm) {
     int li = blockIdx.x * blockDim.x + threadIdx.x;
     if (li >= nleaf) return;
@@ -867,9 +867,11 @@ __global__ void k_item_fill(int nleaf, const int *leaves, const int *beg, const 
     unsigned long long su = 0, sd = 0;
     for (int k = uoff[li]; k < uoff[li + 1]; ++k) su += unsigned(end[uidx[k]] - beg[uidx[k]]);
     for (int k = doff[li]; k < doff[li + 1]; ++k) sd += unsigned(end[didx[k]] - beg[didx[k]]);
-    for (int q = 0, it = ioff[li]; q * kItemTargets < nt; ++q, ++it) {
-        unsigned tc = unsigned(min(kItemTargets, nt - q * kItemTargets));
-        items[it] = make_int2(li, t0 + q * kItemTargets);
+    const int full = nt / kItemTargets, r = nt % kItemTargets, per = rest_in_halves(r) ? (r + 1) / 2 : r;
+    for (int q = 0, it = ioff[li], j = t0; it < ioff[li + 1]; ++q, ++it) {   // as many as item_count has counted
+        const unsigned tc = unsigned(min(q < full ? kItemTargets : per, t0 + nt - j));
+        items[it] = make_int4(li, b, j, j + int(tc));
+        j += int(tc);
         ku[it] = cost_key(su * tc);
         vu[it] = uint32_t(it);
         kd[it] = cost_key(sd * tc);
@@ -879,8 +881,8 @@ __global__ void k_item_fill(int nleaf, const int *leaves, const int *beg, const 
     }
 }
 
-__global__ void k_item_order(int n, const int2 *items, const uint32_t *ou, const uint32_t *od, const uint32_t *om,
-                             int2 *u_items, int2 *d_items, int2 *m_items) {
+__global__ void k_item_order(int n, const int4 *items, const uint32_t *ou, const uint32_t *od, const uint32_t *om,
+                             int4 *u_items, int4 *d_items, int4 *m_items) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     u_items[i] = items[ou[i]];
@@ -1194,12 +1196,12 @@ int tree_build(Tree &t, const double *pos_dev, cudaStream_t st) {
         if (scan_tmp_bytes(nleaf + 1) > sbytes) return RPY_ERR_INTERNAL;
         RPY_TRY(exclusive_scan_i32(icnt, ioff, nleaf + 1, &ni, stmp, sbytes, st));
         t.n_items = ni;
-        int2 *items;
+        int4 *items;
         uint64_t *ku, *kd, *km, *kt;
         uint32_t *vu, *vd, *vm, *vt;
         int *icounts;
         const int itiles = nblk(std::max(ni, 1), kSortTile);
-        RPY_TRY(dev_alloc(scratch, (void **)&items, sizeof(int2) * std::max(ni, 1)));
+        RPY_TRY(dev_alloc(scratch, (void **)&items, sizeof(int4) * std::max(ni, 1)));
         RPY_TRY(dev_alloc(scratch, (void **)&ku, sizeof(uint64_t) * std::max(ni, 1)));
         RPY_TRY(dev_alloc(scratch, (void **)&kd, sizeof(uint64_t) * std::max(ni, 1)));
         RPY_TRY(dev_alloc(scratch, (void **)&km, sizeof(uint64_t) * std::max(ni, 1)));
@@ -1210,9 +1212,9 @@ int tree_build(Tree &t, const double *pos_dev, cudaStream_t st) {
         RPY_TRY(dev_alloc(scratch, (void **)&vt, sizeof(uint32_t) * std::max(ni, 1)));
         RPY_TRY(dev_alloc(scratch, (void **)&icounts, sizeof(int) * 256 * size_t(itiles)));
         if (scan_tmp_bytes(256 * itiles) > sbytes) return RPY_ERR_INTERNAL;
-        RPY_TRY(dev_alloc(t, (void **)&t.u_items, sizeof(int2) * std::max(ni, 1)));
-        RPY_TRY(dev_alloc(t, (void **)&t.d_items, sizeof(int2) * std::max(ni, 1)));
-        RPY_TRY(dev_alloc(t, (void **)&t.m_items, sizeof(int2) * std::max(ni, 1)));
+        RPY_TRY(dev_alloc(t, (void **)&t.u_items, sizeof(int4) * std::max(ni, 1)));
+        RPY_TRY(dev_alloc(t, (void **)&t.d_items, sizeof(int4) * std::max(ni, 1)));
+        RPY_TRY(dev_alloc(t, (void **)&t.m_items, sizeof(int4) * std::max(ni, 1)));
         if (ni > 0) {
             k_item_fill<<<nblk(nleaf, 256), 256, 0, st>>>(nleaf, t.leaves, t.b_begin, t.b_end, t.u_off, t.u_idx,
                                                           t.d_off, t.d_idx, ioff, items, ku, vu, kd, vd, km, vm);

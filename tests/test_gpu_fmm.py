@@ -258,6 +258,23 @@ def test_fp64_near_part_in_double_floats(name, n, leaf_cap):
         assert (np.abs(u[mem] - ref[mem]).max(axis=1) <= 2.0 ** -40 * mag).all(), name
 
 
+@pytest.mark.parametrize("n", [128, 129, 141, 170, 171, 192, 193, 340, 385, 513])
+def test_near_items_of_one_leaf(n):
+    """A leaf's beads fall into full work items and a rest, halved where that fills the block better; both
+    precision forms on both sides of each change of the split.  FP32: coordinates relative to the leaf's
+    centre round at 2^-24, some 10 roundings per pair value."""
+    rng = np.random.default_rng(n)
+    pos, f, a = rng.random((n, 3)), rng.standard_normal((n, 3)), 0.01
+    s = 6 * math.pi * a
+    r = np.linalg.norm(pos[:, None, :] - pos[None, :, :], axis=2)
+    mag = (s / (8 * math.pi)) * (8.0 / 3.0) * (np.linalg.norm(f, axis=1) / np.maximum(r, a))
+    rel = np.where(r > 0, 4 * 2.0 ** -24 / np.maximum(r, a), 0.0)   # of a pair's value, per rounded coordinate
+    for prec, bound in ((0, 2.0 ** -40 * mag.sum(axis=1)), (1, (mag * (10 * 2.0 ** -24 + rel)).sum(axis=1))):
+        u, t = matvec(pos, f, a, s, 3, leaf_cap=600, precision=prec, parts=rp.RPY_PART_NEAR)
+        assert len(rp.rpy_tree_export(t, "leaves")) == 1
+        assert (np.abs(u - _near_oracle(t, pos, f, a, s)).max(axis=1) <= bound).all(), prec
+
+
 def test_fp64_near_part_outside_the_double_float_range():
     """A system whose forces hold an infinity, or lie below the range the double-floats cover, takes the
     all-FP64 form; in a forest the other system is untouched."""
