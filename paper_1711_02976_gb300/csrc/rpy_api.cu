@@ -424,7 +424,7 @@ int tree_alloc_workspace(Tree &t, cudaStream_t st) {
     t.x_frames = (t.params.flags & RPY_FLAG_FRAME_PASSES) ? 1 : plane_wave_frames(double(nb), double(es), h.S);
     RPY_TRY(dev_alloc(t, &t.Xo, es * nb * 2 * t.x_frames * kSets * h.S));
     RPY_TRY(dev_alloc(t, &t.Xi, es * nb * 2 * t.x_frames * kSets * h.S));
-    RPY_TRY(dev_alloc(t, &t.EVg, es * size_t(t.nleaf) * 18 * h.nc));
+    RPY_TRY(dev_alloc(t, &t.EVg, es * size_t(t.nleaf) * (t.params.flags & RPY_FLAG_EVAL_PER_POTENTIAL ? 18 : 6) * h.nc));
     RPY_TRY(dev_alloc(t, (void **)&t.fs, sizeof(double) * 3 * t.n));
     if (t.params.precision == RPY_FP32) {
         RPY_TRY(dev_alloc(t, (void **)&t.p32, sizeof(float) * 6 * t.n));

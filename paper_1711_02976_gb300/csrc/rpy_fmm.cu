@@ -27,10 +27,11 @@
 //                     rotated back to the world frame
 //   k_p2l      S->L   X list
 //   k_l2l_rot  L->L   the same for locals, level by level downward
-//   k_far_eval L->T, M->T   L2P for the leaf and M2P for its W list, with the
-//                     gradients and Hessians of Theorems 1-2 formed as
-//                     derivative expansions per box, combined by Eq. (2.8):
-//                     u = C1 [L1 L2 L3] - C1 sum_k x_k grad L_k + C1 grad L4 - C2 grad L_C.
+//   k_eval_prep, k_eval_apply  L->T   L2P: the gradients and Hessians of Theorems 1-2 formed as derivative
+//                     expansions per leaf, combined by Eq. (2.8):
+//                     u = C1 [L1 L2 L3] - C1 sum_k x_k grad L_k + C1 grad L4 - C2 grad L_C,
+//                     six fields at each bead
+//   k_far_eval M->T   M2P of a leaf's W list, by the same six fields
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -117,6 +118,74 @@ __device__ void eval_fields(T x, T y, T z, int P, const cpx<T> *E, int stride, c
     }
 #pragma unroll
     for (int q = 0; q < NE; ++q) acc[q] = closed(acc[q]);
+}
+
+// Coefficient i of the six fields of fold_fields.
+__device__ __forceinline__ void load_six(const cpx<float> *E, int i, cpx<float> (&e)[6]) {
+    const float4 *q = reinterpret_cast<const float4 *>(E + 6 * i);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float4 v = q[k];
+        e[2 * k] = mk(v.x, v.y);
+        e[2 * k + 1] = mk(v.z, v.w);
+    }
+}
+__device__ __forceinline__ void load_six(const cpx<dfl> *E, int i, cpx<dfl> (&e)[6]) {
+    const float4 *q = reinterpret_cast<const float4 *>(E + 6 * i);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const float4 v = q[k];
+        e[k] = mk(dfl(v.x, v.y), dfl(v.z, v.w));
+    }
+}
+
+// The six fields of fold_fields at one point.  AHEAD: each step's coefficients are loaded a step before, for few warps
+// hide the loads where they come from global memory (k_eval_apply: 20,001 beads, 6 digits, FP64 0.16 -> 0.11 ms
+// together with the bound on its registers) or the registers leave room for few (double-floats); the FP32 k_far_eval has
+// warps enough and gains nothing.
+template <typename T, bool IRREG, bool AHEAD>
+__device__ void eval_six(T x, T y, T z, int P, const cpx<T> *E, const T *ra, const T *rb, const T *rc, T *acc) {
+    const T r2 = fma(z, z, fma(y, y, x * x));
+    const T ir2 = IRREG ? T(1) / r2 : T(0);
+    const cpx<T> w = IRREG ? mk(x * ir2, y * ir2) : mk(x, y);
+    const T zz = IRREG ? z * ir2 : z;
+    const T rr = IRREG ? ir2 : r2;
+    cpx<T> diag = IRREG ? mk<T>(sqrt(ir2), 0) : mk<T>(1, 0);
+    cpx<T> e[6], f[6];
+    if constexpr (AHEAD) load_six(E, 0, e);
+    for (int m = 0; m <= P; ++m) {
+        if (m > 0) diag = rc[m] * (w * diag);
+        cpx<T> p2 = mk<T>(0, 0), p1 = diag;
+#pragma unroll 2
+        for (int n = m;;) {
+            const bool last = n == P;
+            T a, b;
+            if constexpr (AHEAD) {
+                const int i = last ? (m < P ? tri(m + 1, m + 1) : 0) : tri(n + 1, m);
+                load_six(E, i, f);
+                a = ra[i], b = rb[i];
+            } else {
+                load_six(E, tri(n, m), e);
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                macc(acc[q], e[q].x, p1.x);
+                macc(acc[q], -e[q].y, p1.y);
+            }
+            if constexpr (AHEAD)
+#pragma unroll
+                for (int q = 0; q < 6; ++q) e[q] = f[q];
+            if (last) break;
+            ++n;
+            if constexpr (!AHEAD) a = ra[tri(n, m)], b = rb[tri(n, m)];
+            const T A = a * zz, B = b * rr;
+            const cpx<T> c = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
+            p2 = p1;
+            p1 = c;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) acc[q] = closed(acc[q]);
 }
 
 // ---------------------------------------------------------------- derivative expansions
@@ -368,10 +437,20 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
 constexpr int kNE = 18;   // evaluation expansions of Eq. (2.8) per box
 constexpr int kNF = 12;   // evaluated per bead after the fold of k_eval_prep (per-potential form)
 constexpr int kNF2 = 6;   // evaluated per bead in the one-expansion-per-component form
+constexpr int kFarGroups = 4;   // source boxes per round of k_far_eval at most
 
-// Build the 18 evaluation expansions of Eq. (2.8) from 4 source expansions.
-// IRREG = multipole source (degrees grow by one per derivative), else local.
-template <typename T, bool IRREG>
+// tables of k_far_eval (recurrences, ladders, 1 / (2k + 1)) and k_eval_prep (the last two), 16-byte multiples
+template <typename T>
+__host__ __device__ inline int far_tab_floats(int p) {
+    return (tab_floats<T>(p) + p + 4 + 3) & ~3;
+}
+template <typename T>
+__host__ __device__ inline int prep_tab_floats(int p) {
+    return (6 * ncoef(p + 2) + p + 4 + 3) & ~3;
+}
+
+// Build the 18 evaluation expansions of Eq. (2.8) from 4 local expansions (the per-potential form).
+template <typename T>
 __device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<T> *tmp, T cbx, T cby, T cbz,
                                const Lad<T> &G) {
     const int st = ncoef(P);
@@ -383,8 +462,7 @@ __device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<
     // 3..11 gradients of sets 0..2 (index 3 + 3k + a), tmp[0..2] gradient of set 3
     for (int k = 0; k < 4; ++k) {
         cpx<T> *gx = k < 3 ? EV + (3 + 3 * k) * st : tmp;
-        if (IRREG) d_multipole(src + k * ncoef(p), p, gx, gx + st, gx + 2 * st, P, G);
-        else d_local(src + k * ncoef(p), p, gx, gx + st, gx + 2 * st, P, G);
+        d_local(src + k * ncoef(p), p, gx, gx + st, gx + 2 * st, P, G);
     }
     __syncthreads();
     // 12..14: G4'_a = dL4_a - sum_k cb_k dL_k,a ; tmp[3] = L_C = dxL1 + dyL2 + dzL3
@@ -403,94 +481,209 @@ __device__ void build_eval_set(const cpx<T> *src, int p, int P, cpx<T> *EV, cpx<
         tmp[3 * st + i] = lc;
     }
     __syncthreads();
-    int pl = IRREG ? p + 1 : p - 1;
-    if (IRREG) d_multipole(tmp + 3 * st, pl, EV + 15 * st, EV + 16 * st, EV + 17 * st, P, G);
-    else d_local(tmp + 3 * st, pl, EV + 15 * st, EV + 16 * st, EV + 17 * st, P, G);
+    d_local(tmp + 3 * st, p - 1, EV + 15 * st, EV + 16 * st, EV + 17 * st, P, G);
     __syncthreads();
 }
 
-// rb: the multipoles carry q4 about their own box centres (box origin), so the
-// set-4 gradient is re-based from the source box's centre to the leaf's.
-template <typename T>
-__global__ void k_far_eval(const int *leaves, DevTables<T> D, const int *beg, const int *end, const double *ctr,
-                           const double *side, const int *lvl, const int *bsys, const int *woff, const int *widx,
-                           const double *pos, int64_t n, SysConst sc, const cpx<T> *L, const cpx<T> *M,
-                           double *ufar, int rb) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    int li = blockIdx.x;
-    int b = leaves[li];
-    const int p = D.p, nc = ncoef(p), P = p + 2, st = ncoef(P);
-    T *smr = reinterpret_cast<T *>(smem_raw);
-    Rec<T> R = load_rec(D, smr);
-    Lad<T> G = load_lad(D, smr + rec_floats<T>(p));
-    cpx<T> *EV = reinterpret_cast<cpx<T> *>(smr + tab_floats<T>(p));
-    cpx<T> *tmp = EV + kNE * st;
-    cpx<T> *srcs = tmp + 4 * st;
-    int sy = bsys[b];
-    const double C1 = sc.pc[sy].C1, C2 = sc.pc[sy].C2, icube = sc.pc[sy].icube;
-    double c0x = sc.cube[4 * sy], c0y = sc.cube[4 * sy + 1], c0z = sc.cube[4 * sy + 2];
-    double cbx = ctr[3 * b], cby = ctr[3 * b + 1], cbz = ctr[3 * b + 2];
-    float c3b[9];
-    if constexpr (kIsDf<T>)
-        for (int k = 0; k < 9; ++k) c3b[k] = sc.c3[9 * size_t(b) + k];
-    int j0 = beg[b], j1 = end[b];
-    int nw = woff[li + 1] - woff[li];
-    if (nw == 0) return;
-    for (int jc = j0; jc < j1; jc += blockDim.x) {
-        int j = jc + threadIdx.x;
-        bool act = j < j1;
-        double x = act ? pos[j] : cbx, y = act ? pos[n + j] : cby, z = act ? pos[2 * n + j] : cbz;
-        double u[3] = {0, 0, 0};
-        for (int w = 0; w < nw; ++w) {
-            const int C = widx[woff[li] + w];
-            const cpx<T> *E = M + size_t(C) * kSets * nc;
-            __syncthreads();
-            for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) srcs[i] = E[i];
-            __syncthreads();
-            // origin of the source expansion's q4: its own centre (box origin) or the cube centre
-            T acc[kNE];
+// Eq. (2.8) of one expansion of degree p as six fields, with x the offset from the expansion's centre in box sides
+// and o its centre relative to the origin of q4 (Approach 2 of Sec. 2, one expansion per velocity component):
+//   u_d = L_d - sum_k x_k dL_k/dx_d + c4 dS/dx_d - cc dL_C/dx_d,  S = L4 - sum_k o_k L_k,  L_C = sum_k dL_k/dx_k
+// in units of C1/h.  A coordinate times a harmonic function splits into harmonic ones (Kelvin transform): for each
+// degree-n part h of a local expansion, with g = h / (2n + 1),
+//   x_k h = [x_k h - |x|^2 d_k g] + |x|^2 d_k g,
+// where the bracket is -|x|^(2n+3) d_k(g / |x|^(2n+1)): the coefficients of d_k g taken as a multipole expansion's,
+// negated and read as a local one's.  For a multipole expansion the two swap, its local-form
+// derivative being the bracket's part without |x|^2.  So
+//   sum_k x_k L_k = U + |x|^2 V,  sum_k x_k dL_k/dx_d = d_d(U + |x|^2 V) - L_d = d_d U + 2 x_d V + |x|^2 d_d V - L_d,
+// and with x_d V = Y_d + |x|^2 Z_d
+//   u_d = [2 L_d + d_d(c4 S - U - cc L_C) - 2 Y_d] - |x|^2 [d_d V + 2 Z_d].
+// V and Z are the native derivatives (L_C and d_d V) scaled by degree: two scalar expansions are differentiated where
+// the gradients of all three L_k would be three times the work.  inv[k] = 1 / (2k + 1).  The fields
+// carry the factor 2 of the m > 0 terms of Re(sum E h) and stand interleaved, [coefficient][6].
+template <typename T, bool IRREG>
+__device__ __forceinline__ cpx<T> d_native(const cpx<T> *src, int ps, int c, int i, const Lad<T> &G) {
+    return IRREG ? d_mul_one(src, ps, c, i, G) : d_loc_one(src, ps, c, i, G);
+}
+
+template <typename T, bool IRREG>
+__device__ __forceinline__ void fold_scalars(const cpx<T> *src, int p, int i, T c4, T cc, const T *o, const T *inv,
+                                             const Lad<T> &G, cpx<T> *phi, cpx<T> *V) {
+    const int nc = ncoef(p), k = deg_of(i);
+    cpx<T> lc = mk<T>(0, 0), x = lc, S = lc;
 #pragma unroll
-            for (int q = 0; q < kNE; ++q) acc[q] = T(0);
-            if constexpr (kIsDf<T>) {
-                // lengths in the split units; L4 and the C2 term carry their factors here
-                T cb[3], v[3], xi[3];
-                const double ihd = inv_side_u(sc.pc[sy], lvl[C]);
-                const T ihs = T(ihd);
-                for (int a = 0; a < 3; ++a) {
-                    cb[a] = rb ? coord_diff(c3b, sc.c3 + 9 * size_t(C), a) : dfl3(c3b[3 * a], c3b[3 * a + 1], c3b[3 * a + 2]);
-                    v[a] = act ? coord_diff(sc.p3, n, j, a, sc.c3 + 9 * size_t(C)) * ihs : T(1);
-                    xi[a] = act ? coord_diff(sc.p3, n, j, a, c3b) * ihs : T(0);
-                }
-                build_eval_set<T, true>(srcs, p, P, EV, tmp, cb[0], cb[1], cb[2], G);
-                eval_fields<T, kNE, true>(v[0], v[1], v[2], P, EV, st, R.a, R.b, R.c, acc);
-                const T cc = T(double(sc.pc[sy].d_k23h) + double(sc.pc[sy].d_k23l)) * ihs;
-                const double w1 = sc.pc[sy].C1 * sc.pc[sy].d_xs * force_unit(sc.fmax[sy]) * ihd;
-                for (int d = 0; d < 3; ++d) {
-                    T t = acc[d] + ihs * (acc[12 + d] - cc * acc[15 + d]);
-                    for (int k = 0; k < 3; ++k) t -= xi[k] * acc[3 + 3 * k + d];
-                    u[d] += w1 * double(t);
-                }
-            } else {
-                const double ox = rb ? ctr[3 * C] : c0x, oy = rb ? ctr[3 * C + 1] : c0y, oz = rb ? ctr[3 * C + 2] : c0z;
-                build_eval_set<T, true>(srcs, p, P, EV, tmp, T(cbx - ox), T(cby - oy), T(cbz - oz), G);
-                double ih = icube * pow2i(lvl[C]);   // 1 / side[C], exactly
-                T vx = T((x - ctr[3 * C]) * ih), vy = T((y - ctr[3 * C + 1]) * ih), vz = T((z - ctr[3 * C + 2]) * ih);
-                eval_fields<T, kNE, true>(vx, vy, vz, P, EV, st, R.a, R.b, R.c, acc);
-                double xi[3] = {(x - cbx) * ih, (y - cby) * ih, (z - cbz) * ih};
-                for (int d = 0; d < 3; ++d) {
-                    double v = double(acc[d]);
-                    for (int k = 0; k < 3; ++k) v -= xi[k] * double(acc[3 + 3 * k + d]);
-                    u[d] += C1 * ih * v + C1 * ih * ih * double(acc[12 + d]) - C2 * ih * ih * ih * double(acc[15 + d]);
-                }
-            }
+    for (int c = 0; c < 3; ++c) {
+        lc += d_native<T, IRREG>(src + c * nc, p, c, i, G);
+        x += d_native<T, !IRREG>(src + c * nc, p, c, i, G);
+    }
+    if (i < nc) {
+        S = src[3 * nc + i];
+        for (int c = 0; c < 3; ++c) {
+            const cpx<T> v = src[c * nc + i];
+            macc(S.x, -o[c], v.x);
+            macc(S.y, -o[c], v.y);
         }
-        if (act)
-            for (int d = 0; d < 3; ++d) ufar[3 * size_t(j) + d] += u[d];
+        S = mk(closed(S.x), closed(S.y));
+    }
+    const T up = inv[k + 1], dn = inv[max(k - 1, 0)];   // (no derivative raises to degree 0)
+    V[i] = (IRREG ? -dn : up) * lc;
+    const T u = IRREG ? -up : dn;
+    cpx<T> f = mk(c4 * S.x, c4 * S.y);
+    macc(f.x, u, x.x);
+    macc(f.y, u, x.y);
+    macc(f.x, -cc, lc.x);
+    macc(f.y, -cc, lc.y);
+    phi[i] = mk(closed(f.x), closed(f.y));
+}
+
+template <typename T, bool IRREG>
+__device__ __forceinline__ void fold_fields(const cpx<T> *src, int p, int i, const T *inv, const Lad<T> &G,
+                                            const cpx<T> *phi, const cpx<T> *V, cpx<T> *out) {
+    const int nc = ncoef(p), k = deg_of(i), pv = IRREG ? p + 1 : p - 1;
+    const T up = inv[k + 1], dn = inv[max(k - 1, 0)];
+    const float w = i == tri(k, 0) ? 1.f : 2.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const cpx<T> a = d_native<T, IRREG>(V, pv, d, i, G), b = d_native<T, !IRREG>(V, pv, d, i, G);
+        cpx<T> h = d_native<T, IRREG>(phi, p + 1, d, i, G);
+        if (i < nc) {
+            const cpx<T> v = src[d * nc + i];
+            h += mk(scale2(2.f, v.x), scale2(2.f, v.y));
+        }
+        h += scale2(2.f, IRREG ? -up : dn) * b;
+        const T z = T(1) + scale2(2.f, IRREG ? -dn : up);
+        out[6 * i + d] = mk(scale2(w, h.x), scale2(w, h.y));
+        const cpx<T> B = z * a;
+        out[6 * i + 3 + d] = mk(scale2(w, B.x), scale2(w, B.y));
     }
 }
 
-// Per leaf at level >= 2: the 18 derived local expansions of Eq. (2.8),
-// written to global memory for the bead-parallel evaluation.
+template <typename T>
+__device__ const T *load_inv(T *sm, int p) {   // p + 4 entries
+    for (int k = threadIdx.x; k < p + 4; k += blockDim.x) {
+        if constexpr (kIsDf<T>) sm[k] = recip(T(2 * k + 1));
+        else sm[k] = T(1) / T(2 * k + 1);
+    }
+    return sm;
+}
+
+// M2P of the W lists, a near-field work item (at most kItemTargets beads of a leaf) per block: the six fields of
+// `groups` source boxes at a time are formed in shared memory by the whole block, and each box then is evaluated
+// by its own group of threads, one bead each.
+// Bound by the FP32 pipe (the macc of the fields) and the loads of the fields from shared memory.  Eighteen fields per box,
+// formed for every 64 beads of the leaf, took twice the arithmetic and three times the loads; a block per leaf left
+// the large leaves of a cluster to run alone.  Evaluation stage before and now: 1M mixed, 6 digits, FP64 4.72 -> 2.40 ms,
+// FP32 1.86 -> 0.82 ms; 256 systems FP32 4.77 -> 3.29 ms; a Plummer cluster of 30,001 beads 416 -> 180 us.  64 threads: FP32
+// 0.96 ms; 256: 0.78 ms, but 256 systems 3.57 ms, most of whose items have no W list; two boxes a round instead of up to four:
+// the same within 1%.
+constexpr int kFarThreads = 128;
+template <typename T>
+struct FarBox {   // one source box of the round
+    T c4, cc, o[3];
+    double w;     // per velocity: C1 / side, with the force unit
+    int box;
+};
+template <typename T>
+__global__ void __launch_bounds__(kFarThreads) k_far_eval(const int4 *items, DevTables<T> D, const double *ctr,
+                                                          const int *lvl, const int *bsys, const int *woff,
+                                                          const int *widx, const double *pos, int64_t n, SysConst sc,
+                                                          const cpx<T> *M, double *ufar, int rb, int groups) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ FarBox<T> sB[kFarGroups];
+    __shared__ double sU[3][kItemTargets];
+    const int4 item = items[blockIdx.x];
+    const int w0 = woff[item.x], nw = woff[item.x + 1] - w0;
+    if (nw == 0) return;
+    const int p = D.p, nc = ncoef(p), n1 = ncoef(p + 1), P = p + 2, st = ncoef(P), sy = bsys[item.y];
+    T *smr = reinterpret_cast<T *>(smem_raw);
+    const Rec<T> R = load_rec(D, smr);
+    const Lad<T> G = load_lad(D, smr + rec_floats<T>(p));
+    const T *inv = load_inv(smr + tab_floats<T>(p), p);
+    const int per = kSets * nc + 2 * n1 + 6 * st;
+    cpx<T> *box0 = reinterpret_cast<cpx<T> *>(smr + far_tab_floats<T>(p));
+    const PairConst &pc = sc.pc[sy];
+    const int nt = item.w - item.z, rows = min(nt, kFarThreads), ng = min(min(groups, nw), kFarThreads / rows);
+    const int tl = threadIdx.x % rows, g = threadIdx.x / rows;
+    for (int e = threadIdx.x; e < 3 * kItemTargets; e += kFarThreads) sU[0][e] = 0.0;
+    for (int wb = 0; wb < nw; wb += ng) {
+        const int nb = min(ng, nw - wb);
+        __syncthreads();
+        if (threadIdx.x < nb) {
+            FarBox<T> B;
+            const int C = B.box = widx[w0 + wb + threadIdx.x];
+            if constexpr (kIsDf<T>) {   // lengths in the split units: C2 / C1 = 2a^2/3 there
+                const double ihd = inv_side_u(pc, lvl[C]);
+                B.c4 = T(ihd);
+                B.cc = T((double(pc.d_k23h) + double(pc.d_k23l)) * ihd * ihd);
+                const float *c = sc.c3 + 9 * size_t(C);
+                for (int a = 0; a < 3; ++a) B.o[a] = rb ? T(0) : dfl3(c[3 * a], c[3 * a + 1], c[3 * a + 2]);
+                B.w = pc.C1 * pc.d_xs * force_unit(sc.fmax[sy]) * ihd;
+            } else {
+                const double ih = pc.icube * pow2i(lvl[C]);   // 1 / side[C], exactly
+                B.c4 = T(ih);
+                B.cc = T(pc.C2 / pc.C1 * ih * ih);
+                for (int a = 0; a < 3; ++a) B.o[a] = rb ? T(0) : T(ctr[3 * C + a] - sc.cube[4 * sy + a]);
+                B.w = pc.C1 * ih;
+            }
+            sB[threadIdx.x] = B;
+        }
+        for (int e = threadIdx.x; e < nb * kSets * nc; e += kFarThreads) {
+            const int gg = e / (kSets * nc), r = e - gg * kSets * nc;
+            box0[gg * per + r] = M[size_t(widx[w0 + wb + gg]) * kSets * nc + r];
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < nb * n1; e += kFarThreads) {
+            const int gg = e / n1;
+            cpx<T> *src = box0 + gg * per, *phi = src + kSets * nc;
+            fold_scalars<T, true>(src, p, e - gg * n1, sB[gg].c4, sB[gg].cc, sB[gg].o, inv, G, phi, phi + n1);
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < nb * st; e += kFarThreads) {
+            const int gg = e / st;
+            cpx<T> *src = box0 + gg * per, *phi = src + kSets * nc;
+            fold_fields<T, true>(src, p, e - gg * st, inv, G, phi, phi + n1, phi + 2 * n1);
+        }
+        __syncthreads();
+        if (g < nb) {
+            const int C = sB[g].box;
+            const cpx<T> *E = box0 + g * per + kSets * nc + 2 * n1;
+            const double w = sB[g].w;
+            for (int t = tl; t < nt; t += rows) {   // one group takes more than one bead a thread
+                const int j = item.z + t;
+                double *u = &sU[0][g * rows + t];
+                T acc[6];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) acc[q] = T(0);
+                if constexpr (kIsDf<T>) {
+                    const float *c = sc.c3 + 9 * size_t(C);
+                    const T ihs = sB[g].c4;
+                    const T x = coord_diff(sc.p3, n, j, 0, c) * ihs, y = coord_diff(sc.p3, n, j, 1, c) * ihs,
+                            z = coord_diff(sc.p3, n, j, 2, c) * ihs;
+                    eval_six<T, true, kIsDf<T>>(x, y, z, P, E, R.a, R.b, R.c, acc);
+                    const T r2 = fma(z, z, fma(y, y, x * x));
+                    for (int d = 0; d < 3; ++d) u[d * kItemTargets] += w * double(acc[d] - r2 * acc[3 + d]);
+                } else {
+                    const double ih = pc.icube * pow2i(lvl[C]);
+                    const double x = (pos[j] - ctr[3 * C]) * ih, y = (pos[n + j] - ctr[3 * C + 1]) * ih,
+                                 z = (pos[2 * n + j] - ctr[3 * C + 2]) * ih;
+                    eval_six<T, true, kIsDf<T>>(T(x), T(y), T(z), P, E, R.a, R.b, R.c, acc);
+                    const double r2 = x * x + y * y + z * z;
+                    for (int d = 0; d < 3; ++d) u[d * kItemTargets] += w * (double(acc[d]) - r2 * double(acc[3 + d]));
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 3 * nt; e += kFarThreads) {
+        const int t = e / 3, d = e - 3 * t;
+        double v = 0.0;
+        for (int gg = 0; gg < ng; ++gg) v += sU[d][gg * rows + t];
+        ufar[3 * size_t(item.z) + e] += v;
+    }
+}
+
+// Per leaf at level >= 2: the evaluated expansions of Eq. (2.8), written to global memory for the
+// bead-parallel evaluation: six fields per leaf (per velocity component), or by request the twelve of the
+// per-potential form.
 // rb: the local expansions carry q4 about their own box centres (box origin),
 // so set 4 needs no re-basing to the leaf centre.
 template <typename T>
@@ -503,33 +696,41 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
     const int p = D.p, nc = ncoef(p);
     T *smr = reinterpret_cast<T *>(smem_raw);
     Lad<T> G = load_lad(D, smr);
-    cpx<T> *srcs = reinterpret_cast<cpx<T> *>(smr + ((6 * ncoef(p + 2) + 1) & ~1));
+    const T *inv = load_inv(smr + 6 * ncoef(p + 2), p);
+    cpx<T> *srcs = reinterpret_cast<cpx<T> *>(smr + prep_tab_floats<T>(p));
     cpx<T> *tmp = srcs + kSets * nc;
     const cpx<T> *E = L + size_t(b) * kSets * nc;
     for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) srcs[i] = E[i];
-    __syncthreads();
     int sy = bsys[b];
-    cpx<T> *EV = EVg + size_t(li) * kNE * nc;
-    if (rb) {
-        build_eval_set<T, false>(srcs, p, p, EV, tmp, T(0), T(0), T(0), G);
-    } else if constexpr (kIsDf<T>) {
-        const float *c = sc.c3 + 9 * size_t(b);
-        build_eval_set<T, false>(srcs, p, p, EV, tmp, dfl3(c[0], c[1], c[2]), dfl3(c[3], c[4], c[5]),
-                                 dfl3(c[6], c[7], c[8]), G);
-    } else {
-        build_eval_set<T, false>(srcs, p, p, EV, tmp, T(ctr[3 * b] - sc.cube[4 * sy]),
-                                 T(ctr[3 * b + 1] - sc.cube[4 * sy + 1]), T(ctr[3 * b + 2] - sc.cube[4 * sy + 2]), G);
-    }
-    // Fold the terms of Eq. (2.8) that are not multiplied by a coordinate into
-    // fields 0..2 (in units of C1/h):  L_d + h^-1 dL4'_d - (C2/C1) h^-2 dL_C,d.
-    // The bead evaluation then needs fields 0..11 only.
-    const double ih = sc.pc[sy].icube * pow2i(lvl[b]);
-    T c4 = T(ih), cc = T(sc.pc[sy].C2 / sc.pc[sy].C1 * ih * ih);
+    T c4, cc, o[3] = {T(0), T(0), T(0)};
     if constexpr (kIsDf<T>) {   // lengths in the split units: C2 / C1 = 2a^2/3 there
         const double ihs = inv_side_u(sc.pc[sy], lvl[b]);
         c4 = T(ihs);
         cc = T((double(sc.pc[sy].d_k23h) + double(sc.pc[sy].d_k23l)) * ihs * ihs);
+        const float *c = sc.c3 + 9 * size_t(b);
+        if (!rb)
+            for (int a = 0; a < 3; ++a) o[a] = dfl3(c[3 * a], c[3 * a + 1], c[3 * a + 2]);
+    } else {
+        const double ih = sc.pc[sy].icube * pow2i(lvl[b]);   // 1 / side[b], exactly
+        c4 = T(ih);
+        cc = T(sc.pc[sy].C2 / sc.pc[sy].C1 * ih * ih);
+        if (!rb)
+            for (int a = 0; a < 3; ++a) o[a] = T(ctr[3 * b + a] - sc.cube[4 * sy + a]);
     }
+    __syncthreads();
+    if (per_component) {
+        cpx<T> *EV = EVg + size_t(li) * kNF2 * nc, *phi = tmp, *V = phi + ncoef(p + 1);
+        for (int i = threadIdx.x; i < ncoef(p + 1); i += blockDim.x)
+            fold_scalars<T, false>(srcs, p, i, c4, cc, o, inv, G, phi, V);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nc; i += blockDim.x) fold_fields<T, false>(srcs, p, i, inv, G, phi, V, EV);
+        return;
+    }
+    cpx<T> *EV = EVg + size_t(li) * kNE * nc;
+    build_eval_set<T>(srcs, p, p, EV, tmp, o[0], o[1], o[2], G);
+    // Fold the terms of Eq. (2.8) that are not multiplied by a coordinate into
+    // fields 0..2 (in units of C1/h):  L_d + h^-1 dL4'_d - (C2/C1) h^-2 dL_C,d.
+    // The bead evaluation then needs fields 0..11 only.
     for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x) {
         int d = i / nc, c = i - d * nc;
         cpx<T> v = EV[d * nc + c], g4 = EV[(12 + d) * nc + c], gc = EV[(15 + d) * nc + c];
@@ -540,44 +741,9 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
         v = mk(closed(v.x), closed(v.y));
         EV[d * nc + c] = v;
     }
-    int nf = kNF;
-    if (per_component) {
-        // Approach 2 of Sec. 2: one expansion per velocity component.  With
-        // G_kd = dL_k/dx_d (fields 3 + 3k + d, degree <= p - 1) and x the bead
-        // offset in box units, sum_k x_k G_kd = A_d + |x|^2 B_d with A_d, B_d
-        // harmonic: for each degree-n part h of G_kd, with g = h / (2n + 1),
-        //   x_k h = [x_k h - |x|^2 d_k g] + |x|^2 d_k g,
-        // where the bracket is -|x|^(2n+3) d_k(g / |x|^(2n+1)) (Kelvin transform:
-        // the same coefficients read as a multipole expansion), so
-        //   A_d = -sum_k [d_k of g as a multipole, read as a local expansion],
-        //   B_d =  sum_k [d_k of g as a local expansion].
-        // Fields become H_d = F_d - A_d (0..2, degree <= p) and B_d (3..5).
-        __syncthreads();
-        for (int i = threadIdx.x; i < 9 * nc; i += blockDim.x) {
-            const int c = i % nc;
-            const T w = T(1) / T(2 * deg_of(c) + 1);
-            cpx<T> v = EV[3 * nc + i];
-            EV[3 * nc + i] = mk(w * v.x, w * v.y);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x) {
-            const int d = i / nc, c = i - d * nc;
-            cpx<T> a = mk<T>(0, 0), bb = mk<T>(0, 0);
-            for (int k = 0; k < 3; ++k) {
-                const cpx<T> *g = EV + (3 + 3 * k + d) * nc;
-                a += d_mul_one(g, p - 1, k, c, G);
-                bb += d_loc_one(g, p - 1, k, c, G);
-            }
-            EV[d * nc + c] += a;
-            EV[(12 + d) * nc + c] = bb;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 3 * nc; i += blockDim.x) EV[3 * nc + i] = EV[12 * nc + i];
-        nf = kNF2;
-    }
     __syncthreads();
     // the evaluated fields carry the factor 2 of the m > 0 terms of Re(sum E h)
-    for (int i = threadIdx.x; i < nf * nc; i += blockDim.x) {
+    for (int i = threadIdx.x; i < kNF * nc; i += blockDim.x) {
         int c = i % nc, n = deg_of(c);
         if (c != tri(n, 0)) {
             cpx<T> v = EV[i];
@@ -589,10 +755,14 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
 // One thread per bead: L2P of the leaf's derived expansions and Eq. (2.8),
 // per potential (NF = 12: folded values and nine gradients) or per velocity
 // component (NF = 6: u_d = H_d - |x|^2 B_d).
+// Bound by latency on small systems, by the FP32 pipe on large ones.  With k_eval_prep, before the six fields stood
+// interleaved and came from two scalar expansions, and now: 15M-bead cube FP64 5.74 -> 4.71 ms, FP32 2.82 -> 2.36 ms; 200k
+// mixed at 9 digits 1.83 -> 0.98 ms; 4,096 beads FP64 51 -> 40 us.
 template <typename T, int NF>
-__global__ void k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves, DevTables<T> D, const double *ctr,
-                             const double *side, const int *lvl, const int *bsys, const double *pos, SysConst sc,
-                             const cpx<T> *EVg, double *ufar) {
+__global__ void __launch_bounds__(128, 6) k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
+                                                       DevTables<T> D, const double *ctr, const double *side,
+                                                       const int *lvl, const int *bsys, const double *pos, SysConst sc,
+                                                       const cpx<T> *EVg, double *ufar) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int li = bead_leaf[i];
@@ -611,8 +781,12 @@ __global__ void k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
             const T ihs = T(ihd);
             const T xi[3] = {coord_diff(sc.p3, n, i, 0, c) * ihs, coord_diff(sc.p3, n, i, 1, c) * ihs,
                              coord_diff(sc.p3, n, i, 2, c) * ihs};
-            eval_fields<T, NF, false, true>(xi[0], xi[1], xi[2], p, EVg + size_t(li) * kNE * nc, nc, D.rec_a, D.rec_b,
-                                            D.rec_c, acc);
+            if constexpr (NF == kNF2)
+                eval_six<T, false, true>(xi[0], xi[1], xi[2], p, EVg + size_t(li) * kNF2 * nc, D.rec_a, D.rec_b,
+                                         D.rec_c, acc);
+            else
+                eval_fields<T, NF, false, true>(xi[0], xi[1], xi[2], p, EVg + size_t(li) * kNE * nc, nc, D.rec_a,
+                                                D.rec_b, D.rec_c, acc);
             const double w1 = C1 * sc.pc[sy].d_xs * force_unit(sc.fmax[sy]) * ihd;
             const T r2 = fma(xi[2], xi[2], fma(xi[1], xi[1], xi[0] * xi[0]));
             for (int d = 0; d < 3; ++d) {
@@ -626,13 +800,15 @@ __global__ void k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
         const double ih = sc.pc[sy].icube * pow2i(lvl[b]);   // 1 / side[b], exactly
         double xi[3] = {(pos[i] - ctr[3 * b]) * ih, (pos[n + i] - ctr[3 * b + 1]) * ih,
                         (pos[2 * n + i] - ctr[3 * b + 2]) * ih};
-        eval_fields<T, NF, false, true>(T(xi[0]), T(xi[1]), T(xi[2]), p, EVg + size_t(li) * kNE * nc, nc, D.rec_a,
-                                        D.rec_b, D.rec_c, acc);
         if constexpr (NF == kNF2) {
+            eval_six<T, false, true>(T(xi[0]), T(xi[1]), T(xi[2]), p, EVg + size_t(li) * kNF2 * nc, D.rec_a, D.rec_b,
+                                     D.rec_c, acc);
             // fields 0..2: H_d; 3..5: B_d
             const double r2 = xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2];
             for (int d = 0; d < 3; ++d) u[d] = C1 * ih * (double(acc[d]) - r2 * double(acc[3 + d]));
         } else {
+            eval_fields<T, NF, false, true>(T(xi[0]), T(xi[1]), T(xi[2]), p, EVg + size_t(li) * kNE * nc, nc, D.rec_a,
+                                            D.rec_b, D.rec_c, acc);
             // fields 0..2: the folded value terms; 3..11: gradients dL_k / dx_d at 3 + 3k + d
             for (int d = 0; d < 3; ++d) {
                 double v = double(acc[d]);
@@ -744,9 +920,9 @@ static size_t smem_p2x(int p, int threads) {
            sizeof(T) * 4 * chunk + 64;
 }
 template <typename T>
-static size_t smem_far(int p) {
-    int st = ncoef(p + 2);
-    return sizeof(T) * tab_floats<T>(p) + sizeof(cpx<T>) * (kNE * st + 4 * st + kSets * ncoef(p)) + 64;
+static size_t smem_far(int p, int groups) {
+    return sizeof(T) * far_tab_floats<T>(p) +
+           sizeof(cpx<T>) * groups * (kSets * ncoef(p) + 2 * ncoef(p + 1) + 6 * ncoef(p + 2));
 }
 template <typename T>
 static size_t smem_lap(int p) {
@@ -806,7 +982,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     prof_mark(t, RPY_STAGE_EVAL, st);
     if (ufar) {
         cpx<T> *EVg = static_cast<cpx<T> *>(t.EVg);
-        size_t sp2 = sizeof(T) * (((6 * ncoef(p + 2) + 1) & ~1)) + sizeof(cpx<T>) * 2 * kSets * nc + 64;
+        const size_t sp2 = sizeof(T) * prep_tab_floats<T>(p) + sizeof(cpx<T>) * (kSets * nc + kSets * ncoef(p + 1));
         RPY_TRY(set_smem(k_eval_prep<T>, sp2));
         // one expansion per velocity component unless the per-potential form is asked for
         const int per_comp = (t.params.flags & RPY_FLAG_EVAL_PER_POTENTIAL) ? 0 : 1;
@@ -821,11 +997,16 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
             k_eval_apply<T, kNF><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, side, t.b_level,
                                                      t.b_sys, t.pos, sc, EVg, ufar);
         RPY_LAUNCHED(1);
-        size_t sf = smem_far<T>(p);
-        RPY_TRY(set_smem(k_far_eval<T>, sf));
-        k_far_eval<T><<<t.nleaf, 64, sf, st>>>(t.leaves, D, t.b_begin, t.b_end, t.b_center, side, t.b_level,
-                                                t.b_sys, t.w_off, t.w_idx, t.pos, t.n, sc, L, M, ufar, rb);
-        RPY_LAUNCHED(1);
+        if (t.n_w > 0) {
+            // source boxes per round: as many groups as fit a block of an average leaf, in 64 KB
+            int groups = std::min(kFarGroups, std::max(1, int(int64_t(kFarThreads) * t.nleaf / t.n)));
+            while (groups > 1 && smem_far<T>(p, groups) > 64 * 1024) --groups;
+            const size_t sf = smem_far<T>(p, groups);
+            RPY_TRY(set_smem(k_far_eval<T>, sf));
+            k_far_eval<T><<<t.n_items, kFarThreads, sf, st>>>(t.u_items, D, t.b_center, t.b_level, t.b_sys, t.w_off,
+                                                              t.w_idx, t.pos, t.n, sc, M, ufar, rb, groups);
+            RPY_LAUNCHED(1);
+        }
         RPY_CHECK(cudaGetLastError());
     }
     if (lapout) {

@@ -305,7 +305,7 @@ struct Tree {
     // expansions and matvec workspace
     void *M = nullptr, *L = nullptr, *Xo = nullptr, *Xi = nullptr;
     int x_frames = 3;                 // plane-wave frames per pass (3 or 1)
-    void *EVg = nullptr;              // [nleaf][18][ncoef(p)] derived local expansions of Eq. (2.8)
+    void *EVg = nullptr;              // [nleaf][ncoef(p)][6] evaluated local expansions of Eq. (2.8) ([18][ncoef(p)] per potential)
     double *fs = nullptr;             // sorted forces SoA [3][n]
     float *p32 = nullptr;             // FP32 form: sorted positions as hi + lo floats, [6][n] (x,y,z hi; x,y,z lo)
     float *f32 = nullptr;             // FP32 form: sorted forces [3][n]

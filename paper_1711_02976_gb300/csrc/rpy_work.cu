@@ -218,8 +218,8 @@ extern "C" int rpy_tree_work(rpy_tree h, double *flops, double *bytes, int n) {
         B[RPY_STAGE_X2X] = 2 * n2 * 6.0 * 4 * S * ce;
         // L2P with Eq. (2.8) at the beads, the derived expansions per leaf, M2P of large W boxes
         F[RPY_STAGE_EVAL] = bead2 * (harm + 6 * 2 * 2.0 * nc) + leaf2 * 18 * nc * 8.0 +
-                            wpairs * (harm2 + 18 * 2 * 2.0 * nc2);
-        B[RPY_STAGE_EVAL] = leaf2 * (4 * nc + 2 * 18 * nc) * ce + bead2 * 48;
+                            wpairs * (harm2 + 6 * 2 * 2.0 * nc2);
+        B[RPY_STAGE_EVAL] = leaf2 * (4 * nc + 2 * 6 * nc) * ce + bead2 * 48;
     }
     for (int k = 0; k < n; ++k) {
         flops[k] = k < RPY_NUM_STAGES ? F[k] : 0.0;

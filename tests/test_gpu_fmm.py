@@ -454,6 +454,22 @@ def test_both_precision_forms_agree_at_every_order(order, n, leaf_cap):
     assert oracle.rel_l2(u[rp.RPY_FP64, 3], u[rp.RPY_FP64, 6]) < 3e-3
 
 
+@pytest.mark.parametrize("precision,digits,order", [(rp.RPY_FP64, 9, 0), (rp.RPY_FP64, 3, 28), (rp.RPY_FP32, 6, 0),
+                                                    (rp.RPY_FP32, 3, 5)])
+@pytest.mark.parametrize("leaf_cap", [2, 20, 128, 400])
+def test_multipoles_at_the_beads_of_w_lists(leaf_cap, precision, digits, order):
+    """All W boxes by multipoles at the beads of small leaves (several boxes a round), of leaves with more beads than a
+    block has threads, and of several work items.  The sum keeps the accuracy of the setting."""
+    rng = np.random.default_rng(leaf_cap)
+    # sparse beads around a dense clump: leaves of up to leaf_cap beads next to much smaller boxes
+    pos = np.concatenate([rng.random((2700, 3)), 0.375 + 0.02 * rng.standard_normal((1500, 3))])
+    f, a = rng.standard_normal(pos.shape), 1e-4
+    s = 6 * math.pi * a
+    u, t = matvec(pos, f, a, s, digits, leaf_cap=leaf_cap, precision=precision, order_p=order, direct_w=-1, direct_x=-1)
+    assert len(rp.rpy_tree_export(t, "w_idx")) > 0
+    assert oracle.rel_l2(u, oracle.rpy_direct(pos, f, a, s)) < 10.0 ** -digits
+
+
 # ---------------------------------------------------------------- edge cases
 
 @pytest.mark.parametrize("precision", [rp.RPY_FP64, rp.RPY_FP32])
