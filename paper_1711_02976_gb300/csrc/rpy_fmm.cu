@@ -44,34 +44,80 @@
 namespace rpy {
 
 // ---------------------------------------------------------------- harmonics, several points per warp
-// Solid harmonics (regular, or irregular when IRREG) of one point into out[],
-// columns c and P - c of it.
+__device__ __forceinline__ cpx<dfl> from_lane(unsigned mask, cpx<dfl> v, int lane) {
+    return mk(dfl(__shfl_sync(mask, v.x.h, lane), __shfl_sync(mask, v.x.l, lane)),
+              dfl(__shfl_sync(mask, v.y.h, lane), __shfl_sync(mask, v.y.l, lane)));
+}
+
+// Solid harmonics (regular, or irregular when IRREG) of one point into out[], by harm_lanes(P) consecutive lanes of
+// a warp, c = 0, 1, ... : columns c and P - c each.  All lanes of the warp come here; those without a point
+// (!act) store nothing.
+// Double-floats: w^c by binary powers, w^(P - c) as w^(P - H) w^(H - c), H = P / 2, from the lane of column H - c, and
+// the two columns as one sequence of P + 2 steps.  FP32: each lane raises w to both powers and runs its columns
+// one after the other (1.5 P steps in the warp), for the shuffles and the longer loop body cost more there
+// than the products they save.  Both ways in both forms, P2M: 1M mixed FP64 1.70 against 1.82 ms, 15M cube FP64 4.65
+// against 5.12, 1M mixed FP32 0.52 against 0.39, 15M cube FP32 2.43 against 1.85.
 template <typename T, bool IRREG>
-__device__ void lane_harmonics(T x, T y, T z, int P, const T *ra, const T *rb, const T *cm, cpx<T> *out, int c) {
+__device__ void lane_harmonics(T x, T y, T z, int P, const T *ra, const T *rb, const T *cm, cpx<T> *out, int c,
+                               bool act) {
     const T r2 = fma(z, z, fma(y, y, x * x));
     const T ir2 = IRREG ? T(1) / r2 : T(0);
     const cpx<T> w = IRREG ? mk(x * ir2, y * ir2) : mk(x, y);
     const T d0 = IRREG ? sqrt(ir2) : T(1);
     const T zz = IRREG ? z * ir2 : z;   // factor of the a-coefficients
     const T rr = IRREG ? ir2 : r2;      // factor of the b-coefficients
-    for (int h = 0; h < 2; ++h) {
-        const int m = h ? P - c : c;
-        if (h && m == c) break;
-        cpx<T> pw = mk<T>(1, 0), base = w;   // w^m by binary powering
-        for (int e = m; e; e >>= 1) {
-            if (e & 1) pw = pw * base;
+    if constexpr (kIsDf<T>) {
+        const int H = P / 2, lane0 = (threadIdx.x & 31) - c;
+        cpx<T> pw = c & 1 ? w : mk<T>(1, 0), base = w;
+        for (int e = 2; e <= H; e <<= 1) {
             base = base * base;
+            const cpx<T> t = pw * base;
+            if (c & e) pw = t;
         }
-        const T s0 = cm[m] * d0;
+        cpx<T> q = from_lane(0xffffffffu, pw, (lane0 + H) & 31);   // w^H
+        if (P & 1) q = q * w;
+        q = q * from_lane(0xffffffffu, pw, (lane0 + H - c) & 31);
+        if (!act) return;
+        int m = c, n = c;
+        const T s0 = cm[c] * d0, s1 = cm[P - c] * d0;
         cpx<T> p1 = mk(s0 * pw.x, s0 * pw.y), p2 = mk<T>(0, 0);
-        out[tri(m, m)] = p1;
-        for (int n = m + 1; n <= P; ++n) {
-            const int i = tri(n, m);
-            const T A = ra[i] * zz, B = rb[i] * rr;
-            const cpx<T> cn = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
-            out[i] = cn;
-            p2 = p1;
-            p1 = cn;
+        q = mk(s1 * q.x, s1 * q.y);
+        for (int left = 2 * c == P ? P - c + 1 : P + 2; left > 0; --left) {
+            out[tri(n, m)] = p1;
+            if (n == P) {
+                m = n = P - c;
+                p1 = q;
+                p2 = mk<T>(0, 0);
+            } else {
+                ++n;
+                const int i = tri(n, m);
+                const T A = ra[i] * zz, B = rb[i] * rr;
+                const cpx<T> cn = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
+                p2 = p1;
+                p1 = cn;
+            }
+        }
+    } else {
+        if (!act) return;
+        for (int h = 0; h < 2; ++h) {
+            const int m = h ? P - c : c;
+            if (h && m == c) break;
+            cpx<T> pw = mk<T>(1, 0), base = w;   // w^m by binary powering
+            for (int e = m; e; e >>= 1) {
+                if (e & 1) pw = pw * base;
+                base = base * base;
+            }
+            const T s0 = cm[m] * d0;
+            cpx<T> p1 = mk(s0 * pw.x, s0 * pw.y), p2 = mk<T>(0, 0);
+            out[tri(m, m)] = p1;
+            for (int n = m + 1; n <= P; ++n) {
+                const int i = tri(n, m);
+                const T A = ra[i] * zz, B = rb[i] * rr;
+                const cpx<T> cn = mk(mul_diff(A, p1.x, B, p2.x), mul_diff(A, p1.y, B, p2.y));
+                out[i] = cn;
+                p2 = p1;
+                p1 = cn;
+            }
         }
     }
 }
@@ -308,19 +354,91 @@ __host__ __device__ inline int tab_floats(int p) {   // recurrences + ladders, r
 
 // ---------------------------------------------------------------- P2M / P2L
 
-// Beads per chunk of P2M / P2L: one round of harmonics, (warps x points per warp).
-__host__ __device__ inline int p2x_chunk(int p, int threads) { return (threads / 32) * (32 / harm_lanes(p)); }
+// Two charge sets of one value in a packed operand: float2 in FP32, df2 in double-floats.
+template <typename T> struct Pair;
+template <> struct Pair<float> { using V = float2; };
+template <> struct Pair<dfl> { using V = df2; };
+__device__ __forceinline__ float2 pair2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ df2 pair2(dfl a, dfl b) { return df2{make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
+__device__ __forceinline__ float first(float2 v) { return v.x; }
+__device__ __forceinline__ float second(float2 v) { return v.y; }
+__device__ __forceinline__ dfl first(df2 v) { return dfl(v.h.x, v.l.x); }
+__device__ __forceinline__ dfl second(df2 v) { return dfl(v.h.y, v.l.y); }
+__device__ __forceinline__ void macc2(float2 &s, float2 a, float2 b) { s = fma2(a, b, s); }
+__device__ __forceinline__ void macc2(df2 &s, df2 a, df2 b) { macc(s, a, b); }
+__device__ __forceinline__ void add_comp(float2 &s, float2 &c, float2 v) {   // s - c += v (Kahan)
+    const float2 y = sub2(v, c), t = add2(s, y);
+    c = sub2(sub2(t, s), y);
+    s = t;
+}
 
+// Running sums of one coefficient for the four charge sets: re[h], im[h] of sets 2h and 2h + 1; in FP32 with the
+// compensation of each (double-floats are only normalised).
+template <typename T>
+struct Sum4 {
+    typename Pair<T>::V v[4], c[sizeof(T) == 4 ? 4 : 1];
+    __device__ void clear() {
+        const auto z = pair2(T(0), T(0));
+        for (auto &x : v) x = z;
+        for (auto &x : c) x = z;
+    }
+    __device__ void add(const typename Pair<T>::V *u) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if constexpr (sizeof(T) == 4) add_comp(v[k], c[k], u[k]);
+            else v[k] = renorm(sum_raw(v[k], u[k]));
+        }
+    }
+    __device__ void join(const Sum4 &o) {
+        add(o.v);
+        if constexpr (sizeof(T) == 4) {
+            float2 m[4];
+            for (int k = 0; k < 4; ++k) m[k] = neg2(o.c[k]);
+            add(m);
+        }
+    }
+};
+
+// Threads of a P2M / P2L block: G = threads / ncoef groups of one thread per coefficient.  At low orders two warps, for
+// the groups' joining costs as much as their sums (P2M, p = 6, 15M cube: FP64 4.10 ms, FP32 1.49 ms; four warps 4.65 and
+// 1.86); four where there are too few boxes to fill the chip (585 boxes: 15 us against 17).
+inline int p2x_threads(int p, int nbox) {
+    const int nc = ncoef(p);
+    return (std::max(1, (nbox < 1024 ? 128 : 64) / nc) * nc + 31) / 32 * 32;
+}
+// Beads per chunk: one round of harmonics (warps x points per warp) in at most kP2xBuf bytes (9 digits, p = 25, P2M: 32 KB
+// 1.78 ms, 64 KB 1.24, 96 KB 1.10).
+constexpr int kP2xStage = 128;   // beads staged at a time: coordinates and charges
+constexpr int kP2xBuf = 96 * 1024;
+template <typename T>
+__host__ __device__ inline int p2x_chunk(int p, int threads) {
+    const int most = kP2xBuf / int(ncoef(p) * sizeof(cpx<T>)), one = (threads / 32) * (32 / harm_lanes(p));
+    return one < most ? one : most;
+}
+template <typename T>
+__host__ __device__ inline int p2x_buf(int p, int threads) {   // harmonics of a chunk, later the groups' sums
+    const int y = p2x_chunk<T>(p, threads) * ncoef(p) * int(sizeof(cpx<T>)), r = threads * int(sizeof(Sum4<T>));
+    return ((y > r ? y : r) + 15) & ~15;
+}
+
+// Bound by the harmonics (a chain per lane) and, at low orders, by the synchronised phases of each leaf; in FP32 also by
+// the FP64 coordinates, taken once per bead and box: every lane of a point's harmonics took them before.  A
+// coefficient's four sums stay in registers and share each loaded harmonic; they stood in shared memory, a thread per
+// coefficient and set, with two loads for every two products.  P2M and P2L before and now: 1M mixed FP64 1.97 -> 1.70
+// and 2.06 -> 1.95 ms, FP32 0.49 -> 0.39 and 0.89 -> 0.73; 200k at 9 digits 1.21 -> 0.94 and 1.16 -> 0.83; 15M cube P2M
+// FP64 5.05 -> 4.10 and FP32 2.02 -> 1.49; 256 systems FP32 2.57 -> 2.05 and 2.37 -> 2.02.
 // MODE 0: P2M over the leaf's own beads (multipole about its centre)
 // MODE 1: P2L over the beads of every box in X(b) (local about b's centre)
 // The fourth charge q4 = F . (r - o) takes its origin o at the expansion's own
 // centre when rb is set (box origin), else at the system's cube centre.
 template <typename T, int MODE>
-__global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int *end, const double *ctr,
-                      const double *side, const int *lvl, const int *leaf, const int *bsys, const int *xoff,
-                      const int *xidx, const double *pos, const double *fs, const double *lapq, int64_t n,
-                      SysConst sc, cpx<T> *out, int rb) {
-    const int kChunkB = p2x_chunk(D.p, blockDim.x);
+__global__ void __launch_bounds__(512) k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int *end,
+                                             const double *ctr, const double *side, const int *lvl, const int *leaf,
+                                             const int *bsys, const int *xoff, const int *xidx, const double *pos,
+                                             const double *fs, const double *lapq, int64_t n, SysConst sc, cpx<T> *out,
+                                             int rb) {
+    using V = typename Pair<T>::V;
+    const int chunk = p2x_chunk<T>(D.p, blockDim.x);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int b = b0 + blockIdx.x;
     if (b >= b0 + nb) return;
@@ -329,13 +447,10 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
     int nsrc = MODE == 0 ? 1 : xoff[b + 1] - xoff[b];
     if (nsrc == 0) return;
     const int p = D.p, nc = ncoef(p);
-    T *smr = reinterpret_cast<T *>(smem_raw);
-    Rec<T> R = load_rec(D, smr);
-    cpx<T> *ybuf = reinterpret_cast<cpx<T> *>(smr + ((rec_floats<T>(p) + 1) & ~1));
-    cpx<T> *acc = ybuf + kChunkB * nc;
-    cpx<T> *cmp = acc + kSets * nc;   // FP32: compensation of the running sums
-    T *q = reinterpret_cast<T *>(cmp + kSets * nc);
-    for (int i = threadIdx.x; i < kSets * nc; i += blockDim.x) acc[i] = cmp[i] = mk<T>(0, 0);
+    cpx<T> *ybuf = reinterpret_cast<cpx<T> *>(smem_raw);
+    V *q = reinterpret_cast<V *>(smem_raw + p2x_buf<T>(p, blockDim.x));   // [bead][2]
+    T *X = reinterpret_cast<T *>(q + 2 * kP2xStage);   // coordinates in box sides, [3][bead]
+    Rec<T> R = load_rec(D, X + 3 * kP2xStage);
     int sy = bsys[b];
     double cx = ctr[3 * b], cy = ctr[3 * b + 1], cz = ctr[3 * b + 2];
     const double c0x = rb ? cx : sc.cube[4 * sy], c0y = rb ? cy : sc.cube[4 * sy + 1],
@@ -353,83 +468,99 @@ __global__ void k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int 
     int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     // harmonics: hG points per warp, lane -> (point hg, column pair hc)
     const int hL = harm_lanes(p), hG = 32 / hL, hg = (threadIdx.x & 31) / hL, hc = (threadIdx.x & 31) - hg * hL;
+    // sums: this thread's coefficient i, and every G-th bead of a chunk from g on
+    const int G = blockDim.x / nc, g = threadIdx.x / nc, i = threadIdx.x - g * nc;
+    Sum4<T> sum;
+    sum.clear();
     __syncthreads();
     for (int si = 0; si < nsrc; ++si) {
         int src = MODE == 0 ? b : xidx[xoff[b] + si];
-        int j0 = beg[src], j1 = end[src];
-        for (int jc = j0; jc < j1; jc += kChunkB) {
-            int cnt = min(kChunkB, j1 - jc);
-            for (int t0 = warp * hG; t0 < cnt; t0 += nwarp * hG) {
-                const int t = t0 + hg;
-                if (hg < hG && t < cnt) {
-                    int j = jc + t;
-                    T ex, ey, ez;
-                    if constexpr (kIsDf<T>) {
-                        ex = coord_diff(sc.p3, n, j, 0, c3) * ihs;
-                        ey = coord_diff(sc.p3, n, j, 1, c3) * ihs;
-                        ez = coord_diff(sc.p3, n, j, 2, c3) * ihs;
-                    } else {
-                        ex = T((pos[j] - cx) * ih), ey = T((pos[n + j] - cy) * ih), ez = T((pos[2 * n + j] - cz) * ih);
-                    }
-                    lane_harmonics<T, MODE == 1>(ex, ey, ez, p, R.a, R.b, R.cm, ybuf + t * nc, hc);
+        for (int js = beg[src], j1 = end[src]; js < j1; js += kP2xStage) {
+            const int ns = min(kP2xStage, j1 - js);
+            for (int t = threadIdx.x; t < ns; t += blockDim.x) {
+                int j = js + t;
+                if constexpr (kIsDf<T>) {
+                    for (int a = 0; a < 3; ++a) X[a * kP2xStage + t] = coord_diff(sc.p3, n, j, a, c3) * ihs;
+                } else {
+                    X[t] = T((pos[j] - cx) * ih);
+                    X[kP2xStage + t] = T((pos[n + j] - cy) * ih);
+                    X[2 * kP2xStage + t] = T((pos[2 * n + j] - cz) * ih);
                 }
-            }
-            for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-                int j = jc + t;
+                T c[kSets];
                 if (lapq) {
-                    for (int k = 0; k < kSets; ++k) q[4 * t + k] = T(kIsDf<T> ? qs * lapq[4 * j + k] : lapq[4 * j + k]);
+                    for (int k = 0; k < kSets; ++k) c[k] = T(kIsDf<T> ? qs * lapq[4 * j + k] : lapq[4 * j + k]);
                 } else if constexpr (kIsDf<T>) {
                     // scaled forces; q4 in the split units of length, its origin at the cube's or the box's centre
                     float o3[9];
                     for (int k = 0; k < 9; ++k) o3[k] = rb ? c3[k] : 0.f;
                     T q4 = T(0);
                     for (int a = 0; a < 3; ++a) {
-                        const T fa(sc.f2[(2 * a) * n + j], sc.f2[(2 * a + 1) * n + j]);
-                        q[4 * t + a] = fa;
-                        macc(q4, fa, coord_diff(sc.p3, n, j, a, o3));
+                        c[a] = T(sc.f2[(2 * a) * n + j], sc.f2[(2 * a + 1) * n + j]);
+                        macc(q4, c[a], coord_diff(sc.p3, n, j, a, o3));
                     }
-                    q[4 * t + 3] = closed(q4);
+                    c[3] = closed(q4);
                 } else {
                     double fx = fs[j], fy = fs[n + j], fz = fs[2 * n + j];
-                    q[4 * t] = T(fx);
-                    q[4 * t + 1] = T(fy);
-                    q[4 * t + 2] = T(fz);
-                    q[4 * t + 3] = T(fx * (pos[j] - c0x) + fy * (pos[n + j] - c0y) + fz * (pos[2 * n + j] - c0z));
+                    c[0] = T(fx);
+                    c[1] = T(fy);
+                    c[2] = T(fz);
+                    c[3] = T(fx * (pos[j] - c0x) + fy * (pos[n + j] - c0y) + fz * (pos[2 * n + j] - c0z));
                 }
+                q[2 * t] = pair2(c[0], c[1]);
+                q[2 * t + 1] = pair2(c[2], c[3]);
             }
             __syncthreads();
-            for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-                int k = e / nc, i = e - k * nc;
-                cpx<T> a = sizeof(T) == 4 ? mk<T>(0, 0) : acc[e];
-                for (int t = 0; t < cnt; ++t) {
-                    cpx<T> yv = ybuf[t * nc + i];
-                    T qq = q[4 * t + k];
-                    macc(a.x, qq, yv.x);
-                    macc(a.y, -qq, yv.y);   // conj
+            for (int jc = 0; jc < ns; jc += chunk) {
+                const int cnt = min(chunk, ns - jc);
+                for (int t0 = warp * hG; t0 < cnt; t0 += nwarp * hG) {
+                    const int t = t0 + hg;
+                    const bool act = hg < hG && t < cnt;
+                    const T *x = X + jc + (act ? t : 0);
+                    lane_harmonics<T, MODE == 1>(x[0], x[kP2xStage], x[2 * kP2xStage], p, R.a, R.b, R.cm, ybuf + t * nc, hc,
+                                                 act);
                 }
-                if constexpr (sizeof(T) == 4) {
-                    // a leaf (or an X-list source) may hold hundreds to thousands of beads: the
+                __syncthreads();
+                if (g < G) {
+                    const V z = pair2(T(0), T(0));
+                    V u[4] = {z, z, z, z};
+                    for (int t = g; t < cnt; t += G) {
+                        const cpx<T> yv = ybuf[t * nc + i];
+                        const V re = pair2(yv.x, yv.x), im = pair2(-yv.y, -yv.y);   // conj
+    #pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const V c = q[2 * (jc + t) + h];
+                            macc2(u[2 * h], c, re);
+                            macc2(u[2 * h + 1], c, im);
+                        }
+                    }
+                    // a leaf (or an X-list source) may hold hundreds to thousands of beads: in FP32 the
                     // chunk's plain sum enters the running sum by compensated (Kahan) addition
-                    cpx<T> sum = acc[e], c = cmp[e];
-                    const T yx = a.x - c.x, tx = sum.x + yx;
-                    c.x = (tx - sum.x) - yx;
-                    sum.x = tx;
-                    const T yy = a.y - c.y, ty = sum.y + yy;
-                    c.y = (ty - sum.y) - yy;
-                    sum.y = ty;
-                    acc[e] = sum;
-                    cmp[e] = c;
-                } else {
-                    acc[e] = mk(closed(a.x), closed(a.y));
+                    sum.add(u);
                 }
+                __syncthreads();
             }
-            __syncthreads();
         }
     }
-    cpx<T> *o = out + size_t(b) * kSets * nc;
-    for (int e = threadIdx.x; e < kSets * nc; e += blockDim.x) {
-        if (MODE == 0) o[e] = acc[e];
-        else o[e] += acc[e];
+    if (G > 1) {
+        Sum4<T> *red = reinterpret_cast<Sum4<T> *>(smem_raw);
+        if (g > 0 && g < G) red[threadIdx.x] = sum;
+        __syncthreads();
+        if (g == 0)
+            for (int h = 1; h < G; ++h) sum.join(red[h * nc + i]);
+    }
+    if (g > 0) return;
+    cpx<T> *o = out + size_t(b) * kSets * nc + i;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const cpx<T> a = mk(first(sum.v[2 * h]), first(sum.v[2 * h + 1])),
+                     c = mk(second(sum.v[2 * h]), second(sum.v[2 * h + 1]));
+        if (MODE == 0) {
+            o[2 * h * nc] = a;
+            o[(2 * h + 1) * nc] = c;
+        } else {
+            o[2 * h * nc] += a;
+            o[(2 * h + 1) * nc] += c;
+        }
     }
 }
 
@@ -915,9 +1046,7 @@ int raise_smem(const void *kernel, size_t bytes) {
 
 template <typename T>
 static size_t smem_p2x(int p, int threads) {
-    const int nc = ncoef(p), chunk = p2x_chunk(p, threads);
-    return sizeof(T) * ((rec_floats<T>(p) + 1) & ~1) + sizeof(cpx<T>) * (chunk * nc + 2 * kSets * nc) +
-           sizeof(T) * 4 * chunk + 64;
+    return size_t(p2x_buf<T>(p, threads)) + sizeof(T) * (7 * kP2xStage + rec_floats<T>(p));
 }
 template <typename T>
 static size_t smem_far(int p, int groups) {
@@ -956,10 +1085,11 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     // box sides in the units of the expansions' lengths
     const double *side = kIsDf<T> ? t.side_u : t.b_side;
     // upward pass
-    size_t sp = smem_p2x<T>(p, 128);
+    const int tp = p2x_threads(p, n2);
+    const size_t sp = smem_p2x<T>(p, tp);
     RPY_TRY(set_smem(k_p2x<T, 0>, sp));
     RPY_TRY(set_smem(k_p2x<T, 1>, sp));
-    k_p2x<T, 0><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
+    k_p2x<T, 0><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
                                      t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, M, rb);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
@@ -972,7 +1102,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     RPY_TRY(run_waves_t(t, D, M, L, rb, st));
     // X list
     prof_mark(t, RPY_STAGE_P2L, st);
-    k_p2x<T, 1><<<n2, 128, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
+    k_p2x<T, 1><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
                                      t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, L, rb);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());

@@ -459,7 +459,8 @@ def test_both_precision_forms_agree_at_every_order(order, n, leaf_cap):
 @pytest.mark.parametrize("leaf_cap", [2, 20, 128, 400])
 def test_multipoles_at_the_beads_of_w_lists(leaf_cap, precision, digits, order):
     """All W boxes by multipoles at the beads of small leaves (several boxes a round), of leaves with more beads than a
-    block has threads, and of several work items.  The sum keeps the accuracy of the setting."""
+    block has threads, and of several work items, and all X boxes by local expansions of those leaves' beads, staged in
+    several parts.  The sum keeps the accuracy of the setting."""
     rng = np.random.default_rng(leaf_cap)
     # sparse beads around a dense clump: leaves of up to leaf_cap beads next to much smaller boxes
     pos = np.concatenate([rng.random((2700, 3)), 0.375 + 0.02 * rng.standard_normal((1500, 3))])
