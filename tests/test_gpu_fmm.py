@@ -48,6 +48,20 @@ def test_permutation_and_keys_bit_exact():
     np.testing.assert_array_equal(rp.rpy_tree_export(t, "cube")[0], cube)
 
 
+@pytest.mark.parametrize("n", [2, 511, 512, 2049, 8191, 8192, 8193])
+def test_order_of_small_sorts_is_stable(n):
+    """Both sides of the size up to which one block sorts by itself, with runs of equal keys (beads at one point keep the
+    caller's order): order and keys bit-exact."""
+    rng = np.random.default_rng(n)
+    pos = rng.random((n, 3))
+    pos[rng.integers(0, n, n // 3)] = pos[0]
+    t = rp.rpy_tree_build(cuda_tensor(pos), n, 1e-6, 3, leaf_cap=40)
+    keys, _ = oracle.morton_keys(pos)
+    perm = oracle.stable_sort(keys)
+    np.testing.assert_array_equal(rp.rpy_tree_export(t, "perm"), perm)
+    np.testing.assert_array_equal(rp.rpy_tree_export(t, "keys"), keys[perm])
+
+
 def test_morton_keys_exact_on_and_near_grid_points():
     """Coordinates whose scaled value (x - origin) / side * 2^21 is an integer (a cube of side 1
     and coordinates on a 2^-12 grid), or lies within rounding of one (a cube of side 3, offsets of
