@@ -322,12 +322,11 @@ def run_ours(args, ws, rank, local, config=None, steps=None, warmup=None, profil
 
 
 # DRAM bytes per bead of the FP64 near-field launch (the merged pass over U lists and
-# direct substitutes, k_p2p), from one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum) of the 200,000-bead sphere + cube workload at 6 digits, FP64
-# (bench.py --config sphere200k_6digit_fp64): 10,747,648 B per launch.  The traffic is
-# the sources' positions and forces, so it grows with the bead count; it is reported
-# only for that kernel.
-P2P64_DRAM_BYTES_PER_BEAD = 10747648.0 / 200000.0
+# direct substitutes, k_p2p_df), from one ncu capture (dram__bytes_read.sum +
+# dram__bytes_write.sum) of a 200,000-bead sphere + cube system at 6 digits, FP64:
+# 18,009,344 B per launch.  The traffic is the sources' split positions and forces, so
+# it grows with the bead count; it is reported only for that kernel.
+P2P64_DRAM_BYTES_PER_BEAD = 18009344.0 / 200000.0
 
 
 def hbm_peak_gbs():
@@ -345,7 +344,9 @@ def roofline(precision, stage_ms, work, peaks, n_beads=None):
     work[stage] = (algorithmic FLOPs, algorithmic DRAM bytes) of one matvec on the tree
     (rpy_tree_work); the achieved rates divide them by the stage's CUDA-event time.  A
     stage's bound is the roof it is closer to: the FP64 or FP32 FMA peak measured on
-    this GPU (rpy_alu_peak) or the measured HBM copy bandwidth."""
+    this GPU (rpy_alu_peak) or the measured HBM copy bandwidth.  The FP64 form computes
+    its pairs and expansions in double-floats on the FP32 units, so its FP64 operations
+    over the FP64 peak exceed 1 where that is faster than the FP64 units could be."""
     hbm, hbm_src = hbm_peak_gbs()
     alu = peaks["fp64"] if precision == "fp64" else peaks["fp32"]
     per = {}
@@ -371,7 +372,7 @@ def roofline(precision, stage_ms, work, peaks, n_beads=None):
     out["traffic"] = None
     if top == "p2p" and precision == "fp64" and n_beads:
         out["traffic"] = round(P2P64_DRAM_BYTES_PER_BEAD * n_beads)
-        out["traffic_note"] = ("dram__bytes_read.sum + dram__bytes_write.sum of k_p2p per bead from an ncu capture "
+        out["traffic_note"] = ("dram__bytes_read.sum + dram__bytes_write.sum of k_p2p_df per bead from an ncu capture "
                                "of the 200k-bead sphere (6 digits, FP64), scaled by bead count")
     out["stages"] = per
     return out

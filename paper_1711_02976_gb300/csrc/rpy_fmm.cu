@@ -9,24 +9,24 @@
 // FP64 form, whose kernels were bound by the FP64 pipe (91 to 95% busy) at 64 times the cost of an FP32
 // operation; a multiply-add is 12 FP32 operations in dfl.  Lengths are in units of a power of two at the root
 // cube's side and forces in units of each system's largest (SysConst), so that every value lies well
-// inside the FP32 exponent range.  Measured, matvec of the 1M-bead sphere and cube at 6 digits (ms), FP64 -> dfl ->
-// dfl with packed plane waves: 104 -> 45.5 -> 38.1 (M2X 23.4 -> 8.8 -> 5.4, X2L 20.1 -> 8.9 -> 7.4, X2X 11.9 -> 5.4 ->
-// 3.7, L2P and M2P 16.6 -> 4.8, P2M and P2L 14.5 -> 4.0).  The velocities of whole matvecs move by
+// inside the FP32 exponent range.  Measured, matvec of the 1M-bead sphere and cube at 6 digits without its near field
+// (ms), FP64 -> dfl -> now: 95 -> 37 -> 25.5 (M2X 23.4 -> 8.8 -> 5.4, X2L 20.1 -> 8.9 -> 7.3, X2X 11.9 -> 5.4 -> 3.6, L2P
+// and M2P 16.6 -> 4.8 -> 2.4, P2M and P2L 14.5 -> 4.0 -> 3.65).  The velocities of whole matvecs move by
 // 1e-14 ... 1.2e-13; the error of the expansions is 1e-10 at 9 digits.
 //
 // Kernels, in launch order:
-//   k_p2m      S->M   leaves: M_n^m = sum_j q_j conj(y_n^m(eta_j))
-//   k_m2m_child, k_m2m_sum  M->M   per child: rotate to the shift axis, z-shift, rotate back;
-//                      per parent: add the children's shares in octant order
+//   k_p2x<0>   S->M   leaves: M_n^m = sum_j q_j conj(y_n^m(eta_j))
+//   k_m2m, k_m2m_cluster  M->M   per child: rotate to the shift axis, z-shift, rotate back;
+//                      per parent: add the children's shares in octant order (rpy_shift.cu)
 //   k_m2x      M->I   rotate into the frame of each axis, outgoing plane waves
 //                     W_kj = (w_k/M_k) sum_{n,m} M_n^m i^|m| lambda_k^n e^{i m a_kj} / sqrt((n-|m|)!(n+|m|)!)
 //   k_x2x      I->I   merge-and-shift: per parent and direction, sources are
 //                     shifted to the parent centre and summed per group of
 //                     targets they serve, then shifted once to each child
 //   k_x2l      I->L   L_n^m = i^|m| sum_k (-lambda_k)^n / sqrt(...) sum_j I_kj e^{-i m a_kj},
-//                     rotated back to the world frame
-//   k_p2l      S->L   X list
-//   k_l2l_rot  L->L   the same for locals, level by level downward
+//                     rotated back to the world frame (the three: rpy_waves.cu)
+//   k_p2x<1>   S->L   X list
+//   k_l2l      L->L   the same for locals, level by level downward (rpy_shift.cu)
 //   k_eval_prep, k_eval_apply  L->T   L2P: the gradients and Hessians of Theorems 1-2 formed as derivative
 //                     expansions per leaf, combined by Eq. (2.8):
 //                     u = C1 [L1 L2 L3] - C1 sum_k x_k grad L_k + C1 grad L4 - C2 grad L_C,

@@ -20,11 +20,10 @@
 // than 2^-24 of the root cube's side, leaves below level 17 and systems whose
 // lengths or forces lie outside the FP32 exponent range take every operation in FP64 (near64).
 // FP32 form (precision setting, k_p2p32): positions relative to the target
-// leaf centre in FP32; every thread carries two targets as the two lanes of
-// packed FP32x2 operations and takes two staged sources per iteration; an
+// leaf centre in FP32; every thread carries one target and takes two staged sources in
+// the two lanes of packed FP32x2 operations, four sources per iteration; an
 // iteration whose pairs are all far (across the warp) evaluates the far branch
-// alone on the packed pairs, any other evaluates both branches per target with
-// selects; accumulation is Kahan-compensated across blocks of kP32Block sources;
+// alone, any other evaluates both branches with selects; accumulation is Kahan-compensated across blocks of kP32Block sources;
 // pairs closer than 1e-3 a (where the FP32 difference of coordinates loses the
 // direction) are recomputed in FP64 from the FP64 positions.
 #include <cmath>
