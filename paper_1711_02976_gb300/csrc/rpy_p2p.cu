@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int4 *items, con
             for (int e = threadIdx.x; e < 2 * nP; e += kP32Threads) {
                 float *w = reinterpret_cast<float *>(sS + 3 * (e >> 1)) + (e & 1);
                 float px = 1e15f, py = 1e15f, pz = 1e15f, fx = 0.f, fy = 0.f, fz = 0.f;
-                int j = -1;   // an odd last source gets a far partner without force
+                int j = -1;   // an odd last source gets a partner without force, not far at every scale of lengths
                 if (e < nS) {
                     int q = c0 + e, lo = 0, hi = L;   // box: lpre[lo] <= q < lpre[lo + 1]
                     while (hi - lo > 1) {
@@ -800,13 +800,15 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int4 *items, con
                 for (int eb = g; eb < nP; eb += kP32Block * G) {
                     const int ee = min(nP, eb + kP32Block * G);
                     float2 AX = make_float2(0.f, 0.f), AY = AX, AZ = AX;   // lane sums of this block
-                    // pairs at most 1e-3 a apart other than the self pair: to FP64
+                    // pairs at most 1e-3 a apart other than the self pair and the partner (j < 0): to FP64
                     auto close = [&](int e, float2 R2) {
-                        for (int h = 0; h < 2; ++h)
-                            if (!((h ? R2.y : R2.x) > k.tiny2) && sJ[2 * e + h] != i) {
+                        for (int h = 0; h < 2; ++h) {
+                            const int j = sJ[2 * e + h];
+                            if (!((h ? R2.y : R2.x) > k.tiny2) && j >= 0 && j != i) {
                                 const int q = atomicAdd(&sQn[0], 1);
                                 if (q < kP32Queue) sQ[q] = (threadIdx.x << 11) | (2 * e + h);
                             }
+                        }
                     };
                     // both branches with selects
                     auto slow = [&](int e, float2 DX, float2 DY, float2 DZ, float2 R2, float2 FX, float2 FY, float2 FZ) {
@@ -877,7 +879,8 @@ __global__ void __launch_bounds__(kP32Threads, 4) k_p2p32(const int4 *items, con
                             const float dx = xa + (h ? S0.y : S0.x), dy = ya + (h ? S0.w : S0.z), dz = za + (h ? S1.y : S1.x);
                             const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
                             const int jg = sJ[2 * e + h];
-                            if (!(r2 > k.tiny2) && jg != i) pair_tiny64(jg, i, a, co, pos, fs, n, &sD[3 * threadIdx.x]);
+                            if (!(r2 > k.tiny2) && jg >= 0 && jg != i)
+                                pair_tiny64(jg, i, a, co, pos, fs, n, &sD[3 * threadIdx.x]);
                         }
                     }
                 }
