@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kDfThreads, 2)
 #pragma unroll
                     for (int k = 0; k < 6; ++k) w[18 + 2 * k] = f2[k * n + j];
                     reinterpret_cast<int *>(w)[30] = j;
-                } else {   // an odd last source gets a partner outside the cube, without force
+                } else {   // an odd last source gets a partner without force, 3.5 units from every bead or more
 #pragma unroll
                     for (int k = 0; k < 15; ++k) w[2 * k] = k == 0 ? 4.f : 0.f;
                     reinterpret_cast<int *>(w)[30] = -1;
@@ -528,6 +528,8 @@ __global__ void __launch_bounds__(kDfThreads, 2)
                             df2 O1, O2;
                             pair_far(P, k23, T1, T2);
                             pair_overlap(P, pc, O1, O2);
+                            // far, then overlapping, then FP64 (lim = tiny where 2a is below the split's resolution:
+                            // a pair exactly there is far)
                             const bool fx = P.r2.h.x >= lim, fy = P.r2.h.y >= lim;
                             const bool ox = P.r2.h.x > tiny, oy = P.r2.h.y > tiny;
                             auto pick = [&](float2 far, float2 near) {
@@ -537,13 +539,14 @@ __global__ void __launch_bounds__(kDfThreads, 2)
                             T1.l = pick(T1.l, O1.l);
                             T2.h = pick(T2.h, O2.h);
                             T2.l = pick(T2.l, O2.l);
-                            if (!ox || !oy) {
+                            const bool tx = !fx && !ox, ty = !fy && !oy;
+                            if (tx || ty) {
                                 const int jx = __float_as_int(v7.z), jy = __float_as_int(v7.w);
-                                if (!ox && jx != i) {
+                                if (tx && jx != i) {
                                     pair_tiny_f64(jx, i, pc, pos, fs, n, tiny64);
                                     *any64 = 1;
                                 }
-                                if (!oy && jy != i) {
+                                if (ty && jy != i) {
                                     pair_tiny_f64(jy, i, pc, pos, fs, n, tiny64);
                                     *any64 = 1;
                                 }

@@ -287,6 +287,23 @@ def test_fp64_near_part_in_double_floats(name, n, leaf_cap):
         assert (np.abs(u[mem] - ref[mem]).max(axis=1) <= 2.0 ** -40 * mag).all(), name
 
 
+@pytest.mark.parametrize("delta", [-2.0 ** -40, -2.0 ** -53, 0.0, 2.0 ** -53, 2.0 ** -40])
+@pytest.mark.parametrize("a", [1e-9, 2.0 ** -25, 2.0 ** -24])
+@pytest.mark.parametrize("axis", [0, 2])
+def test_fp64_pair_at_the_resolution_of_the_split(axis, a, delta):
+    """Two beads 2^-24 of the unit of length apart along an axis, and one step to either side: the distance at which
+    FP64 takes over from the double-floats, and the smallest radii at which a pair there is a far one.  Such a
+    pair is counted once."""
+    pos = np.full((4, 3), 0.5)
+    pos[1, axis] += 2.0 ** -24 + delta
+    pos[2:] = (0.015625, 0.0625, 0.875), (0.984375, 0.875, 0.125)   # the cube's side lies in (1/2, 1): the unit is 1
+    f = np.random.default_rng(5).standard_normal((4, 3))
+    s = 6 * math.pi * a
+    u, t = matvec(pos, f, a, s, 3, leaf_cap=4, parts=rp.RPY_PART_NEAR)
+    assert 0.5 < rp.rpy_tree_export(t, "cube")[0, 3] < 1.0
+    np.testing.assert_allclose(u, oracle.rpy_direct(pos, f, a, s), rtol=0, atol=1e-13 * np.abs(f).max())
+
+
 @pytest.mark.parametrize("n", [128, 129, 141, 170, 171, 192, 193, 340, 385, 513])
 def test_near_items_of_one_leaf(n):
     """A leaf's beads fall into full work items and a rest, halved where that fills the block better; both
