@@ -92,9 +92,9 @@ typedef struct {
                          the size of the box's own moments; cube origin: one origin per system
                          (the bounding-cube centre), which leaves the far-field combination
                          grad L4 - sum_k x_k grad L_k of Eq. (2.8) to cancel terms of size
-                         |x - o| |grad L|.  Default: box origin for RPY_FP32 at 6 digits, cube
-                         origin for RPY_FP64 and at 3 digits (whose rounding stays far below
-                         the setting there); at most one of the two bits;
+                         |x - o| |grad L|.  Default: box origin for RPY_FP32 at 6 digits and for
+                         RPY_FP64 with quad 9 on trees of depth 10 and more, cube origin
+                         otherwise; at most one of the two bits;
                          bit 5 (RPY_FLAG_CARTESIAN): the polynomial far field that the paper's
                          Sec. 5 proposes for low accuracy: Cartesian Taylor expansions of total
                          degree order_p (default 8, at most 10) with a direct multipole-to-local

@@ -1059,6 +1059,14 @@ static size_t smem_lap(int p) {
     return sizeof(T) * tab_floats<T>(p) + sizeof(cpx<T>) * (13 * st + 3 * st + ncoef(p)) + 64;
 }
 
+// With one origin of q4 per system, Eq. (2.8) cancels terms of size |c - c0| |grad L|, which rounds like 2^level.
+// Double-floats, a cluster of 20,001 beads in a cube 2^0 ... 2^16 times its size, 9 digits, distance of the far field from
+// the same one in FP64: cube centre 2.0e-13 at depth 9, 6.3e-13 at 11, 5e-12 at 12, 6.4e-11 at 16, 1.5e-9 at 20 (its
+// truncation is 6e-10 ... 1.2e-9); box centres 1.5e-13 ... 1.9e-13 at every depth.  With the rules of fewer digits, which
+// truncate at 6e-8 of the far field and more, 1.5e-9 is lost in it, and X2X pays for the moves (k_x2x4; matvec of 200,001 beads,
+// depth 15, cube against box centres: 3 digits 7.5 against 10.8 ms, 6 digits 9.4 against 10.1, 9 digits 20.1 against 21.5).
+constexpr int kBoxOriginDepth = 10;
+
 template <typename T>
 int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *lapq, double *ufar, double *lapout,
               const SysConst &sc, cudaStream_t st) {
@@ -1074,14 +1082,15 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     }
     int b2 = t.level_off[2];
     int n2 = nbx - b2;
-    // origin of q4 (RPY charges only; the Laplace diagnostic takes its charges as given):
-    // each expansion's own box centre by default in the FP32 form at 6 digits, the cube
-    // centre otherwise (in the FP64 form, and at 3 digits, its rounding stays far below the setting)
+    // origin of q4 (RPY charges only; the Laplace diagnostic takes its charges as given): each expansion's own box
+    // centre by default in the FP32 form at 6 digits and in the FP64 form with the 9-digit plane waves on trees of
+    // depth kBoxOriginDepth and more, the cube centre otherwise
     const int fl = t.params.flags;
     const int rb = lapq ? 0
                         : (fl & RPY_FLAG_BOX_ORIGIN) ? 1
                         : (fl & RPY_FLAG_CUBE_ORIGIN) ? 0
-                        : (sizeof(T) == 4 && t.params.digits >= 6);
+                        : kIsDf<T> ? t.params.quad == 9 && t.nlevels - 1 >= kBoxOriginDepth
+                                   : t.params.digits >= 6;
     // box sides in the units of the expansions' lengths
     const double *side = kIsDf<T> ? t.side_u : t.b_side;
     // upward pass

@@ -975,6 +975,41 @@ def test_box_origin_equals_cube_origin_fp64(extra, direct):
     assert oracle.rel_l2(u1, u0) < 1e-12
 
 
+def _cluster_and_strays(n, k):
+    """A cube of beads 2^-k-1 wide, and two beads in opposite corners of the unit cube: a tree of about
+    k + log8(n / leaf_cap) levels."""
+    rng = np.random.default_rng(k)
+    pos = 0.3141 + (rng.random((n, 3)) - 0.5) * 2.0 ** (-k - 1)
+    pos[0], pos[1] = (0.999, 0.998, 0.997), (0.001, 0.002, 0.003)
+    return pos, rng.standard_normal((n, 3)), 1e-4 * 2.0 ** -k
+
+
+def test_fp64_9digit_cluster_in_a_deep_tree():
+    """A cluster 2^-16 of the cube wide: the far field keeps 9 digits of itself.  With one origin of q4 per
+    system its 48 bits lose 19 to the cancellation of Eq. (2.8) at this depth."""
+    pos, f, a = _cluster_and_strays(20001, 16)
+    s = 6 * math.pi * a
+    kw = dict(leaf_cap=60, order_p=27, direct_w=-1, direct_x=-1)
+    far, t0 = matvec(pos, f, a, s, 9, parts=rp.RPY_PART_FAR, **kw)
+    u, t = matvec(pos, f, a, s, 9, **kw)
+    assert rp.rpy_tree_stats(t)["depth"] >= 19
+    assert np.linalg.norm(u - oracle.rpy_direct(pos, f, a, s)) < 1e-9 * np.linalg.norm(far)
+
+
+@pytest.mark.parametrize("digits,quad", [(6, 0), (6, 9), (9, 0), (9, 6)])
+@pytest.mark.parametrize("k", [5, 6, 7])
+def test_fp64_origin_follows_the_depth(k, digits, quad):
+    """The FP64 form takes box centres with the 9-digit plane waves from depth 10 on, the cube centre elsewhere, bit for
+    bit."""
+    pos, f, a = _cluster_and_strays(3000, k)
+    kw = dict(leaf_cap=40, direct_w=-1, direct_x=-1, order_p=20, quad=quad)
+    u, t = matvec(pos, f, a, 6 * math.pi * a, digits, **kw)
+    depth = rp.rpy_tree_stats(t)["depth"]
+    assert depth == k + 4
+    flag = rp.RPY_FLAG_BOX_ORIGIN if (quad or digits) == 9 and depth >= 10 else rp.RPY_FLAG_CUBE_ORIGIN
+    assert np.array_equal(u, matvec(pos, f, a, 6 * math.pi * a, digits, flags=flag, **kw)[0])
+
+
 @pytest.mark.parametrize("digits,order", [(3, 8), (6, 16)])   # dense M2M / L2L below p = 12, rotations above
 def test_fp32_box_origin_rounding_against_fp64(digits, order):
     """The FP32 form's rounding (its difference from the FP64 path at the same tree and
