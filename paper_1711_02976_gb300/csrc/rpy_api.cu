@@ -195,6 +195,16 @@ static int host_tables(int p, int digits, OpTables **out) {
     return RPY_OK;
 }
 
+// Tables that only rpy_debug_table shows, kept from its first call for them.
+static int reference_table(const OpTables &h, int which, const std::vector<double> **out) {
+    static std::map<std::tuple<int, int, int>, std::vector<double>> tabs;   // (p, quadrature rule, which)
+    std::lock_guard<std::mutex> lk(g_mu);
+    std::vector<double> &v = tabs[std::make_tuple(h.p, h.digits, which)];
+    if (v.empty()) RPY_TRY(build_reference_table(h, which, v));
+    *out = &v;
+    return RPY_OK;
+}
+
 // Upload one table set in both precisions into a single device block.
 template <typename T>
 static void pack_tables(const OpTables &h, std::vector<char> &blob, std::vector<size_t> &offs) {
@@ -1122,10 +1132,6 @@ int rpy_debug_table(int p, int digits, int which, double *dst, int64_t capacity,
     std::vector<double> tmp;
     const std::vector<double> *v = nullptr;
     switch (which) {
-        case 1: v = &h->m2m_t; break;
-        case 2: v = &h->l2l_t; break;
-        case 3: v = &h->rot_fwd; break;
-        case 4: v = &h->rot_bwd; break;
         case 5: v = &h->m2x_c; break;
         case 6: v = &h->x2l_c; break;
         case 7:   // stored plane waves: k, cos, sin, w/M per entry
@@ -1152,17 +1158,8 @@ int rpy_debug_table(int p, int digits, int which, double *dst, int64_t capacity,
             }
             v = &tmp;
             break;
-        case 10:   // rotation block offsets
-            for (int o : h->rot_off) tmp.push_back(o);
-            v = &tmp;
-            break;
-        case 12: v = &h->orot_fwd; break;
-        case 13: v = &h->orot_bwd; break;
         case 14: v = &h->zm2m; break;
         case 15: v = &h->zl2l; break;
-        case 16: v = &h->shz; break;
-        case 17: v = &h->shx; break;
-        case 18: v = &h->shy; break;
         case 11:   // quadrature: s, then lambda, weight, M per node
         {
             const ExpQuad &q = exp_quadrature(digits);
@@ -1175,6 +1172,9 @@ int rpy_debug_table(int p, int digits, int which, double *dst, int64_t capacity,
             v = &tmp;
             break;
         }
+        case 1: case 2: case 3: case 4: case 10: case 12: case 13: case 16: case 17: case 18:
+            RPY_TRY(reference_table(*h, which, &v));
+            break;
         default: return RPY_ERR_INVALID;
     }
     if (count) *count = int64_t(v->size());

@@ -117,11 +117,6 @@ int default_leaf_cap(int digits);
 struct OpTables {
     int p = 0, nc = 0, digits = 0, s = 0, S = 0;   // S = stored plane waves (half of sum M_k)
     // host copies (double) ----------------------------------------------
-    std::vector<double> m2m_t;    // [8][D][D] transposed real M2M (D = 2 nc), column = output
-    std::vector<double> l2l_t;    // [8][D][D] transposed real L2L
-    std::vector<double> rot_fwd;  // [2 frames][sum_n (2n+1)^2] real blocks world -> frame (x, y)
-    std::vector<double> rot_bwd;  // [2 frames][...] frame -> world
-    std::vector<int> rot_off;     // [p+1] offset of degree-n block
     std::vector<double> m2x_c;    // [s][nc]  lambda_k^n / sqrt((n-m)!(n+m)!)
     std::vector<double> x2l_c;    // [s][nc]  (-lambda_k)^n / sqrt((n-m)!(n+m)!)
     std::vector<int> e_k;         // [S] node of stored plane wave e
@@ -133,10 +128,6 @@ struct OpTables {
     std::vector<int> u_k;         // [NU] node of unit u
     std::vector<int> u_start;     // [s+1] first unit of node k
     std::vector<double> shift;    // [216][S][2] e^{-lambda dz + i lambda (dx cos a + dy sin a)}
-    // the same shifts per axis: shift(off) = shz[iz] * shx[ix] * shy[iy] with
-    // off = ix + 6 iy + 36 iz (offset d = index - 2.5 along each axis)
-    std::vector<double> shz;      // [6][S] e^{-lambda dz}
-    std::vector<double> shx, shy; // [6][S][2] e^{i lambda dx cos a}, e^{i lambda dy sin a}
     // merge-and-shift groups per direction
     std::vector<int> grp_off;     // [6][G_MAX+1] start of group g in slot list (per direction)
     std::vector<int> grp_n;       // [6] number of groups
@@ -149,18 +140,20 @@ struct OpTables {
     // local:     lz = sqrt((k+1+m)(k+1-m)), lp = sqrt((k-m+1)(k-m+2)), lq = sqrt((k+m+1)(k+m+2))
     // multipole: mz = sqrt((k+m)(k-m)),     mp = sqrt((k+m)(k+m-1)),   mq = sqrt((k-m)(k-m-1))
     std::vector<double> lad;      // [6][ncoef(p+2)] in the order lz lp lq mz mp mq
-    // rotation-based M2M / L2L: per child octant, rotations world -> frame whose z axis is
-    // the shift direction and back, and the m-diagonal z-shift coefficients
-    std::vector<double> orot_fwd, orot_bwd;   // [8][rot_len]
-    // the same rotations factored through z-y-z Euler angles (layout in rpy_tables.cu)
+    // rotations factored through z-y-z Euler angles (layout in rpy_tables.cu): world -> frame (x, y) and back, and per
+    // child octant world -> frame whose z axis is the shift direction and back
     std::vector<double> frot_fwd, frot_bwd;   // [2 frames][frot_len]
     std::vector<double> forot_fwd, forot_bwd; // [8 octants][frot_len]
     std::vector<int> frot_off;                // [p+2] offset of degree n
-    std::vector<double> zm2m, zl2l;           // [ncoef(p)][p+1]: output (n,m), input degree k
+    std::vector<double> zm2m, zl2l;           // m-diagonal z shifts [ncoef(p)][p+1]: output (n,m), input degree k
 };
 constexpr int kGroupMax = 32;
 
 int build_tables(int p, int digits, OpTables &t);   // host computation, no CUDA
+// Other forms of the same operators, which no kernel reads and rpy_debug_table shows (which as there): the dense M2M
+// and L2L, the rotations as real blocks, the shifts per axis.  Formed with the tables of each setting, they took a
+// fifth of their time and at p = 26 73 MB.
+int build_reference_table(const OpTables &t, int which, std::vector<double> &v);
 // The y blocks of the factored rotations, indexed by output m and input k, stand as [k][m] on the device
 // from p = 12 and in double-floats: a warp's lanes take consecutive m, and at a row of 13 and
 // more values the [m][k] order costs a 128-byte line per lane (200k-bead tree at 9 digits: M2M 4.4 -> 1.9, L2L

@@ -206,10 +206,13 @@ static void transpose3(const double A[9], double B[9]) {
 }
 
 // Real per-degree blocks, layout [off_n + out*(2(n+1)) + in], 2-real local index 2m+part.
-static void build_rotations(int p, std::vector<double> &fwd, std::vector<double> &bwd, std::vector<int> &off) {
+static void rotation_offsets(int p, std::vector<int> &off) {
     off.resize(p + 2);
     off[0] = 0;
     for (int n = 0; n <= p; ++n) off[n + 1] = off[n] + 4 * (n + 1) * (n + 1);
+}
+static void build_rotations(int p, std::vector<double> &fwd, std::vector<double> &bwd, std::vector<int> &off) {
+    rotation_offsets(p, off);
     fwd.assign(size_t(2) * off[p + 1], 0.0);
     bwd.assign(size_t(2) * off[p + 1], 0.0);
     for (int f = 0; f < 2; ++f) {
@@ -511,9 +514,6 @@ int build_tables(int p, int qd, OpTables &t) {
     t.digits = qd;
     t.s = q.s;
     t.S = q.half();
-    build_m2m(p, t.m2m_t);
-    build_l2l(p, t.l2l_t);
-    build_rotations(p, t.rot_fwd, t.rot_bwd, t.rot_off);
     t.m2x_c.assign(size_t(q.s) * t.nc, 0.0);
     t.x2l_c.assign(size_t(q.s) * t.nc, 0.0);
     for (int k = 0; k < q.s; ++k)
@@ -555,18 +555,6 @@ int build_tables(int p, int qd, OpTables &t) {
             t.shift[(size_t(off) * t.S + e) * 2 + 1] = mag * std::sin(ph);
         }
     }
-    t.shz.assign(size_t(6) * t.S, 0.0);
-    t.shx.assign(size_t(6) * t.S * 2, 0.0);
-    t.shy.assign(size_t(6) * t.S * 2, 0.0);
-    for (int i = 0; i < 6; ++i)
-        for (int e = 0; e < t.S; ++e) {
-            const double lam = q.lambda[t.e_k[e]], d = i - 2.5;
-            t.shz[size_t(i) * t.S + e] = std::exp(-lam * d);
-            t.shx[(size_t(i) * t.S + e) * 2] = std::cos(lam * d * t.e_cos[e]);
-            t.shx[(size_t(i) * t.S + e) * 2 + 1] = std::sin(lam * d * t.e_cos[e]);
-            t.shy[(size_t(i) * t.S + e) * 2] = std::cos(lam * d * t.e_sin[e]);
-            t.shy[(size_t(i) * t.S + e) * 2 + 1] = std::sin(lam * d * t.e_sin[e]);
-        }
     build_groups(t);
     // factorized rotations: frames (x, y) and the eight child octants, forward and back
     {
@@ -595,16 +583,8 @@ int build_tables(int p, int qd, OpTables &t) {
                 return RPY_ERR_INTERNAL;
         }
     }
-    // rotation-based M2M / L2L
+    // z shifts of M2M / L2L
     {
-        int L = t.rot_off.back();
-        t.orot_fwd.assign(size_t(8) * L, 0.0);
-        t.orot_bwd.assign(size_t(8) * L, 0.0);
-        for (int o = 0; o < 8; ++o) {
-            double Q[9];
-            octant_frame(o, Q);
-            rotation_blocks(Q, p, t.rot_off, &t.orot_fwd[size_t(o) * L], &t.orot_bwd[size_t(o) * L]);
-        }
         // along the frame z axis the shift is delta = sqrt(3)/4 parent sides:
         // M2M  M^p_n^m = sum_{k=m..n} (N_n^m / N_k^m) delta^{n-k} / (n-k)! 2^{-k} M^c_k^m
         // L2L  L^c_k^m = sum_{n=k..p} (N_n^m / N_k^m) delta^{n-k} / (n-k)! 2^{-k-1} L^p_n^m
@@ -649,6 +629,51 @@ int build_tables(int p, int qd, OpTables &t) {
             t.lad[5 * nl + i] = sq(long(k - m) * (k - m - 1));
         }
     return RPY_OK;
+}
+
+int build_reference_table(const OpTables &t, int which, std::vector<double> &v) {
+    const int p = t.p;
+    std::vector<double> other;
+    std::vector<int> off;
+    switch (which) {
+        case 1: build_m2m(p, v); return RPY_OK;
+        case 2: build_l2l(p, v); return RPY_OK;
+        case 3: build_rotations(p, v, other, off); return RPY_OK;
+        case 4: build_rotations(p, other, v, off); return RPY_OK;
+        case 10:
+            rotation_offsets(p, off);
+            v.assign(off.begin(), off.end());
+            return RPY_OK;
+        case 12:
+        case 13: {
+            rotation_offsets(p, off);
+            const size_t L = off.back();
+            v.assign(8 * L, 0.0);
+            other.assign(L, 0.0);
+            for (int o = 0; o < 8; ++o) {
+                double Q[9];
+                octant_frame(o, Q);
+                double *mine = &v[o * L], *rest = other.data();
+                rotation_blocks(Q, p, off, which == 12 ? mine : rest, which == 12 ? rest : mine);
+            }
+            return RPY_OK;
+        }
+        case 16:
+        case 17:
+        case 18: {   // shift(off) = shz[iz] shx[ix] shy[iy], off = ix + 6 iy + 36 iz, offset d = index - 2.5 per axis
+            const ExpQuad &q = exp_quadrature(t.digits);
+            v.clear();
+            for (int i = 0; i < 6; ++i)
+                for (int e = 0; e < t.S; ++e) {
+                    const double lam = q.lambda[t.e_k[e]], d = i - 2.5;
+                    const double ph = lam * d * (which == 17 ? t.e_cos[e] : t.e_sin[e]);
+                    if (which == 16) v.push_back(std::exp(-lam * d));
+                    else v.insert(v.end(), {std::cos(ph), std::sin(ph)});
+                }
+            return RPY_OK;
+        }
+        default: return RPY_ERR_INVALID;
+    }
 }
 
 }  // namespace rpy
