@@ -18,9 +18,7 @@
 //         charge sets accumulated into them (2 FMA per set and coefficient).
 //   M2M, L2L   per child box: the per-octant translation of the four sets, as
 //         the path computes it (rotation to the shift axis, m-diagonal z-shift,
-//         rotation back; or, for the FP32 form below p = 12, the dense operator
-//         restricted to its triangle); bytes: each expansion read and written
-//         once per level pass.
+//         rotation back); bytes: each expansion read and written once per level pass.
 //   M2X   per box: three frames x four sets x [A_k^m = sum_n c M (2 FMA per
 //         coefficient and node) + the waves of a node from A (2 FMA per wave,
 //         m and set, the two waves of angles a and pi - a sharing their
@@ -30,11 +28,11 @@
 //         read once, Xi written once.
 //   X2L   per box: the transpose of M2X; bytes: Xi read, L read and written.
 //   EVAL  per bead of a leaf at level >= 2: harmonics of degree p and six
-//         fields (2 FMA per coefficient each); per leaf the derived
-//         expansions (18 x nc complex multiply-adds); per (bead, W-list box):
-//         harmonics of degree p + 2 and 18 fields; bytes: L read, the derived
-//         expansions written and read once per leaf, positions read and
-//         velocities written.
+//         fields (2 FMA per coefficient each); per leaf and coefficient the
+//         two scalars from six derivatives (72 FLOP) and the six fields from
+//         nine (84); per (bead, W-list box): harmonics of degree p + 2 and six
+//         fields; bytes: L read, the six fields written and read once per
+//         leaf, positions read and velocities written.
 // Polynomial far field (RPY_FLAG_CARTESIAN, N monomials of degree <= P): P2M per
 // bead 2 multiplies and 4 FMA per monomial; M2M and L2L per child box and M2L per
 // V-list pair one FMA per set and operator term (the pair counts of the tables);
@@ -64,18 +62,6 @@ double zshift_fma(int p, bool up) {
     double f = 0;
     for (int n = 0; n <= p; ++n)
         for (int m = 0; m <= n; ++m) f += 2.0 * (up ? n - m + 1 : p - n + 1);
-    return f;
-}
-
-// FMAs of the dense per-octant operator of one set (real layout, triangle only).
-double dense_fma(int p, bool up) {
-    const int nc = ncoef(p), D = 2 * nc;
-    double f = 0;
-    for (int r = 0; r < D; ++r) {
-        int n = 0;
-        while (tri(n + 1, 0) <= (r >> 1)) ++n;
-        f += up ? 2.0 * ncoef(n) : double(D - 2 * tri(n, 0));
-    }
     return f;
 }
 
@@ -186,9 +172,8 @@ extern "C" int rpy_tree_work(rpy_tree h, double *flops, double *bytes, int n) {
         B[RPY_STAGE_P2L] = xpairs * 48 + 2 * xbox * 4 * nc * ce;
         // M2M / L2L: child boxes at level >= 3
         const double nch = t.nlevels > 3 ? double(nb - t.level_off[3]) : 0.0;
-        const bool rot = !f32 || p >= 12;
-        const double m2m = rot ? 2 * rot_fma(p, false) + zshift_fma(p, true) : dense_fma(p, true);
-        const double l2l = rot ? 2 * rot_fma(p, false) + zshift_fma(p, false) : dense_fma(p, false);
+        const double m2m = 2 * rot_fma(p, false) + zshift_fma(p, true);
+        const double l2l = 2 * rot_fma(p, false) + zshift_fma(p, false);
         F[RPY_STAGE_M2M] = nch * 4 * 2 * m2m;
         F[RPY_STAGE_L2L] = nch * 4 * 2 * l2l;
         double npar = 0;
@@ -217,7 +202,7 @@ extern "C" int rpy_tree_work(rpy_tree h, double *flops, double *bytes, int n) {
         F[RPY_STAGE_X2X] = units * 4 * S * 4 * 2.0;
         B[RPY_STAGE_X2X] = 2 * n2 * 6.0 * 4 * S * ce;
         // L2P with Eq. (2.8) at the beads, the derived expansions per leaf, M2P of large W boxes
-        F[RPY_STAGE_EVAL] = bead2 * (harm + 6 * 2 * 2.0 * nc) + leaf2 * 18 * nc * 8.0 +
+        F[RPY_STAGE_EVAL] = bead2 * (harm + 6 * 2 * 2.0 * nc) + leaf2 * nc * (72.0 + 84.0) +
                             wpairs * (harm2 + 6 * 2 * 2.0 * nc2);
         B[RPY_STAGE_EVAL] = leaf2 * (4 * nc + 2 * 6 * nc) * ce + bead2 * 48;
     }

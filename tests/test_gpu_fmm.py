@@ -1186,3 +1186,20 @@ def test_tree_work_counts_match_the_tree():
     assert terms == math.comb(P + 6, 6)
     assert w["x2l"][0] == st["n_vpairs"] * terms * 4 * 2
     assert w["m2x"] == (0.0, 0.0) and w["x2x"] == (0.0, 0.0) and w["p2l"] == (0.0, 0.0)
+
+
+@pytest.mark.parametrize("order", [6, 8, 12])
+def test_tree_work_counts_the_present_operators(order):
+    """M2M and L2L rotate in both precision forms at every order, so both count the same operations; L2P counts 34 FLOP
+    per bead and coefficient and 156 per leaf and coefficient for its six fields."""
+    sysm = synth.config1()
+    w = []
+    for prec in (rp.RPY_FP64, rp.RPY_FP32):
+        u, t = matvec(sysm.pos, sysm.f, sysm.a, sysm.s, 3, leaf_cap=40, precision=prec, order_p=order)
+        st = rp.rpy_tree_stats(t)
+        w.append(rp.rpy_tree_work(t))
+    assert st["n_wlist"] == st["n_dlist"] == 0 and st["depth"] == 3
+    nc = (order + 1) * (order + 2) // 2
+    for k in ("m2m", "l2l", "m2x", "x2x", "x2l", "p2m", "eval"):
+        assert w[0][k][0] == w[1][k][0] > 0, k
+    assert w[0]["eval"][0] == sysm.n * 34 * nc + st["n_leaves"] * 156 * nc
