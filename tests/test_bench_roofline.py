@@ -33,3 +33,10 @@ def test_roofline_hbm_bound_and_fp32_peak():
     assert math.isclose(r["frac"], 20e9 / 0.004 / 1e9 / hbm, rel_tol=1e-3)
     assert r["traffic"] is None   # no capture figure for this kernel
     assert math.isclose(r["stages"]["p2p"]["frac_alu"], 5e9 / 0.001 / 73.0e12, rel_tol=1e-3)
+
+
+def test_double_float_work_counts_fp32_operations():
+    """200 FP32 operations a pair and 12 a multiply-add, at 2 FLOP each; bytes as they are."""
+    w = bench.double_float_work({"p2p": (38.0 * 1e6, 7.0), "x2l": (2.0 * 1e6, 5.0), "gather": (0.0, 3.0)})
+    assert math.isclose(w["p2p"][0], 200e6 * 2) and math.isclose(w["x2l"][0], 12e6 * 2)
+    assert (w["p2p"][1], w["x2l"][1], w["gather"]) == (7.0, 5.0, (0.0, 3.0))
