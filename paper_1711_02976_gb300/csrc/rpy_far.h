@@ -34,6 +34,17 @@ inline int even_threads(int items, int most = 256) {
     return std::max(64, ((items + rounds - 1) / rounds + 31) / 32 * 32);
 }
 
+// Two charge sets of one value in a packed operand (V), and in memory.
+template <typename T> struct PairOf;
+template <> struct PairOf<float> {
+    using V = float2;
+    using Mem = float2;
+};
+template <> struct PairOf<dfl> {
+    using V = df2;
+    using Mem = float4;
+};
+
 // M2X, X2X and X2L of one matvec: M -> L (added), through t.Xo and t.Xi
 template <typename T>
 int run_waves_t(Tree &t, const DevTables<T> &D, const cpx<T> *M, cpx<T> *L, int rb, cudaStream_t st);

@@ -354,10 +354,6 @@ __host__ __device__ inline int tab_floats(int p) {   // recurrences + ladders, r
 
 // ---------------------------------------------------------------- P2M / P2L
 
-// Two charge sets of one value in a packed operand: float2 in FP32, df2 in double-floats.
-template <typename T> struct Pair;
-template <> struct Pair<float> { using V = float2; };
-template <> struct Pair<dfl> { using V = df2; };
 __device__ __forceinline__ float2 pair2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ df2 pair2(dfl a, dfl b) { return df2{make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
 __device__ __forceinline__ float first(float2 v) { return v.x; }
@@ -376,13 +372,13 @@ __device__ __forceinline__ void add_comp(float2 &s, float2 &c, float2 v) {   // 
 // compensation of each (double-floats are only normalised).
 template <typename T>
 struct Sum4 {
-    typename Pair<T>::V v[4], c[sizeof(T) == 4 ? 4 : 1];
+    typename PairOf<T>::V v[4], c[sizeof(T) == 4 ? 4 : 1];
     __device__ void clear() {
         const auto z = pair2(T(0), T(0));
         for (auto &x : v) x = z;
         for (auto &x : c) x = z;
     }
-    __device__ void add(const typename Pair<T>::V *u) {
+    __device__ void add(const typename PairOf<T>::V *u) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             if constexpr (sizeof(T) == 4) add_comp(v[k], c[k], u[k]);
@@ -433,11 +429,11 @@ __host__ __device__ inline int p2x_buf(int p, int threads) {   // harmonics of a
 // centre when rb is set (box origin), else at the system's cube centre.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(512) k_p2x(int b0, int nb, DevTables<T> D, const int *beg, const int *end,
-                                             const double *ctr, const double *side, const int *lvl, const int *leaf,
+                                             const double *ctr, const int *lvl, const int *leaf,
                                              const int *bsys, const int *xoff, const int *xidx, const double *pos,
                                              const double *fs, const double *lapq, int64_t n, SysConst sc, cpx<T> *out,
                                              int rb) {
-    using V = typename Pair<T>::V;
+    using V = typename PairOf<T>::V;
     const int chunk = p2x_chunk<T>(D.p, blockDim.x);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int b = b0 + blockIdx.x;
@@ -891,7 +887,7 @@ __global__ void k_eval_prep(const int *leaves, DevTables<T> D, const double *ctr
 // mixed at 9 digits 1.83 -> 0.98 ms; 4,096 beads FP64 51 -> 40 us.
 template <typename T, int NF>
 __global__ void __launch_bounds__(128, 6) k_eval_apply(int64_t n, const int *bead_leaf, const int *leaves,
-                                                       DevTables<T> D, const double *ctr, const double *side,
+                                                       DevTables<T> D, const double *ctr,
                                                        const int *lvl, const int *bsys, const double *pos, SysConst sc,
                                                        const cpx<T> *EVg, double *ufar) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1091,14 +1087,12 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
                         : (fl & RPY_FLAG_CUBE_ORIGIN) ? 0
                         : kIsDf<T> ? t.params.quad == 9 && t.nlevels - 1 >= kBoxOriginDepth
                                    : t.params.digits >= 6;
-    // box sides in the units of the expansions' lengths
-    const double *side = kIsDf<T> ? t.side_u : t.b_side;
     // upward pass
     const int tp = p2x_threads(p, n2);
     const size_t sp = smem_p2x<T>(p, tp);
     RPY_TRY(set_smem(k_p2x<T, 0>, sp));
     RPY_TRY(set_smem(k_p2x<T, 1>, sp));
-    k_p2x<T, 0><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
+    k_p2x<T, 0><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, t.b_level, t.b_leaf,
                                      t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, M, rb);
     RPY_LAUNCHED(1);
     RPY_CHECK(cudaGetLastError());
@@ -1114,7 +1108,7 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
     // without X lists (a uniform system, or all of its X boxes summed directly) there is nothing to launch: matvec of
     // 4,096 beads 225.2 -> 223.9 us, 12 Lanczos steps of 50,000 6.99 -> 6.95 ms
     if (t.n_x > 0) {
-        k_p2x<T, 1><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, side, t.b_level, t.b_leaf,
+        k_p2x<T, 1><<<n2, tp, sp, st>>>(b2, n2, D, t.b_begin, t.b_end, t.b_center, t.b_level, t.b_leaf,
                                          t.b_sys, t.x_off, t.x_idx, t.pos, fs, lapq, t.n, sc, L, rb);
         RPY_LAUNCHED(1);
         RPY_CHECK(cudaGetLastError());
@@ -1134,10 +1128,10 @@ int run_far_t(Tree &t, const DevTables<T> &D, const double *fs, const double *la
         RPY_LAUNCHED(1);
         const int ga = int((t.n + 127) / 128);
         if (per_comp)
-            k_eval_apply<T, kNF2><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, side, t.b_level,
+            k_eval_apply<T, kNF2><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, t.b_level,
                                                       t.b_sys, t.pos, sc, EVg, ufar);
         else
-            k_eval_apply<T, kNF><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, side, t.b_level,
+            k_eval_apply<T, kNF><<<ga, 128, 0, st>>>(t.n, t.bead_leaf, t.leaves, D, t.b_center, t.b_level,
                                                      t.b_sys, t.pos, sc, EVg, ufar);
         RPY_LAUNCHED(1);
         if (t.n_w > 0) {

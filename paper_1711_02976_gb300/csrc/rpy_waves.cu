@@ -283,16 +283,7 @@ __device__ __forceinline__ int x2x_sources(X2XList &W, const DevTables<T> &D, in
     return nz;
 }
 
-// A pair of sets in one thread: PairOf<float> = float2, PairOf<dfl> = df2.
-template <typename T> struct PairOf;
-template <> struct PairOf<float> {
-    using V = float2;
-    using Mem = float2;
-};
-template <> struct PairOf<dfl> {
-    using V = df2;
-    using Mem = float4;
-};
+// A pair of sets in one thread (PairOf).
 __device__ __forceinline__ float2 get_pair(float2 m) { return m; }
 __device__ __forceinline__ df2 get_pair(float4 m) { return as_df2(m); }
 __device__ __forceinline__ float2 put_pair(float2 v) { return v; }
