@@ -62,7 +62,7 @@ typedef enum {
 typedef enum {
     RPY_FP64 = 0,            /* FP64 accuracy: tree, bounding cube and per-bead sums in FP64; pairs
                                 and expansions in double-floats (two FP32 numbers, about 48 bits),
-                                or all FP64 where their range does not reach */
+                                the near field in FP64 where their range does not reach */
     RPY_FP32 = 1             /* precision form: near field and translations in FP32 with
                                 compensated accumulation; bounding cube, Morton keys,
                                 r ~ 0 overlap pairs and the final per-bead sum in FP64 */

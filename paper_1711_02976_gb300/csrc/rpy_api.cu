@@ -1010,7 +1010,7 @@ int rpy_tree_footprint(int64_t n, int digits, int precision, int leaf_cap, int64
     // boxes: leaves ~ 2n/cap on clustered data, plus internal boxes (< leaves/7 * 8)
     double nbox = 4.0 * double(n) / double(leaf_cap) + 64.0;
     const int xf = plane_wave_frames(nbox, es, q.half());
-    // M, L, plane waves and L2P scratch
+    // M, L, plane waves and L2P scratch (18 fields, of RPY_FLAG_EVAL_PER_POTENTIAL, which this call is not told of)
     double per_box = es * (2.0 * kSets * ncoef(p) + 2.0 * 2 * xf * kSets * q.half() + 18.0 * ncoef(p)) +
                      4.0 * (8 + 27 + 3 + 12) + 32.0 + (precision == RPY_FP32 ? 0.0 : 9 * 4.0 + 8.0 /*c3, side_u*/);
     double per_bead = 3 * 8 /*pos*/ + 8 /*key*/ + 4 + 4 + 9 * 8 /*fs, unear, ufar*/ + 27 * 4 /*U list share*/ +

@@ -7,7 +7,8 @@
 // forms; the scaling is this library's choice).
 //
 // Tables:
-//   M2M / L2L   dense real matrices per child octant, built from the
+//   M2M / L2L   rotations to the shift axis and z shifts; for the host tests also
+//               dense real matrices per child octant, built from the
 //               addition theorem of regular solid harmonics
 //               R_n^m(u + v) = sum_{k,l} R_k^l(u) R_{n-k}^{m-l}(v),
 //               R_n^m = r^n P_n^m e^{i m phi} / (n+m)!, which in the paper's
@@ -335,7 +336,7 @@ static void rot_y(double b, double R[9]) {
 int factor_len(int n) { return 4 * (n + 1) + 2 * (n + 1) * (n + 1); }
 
 // Fills `out` (layout above) for the rotation X; false if a factor does not have the
-// expected structure (then the dense blocks must be used).  With `quarter` (the
+// expected structure.  With `quarter` (the
 // frame rotations, whose middle angle is pi/2) the y blocks must also have the
 // checkerboard structure the kernels rely on: Yre[mo][mi] = 0 unless mo + mi + n
 // is even, Yim[mo][mi] = 0 unless mo + mi + n is odd (rows and columns m >= 1;
